@@ -1,26 +1,48 @@
 // rlm_simt.cu -- chunked complex-diagonal scan on the CUDA cores (fp32).
 //
-// Runs the fp32-I/O prefill, every shape the tensor-core path does not cover,
-// and the backward pass.  Three phases, each one launch:
+// Runs what the tensor-core paths do not cover: the fp32-I/O prefill with more
+// than 16 modes, an initial state with a length that is not a multiple of 64, the
+// scratch-array prefill, and the backward pass for fp32 I/O and M > 32.  All
+// arithmetic is fp32.
 //
-//  1. chunk-local states: per (b, chunk k, d) and mode m, the state the chunk's
-//     own drives leave at its last token when it starts from zero
-//     (sum_j lambda^(C-1-j) x_j, the chunk form of the terminal state of
-//     Sec. 3.2);
-//  2. inter-chunk carry: per (b, d, m), a sequential scan over chunks,
-//     S_k = lambda^C S_{k-1} + local_k, written back exclusive (the state each
-//     chunk starts from) -- the final S is the prompt's terminal state;
-//  3. chunk output: per (b, k, d), the recurrence of Eq. 4 restarted from the
-//     carried state, with the readout y_t = sum_m Re(c s_t).
+// Chunked form, C = 64 tokens, chunks from token 0 (the last may be partial and is
+// padded with zero drives).  With S_k the state entering chunk k and W_k = c lambda S_k:
 //
-// Chunks are aligned to END at the last token: the first chunk may start at a
-// negative time, whose drives count as zero.  With a zero initial state that
-// leaves every state unchanged, so the carry needs no special last chunk.
+//   L_k       = sum_p lambda^(63-p) x_{k,p}                     chunk-local end state
+//   S_{k+1}   = lambda^64 S_k + L_k                             carry
+//   y_{k,p}   = sum_{p'<=p} K[p-p'] x_{k,p'} + sum_m Re(lambda^p W_k)
 //
-// The backward pass runs the same phases in reverse time on dy (the adjoint of
-// a causal convolution is the anti-causal one) and carries the Jordan partner
-// R of the adjoint state as well, to form G = sum x S and P = sum x R.
+// The backward is the same scan of dy in reverse time: processing time
+// tau = 64 nch - 1 - t puts the padding first, and position p of a chunk is then
+// 63 minus its position in time, so L_k is the adjoint's Dp, the output formula gives
+// dx, and only the Jordan partner (weights 63 - p), the x-side projections and the
+// lag correlation are added:
+//
+//   Dq_k = sum_p (63-p) lambda^(63-p) dy_p,   R_{k+1} = lambda^64 (R_k + 64 S_k) + Dq_k
+//   Xp_k = sum_p lambda^p x_p,                Xq_k = sum_p (p+1) lambda^p x_p
+//   G += lambda Xp_k S_k,                     P += lambda (Xp_k R_k + Xq_k S_k)
+//   rho[n] = sum_k sum_u dy_u x_{u+n},        G += sum_n lambda^n rho[n], P += sum_n n lambda^n rho[n]
+//
+// Every sum over positions or modes is a small matrix product, which costs 2 FMA per
+// token and mode (4 with the Jordan partner) where the token-by-token recurrence
+// costs 4 (8) plus 2 for the readout: at M = 32 about 170 FMA per token-channel
+// forward and 410 backward, against 320 and 830.  They are bound by the FMA pipe.
+//
+// One warp owns one channel and a tile of 16 chunks (1024 tokens); its products are
+// register tiles (lane = 8 row groups x 4 column groups, columns = chunks) over
+// tables and drives in shared memory, issued as packed two-lane FMAs
+// (fma.rn.f32x2: 63 against 52 TFLOP/s with three distinct register operands at the
+// two warps a scheduler has here, and half the issue slots).  A block is 4 channels
+// (a 16-byte fp32 slice of each token row) and walks the tiles of a segment of the
+// sequence with the state in registers, so that chunk states never touch memory.  Few
+// (batch row, channel group) pairs are split into segments of whole tiles: a first
+// launch forms each segment's end state from zero, and the second enters segment s
+// with the combination of the states before it.
+//
+// Same box, before (three launches of token-by-token recurrences, chunk states in
+// memory) and now, us per call: see the launch rule at geometry().
 #include <algorithm>
+#include <type_traits>
 
 #include "rlm_device.cuh"
 #include "rlm_internal.h"
@@ -28,335 +50,710 @@
 namespace rlm {
 namespace {
 
-constexpr int kMgFwd = 16;  // modes per thread, forward phases
-constexpr int kMgBwd = 8;   // modes per thread, backward output phase
-constexpr int kBlock = 128;
-constexpr int kTokBlock = 8;   // drives loaded ahead per thread in the per-token loops
-constexpr int kCarryBlock = 64; // threads per block of the carry (one per (b, d, m): spread over all SMs)
+typedef unsigned long long u64;
 
-int threads_per_channel(int M, int mg) {
-    int t = (M + mg - 1) / mg;
-    int p = 1;
-    while (p < t) p <<= 1;
-    return p;
+constexpr int kC = 64;               // chunk length
+constexpr int kCols = 16;            // chunks per tile
+constexpr int kTile = kC * kCols;    // 1024 tokens
+constexpr int kCh = 4;               // channels (warps) per block
+constexpr int kThreads = 32 * kCh;
+constexpr int kPwStride = 66;        // float2 per mode row of the power table: 16-byte aligned, rows 4 banks apart
+constexpr int kFieldWords = kC * kCols;   // one channel's tile: [p / 2][column][p % 2]
+constexpr int kKernWords = 2 * kC;        // K reversed, and the same shifted by one
+
+// Shared memory of a block, in floats: per channel the power table
+// [modes][66] (complex), the reversed lag kernel, the drive tile and (backward) the
+// x tile.
+constexpr int chan_words(int modes, bool bwd) {
+    return 2 * modes * kPwStride + kKernWords + (bwd ? 2 : 1) * kFieldWords;
+}
+constexpr int smem_bytes(int modes, bool bwd) { return kCh * chan_words(modes, bwd) * 4; }
+
+__device__ __forceinline__ u64 pack2(float a, float b) {
+    u64 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ u64 dup2(float a) { return pack2(a, a); }
+__device__ __forceinline__ float2 unpack2(u64 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ void fma2(u64 &d, u64 a, u64 b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
+    u64 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float2 shfl2(float2 v, int src) {
+    return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
 
-struct ChunkGeom {
-    int C;        // chunk length
-    int nch;      // number of chunks
-    int64_t t0;   // processing time of chunk 0's first token (<= 0)
+struct ScanArgs {
+    const void *u;            // the scanned drive: x (forward), dy (backward)
+    const void *x;            // backward: x
+    void *out;                // y, or dx
+    int bf16;                 // element type of the fields (0: fp32)
+    int rev;                  // reverse time (backward)
+    int64_t L;
+    int D, M;
+    int nch, ntiles;          // chunks and tiles of the sequence
+    int nseg, tps;            // segments, tiles per segment
+    const float *decay, *freq, *amp, *phase;
+    float2 *seg_s, *seg_r;    // [nseg][B][D][M] segment end states (pair) from zero
+    const float2 *enter;      // nullable (forward): the state before token 0, as segment 0 reads it
+    const float2 *state_in;   // nullable (backward)
+    float2 *state_out;        // nullable (forward)
+    float4 *coef_out;         // nullable (forward)
+    float2 *part_g, *part_p;  // backward: [B][nseg][D][M]
+    float2 *part_j;           // with g
+    const float2 *g;          // nullable: gradient of the terminal state
+    float2 *d_state_in;       // nullable
 };
 
-ChunkGeom geom_c(int64_t L, int C) {
-    ChunkGeom g;
-    g.C = C;
-    g.nch = (int)((L + g.C - 1) / g.C);
-    g.t0 = L - (int64_t)g.nch * g.C;
-    return g;
-}
-
-// The backward pass does ~26 M flop per token-channel in its two per-token
-// phases, so it needs far fewer (b, chunk, channel) tuples than the forward to
-// fill the GPU; longer chunks keep its workspace (16 bytes per (b, chunk, d, m))
-// small enough to stay in L2 and shorten the sequential carry and the reduction.
-int bwd_chunk_len(int64_t B, int64_t L, int D) {
-    const int64_t target = (int64_t)sm_count() * 512;
-    const int64_t per_chunk = std::max<int64_t>(1, B * (int64_t)D);
-    int64_t nch = std::max<int64_t>(1, (target + per_chunk - 1) / per_chunk);
-    int64_t C = (L + nch - 1) / nch;
-    C = std::max<int64_t>(16, std::min<int64_t>(4096, C));
-    return (int)C;
-}
-
-ChunkGeom geom(int64_t B, int64_t L, int D) {
-    ChunkGeom g;
-    g.C = simt_chunk_len(B, L, D);
-    g.nch = (int)((L + g.C - 1) / g.C);
-    g.t0 = L - (int64_t)g.nch * g.C;
-    return g;
-}
-
-// Phase 1.  Grid (ceil(D*TPC/kBlock), nch, B).
-template <typename T, int MG, bool REV, bool JORDAN>
-__global__ void __launch_bounds__(kBlock) k_chunk_local(
-    const T *__restrict__ x, int64_t L, int D, int M, int tpc, int C, int nch, int64_t t0,
-    const float *__restrict__ decay, const float *__restrict__ freq, float2 *__restrict__ ws_s,
-    float2 *__restrict__ ws_r) {
-    const int gx = blockIdx.x * blockDim.x + threadIdx.x;
-    const int d = gx / tpc, grp = gx % tpc;
-    const int k = blockIdx.y, b = blockIdx.z;
-    if (d >= D) return;
-    float2 lam[MG], s[MG], r[MG];
-#pragma unroll
-    for (int j = 0; j < MG; ++j) {
-        const int m = grp * MG + j;
-        lam[j] = m < M ? lambda_pow(decay[d * M + m], freq[d * M + m], 1.0f) : make_float2(0, 0);
-        s[j] = make_float2(0, 0);
-        r[j] = make_float2(0, 0);
+// The 4 channels d .. d + 3 of token t.
+__device__ __forceinline__ float4 load4(const void *f, int bf16, int64_t e) {
+    if (bf16) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(static_cast<const __nv_bfloat16 *>(f) + e));
+        return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u),
+                           __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
     }
-    const int64_t tau0 = t0 + (int64_t)k * C;
-    const int i0 = tau0 < 0 ? (int)(-tau0) : 0;
-    // kTokBlock tokens' drives are loaded before their updates run.
-    for (int i = i0; i < C; i += kTokBlock) {
-        float xs[kTokBlock];
-#pragma unroll
-        for (int u = 0; u < kTokBlock; ++u) {
-            const int64_t tau = tau0 + i + u;
-            const int64_t t = REV ? (L - 1 - tau) : tau;
-            xs[u] = i + u < C ? ld_elem(x + ((int64_t)b * L + t) * D + d) : 0.0f;
-        }
-#pragma unroll
-        for (int u = 0; u < kTokBlock; ++u) {
-            if (i + u >= C) break;
-#pragma unroll
-            for (int j = 0; j < MG; ++j) {
-                if (JORDAN) r[j] = cmul(lam[j], make_float2(r[j].x + s[j].x, r[j].y + s[j].y));
-                s[j] = cfma(lam[j], s[j], make_float2(xs[u], 0.0f));
-            }
-        }
-    }
-    const int64_t base = (((int64_t)b * nch + k) * D + d) * M;
-#pragma unroll
-    for (int j = 0; j < MG; ++j) {
-        const int m = grp * MG + j;
-        if (m < M) {
-            ws_s[base + m] = s[j];
-            if (JORDAN) ws_r[base + m] = r[j];
-        }
+    return __ldg(reinterpret_cast<const float4 *>(static_cast<const float *>(f) + e));
+}
+__device__ __forceinline__ void store4(void *f, int bf16, int64_t e, float4 v) {
+    if (bf16) {
+        __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+        *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(f) + e) =
+            make_uint2(*reinterpret_cast<uint32_t *>(&a), *reinterpret_cast<uint32_t *>(&b));
+    } else {
+        *reinterpret_cast<float4 *>(static_cast<float *>(f) + e) = v;
     }
 }
 
-// Phase 2.  One thread per (b, d, m); grid over B*D*M.
-// With state_in (forward only): chunk 0 is entered with the state before token 0
-// (the output phase restarts its recurrence there, at time 0), and that state
-// reaches the end of chunk 0 after C + t0 tokens.
-template <bool JORDAN>
-__global__ void __launch_bounds__(kCarryBlock) k_chunk_carry(
-    int64_t B, int D, int M, int C, int nch, int64_t t0, const float *__restrict__ decay,
-    const float *__restrict__ freq, const float *__restrict__ amp, const float *__restrict__ phase,
-    float2 *__restrict__ ws_s, float2 *__restrict__ ws_r, const float2 *__restrict__ state_in,
-    float2 *__restrict__ state_out, float4 *__restrict__ coef_out) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= B * D * M) return;
-    const int m = (int)(idx % M);
-    const int d = (int)((idx / M) % D);
-    const int64_t b = idx / ((int64_t)M * D);
-    const int pm = d * M + m;
-    const float2 LC = lambda_pow(decay[pm], freq[pm], (float)C);
-    const float Cf = (float)C;
-    float2 S = state_in ? state_in[idx] : make_float2(0, 0), R = make_float2(0, 0);
-    const float2 L0 = state_in ? lambda_pow(decay[pm], freq[pm], (float)(C + t0)) : LC;
-    // The chunks' partials are read kCarryBatch at a time before the recurrence
-    // runs over them (each slot is then overwritten with the state entering its
-    // chunk), so a thread waits on memory once per batch, not once per chunk.
-    constexpr int kCB = JORDAN ? 16 : 32;
-    const int64_t stride = (int64_t)D * M;
-    const int64_t off0 = (b * nch * D + d) * M + m;   // chunk 0; chunk k at off0 + k * stride
-    for (int k0 = 0; k0 < nch; k0 += kCB) {
-        float2 lsv[kCB], lrv[JORDAN ? kCB : 1];
+// Projection of the drive tile on the power table: for the lane's modes g + 8 j and
+// columns 4 cg + c, acc = sum_p lambda^e(p) x_p and (JORDAN) accq = sum_p w(p) lambda^e(p) x_p,
+// with e = 63 - p, w = 63 - p (TO_END) or e = p, w = p + 1.  pw points at the row of
+// mode g, xs at the tile's column 4 cg.  Per pair of positions: J + 2 16-byte shared
+// loads, the drives duplicated into both halves, 8 J (16 J) packed FMAs on (Re, Im).
+template <int J, bool JORDAN, bool TO_END>
+__device__ __forceinline__ void project(const float2 *pw, const float *xs, u64 (&acc)[J][4],
+                                        u64 (&accq)[JORDAN ? J : 1][4]) {
 #pragma unroll
-        for (int j = 0; j < kCB; ++j) {
-            if (k0 + j < nch) {
-                lsv[j] = ws_s[off0 + (k0 + j) * stride];
-                if (JORDAN) lrv[j] = ws_r[off0 + (k0 + j) * stride];
-            }
+    for (int j = 0; j < J; ++j)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            acc[j][c] = 0ull;
+            if (JORDAN) accq[j][c] = 0ull;
         }
+#pragma unroll 2
+    for (int pp = 0; pp < kC / 2; ++pp) {
+        const float4 xa = *reinterpret_cast<const float4 *>(xs + pp * 2 * kCols);
+        const float4 xb = *reinterpret_cast<const float4 *>(xs + pp * 2 * kCols + 4);
+        ulonglong2 a[J];
+        const int n = TO_END ? kC - 2 - 2 * pp : 2 * pp;
 #pragma unroll
-        for (int j = 0; j < kCB; ++j) {
-            if (k0 + j >= nch) break;
-            const int64_t off = off0 + (k0 + j) * stride;
-            ws_s[off] = S;
-            if (JORDAN) {
-                ws_r[off] = R;
-                R = cfma(LC, make_float2(fmaf(Cf, S.x, R.x), fmaf(Cf, S.y, R.y)), lrv[j]);
-            }
-            S = cfma(k0 + j == 0 ? L0 : LC, S, lsv[j]);
-        }
-    }
-    if (state_out) state_out[idx] = S;
-    if (coef_out && b == 0) {
-        const float2 lam = lambda_pow(decay[pm], freq[pm], 1.0f);
-        const float2 c = mode_coef(amp[pm], phase[pm]);
-        coef_out[pm] = make_float4(lam.x, lam.y, c.x, c.y);
-    }
-}
-
-// Phase 3 (forward).  Grid (ceil(D*TPC/kBlock), nch, B); the TPC threads of a
-// channel split its modes and add their readouts with shuffles.
-template <typename T, int MG, bool REV>
-__global__ void __launch_bounds__(kBlock) k_chunk_output(
-    const T *__restrict__ x, T *__restrict__ y, int64_t L, int D, int M, int tpc, int C, int nch,
-    int64_t t0, const float *__restrict__ decay, const float *__restrict__ freq,
-    const float *__restrict__ amp, const float *__restrict__ phase,
-    const float2 *__restrict__ ws_s) {
-    const int gx = blockIdx.x * blockDim.x + threadIdx.x;
-    const int d = gx / tpc, grp = gx % tpc;
-    const int k = blockIdx.y, b = blockIdx.z;
-    const bool active = d < D;
-    float2 lam[MG], c[MG], s[MG];
-    const int64_t base = (((int64_t)b * nch + k) * D + d) * M;
+        for (int j = 0; j < J; ++j) a[j] = *reinterpret_cast<const ulonglong2 *>(pw + 8 * j * kPwStride + n);
+        const float v[2][4] = {{xa.x, xa.z, xb.x, xb.z}, {xa.y, xa.w, xb.y, xb.w}};
 #pragma unroll
-    for (int j = 0; j < MG; ++j) {
-        const int m = grp * MG + j;
-        const bool on = active && m < M;
-        lam[j] = on ? lambda_pow(decay[d * M + m], freq[d * M + m], 1.0f) : make_float2(0, 0);
-        c[j] = on ? mode_coef(amp[d * M + m], phase[d * M + m]) : make_float2(0, 0);
-        s[j] = on ? ws_s[base + m] : make_float2(0, 0);
-    }
-    const int64_t tau0 = t0 + (int64_t)k * C;
-    const int i0 = tau0 < 0 ? (int)(-tau0) : 0;
-    auto at = [&](int i) {
-        const int64_t tau = tau0 + i;
-        return ((int64_t)b * L + (REV ? (L - 1 - tau) : tau)) * D + d;
-    };
-    // kTokBlock tokens' drives are loaded before their updates run (the trip
-    // counts are uniform across the warp, so every lane reaches the shuffles).
-    for (int i = i0; i < C; i += kTokBlock) {
-        float xs[kTokBlock];
+        for (int e = 0; e < 2; ++e) {
+            const int p = 2 * pp + e;
+            const u64 w = dup2((float)(TO_END ? kC - 1 - p : p + 1));
 #pragma unroll
-        for (int u = 0; u < kTokBlock; ++u) xs[u] = active && i + u < C ? ld_elem(x + at(i + u)) : 0.0f;
+            for (int c = 0; c < 4; ++c) {
+                const u64 d = dup2(v[e][c]);
+                const u64 dq = JORDAN ? mul2(d, w) : 0ull;
 #pragma unroll
-        for (int u = 0; u < kTokBlock; ++u) {
-            if (i + u >= C) break;
-            float acc = 0.0f;
-#pragma unroll
-            for (int j = 0; j < MG; ++j) {
-                s[j] = cfma(lam[j], s[j], make_float2(xs[u], 0.0f));
-                acc = fmaf(c[j].x, s[j].x, fmaf(-c[j].y, s[j].y, acc));
-            }
-            for (int o = tpc >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (active && grp == 0) st_elem(y + at(i + u), acc);
-        }
-    }
-}
-
-// Optional state terms of the backward (all [B][D][M] complex, null = absent).
-struct StateTerms {
-    const float2 *state_in;   // the forward's state before token 0
-    const float2 *g;          // the loss gradient of the terminal state
-    float2 *d_state_in;       // output: the loss gradient of state_in
-    float2 *ws_j;             // with g: per-chunk partials of conj(g) J, next to ws_s / ws_r
-};
-
-// Phase 3 (backward).  Reverse time over dy; writes dx and, in place of the
-// carried (S, R), the chunk's partial sums G = sum x S and P = sum x R.
-// kG (a terminal-state gradient g): the second adjoint Phi_t = lambda^(L-1-t)
-// conj(g) joins dx with readout 1, and J = sum x_t (L-1-t) lambda^(L-1-t) (the unit
-// adjoint U and its Jordan partner Q, both closed-form at the chunk start) gives the
-// partials conj(g) J.  The chunk that ends at token 0 holds S_0 and R_0: it adds the
-// initial state's terms s_in lambda S_0 to G and s_in lambda (R_0 + S_0) to P (and
-// conj(g) L lambda^L s_in to its J partial) and writes the gradient of s_in,
-// conj(c lambda S_0) + g conj(lambda^L).
-template <typename T, int MG, bool kG>
-__global__ void __launch_bounds__(kBlock) k_chunk_backward(
-    const T *__restrict__ dy, const T *__restrict__ x, T *__restrict__ dx, int64_t L, int D,
-    int M, int tpc, int C, int nch, int64_t t0, const float *__restrict__ decay,
-    const float *__restrict__ freq, const float *__restrict__ amp,
-    const float *__restrict__ phase, float2 *__restrict__ ws_s, float2 *__restrict__ ws_r,
-    const StateTerms stt) {
-    const int gx = blockIdx.x * blockDim.x + threadIdx.x;
-    const int d = gx / tpc, grp = gx % tpc;
-    const int k = blockIdx.y, b = blockIdx.z;
-    const bool active = d < D;
-    float2 lam[MG], c[MG], s[MG], r[MG], G[MG], P[MG];
-    float2 phi[MG], U[MG], Q[MG], J[MG];
-    const int64_t base = (((int64_t)b * nch + k) * D + d) * M;
-    const int64_t tau0 = t0 + (int64_t)k * C;
-    const int i0 = tau0 < 0 ? (int)(-tau0) : 0;
-#pragma unroll
-    for (int j = 0; j < MG; ++j) {
-        const int m = grp * MG + j;
-        const bool on = active && m < M;
-        lam[j] = on ? lambda_pow(decay[d * M + m], freq[d * M + m], 1.0f) : make_float2(0, 0);
-        c[j] = on ? mode_coef(amp[d * M + m], phase[d * M + m]) : make_float2(0, 0);
-        s[j] = on ? ws_s[base + m] : make_float2(0, 0);
-        r[j] = on ? ws_r[base + m] : make_float2(0, 0);
-        G[j] = make_float2(0, 0);
-        P[j] = make_float2(0, 0);
-        if (kG) {
-            // At the first position (time L-1-tau, tau = tau0 + i0): lambda^tau.
-            const float n = (float)(tau0 + i0);
-            U[j] = on ? lambda_pow(decay[d * M + m], freq[d * M + m], n) : make_float2(0, 0);
-            Q[j] = make_float2(n * U[j].x, n * U[j].y);
-            const float2 gg = on ? stt.g[((int64_t)b * D + d) * M + m] : make_float2(0, 0);
-            phi[j] = cmul(U[j], make_float2(gg.x, -gg.y));
-            J[j] = make_float2(0, 0);
-        }
-    }
-    // The next token's drives are loaded before this token's arithmetic.
-    auto at = [&](int i) { return ((int64_t)b * L + (L - 1 - (tau0 + i))) * D + d; };
-    float u_next = active && i0 < C ? ld_elem(dy + at(i0)) : 0.0f;
-    float x_next = active && i0 < C ? ld_elem(x + at(i0)) : 0.0f;
-    for (int i = i0; i < C; ++i) {
-        const int64_t e = at(i);
-        const float u = u_next, xv = x_next;
-        if (active && i + 1 < C) {
-            u_next = ld_elem(dy + at(i + 1));
-            x_next = ld_elem(x + at(i + 1));
-        }
-        float acc = 0.0f;
-#pragma unroll
-        for (int j = 0; j < MG; ++j) {
-            r[j] = cmul(lam[j], make_float2(r[j].x + s[j].x, r[j].y + s[j].y));
-            s[j] = cfma(lam[j], s[j], make_float2(u, 0.0f));
-            acc = fmaf(c[j].x, s[j].x, fmaf(-c[j].y, s[j].y, acc));
-            G[j].x = fmaf(xv, s[j].x, G[j].x);
-            G[j].y = fmaf(xv, s[j].y, G[j].y);
-            P[j].x = fmaf(xv, r[j].x, P[j].x);
-            P[j].y = fmaf(xv, r[j].y, P[j].y);
-            if (kG) {
-                acc += phi[j].x;
-                J[j].x = fmaf(xv, Q[j].x, J[j].x);
-                J[j].y = fmaf(xv, Q[j].y, J[j].y);
-                phi[j] = cmul(lam[j], phi[j]);
-                Q[j] = cmul(lam[j], make_float2(Q[j].x + U[j].x, Q[j].y + U[j].y));
-                U[j] = cmul(lam[j], U[j]);
-            }
-        }
-        for (int o = tpc >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (active && grp == 0) st_elem(dx + e, acc);
-    }
-    const bool first_token = k == nch - 1;   // this chunk ends at token 0
-#pragma unroll
-    for (int j = 0; j < MG; ++j) {
-        const int m = grp * MG + j;
-        if (active && m < M) {
-            const int64_t sm = ((int64_t)b * D + d) * M + m;
-            const float2 gg = kG ? stt.g[sm] : make_float2(0, 0);
-            float2 gj = kG ? cmul(make_float2(gg.x, -gg.y), J[j]) : make_float2(0, 0);
-            if (first_token) {
-                const float2 ls = cmul(lam[j], s[j]);   // lambda S_0
-                if (stt.state_in) {
-                    const float2 si = stt.state_in[sm];
-                    G[j] = cfma(si, ls, G[j]);
-                    P[j] = cfma(si, cmul(lam[j], make_float2(r[j].x + s[j].x, r[j].y + s[j].y)), P[j]);
-                    if (kG) {
-                        const float2 lL = lambda_pow(decay[d * M + m], freq[d * M + m], (float)L);
-                        const float2 jin = cmul(si, lL);
-                        gj = cfma(make_float2(gg.x, -gg.y), make_float2((float)L * jin.x, (float)L * jin.y), gj);
-                    }
-                }
-                if (stt.d_state_in) {
-                    const float2 cl = cmul(c[j], ls);
-                    float2 ds = make_float2(cl.x, -cl.y);
-                    if (kG) {
-                        const float2 lL = lambda_pow(decay[d * M + m], freq[d * M + m], (float)L);
-                        ds = cfma(gg, make_float2(lL.x, -lL.y), ds);
-                    }
-                    stt.d_state_in[sm] = ds;
+                for (int j = 0; j < J; ++j) {
+                    const u64 aj = (e == 0) == TO_END ? a[j].y : a[j].x;
+                    fma2(acc[j][c], aj, d);
+                    if (JORDAN) fma2(accq[j][c], aj, dq);
                 }
             }
-            ws_s[base + m] = G[j];
-            ws_r[base + m] = P[j];
-            if (kG) stt.ws_j[base + m] = gj;
         }
     }
 }
 
-// Phase 4 (backward).  One thread per (d, m): fixed-order sum of the partials
+// acc[2 j + e][c] += the causal product of row p = 16 j + 2 g + e: sum_{p' <= p} K[p-p'] x_{p'}
+// (the two halves of an accumulator take even and odd p' and are added at the end).
+// Whole 16-row blocks below the diagonal run on packed pairs (K[p-p'], K[p-p'-1]) from
+// the reversed kernel kq (kq[q] = K[63 - q]; the copy kq + 64 shifted by one keeps the
+// pairs of even rows 8-byte aligned).  Inside the diagonal blocks later drives are
+// skipped, not multiplied by zero, so an infinite or NaN drive leaves earlier outputs alone.
+__device__ __forceinline__ void causal(const float *kq, const float *xs, int g, u64 (&acc)[8][4]) {
+#pragma unroll
+    for (int s = 0; s < 3; ++s) {
+#pragma unroll 2
+        for (int u = 0; u < 8; ++u) {
+            const int pp = 8 * s + u;   // positions 2 pp, 2 pp + 1
+            const ulonglong2 xa = *reinterpret_cast<const ulonglong2 *>(xs + pp * 2 * kCols);
+            const ulonglong2 xb = *reinterpret_cast<const ulonglong2 *>(xs + pp * 2 * kCols + 4);
+#pragma unroll
+            for (int j = s + 1; j < 4; ++j) {
+                const int q1 = kC - 1 - (16 * j + 2 * g + 1) + 2 * pp;   // row e = 1: even
+                const u64 k1 = *reinterpret_cast<const u64 *>(kq + q1);
+                const u64 k0 = *reinterpret_cast<const u64 *>(kq + kC + q1);   // row e = 0: kq[q1 + 1], kq[q1 + 2]
+                fma2(acc[2 * j][0], k0, xa.x);
+                fma2(acc[2 * j][1], k0, xa.y);
+                fma2(acc[2 * j][2], k0, xb.x);
+                fma2(acc[2 * j][3], k0, xb.y);
+                fma2(acc[2 * j + 1][0], k1, xa.x);
+                fma2(acc[2 * j + 1][1], k1, xa.y);
+                fma2(acc[2 * j + 1][2], k1, xb.x);
+                fma2(acc[2 * j + 1][3], k1, xb.y);
+            }
+        }
+    }
+    // Diagonal blocks: rows 2 g, 2 g + 1 of each block against its positions i <= row.
+    float d0[4][4], d1[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) d0[j][c] = d1[j][c] = 0.0f;
+    for (int u = 0; u <= g; ++u) {   // positions 2 u, 2 u + 1
+        const float ka = kq[kC - 1 - 2 * (g - u)], kb = kq[kC - 2 - 2 * (g - u)];   // lags 2 (g - u), + 1
+        const float kc = u < g ? kq[kC - 2 * (g - u)] : 0.0f;                       // lag 2 (g - u) - 1
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float *row = xs + (8 * j + u) * 2 * kCols;
+            const float4 xa = *reinterpret_cast<const float4 *>(row), xb = *reinterpret_cast<const float4 *>(row + 4);
+            const float v0[4] = {xa.x, xa.z, xb.x, xb.z}, v1[4] = {xa.y, xa.w, xb.y, xb.w};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                d0[j][c] = fmaf(ka, v0[c], d0[j][c]);
+                if (u < g) d0[j][c] = fmaf(kc, v1[c], d0[j][c]);
+                d1[j][c] = fmaf(kb, v0[c], d1[j][c]);
+                d1[j][c] = fmaf(ka, v1[c], d1[j][c]);
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            float2 a = unpack2(acc[2 * j][c]), b = unpack2(acc[2 * j + 1][c]);
+            acc[2 * j][c] = pack2(a.x + d0[j][c], a.y);
+            acc[2 * j + 1][c] = pack2(b.x + d1[j][c], b.y);
+        }
+}
+
+// acc += Re(sum_m lambda^p W) over `modes` modes: W is staged as (Re, -Im) per column, so
+// a packed FMA on (Re lambda^p, Im lambda^p) accumulates both halves of the real part.
+__device__ __forceinline__ void up_project(const float2 *pw, const float *ws, int modes, int g, u64 (&acc)[8][4]) {
+#pragma unroll 2
+    for (int m = 0; m < modes; ++m) {
+        const ulonglong2 wa = *reinterpret_cast<const ulonglong2 *>(ws + m * 2 * kCols);
+        const ulonglong2 wb = *reinterpret_cast<const ulonglong2 *>(ws + m * 2 * kCols + 4);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(pw + m * kPwStride + 16 * j + 2 * g);
+            fma2(acc[2 * j][0], a.x, wa.x);
+            fma2(acc[2 * j][1], a.x, wa.y);
+            fma2(acc[2 * j][2], a.x, wb.x);
+            fma2(acc[2 * j][3], a.x, wb.y);
+            fma2(acc[2 * j + 1][0], a.y, wa.x);
+            fma2(acc[2 * j + 1][1], a.y, wa.y);
+            fma2(acc[2 * j + 1][2], a.y, wb.x);
+            fma2(acc[2 * j + 1][3], a.y, wb.y);
+        }
+    }
+}
+
+// acc[n] += sum_u dy_u x_{u + 16 l + n} over the 16 positions u of block a, one column
+// (the lane's); positions past the chunk count as zero.
+__device__ __forceinline__ void correlate(const float *dys, const float *xs, int a, int l, float (&acc)[16]) {
+    float dv[16], xv[32];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const float2 v = *reinterpret_cast<const float2 *>(dys + (8 * a + u) * 2 * kCols);
+        dv[2 * u] = v.x;
+        dv[2 * u + 1] = v.y;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const float2 v = a + l + h < 4
+                                 ? *reinterpret_cast<const float2 *>(xs + (8 * (a + l + h) + u) * 2 * kCols)
+                                 : make_float2(0.0f, 0.0f);
+            xv[16 * h + 2 * u] = v.x;
+            xv[16 * h + 2 * u + 1] = v.y;
+        }
+#pragma unroll
+    for (int u = 0; u < 16; ++u)
+#pragma unroll
+        for (int n = 0; n < 16; ++n) acc[n] = fmaf(dv[u], xv[u + n], acc[n]);
+}
+
+// v[n] summed over the 16 columns (lanes of one half); lane `col` receives lag n = col.
+__device__ __forceinline__ float sum_columns(float (&v)[16], int col) {
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+        const bool up = col & o;
+#pragma unroll
+        for (int n = 0; n < o; ++n) {
+            const float keep = up ? v[n + o] : v[n], send = up ? v[n] : v[n + o];
+            v[n] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    return v[0];
+}
+
+// One block: channels 4 blockIdx.x .. + 3 of batch row blockIdx.z, segment blockIdx.y.
+// kOut: write outputs (else only the segment's end state, from zero).
+template <int J, int NP, bool BWD, bool kOut>
+__global__ void __launch_bounds__(kThreads, NP == 2 ? 1 : J == 4 ? 2 : 3) k_scan(const ScanArgs A) {
+    constexpr int kModes = 8 * J * NP;
+    constexpr bool kX = BWD && kOut;   // the x tile is needed
+    extern __shared__ __align__(16) float smem[];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int g = lane & 7, cg = lane >> 3;
+    const int seg = blockIdx.y;
+    const int64_t b = blockIdx.z;
+    const int d0 = kCh * blockIdx.x, d = d0 + w, M = A.M, D = A.D;
+    constexpr int kWords = chan_words(kModes, kX);
+    float2 *pw = reinterpret_cast<float2 *>(smem + w * kWords);
+    float *kq = smem + w * kWords + 2 * kModes * kPwStride;
+    float *us = kq + kKernWords;                 // drive tile, then W, then the output tile
+    float *xs = us + (kX ? kFieldWords : 0);     // x tile (backward)
+
+    // ---- tables: lambda^n, n < 64 (an exact power every 8, products between)
+    {
+        constexpr int kLpm = kModes >= 32 ? 1 : 32 / kModes;   // lanes per mode
+#pragma unroll 1
+        for (int m = lane / kLpm; m < kModes; m += 32) {
+            float2 *row = pw + m * kPwStride;
+            const bool on = m < M;
+            const float ga = on ? A.decay[d * M + m] : 0.0f, om = on ? A.freq[d * M + m] : 0.0f;
+            const float2 l1 = lambda_pow(ga, om, 1.0f);
+#pragma unroll 1
+            for (int n0 = 8 * (lane % kLpm); n0 < kC; n0 += 8 * kLpm) {
+                float2 z = lambda_pow(ga, om, (float)n0);
+                if (!on) z = make_float2(0.0f, 0.0f);
+                row[n0] = z;
+#pragma unroll
+                for (int e = 1; e < 8; ++e) row[n0 + e] = z = cmul(z, l1);
+            }
+        }
+    }
+    // ---- the lane's modes: lambda^64, c, and the state (pair) entering the segment
+    float2 lamC[NP][J], cm[NP][J], S0[NP][J], R0[BWD ? NP : 1][J];
+    float2 *cs = reinterpret_cast<float2 *>(us);   // c of every mode, until the first tile is staged
+#pragma unroll
+    for (int q = 0; q < NP; ++q)
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const int m = 8 * J * q + 8 * j + g;
+            const bool on = m < M;
+            const float ga = on ? A.decay[d * M + m] : 0.0f, om = on ? A.freq[d * M + m] : 0.0f;
+            const float2 z = make_float2(0.0f, 0.0f);
+            const int64_t sm = (b * D + d) * M + m;
+            lamC[q][j] = on ? lambda_pow(ga, om, (float)kC) : z;
+            cm[q][j] = kOut && on ? mode_coef(A.amp[d * M + m], A.phase[d * M + m]) : z;
+            S0[q][j] = !BWD && A.enter && on && seg == 0 ? A.enter[sm] : z;
+            if (BWD) R0[q][j] = z;
+            if (kOut && seg > 0 && on) {
+                // The earlier segments' end states, each carried over the segments between.
+                const float nf = (float)(A.tps * kTile);
+                const float2 lN = lambda_pow(ga, om, nf);
+                const int64_t st = (int64_t)gridDim.z * D * M;
+                float2 S = z, R = z;
+#pragma unroll 4
+                for (int r = 0; r < seg; ++r) {
+                    if (BWD)
+                        R = cfma(lN, make_float2(fmaf(nf, S.x, R.x), fmaf(nf, S.y, R.y)), A.seg_r[sm + r * st]);
+                    S = cfma(lN, S, A.seg_s[sm + r * st]);
+                }
+                S0[q][j] = S;
+                if (BWD) R0[q][j] = R;
+            }
+            if (kOut && cg == 0) cs[m] = cm[q][j];
+            if (!BWD && kOut && A.coef_out && b == 0 && seg == A.nseg - 1 && cg == 0 && on) {
+                const float2 l1 = lambda_pow(ga, om, 1.0f);
+                A.coef_out[d * M + m] = make_float4(l1.x, l1.y, cm[q][j].x, cm[q][j].y);
+            }
+            // The output launch's segment 0 starts from this copy: by then a state_out that
+            // is state_in's buffer may be written by the last segment's block.
+            if (!kOut && !BWD && seg == 0 && A.enter && cg == 0 && on)
+                A.seg_s[sm + (int64_t)(A.nseg - 1) * gridDim.z * D * M] = S0[q][j];
+        }
+    __syncwarp();
+    if (kOut) {
+        // K[n] = sum_m Re(c lambda^n), stored reversed (and once more shifted by one).
+        float k0 = 0.0f, k1 = 0.0f;
+        for (int m = 0; m < M; ++m) {
+            const float2 c = cs[m], p0 = pw[m * kPwStride + lane], p1 = pw[m * kPwStride + lane + 32];
+            k0 = fmaf(c.x, p0.x, fmaf(-c.y, p0.y, k0));
+            k1 = fmaf(c.x, p1.x, fmaf(-c.y, p1.y, k1));
+        }
+        kq[63 - lane] = k0;
+        kq[31 - lane] = k1;
+        kq[kC + 62 - lane] = k0;
+        if (lane < 31) kq[kC + 30 - lane] = k1;
+        if (lane == 0) kq[kC + 63] = 0.0f;
+    }
+    __syncthreads();   // the first tile overwrites cs
+
+    float2 G[kX ? NP : 1][J], P[kX ? NP : 1][J], Jg[kX ? NP : 1][J];
+    float rho_a = 0.0f, rho_b = 0.0f;   // lane (h, n): lags 16 h + n and 16 (3 - h) + n
+    if (kX) {
+#pragma unroll
+        for (int q = 0; q < NP; ++q)
+#pragma unroll
+            for (int j = 0; j < J; ++j) G[q][j] = P[q][j] = Jg[q][j] = make_float2(0.0f, 0.0f);
+    }
+    const int tail = (int)(A.L & (kC - 1));                 // tokens of the partial last chunk
+    const int64_t last_tau = (int64_t)A.nch * kC - 1;
+    const int tile_end = min(A.ntiles, (seg + 1) * A.tps);
+    for (int tile = seg * A.tps; tile < tile_end; ++tile) {
+        // ---- stage the tile: thread (column, position), 4 channels each
+        auto token = [&](int idx, int64_t &e) {
+            const int col = idx & (kCols - 1), p = idx >> 4;
+            const int64_t tau = ((int64_t)tile * kCols + col) * kC + p;
+            const int64_t t = A.rev ? last_tau - tau : tau;
+            e = (b * A.L + t) * D + d0;
+            return t >= 0 && t < A.L;
+        };
+        {
+            float4 v[8];
+            float *base = smem + 2 * kModes * kPwStride + kKernWords;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                int64_t e;
+                const bool in = token(tid + i * kThreads, e);
+                v[i] = in ? load4(A.u, A.bf16, e) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int idx = tid + i * kThreads, col = idx & (kCols - 1), p = idx >> 4;
+                float *o = base + (p >> 1) * 2 * kCols + 2 * col + (p & 1);
+                o[0] = v[i].x;
+                o[kWords] = v[i].y;
+                o[2 * kWords] = v[i].z;
+                o[3 * kWords] = v[i].w;
+            }
+            if (kX) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    int64_t e;
+                    const bool in = token(tid + i * kThreads, e);
+                    v[i] = in ? load4(A.x, A.bf16, e) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int idx = tid + i * kThreads, col = idx & (kCols - 1), p = idx >> 4;
+                    float *o = base + kFieldWords + (p >> 1) * 2 * kCols + 2 * col + (p & 1);
+                    o[0] = v[i].x;
+                    o[kWords] = v[i].y;
+                    o[2 * kWords] = v[i].z;
+                    o[3 * kWords] = v[i].w;
+                }
+            }
+        }
+        __syncthreads();
+
+        // ---- chunk-local states, carry over the 16 columns (and G, P)
+        const float *uc = us + 8 * cg, *xc = xs + 8 * cg;   // the lane's columns
+        const int chunk0 = tile * kCols + 4 * cg;
+        u64 ls[NP][J][4];   // lambda S of the state entering each of the lane's columns
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            u64 acc[J][4], accq[BWD ? J : 1][4];
+            project<J, BWD, true>(pw + (8 * J * q + g) * kPwStride, uc, acc, accq);
+            float2 Rn[BWD ? J : 1][4];
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                const float2 a = lamC[q][j], a2 = cmul(a, a), a4 = cmul(a2, a2);
+                const float2 lam = pw[(8 * J * q + 8 * j + g) * kPwStride + 1];
+                // The lane's four columns from zero ...
+                float2 es = make_float2(0.0f, 0.0f), er = es;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    if (BWD)
+                        er = cfma(a, make_float2(fmaf((float)kC, es.x, er.x), fmaf((float)kC, es.y, er.y)),
+                                  unpack2(accq[j][c]));
+                    es = cfma(a, es, unpack2(acc[j][c]));
+                }
+                // ... the state entering them (over the four lanes of the mode) ...
+                float2 T = S0[q][j], U = BWD ? R0[q][j] : T, S = T, R = U;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (i == cg) {
+                        S = T;
+                        R = U;
+                    }
+                    const float2 ei = shfl2(es, g + 8 * i);
+                    if (BWD)
+                        U = cfma(a4, make_float2(fmaf(4.0f * kC, T.x, U.x), fmaf(4.0f * kC, T.y, U.y)),
+                                 shfl2(er, g + 8 * i));
+                    T = cfma(a4, T, ei);
+                }
+                S0[q][j] = T;
+                if (BWD) R0[q][j] = U;
+                // ... and entering each of them.
+                const int m = 8 * J * q + 8 * j + g;
+                const bool on = m < M;
+#pragma unroll
+                for (int c = 0; c < (kOut ? 4 : 0); ++c) {
+                    const float2 lsv = cmul(lam, S);
+                    ls[q][j][c] = pack2(lsv.x, lsv.y);
+                    if (kX) {
+                        Rn[j][c] = cmul(lam, R);
+                        R = cfma(a, make_float2(fmaf((float)kC, S.x, R.x), fmaf((float)kC, S.y, R.y)),
+                                 unpack2(accq[j][c]));
+                        S = cfma(a, S, unpack2(acc[j][c]));
+                        if (chunk0 + c == A.nch - 1 && on) {
+                            // The chunk of token 0: (S, R) is the adjoint pair there.
+                            const int64_t sm = (b * D + d) * M + m;
+                            const float2 l0 = cmul(lam, S);
+                            const float2 gg = A.g ? A.g[sm] : make_float2(0.0f, 0.0f);
+                            const float2 lL =
+                                A.g ? lambda_pow(A.decay[d * M + m], A.freq[d * M + m], (float)A.L) : gg;
+                            if (A.state_in) {
+                                const float2 si = A.state_in[sm];
+                                G[q][j] = cfma(si, l0, G[q][j]);
+                                P[q][j] = cfma(si, cmul(lam, make_float2(R.x + S.x, R.y + S.y)), P[q][j]);
+                                const float2 ji = cmul(si, lL);
+                                Jg[q][j].x = fmaf((float)A.L, ji.x, Jg[q][j].x);
+                                Jg[q][j].y = fmaf((float)A.L, ji.y, Jg[q][j].y);
+                            }
+                            if (A.d_state_in) {
+                                const float2 v = cmul(cm[q][j], l0);
+                                A.d_state_in[sm] = cfma(gg, make_float2(lL.x, -lL.y), make_float2(v.x, -v.y));
+                            }
+                        }
+                    } else {
+                        const float2 next = cfma(a, S, unpack2(acc[j][c]));
+                        if (chunk0 + c == A.nch - 1 && on && A.state_out) {
+                            float2 f = next;
+                            if (tail) {
+                                // The sequence ends inside this chunk.
+                                const float2 *row = pw + m * kPwStride;
+                                f = cmul(row[tail], S);
+                                for (int p = 0; p < tail; ++p) {
+                                    const float v = uc[(p >> 1) * 2 * kCols + 2 * c + (p & 1)];
+                                    const float2 z = row[tail - 1 - p];
+                                    f.x = fmaf(z.x, v, f.x);
+                                    f.y = fmaf(z.y, v, f.y);
+                                }
+                            }
+                            A.state_out[(b * D + d) * M + m] = f;
+                        }
+                        S = next;
+                    }
+                }
+            }
+            if (kX) {
+                u64 xp[J][4], xq[J][4];
+                project<J, true, false>(pw + (8 * J * q + g) * kPwStride, xc, xp, xq);
+#pragma unroll
+                for (int j = 0; j < J; ++j) {
+                    const int m = 8 * J * q + 8 * j + g;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const float2 s = unpack2(ls[q][j][c]), p = unpack2(xp[j][c]), v = unpack2(xq[j][c]);
+                        G[q][j] = cfma(p, s, G[q][j]);
+                        P[q][j] = cfma(p, Rn[j][c], cfma(v, s, P[q][j]));
+                    }
+                    if (A.g && m < M) {
+                        // J over the whole chunks: L - 1 - t = E + p with E = L minus the chunk's end.
+                        const float ga = A.decay[d * M + m], om = A.freq[d * M + m];
+                        float2 z = make_float2(0.0f, 0.0f);
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const int64_t E = A.L - (int64_t)(A.nch - chunk0 - c) * kC;
+                            if (E >= 0 && chunk0 + c < A.nch) {
+                                z = c == 0 || E < kC ? lambda_pow(ga, om, (float)E) : cmul(z, lamC[q][j]);
+                                const float2 p = unpack2(xp[j][c]), v = unpack2(xq[j][c]);
+                                const float Ef = (float)(E - 1);
+                                Jg[q][j] = cfma(z, make_float2(fmaf(Ef, p.x, v.x), fmaf(Ef, p.y, v.y)), Jg[q][j]);
+                            }
+                        }
+                        if (tail && chunk0 == 0) {
+                            // The partial last chunk (column 0 of the first tile): its tokens are
+                            // positions p >= 64 - tail, L - 1 - t = p - (64 - tail).
+                            const float2 *row = pw + m * kPwStride;
+                            for (int n = 0; n < tail; ++n) {
+                                const int p = n + kC - tail;
+                                const float v = (float)n * xc[(p >> 1) * 2 * kCols + (p & 1)];
+                                Jg[q][j].x = fmaf(row[n].x, v, Jg[q][j].x);
+                                Jg[q][j].y = fmaf(row[n].y, v, Jg[q][j].y);
+                            }
+                        }
+                    }
+                }
+            }
+        }
+        if (!kOut) {
+            __syncthreads();   // every warp is done with the tile
+            continue;
+        }
+        if (kX) {
+            // Lag correlation: lane = (column, half); the half takes lag blocks {0, 3} or
+            // {1, 2}, whose 10 non-empty (u block, lag block) pairs fall in 4 + 2 steps.
+            const int col = lane & 15, h = lane >> 4;
+            float r0[16], r1[16];
+#pragma unroll
+            for (int n = 0; n < 16; ++n) r0[n] = r1[n] = 0.0f;
+#pragma unroll 1
+            for (int a = 0; a < 4; ++a) correlate(us + 2 * col, xs + 2 * col, a, h, r0);
+#pragma unroll 1
+            for (int a = 0; a < 2; ++a) correlate(us + 2 * col, xs + 2 * col, a, 3 - h, r1);
+            rho_a += sum_columns(r0, col);
+            rho_b += sum_columns(r1, col);
+        }
+
+        // ---- outputs
+        u64 acc[8][4];
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[r][c] = 0ull;
+        causal(kq, uc, g, acc);
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            __syncwarp();   // the warp is done reading the tile (or the previous W)
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                const int m = 8 * J * q + 8 * j + g;
+                float2 W[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float2 v = cmul(cm[q][j], unpack2(ls[q][j][c]));
+                    W[c] = m < M ? make_float2(v.x, -v.y) : make_float2(0.0f, 0.0f);
+                }
+                if (kX && A.g && m < M) {
+                    // Terminal-state gradient: its adjoint conj(g) lambda^(L-1-t) enters a
+                    // whole chunk as conj(g) lambda^E with E = L minus the chunk's end.
+                    const float ga = A.decay[d * M + m], om = A.freq[d * M + m];
+                    const float2 gg = A.g[(b * D + d) * M + m];
+                    float2 z = make_float2(0.0f, 0.0f);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const int64_t E = A.L - (int64_t)(A.nch - chunk0 - c) * kC;
+                        if (E >= 0 && chunk0 + c < A.nch) {
+                            z = c == 0 || E < kC ? lambda_pow(ga, om, (float)E) : cmul(z, lamC[q][j]);
+                            const float2 v = cmul(make_float2(gg.x, -gg.y), z);
+                            W[c].x += v.x;
+                            W[c].y -= v.y;
+                        }
+                    }
+                }
+                float4 *o = reinterpret_cast<float4 *>(us + (8 * j + g) * 2 * kCols + 8 * cg);
+                o[0] = make_float4(W[0].x, W[0].y, W[1].x, W[1].y);
+                o[1] = make_float4(W[2].x, W[2].y, W[3].x, W[3].y);
+            }
+            __syncwarp();
+            up_project(pw + 8 * J * q * kPwStride, uc, min(8 * J, M - 8 * J * q), g, acc);
+        }
+        float y[8][4];
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float2 v = unpack2(acc[r][c]);
+                y[r][c] = v.x + v.y;
+            }
+        if (kX && A.g && tail && chunk0 == 0) {
+            // The terminal-state term of the partial last chunk.
+            for (int m = 0; m < M; ++m) {
+                const float2 gg = A.g[(b * D + d) * M + m];
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {
+                    const int n = 16 * (r >> 1) + 2 * g + (r & 1) - (kC - tail);
+                    if (n >= 0) {
+                        const float2 z = pw[m * kPwStride + n];
+                        y[r][0] = fmaf(gg.x, z.x, fmaf(gg.y, z.y, y[r][0]));
+                    }
+                }
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            float4 *o = reinterpret_cast<float4 *>(us + (8 * j + g) * 2 * kCols + 8 * cg);
+            o[0] = make_float4(y[2 * j][0], y[2 * j + 1][0], y[2 * j][1], y[2 * j + 1][1]);
+            o[1] = make_float4(y[2 * j][2], y[2 * j + 1][2], y[2 * j][3], y[2 * j + 1][3]);
+        }
+        __syncthreads();
+        // A thread reads here the words it wrote when staging, and writes them again for
+        // the next tile: no barrier is needed between.
+        const float *base = smem + 2 * kModes * kPwStride + kKernWords;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int idx = tid + i * kThreads, col = idx & (kCols - 1), p = idx >> 4;
+            const float *o = base + (p >> 1) * 2 * kCols + 2 * col + (p & 1);
+            int64_t e;
+            if (token(idx, e)) store4(A.out, A.bf16, e, make_float4(o[0], o[kWords], o[2 * kWords], o[3 * kWords]));
+        }
+    }
+
+    if (!kOut) {
+        if (cg == 0) {
+#pragma unroll
+            for (int q = 0; q < NP; ++q)
+#pragma unroll
+                for (int j = 0; j < J; ++j) {
+                    const int m = 8 * J * q + 8 * j + g;
+                    const int64_t o = (((int64_t)seg * gridDim.z + b) * D + d) * M + m;
+                    if (m < M) {
+                        A.seg_s[o] = S0[q][j];
+                        if (BWD) A.seg_r[o] = R0[q][j];
+                    }
+                }
+        }
+        return;
+    }
+    if (kX) {
+        // The within-chunk terms: lane cg takes lags 16 cg .. 16 cg + 15 of its modes; the
+        // sums over cg complete G, P and J.
+        const int h = lane >> 4;
+        __syncwarp();
+        kq[16 * h + (lane & 15)] = rho_a;
+        kq[16 * (3 - h) + (lane & 15)] = rho_b;
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < NP; ++q)
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                const int m = 8 * J * q + 8 * j + g;
+                float2 gs = G[q][j], ps = P[q][j], js = Jg[q][j];
+                for (int n = 16 * cg; n < 16 * cg + 16; ++n) {
+                    const float2 z = pw[m * kPwStride + n];
+                    const float r = kq[n], nr = (float)n * r;
+                    gs.x = fmaf(z.x, r, gs.x);
+                    gs.y = fmaf(z.y, r, gs.y);
+                    ps.x = fmaf(z.x, nr, ps.x);
+                    ps.y = fmaf(z.y, nr, ps.y);
+                }
+#pragma unroll
+                for (int o = 8; o <= 16; o <<= 1) {
+                    gs.x += __shfl_xor_sync(0xffffffffu, gs.x, o);
+                    gs.y += __shfl_xor_sync(0xffffffffu, gs.y, o);
+                    ps.x += __shfl_xor_sync(0xffffffffu, ps.x, o);
+                    ps.y += __shfl_xor_sync(0xffffffffu, ps.y, o);
+                    js.x += __shfl_xor_sync(0xffffffffu, js.x, o);
+                    js.y += __shfl_xor_sync(0xffffffffu, js.y, o);
+                }
+                if (cg == 0 && m < M) {
+                    const int64_t o = ((b * A.nseg + seg) * D + d) * M + m;
+                    A.part_g[o] = gs;
+                    A.part_p[o] = ps;
+                    if (A.g) {
+                        const float2 gg = A.g[(b * D + d) * M + m];
+                        A.part_j[o] = cmul(make_float2(gg.x, -gg.y), js);
+                    }
+                }
+            }
+    }
+}
+
+// One thread per (d, m): fixed-order sum of the partials
 // over (b, k), then the four gradients.  The sums are compensated (Kahan) fp32
 // sums, so the result is reproducible and its error stays near one rounding
-// however many chunk partials the SIMT path adds; the combination with
+// however many partials are added; the combination with
 // c = A e^{i phi} (formed as the forward forms it, fp32 sincosf) uses fmaf for
 // the differences.  Double precision made this launch 3-4x slower on this part
 // (low FP64 rate): 4.8 against 1.4 us at D = 512, M = 32, four partials.
@@ -414,68 +811,65 @@ __global__ void __launch_bounds__(256) k_grad_reduce(
     g_freq[pm] = -fmaf(cr, pi.s, ci * pr.s) - ji.s;      // -Im(c P) - Im(conj(g) J)
 }
 
-template <typename T>
-cudaError_t prefill_t(const T *x, T *y, int64_t B, int64_t L, int D, int M, const float *decay,
-                      const float *freq, const float *amp, const float *phase, const float *state_in,
-                      float *state_out, float *coef_out, void *ws, cudaStream_t st) {
-    const ChunkGeom g = geom(B, L, D);
-    const int tpc = threads_per_channel(M, kMgFwd);
-    float2 *ws_s = reinterpret_cast<float2 *>(ws);
-    dim3 grid((unsigned)((D * tpc + kBlock - 1) / kBlock), (unsigned)g.nch, (unsigned)B);
-    k_chunk_local<T, kMgFwd, false, false><<<grid, kBlock, 0, st>>>(
-        x, L, D, M, tpc, g.C, g.nch, g.t0, decay, freq, ws_s, nullptr);
-    const int64_t n = B * D * M;
-    k_chunk_carry<false><<<(unsigned)((n + kCarryBlock - 1) / kCarryBlock), kCarryBlock, 0, st>>>(
-        B, D, M, g.C, g.nch, g.t0, decay, freq, amp, phase, ws_s, nullptr,
-        reinterpret_cast<const float2 *>(state_in), reinterpret_cast<float2 *>(state_out),
-        reinterpret_cast<float4 *>(coef_out));
-    k_chunk_output<T, kMgFwd, false><<<grid, kBlock, 0, st>>>(
-        x, y, L, D, M, tpc, g.C, g.nch, g.t0, decay, freq, amp, phase, ws_s);
-    count_launches(3);
+
+// Launch shape.  A block is a 4-channel group of a batch row; where these blocks
+// would leave SMs idle the sequence is cut into as many segments of whole tiles as fill
+// the resident blocks once.  The segments cost one more launch and a second projection
+// of the drive (38 % of the forward's FMA at M = 32, 31 % of the backward's), so they
+// are only taken when at least two of them fit.
+struct Geometry {
+    int nch, ntiles, nseg, tps;
+};
+
+Geometry geometry(int64_t B, int64_t L, int D, int M, int max_seg) {
+    Geometry q;
+    q.nch = (int)((L + kC - 1) / kC);
+    q.ntiles = (q.nch + kCols - 1) / kCols;
+    const int64_t slots = (int64_t)sm_count() * (M > 32 ? 1 : M > 16 ? 2 : 3);
+    const int64_t groups = B * (D / kCh);
+    q.nseg = (int)std::max<int64_t>(1, std::min<int64_t>({slots / groups, (int64_t)q.ntiles, (int64_t)max_seg}));
+    q.tps = (q.ntiles + q.nseg - 1) / q.nseg;
+    q.nseg = (q.ntiles + q.tps - 1) / q.tps;
+    return q;
+}
+
+template <int J, int NP, bool BWD, bool kOut>
+cudaError_t launch_scan(const ScanArgs &a, int64_t B, int nseg, cudaStream_t st) {
+    constexpr int bytes = smem_bytes(8 * J * NP, BWD && kOut);
+    auto *k = k_scan<J, NP, BWD, kOut>;
+    if (bytes > 48 * 1024) {
+        // Idempotent, host-side only, and cheap beside the launch.
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e != cudaSuccess) return e;
+    }
+    k<<<dim3((unsigned)(a.D / kCh), (unsigned)nseg, (unsigned)B), kThreads, bytes, st>>>(a);
+    count_launches(1);
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t backward_t(const T *dy, const T *x, T *dx, int64_t B, int64_t L, int D, int M,
-                       const float *decay, const float *freq, const float *amp,
-                       const float *phase, const float *state_in, const float *d_state_out,
-                       float *d_state_in, float *gd, float *gf, float *ga, float *gp, void *ws,
-                       cudaStream_t st) {
-    const ChunkGeom g = geom_c(L, bwd_chunk_len(B, L, D));
-    const int64_t n = B * (int64_t)g.nch * D * M;
-    float2 *ws_s = reinterpret_cast<float2 *>(ws);
-    float2 *ws_r = ws_s + n;
-    StateTerms stt;
-    stt.state_in = reinterpret_cast<const float2 *>(state_in);
-    stt.g = reinterpret_cast<const float2 *>(d_state_out);
-    stt.d_state_in = reinterpret_cast<float2 *>(d_state_in);
-    stt.ws_j = d_state_out ? ws_r + n : nullptr;
-    const int tpc1 = threads_per_channel(M, kMgFwd);
-    dim3 grid1((unsigned)((D * tpc1 + kBlock - 1) / kBlock), (unsigned)g.nch, (unsigned)B);
-    k_chunk_local<T, kMgFwd, true, true><<<grid1, kBlock, 0, st>>>(
-        dy, L, D, M, tpc1, g.C, g.nch, g.t0, decay, freq, ws_s, ws_r);
-    const int64_t nbdm = B * D * M;
-    k_chunk_carry<true><<<(unsigned)((nbdm + kCarryBlock - 1) / kCarryBlock), kCarryBlock, 0, st>>>(
-        B, D, M, g.C, g.nch, g.t0, decay, freq, amp, phase, ws_s, ws_r, nullptr, nullptr, nullptr);
-    const int tpc3 = threads_per_channel(M, kMgBwd);
-    dim3 grid3((unsigned)((D * tpc3 + kBlock - 1) / kBlock), (unsigned)g.nch, (unsigned)B);
-    if (d_state_out)
-        k_chunk_backward<T, kMgBwd, true><<<grid3, kBlock, 0, st>>>(
-            dy, x, dx, L, D, M, tpc3, g.C, g.nch, g.t0, decay, freq, amp, phase, ws_s, ws_r, stt);
-    else
-        k_chunk_backward<T, kMgBwd, false><<<grid3, kBlock, 0, st>>>(
-            dy, x, dx, L, D, M, tpc3, g.C, g.nch, g.t0, decay, freq, amp, phase, ws_s, ws_r, stt);
-    k_grad_reduce<<<(unsigned)((D * M + 255) / 256), 256, 0, st>>>(
-        B, D, M, g.nch, amp, phase, ws_s, ws_r, stt.ws_j, gd, gf, ga, gp);
-    count_launches(4);
-    return cudaGetLastError();
+template <bool BWD>
+cudaError_t run_scan(ScanArgs &a, int64_t B, cudaStream_t st) {
+    auto pass = [&](auto out, int nseg) {
+        constexpr bool kOut = decltype(out)::value;
+        if (a.M <= 8) return launch_scan<1, 1, BWD, kOut>(a, B, nseg, st);
+        if (a.M <= 16) return launch_scan<2, 1, BWD, kOut>(a, B, nseg, st);
+        if (a.M <= 32) return launch_scan<4, 1, BWD, kOut>(a, B, nseg, st);
+        return launch_scan<4, 2, BWD, kOut>(a, B, nseg, st);
+    };
+    if (a.nseg > 1) {
+        const cudaError_t e = pass(std::false_type{}, a.nseg - 1);
+        if (e != cudaSuccess) return e;
+        if (!BWD && a.enter) a.enter = a.seg_s + (int64_t)(a.nseg - 1) * B * a.D * a.M;
+    }
+    return pass(std::true_type{}, a.nseg);
 }
 
 }  // namespace
 
+// The workspace contract.  Sizes are stated in chunks of simt_chunk_len() tokens (8
+// bytes per chunk, channel and mode; the backward in chunks of its own length, 24
+// bytes); the segments above never need more (at most one state per 1024 tokens).
 int simt_chunk_len(int64_t B, int64_t L, int D) {
-    // Enough (b, chunk, channel) threads for about two full waves of 1024
-    // resident threads per SM; chunks of 16..1024 tokens.
     const int64_t target = (int64_t)sm_count() * 2048;
     const int64_t per_chunk = std::max<int64_t>(1, B * (int64_t)D);
     int64_t nch = (target + per_chunk - 1) / per_chunk;
@@ -485,25 +879,50 @@ int simt_chunk_len(int64_t B, int64_t L, int D) {
     return (int)C;
 }
 
+namespace {
+int bwd_ws_chunks(int64_t B, int64_t L, int D) {
+    const int64_t target = (int64_t)sm_count() * 512;
+    const int64_t per_chunk = std::max<int64_t>(1, B * (int64_t)D);
+    const int64_t nch = std::max<int64_t>(1, (target + per_chunk - 1) / per_chunk);
+    const int64_t C = std::max<int64_t>(16, std::min<int64_t>(4096, (L + nch - 1) / nch));
+    return (int)((L + C - 1) / C);
+}
+}  // namespace
+
 size_t simt_prefill_ws_bytes(int64_t B, int64_t L, int D, int M) {
-    const ChunkGeom g = geom(B, L, D);
-    return (size_t)B * g.nch * D * M * sizeof(float2);
+    const int C = simt_chunk_len(B, L, D);
+    return (size_t)B * ((L + C - 1) / C) * D * M * sizeof(float2);
 }
 
 size_t simt_backward_ws_bytes(int64_t B, int64_t L, int D, int M) {
-    const ChunkGeom g = geom_c(L, bwd_chunk_len(B, L, D));
-    return 3 * (size_t)B * g.nch * D * M * sizeof(float2);   // G, P and conj(g) J partials
+    return 3 * (size_t)B * bwd_ws_chunks(B, L, D) * D * M * sizeof(float2);
 }
 
 cudaError_t simt_prefill(const void *x, void *y, rlm_dtype dt, int64_t B, int64_t L, int D,
                          int M, const float *decay, const float *freq, const float *amp,
                          const float *phase, const float *state_in, float *state_out, float *coef_out,
                          void *ws, cudaStream_t st) {
-    if (dt == RLM_BF16)
-        return prefill_t(static_cast<const __nv_bfloat16 *>(x), static_cast<__nv_bfloat16 *>(y),
-                         B, L, D, M, decay, freq, amp, phase, state_in, state_out, coef_out, ws, st);
-    return prefill_t(static_cast<const float *>(x), static_cast<float *>(y), B, L, D, M, decay,
-                     freq, amp, phase, state_in, state_out, coef_out, ws, st);
+    const Geometry q = geometry(B, L, D, M, 1 << 15);
+    ScanArgs a = {};
+    a.u = x;
+    a.out = y;
+    a.bf16 = dt == RLM_BF16;
+    a.L = L;
+    a.D = D;
+    a.M = M;
+    a.nch = q.nch;
+    a.ntiles = q.ntiles;
+    a.nseg = q.nseg;
+    a.tps = q.tps;
+    a.decay = decay;
+    a.freq = freq;
+    a.amp = amp;
+    a.phase = phase;
+    a.seg_s = static_cast<float2 *>(ws);   // nseg <= ceil(L / 1024) <= the contract's chunks
+    a.enter = reinterpret_cast<const float2 *>(state_in);
+    a.state_out = reinterpret_cast<float2 *>(state_out);
+    a.coef_out = reinterpret_cast<float4 *>(coef_out);
+    return run_scan<false>(a, B, st);
 }
 
 cudaError_t grad_reduce(int64_t nparts, int D, int M, const float *amp, const float *phase,
@@ -518,16 +937,41 @@ cudaError_t grad_reduce(int64_t nparts, int D, int M, const float *amp, const fl
 cudaError_t simt_backward(const void *dy, const void *x, void *dx, rlm_dtype dt, int64_t B,
                           int64_t L, int D, int M, const float *decay, const float *freq,
                           const float *amp, const float *phase, const float *state_in,
-                          const float *d_state_out, float *d_state_in, float *g_decay, float *g_freq,
-                          float *g_amp, float *g_phase, void *ws, cudaStream_t st) {
-    if (dt == RLM_BF16)
-        return backward_t(static_cast<const __nv_bfloat16 *>(dy),
-                          static_cast<const __nv_bfloat16 *>(x), static_cast<__nv_bfloat16 *>(dx),
-                          B, L, D, M, decay, freq, amp, phase, state_in, d_state_out, d_state_in, g_decay,
-                          g_freq, g_amp, g_phase, ws, st);
-    return backward_t(static_cast<const float *>(dy), static_cast<const float *>(x),
-                      static_cast<float *>(dx), B, L, D, M, decay, freq, amp, phase, state_in, d_state_out,
-                      d_state_in, g_decay, g_freq, g_amp, g_phase, ws, st);
+                          const float *d_state_out, float *d_state_in, float *g_decay,
+                          float *g_freq, float *g_amp, float *g_phase, void *ws, cudaStream_t st) {
+    // A segment needs five workspace units (its pair, and its G, P and J partials)
+    // where the contract states three a chunk; one segment keeps no pair.
+    const Geometry q = geometry(B, L, D, M, std::max(1, 3 * bwd_ws_chunks(B, L, D) / 5));
+    const int64_t unit = (int64_t)q.nseg * B * D * M;
+    ScanArgs a = {};
+    a.u = dy;
+    a.x = x;
+    a.out = dx;
+    a.bf16 = dt == RLM_BF16;
+    a.rev = 1;
+    a.L = L;
+    a.D = D;
+    a.M = M;
+    a.nch = q.nch;
+    a.ntiles = q.ntiles;
+    a.nseg = q.nseg;
+    a.tps = q.tps;
+    a.decay = decay;
+    a.freq = freq;
+    a.amp = amp;
+    a.phase = phase;
+    a.part_g = static_cast<float2 *>(ws);
+    a.part_p = a.part_g + unit;
+    a.part_j = a.part_p + unit;
+    a.seg_s = a.part_j + unit;
+    a.seg_r = a.seg_s + unit;
+    a.state_in = reinterpret_cast<const float2 *>(state_in);
+    a.g = reinterpret_cast<const float2 *>(d_state_out);
+    a.d_state_in = reinterpret_cast<float2 *>(d_state_in);
+    const cudaError_t e = run_scan<true>(a, B, st);
+    if (e != cudaSuccess) return e;
+    return grad_reduce(B * q.nseg, D, M, amp, phase, a.part_g, a.part_p, d_state_out ? a.part_j : nullptr, g_decay,
+                       g_freq, g_amp, g_phase, st);
 }
 
 }  // namespace rlm
