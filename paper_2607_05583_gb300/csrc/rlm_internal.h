@@ -20,14 +20,12 @@ int sm_count();
 void count_launches(int n);
 
 // ---- SIMT chunked scan (rlm_simt.cu) --------------------------------------
-// Chunk length the SIMT path uses for a problem; workspace and launch agree.
+// The chunk length in which the SIMT path's workspace contract is stated.
 int simt_chunk_len(int64_t B, int64_t L, int D);
 size_t simt_prefill_ws_bytes(int64_t B, int64_t L, int D, int M);
 size_t simt_backward_ws_bytes(int64_t B, int64_t L, int D, int M);
 
-// y = causal mixing of x (reverse=false) or the anti-causal mixing used by the
-// backward pass for dx (reverse=true: time runs from L-1 down to 0).
-// state_out/coef_out may be null.  ws must hold simt_prefill_ws_bytes().
+// y = causal mixing of x.  ws must hold simt_prefill_ws_bytes().
 // state_in ([B][D][M] complex, the state before token 0), state_out and
 // coef_out may be null; state_out may alias state_in.
 cudaError_t simt_prefill(const void *x, void *y, rlm_dtype dt, int64_t B, int64_t L, int D,

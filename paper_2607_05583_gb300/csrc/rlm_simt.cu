@@ -39,8 +39,17 @@
 // launch forms each segment's end state from zero, and the second enters segment s
 // with the combination of the states before it.
 //
-// Same box, before (three launches of token-by-token recurrences, chunk states in
-// memory) and now, us per call: see the launch rule at geometry().
+// What bounds it: the FMA pipe's floor is a third of the time; with two warps a
+// scheduler (tables and accumulators allow no more at M = 32) shared-load latency and
+// instruction fetch are not hidden.  GB300, us per call, against the three launches of
+// token-by-token recurrences with chunk states in memory that this replaces:
+//
+//   fp32, B = 2, L = 4096, D = 512, M = 32: forward 247 -> 62, backward 303 -> 134
+//   bf16 from a state, B = 8, L = 1000, D = 256, M = 16: 75 -> 30
+//   fp32 backward with state terms, B = 3, L = 1521, D = 536, M = 32: 347 -> 197
+//
+// and the error against 64 bits is a half to a third of the recurrences' (3e-6 -> 1e-6 for
+// the gradients of the first line).
 #include <algorithm>
 #include <type_traits>
 
@@ -58,14 +67,19 @@ constexpr int kTile = kC * kCols;    // 1024 tokens
 constexpr int kCh = 4;               // channels (warps) per block
 constexpr int kThreads = 32 * kCh;
 constexpr int kPwStride = 66;        // float2 per mode row of the power table: 16-byte aligned, rows 4 banks apart
-constexpr int kFieldWords = kC * kCols;   // one channel's tile: [p / 2][column][p % 2]
-constexpr int kKernWords = 2 * kC;        // K reversed, and the same shifted by one
+constexpr int kFieldWords = kC * kCols;   // one channel's tile: [p / 2][column][p % 2], see slot()
+constexpr int kKernCopy = kC + 16;        // K reversed, then zeros (negative lags)
+constexpr int kKernWords = 2 * kKernCopy; // that, and the same shifted by one
 
 // Shared memory of a block, in floats: per channel the power table
 // [modes][66] (complex), the reversed lag kernel, the drive tile and (backward) the
 // x tile.
 constexpr int chan_words(int modes, bool bwd) {
     return 2 * modes * kPwStride + kKernWords + (bwd ? 2 : 1) * kFieldWords;
+}
+// Resident blocks a SM (registers and shared memory both allow them).
+__host__ __device__ constexpr int blocks_per_sm(int modes, bool bwd) {
+    return modes > 32 ? 1 : modes > 16 ? 2 : bwd ? 3 : 4;
 }
 constexpr int smem_bytes(int modes, bool bwd) { return kCh * chan_words(modes, bwd) * 4; }
 
@@ -88,6 +102,10 @@ __device__ __forceinline__ u64 mul2(u64 a, u64 b) {
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
+// Word of columns 2 h, 2 h + 1 in row r of a field tile (rows of 32 words: position pairs,
+// or modes of W).  The 16-byte slots of a row are permuted by its number, so that the
+// column groups that eight lanes write into eight rows fall into different banks.
+__device__ __forceinline__ int slot(int r, int h) { return r * 2 * kCols + ((h ^ (r & 7)) << 2); }
 __device__ __forceinline__ float2 shfl2(float2 v, int src) {
     return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
@@ -136,10 +154,10 @@ __device__ __forceinline__ void store4(void *f, int bf16, int64_t e, float4 v) {
 // Projection of the drive tile on the power table: for the lane's modes g + 8 j and
 // columns 4 cg + c, acc = sum_p lambda^e(p) x_p and (JORDAN) accq = sum_p w(p) lambda^e(p) x_p,
 // with e = 63 - p, w = 63 - p (TO_END) or e = p, w = p + 1.  pw points at the row of
-// mode g, xs at the tile's column 4 cg.  Per pair of positions: J + 2 16-byte shared
+// mode g.  Per pair of positions: J + 2 16-byte shared
 // loads, the drives duplicated into both halves, 8 J (16 J) packed FMAs on (Re, Im).
 template <int J, bool JORDAN, bool TO_END>
-__device__ __forceinline__ void project(const float2 *pw, const float *xs, u64 (&acc)[J][4],
+__device__ __forceinline__ void project(const float2 *pw, const float *xs, int cg, u64 (&acc)[J][4],
                                         u64 (&accq)[JORDAN ? J : 1][4]) {
 #pragma unroll
     for (int j = 0; j < J; ++j)
@@ -150,8 +168,8 @@ __device__ __forceinline__ void project(const float2 *pw, const float *xs, u64 (
         }
 #pragma unroll 2
     for (int pp = 0; pp < kC / 2; ++pp) {
-        const float4 xa = *reinterpret_cast<const float4 *>(xs + pp * 2 * kCols);
-        const float4 xb = *reinterpret_cast<const float4 *>(xs + pp * 2 * kCols + 4);
+        const float4 xa = *reinterpret_cast<const float4 *>(xs + slot(pp, 2 * cg));
+        const float4 xb = *reinterpret_cast<const float4 *>(xs + slot(pp, 2 * cg + 1));
         ulonglong2 a[J];
         const int n = TO_END ? kC - 2 - 2 * pp : 2 * pp;
 #pragma unroll
@@ -177,75 +195,61 @@ __device__ __forceinline__ void project(const float2 *pw, const float *xs, u64 (
 }
 
 // acc[2 j + e][c] += the causal product of row p = 16 j + 2 g + e: sum_{p' <= p} K[p-p'] x_{p'}
-// (the two halves of an accumulator take even and odd p' and are added at the end).
-// Whole 16-row blocks below the diagonal run on packed pairs (K[p-p'], K[p-p'-1]) from
-// the reversed kernel kq (kq[q] = K[63 - q]; the copy kq + 64 shifted by one keeps the
-// pairs of even rows 8-byte aligned).  Inside the diagonal blocks later drives are
-// skipped, not multiplied by zero, so an infinite or NaN drive leaves earlier outputs alone.
-__device__ __forceinline__ void causal(const float *kq, const float *xs, int g, u64 (&acc)[8][4]) {
+// (the two halves of an accumulator take even and odd p' and are added at the end), on
+// packed pairs (K[p-p'], K[p-p'-1]) of the reversed kernel kq (kq[q] = K[63 - q], zeros
+// after; the copy behind it, shifted by one, keeps the pairs of even rows aligned).
+// In the diagonal 16-row blocks the zeros stand for the later drives.  kGuard: a tile
+// with an infinite or NaN drive skips them instead, so that earlier outputs stay clean.
+template <bool kGuard>
+__device__ __forceinline__ void causal(const float *kq, const float *xs, int g, int cg, u64 (&acc)[8][4]) {
 #pragma unroll
-    for (int s = 0; s < 3; ++s) {
+    for (int s = 0; s < 4; ++s) {
 #pragma unroll 2
         for (int u = 0; u < 8; ++u) {
             const int pp = 8 * s + u;   // positions 2 pp, 2 pp + 1
-            const ulonglong2 xa = *reinterpret_cast<const ulonglong2 *>(xs + pp * 2 * kCols);
-            const ulonglong2 xb = *reinterpret_cast<const ulonglong2 *>(xs + pp * 2 * kCols + 4);
+            const ulonglong2 xa = *reinterpret_cast<const ulonglong2 *>(xs + slot(pp, 2 * cg));
+            const ulonglong2 xb = *reinterpret_cast<const ulonglong2 *>(xs + slot(pp, 2 * cg + 1));
+            const u64 x[4] = {xa.x, xa.y, xb.x, xb.y};
 #pragma unroll
-            for (int j = s + 1; j < 4; ++j) {
+            for (int j = s; j < 4; ++j) {
                 const int q1 = kC - 1 - (16 * j + 2 * g + 1) + 2 * pp;   // row e = 1: even
                 const u64 k1 = *reinterpret_cast<const u64 *>(kq + q1);
-                const u64 k0 = *reinterpret_cast<const u64 *>(kq + kC + q1);   // row e = 0: kq[q1 + 1], kq[q1 + 2]
-                fma2(acc[2 * j][0], k0, xa.x);
-                fma2(acc[2 * j][1], k0, xa.y);
-                fma2(acc[2 * j][2], k0, xb.x);
-                fma2(acc[2 * j][3], k0, xb.y);
-                fma2(acc[2 * j + 1][0], k1, xa.x);
-                fma2(acc[2 * j + 1][1], k1, xa.y);
-                fma2(acc[2 * j + 1][2], k1, xb.x);
-                fma2(acc[2 * j + 1][3], k1, xb.y);
+                const u64 k0 = *reinterpret_cast<const u64 *>(kq + kKernCopy + q1);   // row e = 0: kq[q1 + 1], kq[q1 + 2]
+                if (kGuard && j == s) {
+                    // Rows 2 g, 2 g + 1 of the block against its positions 2 u, 2 u + 1.
+                    const float2 f0 = unpack2(k0), f1 = unpack2(k1);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const float2 v = unpack2(x[c]);
+                        float2 a0 = unpack2(acc[2 * j][c]), a1 = unpack2(acc[2 * j + 1][c]);
+                        if (u <= g) {
+                            a0.x = fmaf(f0.x, v.x, a0.x);
+                            a1.x = fmaf(f1.x, v.x, a1.x);
+                            a1.y = fmaf(f1.y, v.y, a1.y);
+                        }
+                        if (u < g) a0.y = fmaf(f0.y, v.y, a0.y);
+                        acc[2 * j][c] = pack2(a0.x, a0.y);
+                        acc[2 * j + 1][c] = pack2(a1.x, a1.y);
+                    }
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        fma2(acc[2 * j][c], k0, x[c]);
+                        fma2(acc[2 * j + 1][c], k1, x[c]);
+                    }
+                }
             }
         }
     }
-    // Diagonal blocks: rows 2 g, 2 g + 1 of each block against its positions i <= row.
-    float d0[4][4], d1[4][4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) d0[j][c] = d1[j][c] = 0.0f;
-    for (int u = 0; u <= g; ++u) {   // positions 2 u, 2 u + 1
-        const float ka = kq[kC - 1 - 2 * (g - u)], kb = kq[kC - 2 - 2 * (g - u)];   // lags 2 (g - u), + 1
-        const float kc = u < g ? kq[kC - 2 * (g - u)] : 0.0f;                       // lag 2 (g - u) - 1
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float *row = xs + (8 * j + u) * 2 * kCols;
-            const float4 xa = *reinterpret_cast<const float4 *>(row), xb = *reinterpret_cast<const float4 *>(row + 4);
-            const float v0[4] = {xa.x, xa.z, xb.x, xb.z}, v1[4] = {xa.y, xa.w, xb.y, xb.w};
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                d0[j][c] = fmaf(ka, v0[c], d0[j][c]);
-                if (u < g) d0[j][c] = fmaf(kc, v1[c], d0[j][c]);
-                d1[j][c] = fmaf(kb, v0[c], d1[j][c]);
-                d1[j][c] = fmaf(ka, v1[c], d1[j][c]);
-            }
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            float2 a = unpack2(acc[2 * j][c]), b = unpack2(acc[2 * j + 1][c]);
-            acc[2 * j][c] = pack2(a.x + d0[j][c], a.y);
-            acc[2 * j + 1][c] = pack2(b.x + d1[j][c], b.y);
-        }
 }
 
 // acc += Re(sum_m lambda^p W) over `modes` modes: W is staged as (Re, -Im) per column, so
 // a packed FMA on (Re lambda^p, Im lambda^p) accumulates both halves of the real part.
-__device__ __forceinline__ void up_project(const float2 *pw, const float *ws, int modes, int g, u64 (&acc)[8][4]) {
+__device__ __forceinline__ void up_project(const float2 *pw, const float *ws, int modes, int g, int cg, u64 (&acc)[8][4]) {
 #pragma unroll 2
     for (int m = 0; m < modes; ++m) {
-        const ulonglong2 wa = *reinterpret_cast<const ulonglong2 *>(ws + m * 2 * kCols);
-        const ulonglong2 wb = *reinterpret_cast<const ulonglong2 *>(ws + m * 2 * kCols + 4);
+        const ulonglong2 wa = *reinterpret_cast<const ulonglong2 *>(ws + slot(m, 2 * cg));
+        const ulonglong2 wb = *reinterpret_cast<const ulonglong2 *>(ws + slot(m, 2 * cg + 1));
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(pw + m * kPwStride + 16 * j + 2 * g);
@@ -263,11 +267,11 @@ __device__ __forceinline__ void up_project(const float2 *pw, const float *ws, in
 
 // acc[n] += sum_u dy_u x_{u + 16 l + n} over the 16 positions u of block a, one column
 // (the lane's); positions past the chunk count as zero.
-__device__ __forceinline__ void correlate(const float *dys, const float *xs, int a, int l, float (&acc)[16]) {
+__device__ __forceinline__ void correlate(const float *dys, const float *xs, int col, int a, int l, float (&acc)[16]) {
     float dv[16], xv[32];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-        const float2 v = *reinterpret_cast<const float2 *>(dys + (8 * a + u) * 2 * kCols);
+        const float2 v = *reinterpret_cast<const float2 *>(dys + slot(8 * a + u, col >> 1) + 2 * (col & 1));
         dv[2 * u] = v.x;
         dv[2 * u + 1] = v.y;
     }
@@ -276,7 +280,7 @@ __device__ __forceinline__ void correlate(const float *dys, const float *xs, int
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const float2 v = a + l + h < 4
-                                 ? *reinterpret_cast<const float2 *>(xs + (8 * (a + l + h) + u) * 2 * kCols)
+                                 ? *reinterpret_cast<const float2 *>(xs + slot(8 * (a + l + h) + u, col >> 1) + 2 * (col & 1))
                                  : make_float2(0.0f, 0.0f);
             xv[16 * h + 2 * u] = v.x;
             xv[16 * h + 2 * u + 1] = v.y;
@@ -304,9 +308,10 @@ __device__ __forceinline__ float sum_columns(float (&v)[16], int col) {
 // One block: channels 4 blockIdx.x .. + 3 of batch row blockIdx.z, segment blockIdx.y.
 // kOut: write outputs (else only the segment's end state, from zero).
 template <int J, int NP, bool BWD, bool kOut>
-__global__ void __launch_bounds__(kThreads, NP == 2 ? 1 : J == 4 ? 2 : 3) k_scan(const ScanArgs A) {
+__global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_scan(const ScanArgs A) {
     constexpr int kModes = 8 * J * NP;
     constexpr bool kX = BWD && kOut;   // the x tile is needed
+    constexpr bool kAhead = !BWD && J == 4;   // the next tile's drive is loaded a tile ahead
     extern __shared__ __align__(16) float smem[];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int g = lane & 7, cg = lane >> 3;
@@ -390,9 +395,10 @@ __global__ void __launch_bounds__(kThreads, NP == 2 ? 1 : J == 4 ? 2 : 3) k_scan
         }
         kq[63 - lane] = k0;
         kq[31 - lane] = k1;
-        kq[kC + 62 - lane] = k0;
-        if (lane < 31) kq[kC + 30 - lane] = k1;
-        if (lane == 0) kq[kC + 63] = 0.0f;
+        kq[kKernCopy + 62 - lane] = k0;
+        if (lane < 31) kq[kKernCopy + 30 - lane] = k1;
+        if (lane < 16) kq[kC + lane] = kq[kKernCopy + kC + lane] = 0.0f;
+        if (lane == 0) kq[kKernCopy + kC - 1] = 0.0f;
     }
     __syncthreads();   // the first tile overwrites cs
 
@@ -405,63 +411,58 @@ __global__ void __launch_bounds__(kThreads, NP == 2 ? 1 : J == 4 ? 2 : 3) k_scan
             for (int j = 0; j < J; ++j) G[q][j] = P[q][j] = Jg[q][j] = make_float2(0.0f, 0.0f);
     }
     const int tail = (int)(A.L & (kC - 1));                 // tokens of the partial last chunk
-    const int64_t last_tau = (int64_t)A.nch * kC - 1;
     const int tile_end = min(A.ntiles, (seg + 1) * A.tps);
+    // The thread's 8 tokens of a tile, 4 channels each (zeros outside the sequence).
+    const int Li = (int)A.L, t_last = A.nch * kC - 1;
+    auto fetch = [&](const void *f, int tile, float4 (&v)[8]) {
+        const int tau = tile * kTile + (tid & (kCols - 1)) * kC + (tid >> 4);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int t = A.rev ? t_last - tau - 8 * i : tau + 8 * i;
+            v[i] = t >= 0 && t < Li ? load4(f, A.bf16, (b * A.L + t) * D + d0) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+    };
+    // The 32-mode forward loads the next tile's drive ahead of this tile's outputs (67 -> 62
+    // us at B = 2, L = 4096, D = 512, M = 32 fp32).  The backward has no registers for it
+    // (132 -> 143 us), the smaller forward needs them for its fourth block a SM.
+    float4 nextu[8], nextx[kX ? 8 : 1];
+    if (kAhead) fetch(A.u, seg * A.tps, nextu);
     for (int tile = seg * A.tps; tile < tile_end; ++tile) {
         // ---- stage the tile: thread (column, position), 4 channels each
-        auto token = [&](int idx, int64_t &e) {
-            const int col = idx & (kCols - 1), p = idx >> 4;
-            const int64_t tau = ((int64_t)tile * kCols + col) * kC + p;
-            const int64_t t = A.rev ? last_tau - tau : tau;
-            e = (b * A.L + t) * D + d0;
-            return t >= 0 && t < A.L;
-        };
-        {
-            float4 v[8];
-            float *base = smem + 2 * kModes * kPwStride + kKernWords;
+        const int t0 = tile * kTile + (tid & (kCols - 1)) * kC + (tid >> 4);   // tau of the thread's first token
+        bool odd = false;   // an infinite or NaN drive
+        auto stage = [&](const float4 (&v)[8], float *base) {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                int64_t e;
-                const bool in = token(tid + i * kThreads, e);
-                v[i] = in ? load4(A.u, A.bf16, e) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int idx = tid + i * kThreads, col = idx & (kCols - 1), p = idx >> 4;
-                float *o = base + (p >> 1) * 2 * kCols + 2 * col + (p & 1);
+                const int p = (tid >> 4) + 8 * i, col = tid & (kCols - 1);
+                float *o = base + slot(p >> 1, col >> 1) + 2 * (col & 1) + (p & 1);
                 o[0] = v[i].x;
                 o[kWords] = v[i].y;
                 o[2 * kWords] = v[i].z;
                 o[3 * kWords] = v[i].w;
             }
-            if (kX) {
+        };
+        float *base = smem + 2 * kModes * kPwStride + kKernWords;
+        if (!kAhead) fetch(A.u, tile, nextu);
+        if constexpr (kX) fetch(A.x, tile, nextx);
+        stage(nextu, base);
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    int64_t e;
-                    const bool in = token(tid + i * kThreads, e);
-                    v[i] = in ? load4(A.x, A.bf16, e) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                }
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int idx = tid + i * kThreads, col = idx & (kCols - 1), p = idx >> 4;
-                    float *o = base + kFieldWords + (p >> 1) * 2 * kCols + 2 * col + (p & 1);
-                    o[0] = v[i].x;
-                    o[kWords] = v[i].y;
-                    o[2 * kWords] = v[i].z;
-                    o[3 * kWords] = v[i].w;
-                }
-            }
+        for (int i = 0; i < 8; ++i) {
+            // x - x is zero for a finite x.
+            const float z = (nextu[i].x - nextu[i].x) + (nextu[i].y - nextu[i].y) + (nextu[i].z - nextu[i].z) +
+                            (nextu[i].w - nextu[i].w);
+            odd |= !(z == 0.0f);
         }
-        __syncthreads();
+        if constexpr (kX) stage(nextx, base + kFieldWords);
+        const bool guard = __syncthreads_or(kOut && odd);
 
         // ---- chunk-local states, carry over the 16 columns (and G, P)
-        const float *uc = us + 8 * cg, *xc = xs + 8 * cg;   // the lane's columns
         const int chunk0 = tile * kCols + 4 * cg;
         u64 ls[NP][J][4];   // lambda S of the state entering each of the lane's columns
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
             u64 acc[J][4], accq[BWD ? J : 1][4];
-            project<J, BWD, true>(pw + (8 * J * q + g) * kPwStride, uc, acc, accq);
+            project<J, BWD, true>(pw + (8 * J * q + g) * kPwStride, us, cg, acc, accq);
             float2 Rn[BWD ? J : 1][4];
 #pragma unroll
             for (int j = 0; j < J; ++j) {
@@ -533,7 +534,7 @@ __global__ void __launch_bounds__(kThreads, NP == 2 ? 1 : J == 4 ? 2 : 3) k_scan
                                 const float2 *row = pw + m * kPwStride;
                                 f = cmul(row[tail], S);
                                 for (int p = 0; p < tail; ++p) {
-                                    const float v = uc[(p >> 1) * 2 * kCols + 2 * c + (p & 1)];
+                                    const float v = us[slot(p >> 1, 2 * cg + (c >> 1)) + 2 * (c & 1) + (p & 1)];
                                     const float2 z = row[tail - 1 - p];
                                     f.x = fmaf(z.x, v, f.x);
                                     f.y = fmaf(z.y, v, f.y);
@@ -547,7 +548,7 @@ __global__ void __launch_bounds__(kThreads, NP == 2 ? 1 : J == 4 ? 2 : 3) k_scan
             }
             if (kX) {
                 u64 xp[J][4], xq[J][4];
-                project<J, true, false>(pw + (8 * J * q + g) * kPwStride, xc, xp, xq);
+                project<J, true, false>(pw + (8 * J * q + g) * kPwStride, xs, cg, xp, xq);
 #pragma unroll
                 for (int j = 0; j < J; ++j) {
                     const int m = 8 * J * q + 8 * j + g;
@@ -577,7 +578,7 @@ __global__ void __launch_bounds__(kThreads, NP == 2 ? 1 : J == 4 ? 2 : 3) k_scan
                             const float2 *row = pw + m * kPwStride;
                             for (int n = 0; n < tail; ++n) {
                                 const int p = n + kC - tail;
-                                const float v = (float)n * xc[(p >> 1) * 2 * kCols + (p & 1)];
+                                const float v = (float)n * xs[slot(p >> 1, 0) + (p & 1)];
                                 Jg[q][j].x = fmaf(row[n].x, v, Jg[q][j].x);
                                 Jg[q][j].y = fmaf(row[n].y, v, Jg[q][j].y);
                             }
@@ -587,6 +588,7 @@ __global__ void __launch_bounds__(kThreads, NP == 2 ? 1 : J == 4 ? 2 : 3) k_scan
             }
         }
         if (!kOut) {
+            if (kAhead && tile + 1 < tile_end) fetch(A.u, tile + 1, nextu);
             __syncthreads();   // every warp is done with the tile
             continue;
         }
@@ -598,9 +600,9 @@ __global__ void __launch_bounds__(kThreads, NP == 2 ? 1 : J == 4 ? 2 : 3) k_scan
 #pragma unroll
             for (int n = 0; n < 16; ++n) r0[n] = r1[n] = 0.0f;
 #pragma unroll 1
-            for (int a = 0; a < 4; ++a) correlate(us + 2 * col, xs + 2 * col, a, h, r0);
+            for (int a = 0; a < 4; ++a) correlate(us, xs, col, a, h, r0);
 #pragma unroll 1
-            for (int a = 0; a < 2; ++a) correlate(us + 2 * col, xs + 2 * col, a, 3 - h, r1);
+            for (int a = 0; a < 2; ++a) correlate(us, xs, col, a, 3 - h, r1);
             rho_a += sum_columns(r0, col);
             rho_b += sum_columns(r1, col);
         }
@@ -611,7 +613,10 @@ __global__ void __launch_bounds__(kThreads, NP == 2 ? 1 : J == 4 ? 2 : 3) k_scan
         for (int r = 0; r < 8; ++r)
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[r][c] = 0ull;
-        causal(kq, uc, g, acc);
+        if (guard)
+            causal<true>(kq, us, g, cg, acc);
+        else
+            causal<false>(kq, us, g, cg, acc);
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
             __syncwarp();   // the warp is done reading the tile (or the previous W)
@@ -641,12 +646,13 @@ __global__ void __launch_bounds__(kThreads, NP == 2 ? 1 : J == 4 ? 2 : 3) k_scan
                         }
                     }
                 }
-                float4 *o = reinterpret_cast<float4 *>(us + (8 * j + g) * 2 * kCols + 8 * cg);
-                o[0] = make_float4(W[0].x, W[0].y, W[1].x, W[1].y);
-                o[1] = make_float4(W[2].x, W[2].y, W[3].x, W[3].y);
+                *reinterpret_cast<float4 *>(us + slot(8 * j + g, 2 * cg)) = make_float4(W[0].x, W[0].y, W[1].x, W[1].y);
+                *reinterpret_cast<float4 *>(us + slot(8 * j + g, 2 * cg + 1)) =
+                    make_float4(W[2].x, W[2].y, W[3].x, W[3].y);
             }
             __syncwarp();
-            up_project(pw + 8 * J * q * kPwStride, uc, min(8 * J, M - 8 * J * q), g, acc);
+            if (kAhead && q == NP - 1 && tile + 1 < tile_end) fetch(A.u, tile + 1, nextu);
+            up_project(pw + 8 * J * q * kPwStride, us, min(8 * J, M - 8 * J * q), g, cg, acc);
         }
         float y[8][4];
 #pragma unroll
@@ -673,20 +679,21 @@ __global__ void __launch_bounds__(kThreads, NP == 2 ? 1 : J == 4 ? 2 : 3) k_scan
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            float4 *o = reinterpret_cast<float4 *>(us + (8 * j + g) * 2 * kCols + 8 * cg);
-            o[0] = make_float4(y[2 * j][0], y[2 * j + 1][0], y[2 * j][1], y[2 * j + 1][1]);
-            o[1] = make_float4(y[2 * j][2], y[2 * j + 1][2], y[2 * j][3], y[2 * j + 1][3]);
+            *reinterpret_cast<float4 *>(us + slot(8 * j + g, 2 * cg)) =
+                make_float4(y[2 * j][0], y[2 * j + 1][0], y[2 * j][1], y[2 * j + 1][1]);
+            *reinterpret_cast<float4 *>(us + slot(8 * j + g, 2 * cg + 1)) =
+                make_float4(y[2 * j][2], y[2 * j + 1][2], y[2 * j][3], y[2 * j + 1][3]);
         }
         __syncthreads();
         // A thread reads here the words it wrote when staging, and writes them again for
         // the next tile: no barrier is needed between.
-        const float *base = smem + 2 * kModes * kPwStride + kKernWords;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const int idx = tid + i * kThreads, col = idx & (kCols - 1), p = idx >> 4;
-            const float *o = base + (p >> 1) * 2 * kCols + 2 * col + (p & 1);
-            int64_t e;
-            if (token(idx, e)) store4(A.out, A.bf16, e, make_float4(o[0], o[kWords], o[2 * kWords], o[3 * kWords]));
+            const int p = (tid >> 4) + 8 * i, col = tid & (kCols - 1);
+            const float *o = base + slot(p >> 1, col >> 1) + 2 * (col & 1) + (p & 1);
+            const int t = A.rev ? t_last - t0 - 8 * i : t0 + 8 * i;
+            if (t >= 0 && t < Li)
+                store4(A.out, A.bf16, (b * A.L + t) * D + d0, make_float4(o[0], o[kWords], o[2 * kWords], o[3 * kWords]));
         }
     }
 
@@ -821,11 +828,11 @@ struct Geometry {
     int nch, ntiles, nseg, tps;
 };
 
-Geometry geometry(int64_t B, int64_t L, int D, int M, int max_seg) {
+Geometry geometry(int64_t B, int64_t L, int D, int M, bool bwd, int max_seg) {
     Geometry q;
     q.nch = (int)((L + kC - 1) / kC);
     q.ntiles = (q.nch + kCols - 1) / kCols;
-    const int64_t slots = (int64_t)sm_count() * (M > 32 ? 1 : M > 16 ? 2 : 3);
+    const int64_t slots = (int64_t)sm_count() * blocks_per_sm(M, bwd);
     const int64_t groups = B * (D / kCh);
     q.nseg = (int)std::max<int64_t>(1, std::min<int64_t>({slots / groups, (int64_t)q.ntiles, (int64_t)max_seg}));
     q.tps = (q.ntiles + q.nseg - 1) / q.nseg;
@@ -902,7 +909,7 @@ cudaError_t simt_prefill(const void *x, void *y, rlm_dtype dt, int64_t B, int64_
                          int M, const float *decay, const float *freq, const float *amp,
                          const float *phase, const float *state_in, float *state_out, float *coef_out,
                          void *ws, cudaStream_t st) {
-    const Geometry q = geometry(B, L, D, M, 1 << 15);
+    const Geometry q = geometry(B, L, D, M, false, 1 << 15);
     ScanArgs a = {};
     a.u = x;
     a.out = y;
@@ -941,7 +948,7 @@ cudaError_t simt_backward(const void *dy, const void *x, void *dx, rlm_dtype dt,
                           float *g_freq, float *g_amp, float *g_phase, void *ws, cudaStream_t st) {
     // A segment needs five workspace units (its pair, and its G, P and J partials)
     // where the contract states three a chunk; one segment keeps no pair.
-    const Geometry q = geometry(B, L, D, M, std::max(1, 3 * bwd_ws_chunks(B, L, D) / 5));
+    const Geometry q = geometry(B, L, D, M, true, std::max(1, 3 * bwd_ws_chunks(B, L, D) / 5));
     const int64_t unit = (int64_t)q.nseg * B * D * M;
     ScanArgs a = {};
     a.u = dy;

@@ -1,0 +1,90 @@
+"""The CUDA-core scan (fp32 with M > 16, M > 32, a ragged length from a state, fp32
+backward) at the edges of its tiles: chunks of 64 tokens, tiles of 1024, mode groups of
+8, 16, 32 and 64, segments of whole tiles.  Tolerances are the operator's parity bar."""
+import numpy as np
+import pytest
+
+import oracle
+from synth import make_inputs
+from tests._util import TOL, assert_close, to_dev, to_np
+
+torch = pytest.importorskip("torch")
+rlm = pytest.importorskip("paper_2607_05583_gb300")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    from paper_2607_05583_gb300 import build
+    build.build()
+    return rlm.load_library()
+
+
+def _state(B, D, M, seed):
+    rng = np.random.default_rng(seed)
+    s = (3.0 * rng.standard_normal((B, D, M, 2))).astype(np.float32)
+    st = rlm.State(torch.from_numpy(s).cuda(), torch.empty(D, M, 4, device="cuda"))
+    return st, s[..., 0].astype(np.float64) + 1j * s[..., 1]
+
+
+# Lengths at chunk and tile edges; the last two rows are long enough for several segments
+# (B * D / 4 blocks against a few hundred resident ones).
+@pytest.mark.parametrize("B,L,D,M,dtype", [
+    (2, 1, 16, 9, "f32"), (1, 63, 8, 33, "f32"), (3, 65, 16, 17, "f32"), (2, 127, 8, 64, "bf16"),
+    (2, 1023, 16, 8, "bf16"), (1, 1025, 24, 1, "f32"), (2, 1087, 8, 16, "bf16"), (1, 2049, 16, 32, "f32"),
+    (1, 20001, 8, 5, "f32"), (1, 9999, 8, 40, "bf16"),
+])
+def test_prefill_from_a_state_at_tile_edges(B, L, D, M, dtype):
+    inp = make_inputs(B, L, D, M, dtype, seed=L + M)
+    x = to_dev(inp.x, dtype)
+    p = rlm.Params.from_arrays(*inp.params())
+    st, s0 = _state(B, D, M, L)
+    y = torch.full_like(x, float("nan"))
+    # In place: the terminal state overwrites the initial one.
+    rlm.rlm_mix_prefill_from(x, p, st, y, st)
+    torch.cuda.synchronize()
+    y_ref, s_ref = oracle.rec_prefill(inp.x, *inp.params(), state_in=s0)
+    assert_close(to_np(y), y_ref, TOL[dtype], "y")
+    s = st.complex().cpu().numpy()
+    assert_close(s.real, s_ref.real, TOL["f32"], "state re")
+    assert_close(s.imag, s_ref.imag, TOL["f32"], "state im")
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("t", [0, 70, 1030])
+def test_a_non_finite_drive_leaves_earlier_outputs_alone(bad, t):
+    B, L, D, M = 1, 1200, 8, 20
+    inp = make_inputs(B, L, D, M, "f32", seed=3)
+    p = rlm.Params.from_arrays(*inp.params())
+    x = to_dev(inp.x, "f32")
+    y0, y1 = torch.empty_like(x), torch.empty_like(x)
+    rlm.rlm_mix_prefill(x, p, y0)
+    x[0, t, 2] = bad
+    rlm.rlm_mix_prefill(x, p, y1)
+    other = [c for c in range(D) if c != 2]
+    assert torch.equal(y0[..., other], y1[..., other])
+    # The guarded and the plain product add in the same order up to rounding.
+    assert_close(to_np(y1[0, :t, 2]), to_np(y0[0, :t, 2]), 1e-5) if t else None
+    assert not torch.isfinite(y1[0, t, 2])
+
+
+@pytest.mark.parametrize("B,L,D,M,dtype", [
+    (1, 1, 8, 4, "f32"), (2, 63, 8, 8, "f32"), (1, 64, 16, 16, "f32"), (2, 100, 8, 33, "bf16"),
+    (2, 1024, 8, 17, "f32"), (1, 1090, 16, 32, "f32"), (1, 12345, 8, 9, "f32"), (1, 4096, 8, 64, "f32"),
+])
+def test_backward_with_state_terms_at_tile_edges(B, L, D, M, dtype):
+    inp = make_inputs(B, L, D, M, dtype, seed=L + 3 * M, with_dy=True)
+    p = rlm.Params.from_arrays(*inp.params())
+    x, dy = to_dev(inp.x, dtype), to_dev(inp.dy, dtype)
+    (st, s0), (gs, g) = _state(B, D, M, L), _state(B, D, M, L + 1)
+    dx, gr, ds = torch.empty_like(x), rlm.Grads.empty(D, M), rlm.State.empty(B, D, M)
+    rlm.rlm_mix_backward_from(dy, x, p, st, gs, dx, gr, ds)
+    torch.cuda.synchronize()
+    ref = oracle.backward_rec(inp.x, inp.dy, *inp.params(), state_in=s0, d_state_out=g)
+    assert_close(to_np(dx), ref[0], TOL[dtype], "dx")
+    for k in ("decay", "freq", "amp", "phase"):
+        assert_close(getattr(gr, k).cpu().numpy(), ref[1][k], TOL["f32"], k)
+    d = ds.complex().cpu().numpy()
+    assert_close(d.real, ref[1]["state_in"].real, TOL["f32"], "d_state re")
+    assert_close(d.imag, ref[1]["state_in"].imag, TOL["f32"], "d_state im")
