@@ -2,7 +2,9 @@
 
 Argument marshalling only: every step of the operator runs in the library's
 CUDA kernels, reached through the C ABI declared in ``include/rlm.h`` with the
-same function names.  PyTorch supplies device memory and the current stream.
+same function names.  Calls with plain arguments (contiguous CUDA tensors) are
+marshalled by ``_rlm_py`` (``csrc/py/rlm_py.cpp``); what it hands back (None) takes the
+ctypes route below, which also raises the errors.  PyTorch supplies device memory and the current stream.
 There is no fallback: if the compiled library is missing the calls raise.
 
 Names follow the paper (ResonatorLM, arxiv 2607.05583): x is the drive field
@@ -13,6 +15,8 @@ of Sec. 3.3, [B][D][M] complex fp32 plus its mode coefficients.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from dataclasses import dataclass
 
@@ -80,6 +84,7 @@ class RlmError(RuntimeError):
 
 
 _lib = None
+_native = None   # the _rlm_py module, loaded with the library
 
 
 def library_path() -> str:
@@ -88,7 +93,7 @@ def library_path() -> str:
 
 def load_library(build_if_missing: bool = False) -> ctypes.CDLL:
     """Load librlm.so (raises if it has not been built)."""
-    global _lib
+    global _lib, _native
     if _lib is not None:
         return _lib
     path = _build_mod.LIB
@@ -132,7 +137,11 @@ def load_library(build_if_missing: bool = False) -> ctypes.CDLL:
     lib.rlm_mix_prefill_noalloc.argtypes = [P(_Tensor), P(_Params), P(_Tensor), P(_State),
                                             ctypes.c_void_p]
     lib.rlm_mix_prefill_noalloc.restype = ctypes.c_int
-    _lib = lib
+    spec = importlib.util.spec_from_file_location(
+        "_rlm_py", _build_mod.PYLIB, loader=importlib.machinery.ExtensionFileLoader("_rlm_py", _build_mod.PYLIB))
+    native = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(native)
+    _native, _lib = native, lib
     return lib
 
 
@@ -348,7 +357,12 @@ def rlm_mix_prefill(x: torch.Tensor, params: Params, y: torch.Tensor,
     """Causal mixing y = K * x (Eq. 2) from a zero state; optional terminal state.
 
     ``workspace`` defaults to a fresh buffer of rlm_prefill_workspace_size bytes."""
-    lib = load_library()
+    lib = _lib or load_library()
+    status = _native.mix_prefill(x, params, None, y, state_out, workspace, stream)
+    if status is not None:
+        if status:
+            _check(status, "rlm_mix_prefill")
+        return
     xt, yt = _field(x), _field(y)
     if workspace is None:
         workspace = _workspace(lib.rlm_prefill_workspace_size(xt.B, xt.L, xt.D, params.M, xt.dtype),
@@ -365,7 +379,12 @@ def rlm_mix_prefill_from(x: torch.Tensor, params: Params, state_in: State | None
     """Causal mixing from an initial state (chunked or continued prefill): y = K * x
     plus the free response of ``state_in`` (its ``s``; None = zero state).
     ``state_out`` may be ``state_in`` itself (in-place continuation)."""
-    lib = load_library()
+    lib = _lib or load_library()
+    status = _native.mix_prefill(x, params, state_in, y, state_out, workspace, stream)
+    if status is not None:
+        if status:
+            _check(status, "rlm_mix_prefill_from")
+        return
     xt, yt = _field(x), _field(y)
     if workspace is None:
         workspace = _workspace(lib.rlm_prefill_workspace_size(xt.B, xt.L, xt.D, params.M, xt.dtype),
@@ -394,7 +413,12 @@ def rlm_mix_prefill_noalloc(x: torch.Tensor, params: Params, y: torch.Tensor,
 
 def rlm_mix_decode(x_t: torch.Tensor, state: State, y_t: torch.Tensor, stream=None) -> None:
     """One decode step (Eq. 4-5); the state is updated in place."""
-    lib = load_library()
+    lib = _lib or load_library()
+    status = _native.mix_decode(x_t, state, y_t, stream)
+    if status is not None:
+        if status:
+            _check(status, "rlm_mix_decode")
+        return
     xt, yt = _field(x_t), _field(y_t)
     _check(lib.rlm_mix_decode(ctypes.byref(xt), ctypes.byref(state._c()), ctypes.byref(yt),
                               ctypes.byref(_launch(stream, None))), "rlm_mix_decode")
@@ -409,7 +433,12 @@ def rlm_state_init(state: State, params: Params, stream=None) -> None:
 def rlm_mix_backward(dy: torch.Tensor, x: torch.Tensor, params: Params, dx: torch.Tensor,
                      dparams: Grads, workspace: torch.Tensor | None = None, stream=None) -> None:
     """dx and the four parameter gradients of l given dy = dl/dy."""
-    lib = load_library()
+    lib = _lib or load_library()
+    status = _native.mix_backward(dy, x, params, None, None, dx, dparams, None, workspace, stream)
+    if status is not None:
+        if status:
+            _check(status, "rlm_mix_backward")
+        return
     dyt, xt, dxt = _field(dy), _field(x), _field(dx)
     if workspace is None:
         workspace = _workspace(lib.rlm_backward_workspace_size(xt.B, xt.L, xt.D, params.M,
@@ -427,7 +456,12 @@ def rlm_mix_backward_from(dy: torch.Tensor, x: torch.Tensor, params: Params, sta
     ``d_state_in`` is given) the gradient of the initial state, for a loss that may
     also depend on the terminal state (its gradient ``d_state_out``).  Only the
     ``s`` buffers of the state arguments are used."""
-    lib = load_library()
+    lib = _lib or load_library()
+    status = _native.mix_backward(dy, x, params, state_in, d_state_out, dx, dparams, d_state_in, workspace, stream)
+    if status is not None:
+        if status:
+            _check(status, "rlm_mix_backward_from")
+        return
     dyt, xt, dxt = _field(dy), _field(x), _field(dx)
     if workspace is None:
         workspace = _workspace(lib.rlm_backward_workspace_size(xt.B, xt.L, xt.D, params.M, xt.dtype),
@@ -457,7 +491,13 @@ def rlm_mixer_prefill(x: torch.Tensor, g: torch.Tensor | None, params: Params, l
     resonant mixing of x from ``state_in``; the local path reads its drives before
     token 0 from ``conv_in``.  ``state_out`` / ``conv_out`` receive the terminal
     state and drive history (each may be its input, for in-place continuation)."""
-    lib = load_library()
+    lib = _lib or load_library()
+    status = _native.mixer_prefill(x, g, params, local, coupling, state_in, conv_in, z, state_out, conv_out,
+                                   workspace, stream)
+    if status is not None:
+        if status:
+            _check(status, "rlm_mixer_prefill")
+        return
     xt, zt = _field(x), _field(z)
     gt = _field(g) if g is not None else None
     if workspace is None:
@@ -475,7 +515,12 @@ def rlm_mixer_decode(x_t: torch.Tensor, g_t: torch.Tensor | None, state: State, 
                      conv: ConvState | None, z_t: torch.Tensor, stream=None, coupling: Coupling | None = None) -> None:
     """One mixer decode step: recurrence, gate and local path in one kernel; the state
     and the drive history advance in place."""
-    lib = load_library()
+    lib = _lib or load_library()
+    status = _native.mixer_decode(x_t, g_t, state, local, coupling, conv, z_t, stream)
+    if status is not None:
+        if status:
+            _check(status, "rlm_mixer_decode")
+        return
     xt, zt = _field(x_t), _field(z_t)
     gt = _field(g_t) if g_t is not None else None
     ref = lambda c: ctypes.byref(c) if c is not None else None

@@ -1,4 +1,5 @@
-"""Compile the CUDA sources into the in-tree shared library ``_build/librlm.so``.
+"""Compile the CUDA sources into the in-tree shared library ``_build/librlm.so`` and the
+Python binding's native call path into ``_build/_rlm_py.so``.
 
 One nvcc invocation per translation unit (run in parallel), one link step.
 Target: sm_103a only (``-gencode arch=compute_103a,code=sm_103a``); the CUDA
@@ -12,6 +13,7 @@ import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -20,6 +22,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(BUILD, "librlm.so")
+PYSRC = os.path.join(CSRC, "py", "rlm_py.cpp")
+PYLIB = os.path.join(BUILD, "_rlm_py.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr",
@@ -39,10 +43,10 @@ def sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(PYLIB):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh"))
+    t = min(os.path.getmtime(LIB), os.path.getmtime(PYLIB))
+    deps = [PYSRC] + sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh"))
     deps += glob.glob(os.path.join(INCLUDE, "*.h"))
     return any(os.path.getmtime(p) > t for p in deps)
 
@@ -70,11 +74,20 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     with ThreadPoolExecutor(max_workers=min(8, os.cpu_count() or 4)) as ex:
         objs = list(ex.map(compile_one, sources()))
     tmp = LIB + f".{os.getpid()}.tmp"
-    cmd = [nvcc, *ARCH, "-shared", "-o", tmp, *objs, "-lpthread"]
+    cmd = [nvcc, *ARCH, "-shared", "-o", tmp, *objs, "-lpthread", "-Xlinker", "-soname=librlm.so"]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError(f"link failed:\n{res.stdout}\n{res.stderr}")
     os.replace(tmp, LIB)
+    # The binding's call path links against librlm.so beside it.
+    tmp = PYLIB + f".{os.getpid()}.tmp"
+    cmd = [nvcc, "-O2", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "-cudart", "none",
+           "-I", sysconfig.get_paths()["include"], "-shared", PYSRC, "-o", tmp, LIB,
+           "-Xlinker", "-rpath", "-Xlinker", "$ORIGIN"]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError(f"building the Python call path failed:\n{res.stdout}\n{res.stderr}")
+    os.replace(tmp, PYLIB)
     return LIB
 
 

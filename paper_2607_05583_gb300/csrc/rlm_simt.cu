@@ -51,6 +51,7 @@
 // and the error against 64 bits is a half to a third of the recurrences' (3e-6 -> 1e-6 for
 // the gradients of the first line).
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "rlm_device.cuh"
@@ -845,9 +846,17 @@ cudaError_t launch_scan(const ScanArgs &a, int64_t B, int nseg, cudaStream_t st)
     constexpr int bytes = smem_bytes(8 * J * NP, BWD && kOut);
     auto *k = k_scan<J, NP, BWD, kOut>;
     if (bytes > 48 * 1024) {
-        // Idempotent, host-side only, and cheap beside the launch.
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        // Once per device (a bit each; devices past 64 set it on every call).
+        static std::atomic<unsigned long long> done{0};
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return e;
+        const unsigned long long bit = dev < 64 ? 1ull << dev : 0;
+        if (!(done.load(std::memory_order_acquire) & bit)) {
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+            if (e != cudaSuccess) return e;
+            done.fetch_or(bit, std::memory_order_release);
+        }
     }
     k<<<dim3((unsigned)(a.D / kCh), (unsigned)nseg, (unsigned)B), kThreads, bytes, st>>>(a);
     count_launches(1);
