@@ -118,8 +118,9 @@ struct ScanArgs {
     int bf16;                 // element type of the fields (0: fp32)
     int rev;                  // reverse time (backward)
     int64_t L;
-    int D, M;
+    int B, D, M;
     int nch, ntiles;          // chunks and tiles of the sequence
+    int gpr;                  // column groups (of 4) of a tile that one batch row takes: 4, or 1 / 2 (packed)
     int nseg, tps;            // segments, tiles per segment
     const float *decay, *freq, *amp, *phase;
     float2 *seg_s, *seg_r;    // [nseg][B][D][M] segment end states (pair) from zero
@@ -127,7 +128,7 @@ struct ScanArgs {
     const float2 *state_in;   // nullable (backward)
     float2 *state_out;        // nullable (forward)
     float4 *coef_out;         // nullable (forward)
-    float2 *part_g, *part_p;  // backward: [B][nseg][D][M]
+    float2 *part_g, *part_p;  // backward: [tiles of rows][nseg][D][M]
     float2 *part_j;           // with g
     const float2 *g;          // nullable: gradient of the terminal state
     float2 *d_state_in;       // nullable
@@ -307,6 +308,9 @@ __device__ __forceinline__ float sum_columns(float (&v)[16], int col) {
 }
 
 // One block: channels 4 blockIdx.x .. + 3 of batch row blockIdx.z, segment blockIdx.y.
+// Sequences of at most 4 (8) chunks leave most of a tile's 16 columns empty, so there a
+// tile holds 4 (2) batch rows, one (two) column groups each, and blockIdx.z counts
+// tiles: b below is then the lane's own row, clamped; `mine` says whether it exists.
 // kOut: write outputs (else only the segment's end state, from zero).
 template <int J, int NP, bool BWD, bool kOut>
 __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_scan(const ScanArgs A) {
@@ -317,7 +321,9 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int g = lane & 7, cg = lane >> 3;
     const int seg = blockIdx.y;
-    const int64_t b = blockIdx.z;
+    const int rpt = 4 / A.gpr, gbase = cg & ~(A.gpr - 1);   // batch rows of a tile; the row's first column group
+    const bool mine = (int)blockIdx.z * rpt + cg / A.gpr < A.B;
+    const int64_t b = min((int)blockIdx.z * rpt + cg / A.gpr, A.B - 1);
     const int d0 = kCh * blockIdx.x, d = d0 + w, M = A.M, D = A.D;
     constexpr int kWords = chan_words(kModes, kX);
     float2 *pw = reinterpret_cast<float2 *>(smem + w * kWords);
@@ -358,13 +364,13 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
             const int64_t sm = (b * D + d) * M + m;
             lamC[q][j] = on ? lambda_pow(ga, om, (float)kC) : z;
             cm[q][j] = kOut && on ? mode_coef(A.amp[d * M + m], A.phase[d * M + m]) : z;
-            S0[q][j] = !BWD && A.enter && on && seg == 0 ? A.enter[sm] : z;
+            S0[q][j] = !BWD && A.enter && on && mine && seg == 0 ? A.enter[sm] : z;
             if (BWD) R0[q][j] = z;
             if (kOut && seg > 0 && on) {
                 // The earlier segments' end states, each carried over the segments between.
                 const float nf = (float)(A.tps * kTile);
                 const float2 lN = lambda_pow(ga, om, nf);
-                const int64_t st = (int64_t)gridDim.z * D * M;
+                const int64_t st = (int64_t)A.B * D * M;
                 float2 S = z, R = z;
 #pragma unroll 4
                 for (int r = 0; r < seg; ++r) {
@@ -376,14 +382,14 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                 if (BWD) R0[q][j] = R;
             }
             if (kOut && cg == 0) cs[m] = cm[q][j];
-            if (!BWD && kOut && A.coef_out && b == 0 && seg == A.nseg - 1 && cg == 0 && on) {
+            if (!BWD && kOut && A.coef_out && blockIdx.z == 0 && seg == A.nseg - 1 && cg == 0 && on) {
                 const float2 l1 = lambda_pow(ga, om, 1.0f);
                 A.coef_out[d * M + m] = make_float4(l1.x, l1.y, cm[q][j].x, cm[q][j].y);
             }
             // The output launch's segment 0 starts from this copy: by then a state_out that
             // is state_in's buffer may be written by the last segment's block.
             if (!kOut && !BWD && seg == 0 && A.enter && cg == 0 && on)
-                A.seg_s[sm + (int64_t)(A.nseg - 1) * gridDim.z * D * M] = S0[q][j];
+                A.seg_s[sm + (int64_t)(A.nseg - 1) * A.B * D * M] = S0[q][j];
         }
     __syncwarp();
     if (kOut) {
@@ -415,12 +421,17 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
     const int tile_end = min(A.ntiles, (seg + 1) * A.tps);
     // The thread's 8 tokens of a tile, 4 channels each (zeros outside the sequence).
     const int Li = (int)A.L, t_last = A.nch * kC - 1;
+    // The thread's column: its batch row, and its first token's tau in tile 0.
+    const int fcol = tid & (kCols - 1), frow = (int)blockIdx.z * rpt + fcol / (4 * A.gpr);
+    const int ftau = (fcol & (4 * A.gpr - 1)) * kC + (tid >> 4);
+    const int64_t fbase = (int64_t)frow * A.L;
     auto fetch = [&](const void *f, int tile, float4 (&v)[8]) {
-        const int tau = tile * kTile + (tid & (kCols - 1)) * kC + (tid >> 4);
+        const int tau = tile * kTile + ftau;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int t = A.rev ? t_last - tau - 8 * i : tau + 8 * i;
-            v[i] = t >= 0 && t < Li ? load4(f, A.bf16, (b * A.L + t) * D + d0) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            v[i] = t >= 0 && t < Li && frow < A.B ? load4(f, A.bf16, (fbase + t) * D + d0)
+                                                  : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
     };
     // The 32-mode forward loads the next tile's drive ahead of this tile's outputs (67 -> 62
@@ -430,7 +441,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
     if (kAhead) fetch(A.u, seg * A.tps, nextu);
     for (int tile = seg * A.tps; tile < tile_end; ++tile) {
         // ---- stage the tile: thread (column, position), 4 channels each
-        const int t0 = tile * kTile + (tid & (kCols - 1)) * kC + (tid >> 4);   // tau of the thread's first token
+        const int t0 = tile * kTile + ftau;   // tau of the thread's first token
         bool odd = false;   // an infinite or NaN drive
         auto stage = [&](const float4 (&v)[8], float *base) {
 #pragma unroll
@@ -458,7 +469,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
         const bool guard = __syncthreads_or(kOut && odd);
 
         // ---- chunk-local states, carry over the 16 columns (and G, P)
-        const int chunk0 = tile * kCols + 4 * cg;
+        const int chunk0 = tile * kCols + 4 * (cg - gbase);   // the lane's first chunk
         u64 ls[NP][J][4];   // lambda S of the state entering each of the lane's columns
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
@@ -478,18 +489,19 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                                   unpack2(accq[j][c]));
                     es = cfma(a, es, unpack2(acc[j][c]));
                 }
-                // ... the state entering them (over the four lanes of the mode) ...
+                // ... the state entering them (over the mode's lanes in this row) ...
                 float2 T = S0[q][j], U = BWD ? R0[q][j] : T, S = T, R = U;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    if (i == cg) {
+                    if (i >= A.gpr) break;   // the same for every lane
+                    if (gbase + i == cg) {
                         S = T;
                         R = U;
                     }
-                    const float2 ei = shfl2(es, g + 8 * i);
+                    const float2 ei = shfl2(es, g + 8 * (gbase + i));
                     if (BWD)
                         U = cfma(a4, make_float2(fmaf(4.0f * kC, T.x, U.x), fmaf(4.0f * kC, T.y, U.y)),
-                                 shfl2(er, g + 8 * i));
+                                 shfl2(er, g + 8 * (gbase + i)));
                     T = cfma(a4, T, ei);
                 }
                 S0[q][j] = T;
@@ -506,7 +518,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                         R = cfma(a, make_float2(fmaf((float)kC, S.x, R.x), fmaf((float)kC, S.y, R.y)),
                                  unpack2(accq[j][c]));
                         S = cfma(a, S, unpack2(acc[j][c]));
-                        if (chunk0 + c == A.nch - 1 && on) {
+                        if (chunk0 + c == A.nch - 1 && on && mine) {
                             // The chunk of token 0: (S, R) is the adjoint pair there.
                             const int64_t sm = (b * D + d) * M + m;
                             const float2 l0 = cmul(lam, S);
@@ -528,7 +540,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                         }
                     } else {
                         const float2 next = cfma(a, S, unpack2(acc[j][c]));
-                        if (chunk0 + c == A.nch - 1 && on && A.state_out) {
+                        if (chunk0 + c == A.nch - 1 && on && mine && A.state_out) {
                             float2 f = next;
                             if (tail) {
                                 // The sequence ends inside this chunk.
@@ -574,12 +586,12 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                             }
                         }
                         if (tail && chunk0 == 0) {
-                            // The partial last chunk (column 0 of the first tile): its tokens are
+                            // The partial last chunk (the row's first column): its tokens are
                             // positions p >= 64 - tail, L - 1 - t = p - (64 - tail).
                             const float2 *row = pw + m * kPwStride;
                             for (int n = 0; n < tail; ++n) {
                                 const int p = n + kC - tail;
-                                const float v = (float)n * xs[slot(p >> 1, 0) + (p & 1)];
+                                const float v = (float)n * xs[slot(p >> 1, 2 * cg) + (p & 1)];
                                 Jg[q][j].x = fmaf(row[n].x, v, Jg[q][j].x);
                                 Jg[q][j].y = fmaf(row[n].y, v, Jg[q][j].y);
                             }
@@ -693,8 +705,8 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
             const int p = (tid >> 4) + 8 * i, col = tid & (kCols - 1);
             const float *o = base + slot(p >> 1, col >> 1) + 2 * (col & 1) + (p & 1);
             const int t = A.rev ? t_last - t0 - 8 * i : t0 + 8 * i;
-            if (t >= 0 && t < Li)
-                store4(A.out, A.bf16, (b * A.L + t) * D + d0, make_float4(o[0], o[kWords], o[2 * kWords], o[3 * kWords]));
+            if (t >= 0 && t < Li && frow < A.B)
+                store4(A.out, A.bf16, (fbase + t) * D + d0, make_float4(o[0], o[kWords], o[2 * kWords], o[3 * kWords]));
         }
     }
 
@@ -705,7 +717,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
 #pragma unroll
                 for (int j = 0; j < J; ++j) {
                     const int m = 8 * J * q + 8 * j + g;
-                    const int64_t o = (((int64_t)seg * gridDim.z + b) * D + d) * M + m;
+                    const int64_t o = (((int64_t)seg * A.B + b) * D + d) * M + m;
                     if (m < M) {
                         A.seg_s[o] = S0[q][j];
                         if (BWD) A.seg_r[o] = R0[q][j];
@@ -728,6 +740,11 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
             for (int j = 0; j < J; ++j) {
                 const int m = 8 * J * q + 8 * j + g;
                 float2 gs = G[q][j], ps = P[q][j], js = Jg[q][j];
+                if (A.g && m < M) {
+                    // conj(g) J, g the lane's row's (Jg of a row that does not exist is zero).
+                    const float2 gg = A.g[(b * D + d) * M + m];
+                    js = cmul(make_float2(gg.x, -gg.y), js);
+                }
                 for (int n = 16 * cg; n < 16 * cg + 16; ++n) {
                     const float2 z = pw[m * kPwStride + n];
                     const float r = kq[n], nr = (float)n * r;
@@ -746,13 +763,10 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                     js.y += __shfl_xor_sync(0xffffffffu, js.y, o);
                 }
                 if (cg == 0 && m < M) {
-                    const int64_t o = ((b * A.nseg + seg) * D + d) * M + m;
+                    const int64_t o = (((int64_t)blockIdx.z * A.nseg + seg) * D + d) * M + m;
                     A.part_g[o] = gs;
                     A.part_p[o] = ps;
-                    if (A.g) {
-                        const float2 gg = A.g[(b * D + d) * M + m];
-                        A.part_j[o] = cmul(make_float2(gg.x, -gg.y), js);
-                    }
+                    if (A.g) A.part_j[o] = js;
                 }
             }
     }
@@ -826,7 +840,8 @@ __global__ void __launch_bounds__(256) k_grad_reduce(
 // of the drive (38 % of the forward's FMA at M = 32, 31 % of the backward's), so they
 // are only taken when at least two of them fit.
 struct Geometry {
-    int nch, ntiles, nseg, tps;
+    int nch, ntiles, nseg, tps, gpr;
+    int zdim;   // blocks along the batch
 };
 
 Geometry geometry(int64_t B, int64_t L, int D, int M, bool bwd, int max_seg) {
@@ -838,11 +853,16 @@ Geometry geometry(int64_t B, int64_t L, int D, int M, bool bwd, int max_seg) {
     q.nseg = (int)std::max<int64_t>(1, std::min<int64_t>({slots / groups, (int64_t)q.ntiles, (int64_t)max_seg}));
     q.tps = (q.ntiles + q.nseg - 1) / q.nseg;
     q.nseg = (q.ntiles + q.tps - 1) / q.tps;
+    // Packed rows cost a block nothing and divide their number by up to four: at B = 22,
+    // L = 74, D = 88, M = 16 (fp32 backward with state terms) 484 blocks, just over one
+    // wave, become 132: 63.6 -> 32.8 us.
+    q.gpr = q.nch <= 4 ? 1 : q.nch <= 8 ? 2 : 4;
+    q.zdim = (int)((B * q.gpr + 3) / 4);
     return q;
 }
 
 template <int J, int NP, bool BWD, bool kOut>
-cudaError_t launch_scan(const ScanArgs &a, int64_t B, int nseg, cudaStream_t st) {
+cudaError_t launch_scan(const ScanArgs &a, int nseg, int zdim, cudaStream_t st) {
     constexpr int bytes = smem_bytes(8 * J * NP, BWD && kOut);
     auto *k = k_scan<J, NP, BWD, kOut>;
     if (bytes > 48 * 1024) {
@@ -858,24 +878,24 @@ cudaError_t launch_scan(const ScanArgs &a, int64_t B, int nseg, cudaStream_t st)
             done.fetch_or(bit, std::memory_order_release);
         }
     }
-    k<<<dim3((unsigned)(a.D / kCh), (unsigned)nseg, (unsigned)B), kThreads, bytes, st>>>(a);
+    k<<<dim3((unsigned)(a.D / kCh), (unsigned)nseg, (unsigned)zdim), kThreads, bytes, st>>>(a);
     count_launches(1);
     return cudaGetLastError();
 }
 
 template <bool BWD>
-cudaError_t run_scan(ScanArgs &a, int64_t B, cudaStream_t st) {
+cudaError_t run_scan(ScanArgs &a, int zdim, cudaStream_t st) {
     auto pass = [&](auto out, int nseg) {
         constexpr bool kOut = decltype(out)::value;
-        if (a.M <= 8) return launch_scan<1, 1, BWD, kOut>(a, B, nseg, st);
-        if (a.M <= 16) return launch_scan<2, 1, BWD, kOut>(a, B, nseg, st);
-        if (a.M <= 32) return launch_scan<4, 1, BWD, kOut>(a, B, nseg, st);
-        return launch_scan<4, 2, BWD, kOut>(a, B, nseg, st);
+        if (a.M <= 8) return launch_scan<1, 1, BWD, kOut>(a, nseg, zdim, st);
+        if (a.M <= 16) return launch_scan<2, 1, BWD, kOut>(a, nseg, zdim, st);
+        if (a.M <= 32) return launch_scan<4, 1, BWD, kOut>(a, nseg, zdim, st);
+        return launch_scan<4, 2, BWD, kOut>(a, nseg, zdim, st);
     };
     if (a.nseg > 1) {
         const cudaError_t e = pass(std::false_type{}, a.nseg - 1);
         if (e != cudaSuccess) return e;
-        if (!BWD && a.enter) a.enter = a.seg_s + (int64_t)(a.nseg - 1) * B * a.D * a.M;
+        if (!BWD && a.enter) a.enter = a.seg_s + (int64_t)(a.nseg - 1) * a.B * a.D * a.M;
     }
     return pass(std::true_type{}, a.nseg);
 }
@@ -924,6 +944,8 @@ cudaError_t simt_prefill(const void *x, void *y, rlm_dtype dt, int64_t B, int64_
     a.out = y;
     a.bf16 = dt == RLM_BF16;
     a.L = L;
+    a.B = (int)B;
+    a.gpr = q.gpr;
     a.D = D;
     a.M = M;
     a.nch = q.nch;
@@ -938,7 +960,7 @@ cudaError_t simt_prefill(const void *x, void *y, rlm_dtype dt, int64_t B, int64_
     a.enter = reinterpret_cast<const float2 *>(state_in);
     a.state_out = reinterpret_cast<float2 *>(state_out);
     a.coef_out = reinterpret_cast<float4 *>(coef_out);
-    return run_scan<false>(a, B, st);
+    return run_scan<false>(a, q.zdim, st);
 }
 
 cudaError_t grad_reduce(int64_t nparts, int D, int M, const float *amp, const float *phase,
@@ -966,6 +988,8 @@ cudaError_t simt_backward(const void *dy, const void *x, void *dx, rlm_dtype dt,
     a.bf16 = dt == RLM_BF16;
     a.rev = 1;
     a.L = L;
+    a.B = (int)B;
+    a.gpr = q.gpr;
     a.D = D;
     a.M = M;
     a.nch = q.nch;
@@ -984,9 +1008,9 @@ cudaError_t simt_backward(const void *dy, const void *x, void *dx, rlm_dtype dt,
     a.state_in = reinterpret_cast<const float2 *>(state_in);
     a.g = reinterpret_cast<const float2 *>(d_state_out);
     a.d_state_in = reinterpret_cast<float2 *>(d_state_in);
-    const cudaError_t e = run_scan<true>(a, B, st);
+    const cudaError_t e = run_scan<true>(a, q.zdim, st);
     if (e != cudaSuccess) return e;
-    return grad_reduce(B * q.nseg, D, M, amp, phase, a.part_g, a.part_p, d_state_out ? a.part_j : nullptr, g_decay,
+    return grad_reduce((int64_t)q.zdim * q.nseg, D, M, amp, phase, a.part_g, a.part_p, d_state_out ? a.part_j : nullptr, g_decay,
                        g_freq, g_amp, g_phase, st);
 }
 

@@ -34,6 +34,8 @@ def _state(B, D, M, seed):
     (2, 1, 16, 9, "f32"), (1, 63, 8, 33, "f32"), (3, 65, 16, 17, "f32"), (2, 127, 8, 64, "bf16"),
     (2, 1023, 16, 8, "bf16"), (1, 1025, 24, 1, "f32"), (2, 1087, 8, 16, "bf16"), (1, 2049, 16, 32, "f32"),
     (1, 20001, 8, 5, "f32"), (1, 9999, 8, 40, "bf16"),
+    # several batch rows in a tile (at most 4 or 8 chunks), the last tile partly empty
+    (5, 100, 8, 16, "bf16"), (6, 255, 16, 3, "f32"), (3, 257, 8, 20, "f32"), (5, 511, 8, 33, "f32"),
 ])
 def test_prefill_from_a_state_at_tile_edges(B, L, D, M, dtype):
     inp = make_inputs(B, L, D, M, dtype, seed=L + M)
@@ -72,6 +74,7 @@ def test_a_non_finite_drive_leaves_earlier_outputs_alone(bad, t):
 @pytest.mark.parametrize("B,L,D,M,dtype", [
     (1, 1, 8, 4, "f32"), (2, 63, 8, 8, "f32"), (1, 64, 16, 16, "f32"), (2, 100, 8, 33, "bf16"),
     (2, 1024, 8, 17, "f32"), (1, 1090, 16, 32, "f32"), (1, 12345, 8, 9, "f32"), (1, 4096, 8, 64, "f32"),
+    (9, 74, 8, 16, "f32"), (4, 256, 16, 32, "f32"), (3, 300, 8, 5, "f32"), (5, 512, 8, 40, "bf16"),
 ])
 def test_backward_with_state_terms_at_tile_edges(B, L, D, M, dtype):
     inp = make_inputs(B, L, D, M, dtype, seed=L + 3 * M, with_dy=True)
@@ -88,3 +91,28 @@ def test_backward_with_state_terms_at_tile_edges(B, L, D, M, dtype):
     d = ds.complex().cpu().numpy()
     assert_close(d.real, ref[1]["state_in"].real, TOL["f32"], "d_state re")
     assert_close(d.imag, ref[1]["state_in"].imag, TOL["f32"], "d_state im")
+
+
+# The tensor-core backward with several rows of a channel per block: one level of rows
+# (many short rows), three levels (few tiles, more blocks than fit at once), a ragged
+# length, and one row per block.  Rows must not see one another's carry: dx of each row
+# equals the row's own backward, and the gradients are the rows' sum.
+@pytest.mark.parametrize("B,L,D,M", [(7, 130, 96, 32), (40, 100, 64, 16), (9, 2049, 256, 8), (3, 64, 8, 1)])
+def test_backward_rows_sharing_a_block(B, L, D, M):
+    inp = make_inputs(B, L, D, M, "bf16", seed=B + L, with_dy=True)
+    p = rlm.Params.from_arrays(*inp.params())
+    x, dy = to_dev(inp.x, "bf16"), to_dev(inp.dy, "bf16")
+    (st, _), (gs, _) = _state(B, D, M, L), _state(B, D, M, L + 1)
+    dx, gr, ds = torch.empty_like(x), rlm.Grads.empty(D, M), rlm.State.empty(B, D, M)
+    rlm.rlm_mix_backward_from(dy, x, p, st, gs, dx, gr, ds)
+    total = {k: torch.zeros(D, M, dtype=torch.float64, device="cuda") for k in ("decay", "freq", "amp", "phase")}
+    for b in range(B):
+        one = lambda s: rlm.State(s.s[b:b + 1].contiguous(), s.coef)
+        dx1, g1, ds1 = torch.empty_like(x[b:b + 1]), rlm.Grads.empty(D, M), rlm.State.empty(1, D, M)
+        rlm.rlm_mix_backward_from(dy[b:b + 1].contiguous(), x[b:b + 1].contiguous(), p, one(st), one(gs), dx1, g1, ds1)
+        assert torch.equal(dx1[0], dx[b]) and torch.equal(ds1.s[0], ds.s[b])
+        for k in total:
+            total[k] += getattr(g1, k).double()
+    for k in total:
+        # fp32 sums of the same terms in another order.
+        assert_close(getattr(gr, k).cpu().numpy(), total[k].cpu().numpy(), 2e-5, k)
