@@ -52,7 +52,9 @@
 // written channel-major (64-byte runs per warp store) and a second transpose
 // writes the [B][L][D] field.
 //
-// One CTA = one (batch row, channel), two CTAs per SM (256 TMEM columns each):
+// One CTA = one channel of one or more batch rows (RowPlan below; the tables are the
+// channel's, Q and E accumulate over all rows, the carry restarts at each), two CTAs per
+// SM (256 TMEM columns each):
 //   warps 0-3  reverse scan; at the end they read E and form the cross-chunk
 //              (G, P).
 //   warps 4-5  dx epilogue (quarters 0, 1: positions 0-63), then the diagonal
@@ -298,13 +300,36 @@ __device__ __forceinline__ void store_pair_row(uint32_t buf, int r, int g, const
     st_shared_v4(a + 8192, l[0], l[1], l[2], l[3]);
 }
 
+// Which rows a CTA takes.  A CTA spends about 6 tiles' time on its tables, the pipeline's
+// fill and drain, so short sequences of many rows run several rows of a channel per CTA;
+// the grid then shrinks, and a last wave that is nearly empty costs more than the
+// prologues saved.  Up to three levels: blocks below end[0] take r[0] rows each, of
+// channels from 0 on, the next ones r[1] rows of channels from ch[1] on, and so on, fewer
+// rows each, so that the large units start first and small ones fill the tail.  Same box,
+// one row per block and now: B = 8, L = 4096, D = 256, M = 16 with both state terms (this
+// kernel and k_terminal_tc) 157 -> 96 us; B = 4, L = 32768, D = 512, M = 32 (16 tiles a
+// row) with the forward 445 -> 416; B = 7, L = 465, D = 160, M = 32 66 -> 49.
+struct RowPlan {
+    int r[3];       // rows per block of the level
+    int end[3];     // one past the level's last block
+    int ch[3];      // the level's first channel
+    int B, D;
+};
+__device__ __forceinline__ void rows_of(const RowPlan &p, int blk, int &d, int &b0, int &nrows) {
+    const int l = blk < p.end[0] ? 0 : blk < p.end[1] ? 1 : 2;
+    const int r = p.r[l], u = (p.B + r - 1) / r, at = blk - (l ? p.end[l - 1] : 0);
+    d = p.ch[l] + at / u;
+    b0 = at % u * r;
+    nrows = min(r, p.B - b0);
+}
+
 struct BwdArgs {
     const float *decay, *freq, *amp, *phase;
     float2 *part_g, *part_p;  // [B*D][M] (backward)
     const float2 *state_in;   // nullable, [B*D][M] (time-reversed prefill: state before token 0)
     float2 *state_out;        // nullable, [B*D][M] (time-reversed prefill)
     int64_t L;
-    int row0;                 // first (b * D + d) row of this launch (0: the whole problem)
+    RowPlan plan;
     float4 *coef_out;         // nullable, [D][M]   (time-reversed prefill)
     float2 *d_state_in;       // nullable, [B*D][M] (backward: gradient of the forward's state_in)
     __nv_bfloat16 *dxT;       // [B*D][Lp]
@@ -329,9 +354,13 @@ __global__ void __launch_bounds__(kThreads, 2)
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int row = args.row0 + blockIdx.x;     // b * D + d
-    const int d = row % args.D;
+    // The time-reversed prefill keeps one row per CTA: it serves few rows, and the row
+    // bookkeeping cost it 3 %.
+    int d = blockIdx.x % args.D, b0 = blockIdx.x / args.D, nrows = 1;
+    if (kGrad) rows_of(args.plan, blockIdx.x, d, b0, nrows);
+    const int row0 = b0 * args.D + d;           // b * D + d of the first row; the next ones D apart
     const int M = args.M, ntiles = args.ntiles;
+    const int nv = kGrad ? nrows * ntiles : ntiles;   // tiles of the walk: each row's in reverse, row after row
     const int w_prod = 6;
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kOffBar);
     auto bar = [&](int i) { return smem_u32(bars + i); };
@@ -365,10 +394,10 @@ __global__ void __launch_bounds__(kThreads, 2)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    // Tile v of the reverse walk is tile ntiles - 1 - v of the sequence.
+    // Tile v of the walk is tile ntiles - 1 - v % ntiles of row v / ntiles.
     auto load_tile = [&](int v) {
-        const int slot = v % kSlots;
-        const int chunk0 = (ntiles - 1 - v) * kNT;
+        const int slot = v % kSlots, rr = kGrad ? v / ntiles : 0;
+        const int chunk0 = (ntiles - 1 - (v - rr * ntiles)) * kNT, row = row0 + rr * args.D;
         const uint32_t dst = sbase + kOffRing + slot * kSlotBytes;
         bar_expect_tx(bar(kBarSlotFull + slot), kGrad ? 8192u : 4096u);
         tma_load_3d(dst, &tmap_dy, 0, chunk0, row, bar(kBarSlotFull + slot));
@@ -376,7 +405,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     };
     int issued = 0;
     if (warp == w_prod && lane == 0)
-        for (; issued < ntiles && issued < kSlots; ++issued) load_tile(issued);
+        for (; issued < nv && issued < kSlots; ++issued) load_tile(issued);
 
     // ------------------------------------------------------------ constants
     // Stage 1: lambda^n (n = 0..64) and c for every mode slot (zero past M):
@@ -475,7 +504,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     __syncthreads();
     tc_fence_after();
 
-    const int last = ntiles - 1;
+    const int last = nv - 1;
     // Scan lanes: lane l of quarter q owns row 32 q + l of the projections and of
     // [S^n ; R^n] (mode mE = 8 q + (l % 16) / 2; role s = 2 (l >= 16) + l % 2:
     // Re / Im of Dp and S^n, of Dq and R^n); their cross-chunk (G, P) from E is
@@ -484,7 +513,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     const bool onE = warp < 4 && mE < M;
     const float gamE = onE ? args.decay[d * M + mE] : 0.0f, omgE = onE ? args.freq[d * M + mE] : 0.0f;
     float gr = 0.0f, gi = 0.0f, pr = 0.0f, pi = 0.0f;
-    // The adjoint pair of the scan lanes; after the last tile it is (S_0, R_0).
+    // The adjoint pair of the scan lanes; after a row's last tile it is (S_0, R_0).
     float2 S = make_float2(0.0f, 0.0f), R = make_float2(0.0f, 0.0f);
     if (warp < 4) {
         // ---------------------------------------------------- reverse chunk scan
@@ -499,11 +528,13 @@ __global__ void __launch_bounds__(kThreads, 2)
             const int64_t Lr = (args.L + kC - 1) / kC * kC;
             kinj = (int)(Lr / kC) - 1;
             if (onE)
-                inj = cmul(lambda_pow(gamE, omgE, (float)(args.L - Lr)), args.state_in[(int64_t)row * M + mE]);
+                inj = cmul(lambda_pow(gamE, omgE, (float)(args.L - Lr)), args.state_in[(int64_t)row0 * M + mE]);
         }
         bool ok = true;
-        for (int v = 0; v < ntiles && ok; ++v) {
+        int row = row0, tv = 0;   // the current row and its tile
+        for (int v = 0; v < nv && ok; ++v) {
             const int bb = v & 1;
+            if (kGrad && tv == 0) S = R = make_float2(0.0f, 0.0f);
             if (!wait_bar(bar(kBarPFull + bb), (v >> 1) & 1, abort_flag)) break;
             tc_fence_after();
             if (warp == 0 && lane == 0) bar_arrive(bar(kBarSlotEmpty + v % kSlots));
@@ -548,18 +579,42 @@ __global__ void __launch_bounds__(kThreads, 2)
             fence_async_smem();
             __syncwarp();
             if (lane == 0) bar_arrive(bar(kBarSFull + bb));
-        }
-        if (!kGrad) {
-            // The adjoint state after the first chunk is the prompt's terminal state.
-            if (ok && s == 0 && onE) {
-                if (args.state_out) args.state_out[(int64_t)row * M + mE] = S;
-                if (args.coef_out && row < args.D) {
-                    const float2 l1 = lambda_pow(gamE, omgE, 1.0f);
+            if (!kGrad || ++tv < ntiles) continue;
+            // The row's end: (S, R) is the adjoint pair at token 0.  The forward's initial
+            // state s_in (Sec. 3.2-3.3): G += s_in lambda S_0, P += s_in lambda (R_0 + S_0),
+            // once per mode; the gradient of s_in is conj(c lambda S_0).
+            if (s == 0 && onE && (args.state_in || args.d_state_in)) {
+                const int64_t at = (int64_t)row * M + mE;
+                const float2 l1 = lambda_pow(gamE, omgE, 1.0f);
+                const float2 ls = cmul(l1, S);
+                if (args.state_in) {
+                    const float2 si = args.state_in[at];
+                    const float2 gin = cmul(si, ls), pin = cmul(si, cmul(l1, make_float2(R.x + S.x, R.y + S.y)));
+                    gr += gin.x;
+                    gi += gin.y;
+                    pr += pin.x;
+                    pi += pin.y;
+                }
+                if (args.d_state_in) {
                     const float2 c = mode_coef(args.amp[d * M + mE], args.phase[d * M + mE]);
-                    args.coef_out[d * M + mE] = make_float4(l1.x, l1.y, c.x, c.y);
+                    const float2 cls = cmul(c, ls);
+                    args.d_state_in[at] = make_float2(cls.x, -cls.y);
                 }
             }
-        } else if (ok && wait_bar(bar(kBarDFull + (last & 1)), (last >> 1) & 1, abort_flag)) {
+            __syncwarp();   // the next tile's tensor-memory loads are warp-wide
+            tv = 0;
+            row += args.D;
+        }
+        if (!kGrad && ok && s == 0 && onE) {
+            // The adjoint state after the first chunk is the prompt's terminal state.
+            if (args.state_out) args.state_out[(int64_t)row0 * M + mE] = S;
+            if (args.coef_out && row0 < args.D) {
+                const float2 l1 = lambda_pow(gamE, omgE, 1.0f);
+                const float2 c = mode_coef(args.amp[d * M + mE], args.phase[d * M + mE]);
+                args.coef_out[d * M + mE] = make_float4(l1.x, l1.y, c.x, c.y);
+            }
+        }
+        if (kGrad && ok && wait_bar(bar(kBarDFull + (last & 1)), (last >> 1) & 1, abort_flag)) {
             // E = [S^n ; R^n] X over the sequence, complete with the last dx product.
             tc_fence_after();
             // Weights lambda^(C-i), i = 63 .. 0, by successive products.
@@ -583,7 +638,7 @@ __global__ void __launch_bounds__(kThreads, 2)
                 }
             }
             // G = sum w (E_S.re + i E_S.im), P = sum w E_R + sum (C - i) w E_S.
-            if (s == 0) { gr = a1; gi = a2; pr = a3; pi = a4; }
+            if (s == 0) { gr += a1; gi += a2; pr += a3; pi += a4; }
             else if (s == 1) { gr = -a2; gi = a1; pr = -a4; pi = a3; }
             else if (s == 2) { pr = a1; pi = a2; }
             else { pr = -a2; pi = a1; }
@@ -593,7 +648,10 @@ __global__ void __launch_bounds__(kThreads, 2)
         const int q = warp & 3;   // 0 or 1: positions 32 q + lane
         const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16);
         bool ok = true;
-        for (int v = 0; v < ntiles; ++v) {
+        // The tile's positions in dxT: rows D apart, tiles from the end of each.
+        __nv_bfloat16 *rowp = args.dxT + (int64_t)row0 * args.Lp + 32 * q + lane;
+        int tile = ntiles - 1;
+        for (int v = 0; v < nv; ++v) {
             const int bb = v & 1;
             if (!wait_bar(bar(kBarDFull + bb), (v >> 1) & 1, abort_flag)) {
                 ok = false;
@@ -614,11 +672,15 @@ __global__ void __launch_bounds__(kThreads, 2)
                 }
             }
             // Channel-major dx: each store instruction writes 64 contiguous bytes.
-            __nv_bfloat16 *out = args.dxT + (int64_t)row * args.Lp + (int64_t)(last - v) * kTile + 32 * q + lane;
+            __nv_bfloat16 *out = rowp + (int64_t)tile * kTile;
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
                 out[k * kC] = __float2bfloat16_rn(__uint_as_float(r0[k]));
                 out[(k + 16) * kC] = __float2bfloat16_rn(__uint_as_float(r1[k]));
+            }
+            if (--tile < 0 && kGrad) {
+                tile = ntiles - 1;
+                rowp += (int64_t)args.D * args.Lp;
             }
         }
         // Diagonal sums of Q (accumulated over the whole sequence; its last
@@ -658,7 +720,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     } else if (warp == w_prod) {
         // ---------------------------------------------------- TMA producer
         if (lane == 0) {
-            for (; issued < ntiles; ++issued) {
+            for (; issued < nv; ++issued) {
                 const int slot = issued % kSlots;
                 if (!wait_bar(bar(kBarSlotEmpty + slot), ((issued / kSlots) & 1) ^ 1, abort_flag)) break;
                 load_tile(issued);
@@ -674,7 +736,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             const uint64_t dap = desc_plain(sbase + kOffAP, 128, 1024);
             const uint64_t dapl = desc_plain(sbase + kOffAPlo, 128, 1024);
             int v = 0;
-            for (; v < ntiles; ++v) {
+            for (; v < nv; ++v) {
                 const int slot = v % kSlots, bb = v & 1;
                 if (!wait_bar(bar(kBarSlotFull + slot), (v / kSlots) & 1, abort_flag)) break;
                 if (!wait_bar(bar(kBarPEmpty + bb), ((v >> 1) & 1) ^ 1, abort_flag)) break;
@@ -709,7 +771,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             const uint64_t dt = desc_plain(sbase + kOffT, 128, 1024);
             const uint64_t du = desc_plain(sbase + kOffU, 128, 1024);
             int v = 0;
-            for (; v < ntiles; ++v) {
+            for (; v < nv; ++v) {
                 const int slot = v % kSlots, bb = v & 1;
                 if (!wait_bar(bar(kBarSlotFull + slot), (v / kSlots) & 1, abort_flag)) break;
                 if (!wait_bar(bar(kBarDEmpty + bb), ((v >> 1) & 1) ^ 1, abort_flag)) break;
@@ -773,26 +835,6 @@ __global__ void __launch_bounds__(kThreads, 2)
             pi = fmaf(r * (float)n, ln.y, pi);
             ln = cmul(ln, l4);
         }
-        // The forward's initial state s_in (Sec. 3.2-3.3): G += s_in lambda S_0,
-        // P += s_in lambda (R_0 + S_0), added once per mode before the lanes' sum; the
-        // gradient of s_in is conj(c lambda S_0).
-        if (s == 0 && onE && (args.state_in || args.d_state_in)) {
-            const float2 l1 = lambda_pow(gamE, omgE, 1.0f);
-            const float2 ls = cmul(l1, S);
-            if (args.state_in) {
-                const float2 si = args.state_in[(int64_t)row * M + mE];
-                const float2 gin = cmul(si, ls), pin = cmul(si, cmul(l1, make_float2(R.x + S.x, R.y + S.y)));
-                gr += gin.x;
-                gi += gin.y;
-                pr += pin.x;
-                pi += pin.y;
-            }
-            if (args.d_state_in) {
-                const float2 c = mode_coef(args.amp[d * M + mE], args.phase[d * M + mE]);
-                const float2 cls = cmul(c, ls);
-                args.d_state_in[(int64_t)row * M + mE] = make_float2(cls.x, -cls.y);
-            }
-        }
 #pragma unroll
         for (int o = 1; o <= 16; o <<= 4) {
             gr += __shfl_xor_sync(0xffffffffu, gr, o);
@@ -801,8 +843,12 @@ __global__ void __launch_bounds__(kThreads, 2)
             pi += __shfl_xor_sync(0xffffffffu, pi, o);
         }
         if (s == 0 && onE) {
-            args.part_g[(int64_t)row * M + mE] = make_float2(gr, gi);
-            args.part_p[(int64_t)row * M + mE] = make_float2(pr, pi);
+            // The sums of all rows in the first one's place, zeros in the others'.
+            for (int r = 0; r < nrows; ++r) {
+                const int64_t at = (int64_t)(row0 + r * args.D) * M + mE;
+                args.part_g[at] = r ? make_float2(0.0f, 0.0f) : make_float2(gr, gi);
+                args.part_p[at] = r ? make_float2(0.0f, 0.0f) : make_float2(pr, pi);
+            }
         }
     }
 }
@@ -822,8 +868,8 @@ __global__ void __launch_bounds__(kThreads, 2)
 // both on the tensor cores (p, q: the projections of the main pass with the
 // table reversed in i; dx: an up-projection of W).  The one chunk that holds
 // token L - 1 without ending there (L % 64 != 0) is evaluated directly in fp32,
-// so no negative power of lambda is ever formed.  One CTA per row, walking the
-// tiles from the end of the sequence:
+// so no negative power of lambda is ever formed.  One CTA per row or run of rows of
+// one channel (RowPlan), walking each row's tiles from the end of the sequence:
 //   warps 0-3  per tile: the chunk weights W_n = conj(g) lambda^E_n (steps of
 //              lambda^64 in four chains; each tile's first weight carried from
 //              the previous tile by lambda^2048), the W rows, and conj(g) J from
@@ -847,9 +893,7 @@ constexpr int kTmOffRing = 32768;                           // [kTmSlots] x (4 K
 constexpr int kTmSlotBytes = 8192;
 constexpr int kTmOffW = kTmOffRing + kTmSlots * kTmSlotBytes;   // [2] W buffers, 8 KB each (pair layout)
 constexpr int kTmOffPw = kTmOffW + 2 * 8192;                // [32][65] float2: lambda^s, s = 0..64
-constexpr int kTmOffG = kTmOffPw + kMaxModes * kPwStride * 8;   // [32] float2: g
-constexpr int kTmOffXp = kTmOffG + kMaxModes * 8;          // [64] fp32: x of the chunk holding token L - 1
-constexpr int kTmOffBar = kTmOffXp + kC * 4;
+constexpr int kTmOffBar = kTmOffPw + kMaxModes * kPwStride * 8;
 constexpr int kTmNumBars = 24;
 constexpr int kTmOffMisc = kTmOffBar + kTmNumBars * 8;
 constexpr int kTmSmemBytes = kTmOffMisc + 64 + 1024;        // + alignment slack
@@ -871,6 +915,7 @@ struct TermArgs {
     __nv_bfloat16 *dxT;            // [B*D][Lp]: += the g term of dx
     int64_t L, Lp;
     int D, M, ntiles;
+    RowPlan plan;
 };
 
 __global__ void __launch_bounds__(kTmThreads, 2)
@@ -880,16 +925,16 @@ __global__ void __launch_bounds__(kTmThreads, 2)
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const uint32_t sbase = smem_u32(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int row = blockIdx.x;     // b * D + d
-    const int d = row % args.D;
-    const int M = args.M, ntiles = args.ntiles;
+    int d, b0, nrows;
+    rows_of(args.plan, blockIdx.x, d, b0, nrows);
+    const int row0 = b0 * args.D + d;   // b * D + d of the first row; the next ones D apart
+    const int M = args.M, ntiles = args.ntiles, nv = nrows * ntiles;
     const int64_t L = args.L;
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kTmOffBar);
     auto bar = [&](int i) { return smem_u32(bars + i); };
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + kTmOffMisc);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + kTmOffMisc + 16);
     float2 *pw = reinterpret_cast<float2 *>(smem + kTmOffPw);
-    float2 *gs = reinterpret_cast<float2 *>(smem + kTmOffG);
 
     if (tid == 0) {
         *abort_flag = 0;
@@ -932,13 +977,6 @@ __global__ void __launch_bounds__(kTmThreads, 2)
 #pragma unroll
             for (int k = 0; k < 8; ++k) o[k] = make_float2(0.0f, 0.0f);
             if (e == 7) o[8] = make_float2(0.0f, 0.0f);
-        }
-        if (tid < kMaxModes) gs[tid] = tid < M ? args.g[(int64_t)row * M + tid] : make_float2(0.0f, 0.0f);
-        // x of the chunk holding token L - 1 when it does not end there.
-        if (tid >= 64 && tid < 64 + kC && (L % kC) != 0) {
-            const int64_t j = (L - 1) / kC * kC + (tid - 64);
-            reinterpret_cast<float *>(smem + kTmOffXp)[tid - 64] =
-                j < L ? __bfloat162float(args.xT[(int64_t)row * args.Lp + j]) : 0.0f;
         }
     }
     __syncthreads();
@@ -984,7 +1022,6 @@ __global__ void __launch_bounds__(kTmThreads, 2)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const int last = ntiles - 1;
     // The chunk holding token L - 1 when it does not end there (-1: none).
     const int64_t n_part = (L % kC) ? (L - 1) / kC : -1;
 
@@ -998,7 +1035,6 @@ __global__ void __launch_bounds__(kTmThreads, 2)
         const float2 l64 = lambda_pow(gam, omg, (float)kC), l2048 = lambda_pow(gam, omg, (float)kTile);
         const float2 l512 = lambda_pow(gam, omg, 512.0f), l1024 = lambda_pow(gam, omg, 1024.0f),
                      l1536 = lambda_pow(gam, omg, 1536.0f);
-        const float2 gc = on ? conj2(gs[m]) : make_float2(0.0f, 0.0f);
         const int prow = 32 * q + (l & 15);   // this lane's W row
         // The last chunk that ends at or before token L - 1 (-1: none).
         const int64_t nfull = L >= kC ? (L - kC) / kC : -1;
@@ -1006,9 +1042,15 @@ __global__ void __launch_bounds__(kTmThreads, 2)
         float2 T = make_float2(0.0f, 0.0f);   // lambda^E of the next tile's chunk 31, once known
         bool haveT = false;
         bool ok = true;
-        for (int v = 0; v < ntiles && ok; ++v) {
+        int row = row0, tv = 0;   // the current row and its tile
+        float2 gc = make_float2(0.0f, 0.0f);   // conj(g) of the row
+        for (int v = 0; v < nv && ok; ++v) {
             const int bb = v & 1;
-            const int64_t n0 = (int64_t)(last - v) * kNT;   // the tile's first chunk
+            if (tv == 0) {
+                haveT = false;
+                if (on) gc = conj2(args.g[(int64_t)row * M + m]);
+            }
+            const int64_t n0 = (int64_t)(ntiles - 1 - tv) * kNT;   // the tile's first chunk
             // Weights W_n = conj(g) lambda^E_n of the tile's chunks, E_n = L - 64 - 64 n
             // (zero where E_n < 0), from the tile's last full chunk ctop down by steps
             // of lambda^64.  lambda^E at ctop is an exact power in the first one or
@@ -1096,50 +1138,60 @@ __global__ void __launch_bounds__(kTmThreads, 2)
                 jr[c & 3] = fmaf(ri ? -w[c].y : w[c].x, val, jr[c & 3]);
                 ji[c & 3] = fmaf(ri ? w[c].x : w[c].y, val, ji[c & 3]);
             }
-        }
-        // The chunk holding token L - 1 (L % 64 != 0): its part of J directly, one
-        // lane per mode.
-        if (ok && on && !jordan && ri == 0 && n_part >= 0) {
-            const float *xp = reinterpret_cast<const float *>(smem + kTmOffXp);
-            const int cnt = (int)(L - n_part * kC);   // tokens of the chunk before L
-            float pr = 0.0f, pi = 0.0f;
-            for (int i = 0; i < cnt; ++i) {
-                const int s = cnt - 1 - i;
-                const float xv = xp[i] * (float)s;
-                const float2 p = pw[m * kPwStride + s];
-                pr = fmaf(p.x, xv, pr);
-                pi = fmaf(p.y, xv, pi);
+            if (++tv < ntiles) continue;
+            // The row's end, one lane per mode: the part of J of the chunk that holds
+            // token L - 1 (L % 64 != 0) directly, and the state terms.
+            if (on && !jordan && ri == 0) {
+                if (n_part >= 0) {
+                    const __nv_bfloat16 *xp = args.xT + (int64_t)row * args.Lp + n_part * kC;
+                    const int cnt = (int)(L - n_part * kC);   // tokens of the chunk before L
+                    float pr = 0.0f, pi = 0.0f;
+                    for (int i = 0; i < cnt; ++i) {
+                        const int e = cnt - 1 - i;
+                        const float xv = __bfloat162float(xp[i]) * (float)e;
+                        const float2 p = pw[m * kPwStride + e];
+                        pr = fmaf(p.x, xv, pr);
+                        pi = fmaf(p.y, xv, pi);
+                    }
+                    const float2 t = cmul(gc, make_float2(pr, pi));
+                    jr[0] += t.x;
+                    ji[0] += t.y;
+                }
+                const float2 lL = lambda_pow(gam, omg, (float)L);
+                const int64_t at = (int64_t)row * M + m;
+                if (args.state_in) {
+                    const float2 t = cmul(gc, cmul(args.state_in[at], lL));
+                    jr[1] = fmaf((float)L, t.x, jr[1]);
+                    ji[1] = fmaf((float)L, t.y, ji[1]);
+                }
+                if (args.d_state_in) {
+                    const float2 prev = args.d_state_in[at];
+                    args.d_state_in[at] = cfma(conj2(gc), conj2(lL), prev);
+                }
             }
-            const float2 t = cmul(gc, make_float2(pr, pi));
-            jr[0] += t.x;
-            ji[0] += t.y;
+            __syncwarp();   // the next tile's tensor-memory loads are warp-wide
+            tv = 0;
+            row += args.D;
         }
         float jsr = (jr[0] + jr[1]) + (jr[2] + jr[3]), jsi = (ji[0] + ji[1]) + (ji[2] + ji[3]);
-        // The mode's four rows, then the state terms.
+        // The mode's four rows.
         jsr += __shfl_xor_sync(0xffffffffu, jsr, 1);
         jsi += __shfl_xor_sync(0xffffffffu, jsi, 1);
         jsr += __shfl_xor_sync(0xffffffffu, jsr, 16);
         jsi += __shfl_xor_sync(0xffffffffu, jsi, 16);
         if (ok && on && !jordan && ri == 0) {
-            const float2 lL = lambda_pow(gam, omg, (float)L);
-            float2 J = make_float2(jsr, jsi);   // conj(g) J
-            const int64_t at = (int64_t)row * M + m;
-            if (args.state_in) {
-                const float2 t = cmul(gc, cmul(args.state_in[at], lL));
-                J = make_float2(fmaf((float)L, t.x, J.x), fmaf((float)L, t.y, J.y));
-            }
-            args.part_j[at] = J;
-            if (args.d_state_in) {
-                const float2 gg = gs[m], prev = args.d_state_in[at];
-                args.d_state_in[at] = cfma(gg, conj2(lL), prev);
-            }
+            // The sum of all rows in the first one's place, zeros in the others'.
+            for (int r = 0; r < nrows; ++r)
+                args.part_j[(int64_t)(row0 + r * args.D) * M + m] =
+                    r ? make_float2(0.0f, 0.0f) : make_float2(jsr, jsi);   // conj(g) J
         }
     } else if (warp < 6) {
         // ---------------------------------------------------- dx epilogue
         const int q = warp & 3;   // positions 32 q + lane
         const int i = 32 * q + lane;
         const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16);
-        for (int v = 0; v < ntiles; ++v) {
+        int row = row0, tile = ntiles - 1;
+        for (int v = 0; v < nv; ++v) {
             const int bb = v & 1, slot = v % kTmSlots;
             // The old dx values of this tile (plain [chunk][position] layout).
             if (!wait_bar(bar(kTmSlotFull + slot), (v / kTmSlots) & 1, abort_flag)) break;
@@ -1159,7 +1211,7 @@ __global__ void __launch_bounds__(kTmThreads, 2)
             tc_fence_before();
             __syncwarp();
             if (lane == 0) bar_arrive(bar(kTmDEmpty + bb));
-            const int64_t n0 = (int64_t)(last - v) * kNT;
+            const int64_t n0 = (int64_t)tile * kNT;
             float add[kNT];
 #pragma unroll
             for (int c = 0; c < 16; ++c) {
@@ -1173,7 +1225,7 @@ __global__ void __launch_bounds__(kTmThreads, 2)
                 if (j < L) {
                     const int s = (int)(L - 1 - j);
                     for (int mm = 0; mm < M; ++mm) {
-                        const float2 p = pw[mm * kPwStride + s], gg = gs[mm];
+                        const float2 p = pw[mm * kPwStride + s], gg = args.g[(int64_t)row * M + mm];
                         fx = fmaf(gg.x, p.x, fmaf(gg.y, p.y, fx));   // Re(conj(g) lambda^s)
                     }
                 }
@@ -1187,19 +1239,28 @@ __global__ void __launch_bounds__(kTmThreads, 2)
             __nv_bfloat16 *out = args.dxT + (int64_t)row * args.Lp + n0 * kC + i;
 #pragma unroll
             for (int c = 0; c < kNT; ++c) out[c * kC] = __float2bfloat16_rn(prev[c] + add[c]);
+            if (--tile < 0) {
+                tile = ntiles - 1;
+                row += args.D;
+            }
         }
     } else if (warp == 6) {
         // ---------------------------------------------------- TMA producer
         if (lane == 0) {
             int issued = 0;
-            for (; issued < ntiles; ++issued) {
+            int row = row0, tile = ntiles - 1;
+            for (; issued < nv; ++issued) {
                 const int slot = issued % kTmSlots;
                 if (!wait_bar(bar(kTmSlotEmpty + slot), ((issued / kTmSlots) & 1) ^ 1, abort_flag)) break;
                 bar_expect_tx(bar(kTmSlotFull + slot), 8192u);
-                tma_load_3d(sbase + kTmOffRing + slot * kTmSlotBytes, &tmap_x, 0, (last - issued) * kNT, row,
+                tma_load_3d(sbase + kTmOffRing + slot * kTmSlotBytes, &tmap_x, 0, tile * kNT, row,
                             bar(kTmSlotFull + slot));
-                tma_load_3d(sbase + kTmOffRing + slot * kTmSlotBytes + 4096, &tmap_dx, 0, (last - issued) * kNT, row,
+                tma_load_3d(sbase + kTmOffRing + slot * kTmSlotBytes + 4096, &tmap_dx, 0, tile * kNT, row,
                             bar(kTmSlotFull + slot));
+                if (--tile < 0) {
+                    tile = ntiles - 1;
+                    row += args.D;
+                }
             }
             for (int k = issued > kTmSlots ? issued - kTmSlots : 0; k < issued; ++k)
                 drain_bar(bar(kTmSlotFull + k % kTmSlots), (k / kTmSlots) & 1);
@@ -1213,7 +1274,7 @@ __global__ void __launch_bounds__(kTmThreads, 2)
             const uint64_t du = desc_plain(sbase + kTmOffU, 128, 1024);
             int last_bar = -1;
             uint32_t last_par = 0;
-            for (int v = 0; v < ntiles; ++v) {
+            for (int v = 0; v < nv; ++v) {
                 const int slot = v % kTmSlots, bb = v & 1;
                 if (!wait_bar(bar(kTmSlotFull + slot), (v / kTmSlots) & 1, abort_flag)) break;
                 if (!wait_bar(bar(kTmPEmpty + bb), ((v >> 1) & 1) ^ 1, abort_flag)) break;
@@ -1484,6 +1545,9 @@ size_t tc_backward_ws_bytes(int64_t B, int64_t L, int D, int M) {
 
 namespace {
 
+// Longest walk of a block over several rows, in tiles (Q and E accumulate over it).
+constexpr int kMaxWalk = 64;
+
 cudaError_t configure_once() {
     static std::mutex mu;
     static std::vector<int> configured;
@@ -1522,8 +1586,46 @@ BwdArgs base_args(const float *decay, const float *freq, const float *amp, const
     a.M = M;
     a.ntiles = (int)(Lp / kTile);
     a.L = 0;
-    a.row0 = 0;
     return a;
+}
+
+// The row plan with the shortest estimated walk, in units of one tile: the plain waves of
+// every number of blocks per channel, and the descending levels r, r / 2, 1 that each
+// fill whole waves of the resident blocks.  kFill: tables, fill and drain of a block.
+RowPlan row_plan(int64_t B, int D, int ntiles) {
+    constexpr int64_t kFill = 6;
+    const int64_t slots = 2 * sm_count();
+    RowPlan best = {{1, 1, 1}, {(int)(B * D), (int)(B * D), (int)(B * D)}, {0, 0, 0}, (int)B, D};
+    int64_t cost = (B * D + slots - 1) / slots * (kFill + ntiles);
+    if (ntiles > kMaxWalk / 2) return best;
+    for (int64_t r = B; r > 1; r = (r + 1) / 2) {
+        if (r * ntiles > kMaxWalk) continue;
+        RowPlan p = {{1, 1, 1}, {0, 0, 0}, {0, 0, 0}, (int)B, D};
+        int64_t left = D, blocks = 0, c = 0, rl = r;
+        for (int l = 0; l < 3; ++l, rl = l == 2 ? 1 : (rl + 1) / 2) {
+            const int64_t u = (B + rl - 1) / rl, per = kFill + rl * ntiles;
+            // Whole waves of this level (the last one takes what is left).
+            const int64_t waves = l < 2 && rl > 1 ? left * u / slots : (left * u + slots - 1) / slots;
+            const int64_t chans = l < 2 && rl > 1 ? std::min(left, waves * slots / u) : left;
+            p.r[l] = (int)rl;
+            p.ch[l] = (int)(D - left);
+            left -= chans;
+            blocks += chans * u;
+            p.end[l] = (int)blocks;
+            c += (chans > 0 ? waves : 0) * per;
+        }
+        if (c < cost) {
+            cost = c;
+            best = p;
+        }
+        const int64_t u = (B + r - 1) / r, cs = (D * u + slots - 1) / slots * (kFill + r * ntiles);
+        if (cs < cost) {
+            cost = cs;
+            const int n = (int)(D * u);
+            best = RowPlan{{(int)r, (int)r, (int)r}, {n, n, n}, {0, 0, 0}, (int)B, D};
+        }
+    }
+    return best;
 }
 
 // One call: transpose in (nf fields: x, or x and dy), the tcgen05 kernel, transpose
@@ -1539,8 +1641,8 @@ cudaError_t run_layout_and_scan(const CUtensorMap &mdy, const CUtensorMap &mx, B
     const unsigned cg = (unsigned)((D + 63) / 64);
     k_to_channel_major<<<dim3((unsigned)(Lp / 64), cg, (unsigned)(B * nf)), 128, 0, st>>>(
         src0, src1, dst0, dst1, L, D, Lp, nf, rev);
-    a.row0 = 0;
-    k_backward_tc<kGrad><<<(unsigned)(B * D), kThreads, kSmemBytes, st>>>(mdy, mx, a);
+    if (kGrad) a.plan = row_plan(B, D, a.ntiles);
+    k_backward_tc<kGrad><<<(unsigned)(kGrad ? a.plan.end[2] : B * D), kThreads, kSmemBytes, st>>>(mdy, mx, a);
     if (rev)
         k_to_row_major<<<dim3((unsigned)((L + 63) / 64), cg, (unsigned)B), 128, 0, st>>>(outT, out, L, D, Lp, rev);
     else
@@ -1590,8 +1692,10 @@ cudaError_t tc_backward(const void *dy, const void *x, void *dx, int64_t B, int6
         const unsigned cg = (unsigned)((D + 63) / 64);
         k_to_channel_major<<<dim3((unsigned)(Lp / 64), cg, (unsigned)(B * 2)), 128, 0, st>>>(
             static_cast<const __nv_bfloat16 *>(x), static_cast<const __nv_bfloat16 *>(dy), xT, dyT, L, D, Lp, 2, 0);
-        k_backward_tc<true><<<(unsigned)rows, kThreads, kSmemBytes, st>>>(mdy, mx, a);
+        a.plan = row_plan(B, D, a.ntiles);
+        k_backward_tc<true><<<(unsigned)a.plan.end[2], kThreads, kSmemBytes, st>>>(mdy, mx, a);
         TermArgs ta;
+        ta.plan = a.plan;
         ta.decay = decay;
         ta.freq = freq;
         ta.g = reinterpret_cast<const float2 *>(d_state_out);
@@ -1607,7 +1711,7 @@ cudaError_t tc_backward(const void *dy, const void *x, void *dx, int64_t B, int6
         ta.ntiles = (int)(Lp / kTile);
         CUtensorMap mdx;
         if (!make_chunk_map(&mdx, dxT, rows, Lp, false)) return cudaErrorInvalidValue;
-        k_terminal_tc<<<(unsigned)rows, kTmThreads, kTmSmemBytes, st>>>(mx, mdx, ta);
+        k_terminal_tc<<<(unsigned)ta.plan.end[2], kTmThreads, kTmSmemBytes, st>>>(mx, mdx, ta);
         row_major_wide(dxT, static_cast<__nv_bfloat16 *>(dx), B, L, D, Lp, st);
         count_launches(4);   // transpose, pass, terminal-state terms, transpose
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
