@@ -59,7 +59,14 @@
 //              (G, P).
 //   warps 4-5  dx epilogue (quarters 0, 1: positions 0-63), then the diagonal
 //              sums of Q.
-//   warp 6     TMA producer and TMEM allocation; warp 7 idle.
+//   warp 6     TMA producer, which loads while the others build the tables (with the
+//              producer in warp 7 the call at B = 4, L = 32768, D = 512 took 329 us
+//              against 319; the MMA warps in 6-7 or exchanged, 325-333).
+//   warp 7     TMEM allocation (and the tables, with warps 0-5 and 8-9).
+//   The kernel may start while the input transposes drain (pdl_wait): only the producer
+//   waits for them, so the tables are built meanwhile.  Backward calls, launches one after
+//   the other and now (us): B = 1, L = 122, D = 424, M = 8 33 -> 26; B = 8, L = 2048, D = 256,
+//   M = 16 42 -> 35; B = 8, L = 4096, D = 256, M = 16 with state terms 97 -> 88.
 //   warp 8     MMA issue: projections and Q; warp 9: T', U' and E.
 //
 // Every wait is bounded: after kWaitLimitCycles the waiting thread sets a shared
@@ -361,7 +368,11 @@ __global__ void __launch_bounds__(kThreads, 2)
     const int row0 = b0 * args.D + d;           // b * D + d of the first row; the next ones D apart
     const int M = args.M, ntiles = args.ntiles;
     const int nv = kGrad ? nrows * ntiles : ntiles;   // tiles of the walk: each row's in reverse, row after row
-    const int w_prod = 6;
+    constexpr int w_prod = 6, w_alloc = 7, w_mma_p = 8, w_mma_d = 9;
+    // Threads that build the tables: all but the producer's.
+    constexpr int kBuilders = kThreads - 32;
+    const int bt = warp < w_prod ? tid : tid - 32;
+    auto sync_builders = [] { asm volatile("bar.sync 2, %0;" ::"n"(kBuilders) : "memory"); };
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kOffBar);
     auto bar = [&](int i) { return smem_u32(bars + i); };
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + kOffMisc);
@@ -383,7 +394,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == w_prod) {
+    if (warp == w_alloc) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(tmem_slot)),
                      "r"(kTmemCols));
@@ -403,10 +414,9 @@ __global__ void __launch_bounds__(kThreads, 2)
         tma_load_3d(dst, &tmap_dy, 0, chunk0, row, bar(kBarSlotFull + slot));
         if (kGrad) tma_load_3d(dst + 4096, &tmap_x, 0, chunk0, row, bar(kBarSlotFull + slot));
     };
-    int issued = 0;
-    if (warp == w_prod && lane == 0)
-        for (; issued < nv && issued < kSlots; ++issued) load_tile(issued);
-
+    // (No pdl_launch_dependents() here: blocks of the output transpose beside the last wave
+    // cost 5 us at B = 4, L = 32768, D = 512.)
+    if (warp != w_prod) {
     // ------------------------------------------------------------ constants
     // Stage 1: lambda^n (n = 0..64) and c for every mode slot (zero past M):
     // thread (m, g) runs n = 8g .. 8g+7 as one exact power and seven products
@@ -414,8 +424,9 @@ __global__ void __launch_bounds__(kThreads, 2)
     float2 *pw = reinterpret_cast<float2 *>(smem + kOffPw);
     float2 *cf = reinterpret_cast<float2 *>(smem + kOffCf);
     float *kt = reinterpret_cast<float *>(smem + kOffK);
-    if (tid < kMaxModes * 9) {
-        const int m = tid / 9, g = tid % 9;
+    static_assert(kMaxModes * 9 == kBuilders, "one builder per mode and group of powers");
+    {
+        const int m = bt / 9, g = bt % 9;
         float2 *o = pw + m * kPwStride + 8 * g;
         if (m < M) {
             const float ga = args.decay[d * M + m], om = args.freq[d * M + m];
@@ -432,26 +443,31 @@ __global__ void __launch_bounds__(kThreads, 2)
         } else {
             for (int e = 0; e < (g < 8 ? 8 : 1); ++e) o[e] = make_float2(0.0f, 0.0f);
         }
-    } else if (tid >= 288 && tid < 288 + kMaxModes) {
-        const int m = tid - 288;
+    }
+    if (bt >= kBuilders - kMaxModes) {
+        const int m = bt - (kBuilders - kMaxModes);
         cf[m] = m >= M ? make_float2(0.0f, 0.0f)
                              : mode_coef(args.amp[d * M + m], args.phase[d * M + m]);
     }
-    if (tid < 64) reinterpret_cast<float *>(smem + kOffRho)[tid] = 0.0f;
-    __syncthreads();
+    if (bt < 64) reinterpret_cast<float *>(smem + kOffRho)[bt] = 0.0f;
+    sync_builders();
     // Stage 2: K[n] (Eq. 1 at integer lags, modes summed in a fixed order), the
     // projection table and the up-projection U', one 16-byte core-matrix row
     // (8 consecutive K elements of one row) per task; consecutive tasks take
     // consecutive rows, so each quarter-warp's stores fill 128 contiguous bytes.
-    if (tid < kC) {
+    if (bt < 4 * kC) {   // whole warps: four lanes a lag, eight modes each
+        const int n = bt >> 2, m0 = 8 * (bt & 3);
         float acc = 0.0f;
-        for (int m = 0; m < kMaxModes; ++m) {
-            const float2 p = pw[m * kPwStride + tid], c = cf[m];
+#pragma unroll
+        for (int m = m0; m < m0 + 8; ++m) {
+            const float2 p = pw[m * kPwStride + n], c = cf[m];
             acc = fmaf(c.x, p.x, fmaf(-c.y, p.y, acc));
         }
-        kt[tid] = acc;
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        if ((bt & 3) == 0) kt[n] = acc;
     }
-    for (int t = tid; t < 1024 + 512; t += kThreads) {
+    for (int t = bt; t < 1024 + 512; t += kBuilders) {
         if (t < 1024) {
             // A_P row r, k = 8 kg .. 8 kg + 7: lambda^k (Vp rows, with low parts) or
             // k lambda^k (Vq rows).
@@ -487,9 +503,9 @@ __global__ void __launch_bounds__(kThreads, 2)
             st_shared_v4(sbase + kOffU + kmaj(i, 8 * kg), w[0], w[1], w[2], w[3]);
         }
     }
-    __syncthreads();
+    sync_builders();
     // Stage 3: the transposed Toeplitz block T'[i][j] = K[j - i] (j >= i).
-    for (int t = tid; t < 512; t += kThreads) {
+    for (int t = bt; t < 512; t += kBuilders) {
         const int kg = t >> 6, i = t & 63;
         uint32_t w[4];
 #pragma unroll
@@ -501,8 +517,9 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     fence_async_smem();
     tc_fence_before();
-    __syncthreads();
+    sync_builders();
     tc_fence_after();
+    }
 
     const int last = nv - 1;
     // Scan lanes: lane l of quarter q owns row 32 q + l of the projections and of
@@ -720,6 +737,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     } else if (warp == w_prod) {
         // ---------------------------------------------------- TMA producer
         if (lane == 0) {
+            pdl_wait();
+            int issued = 0;
             for (; issued < nv; ++issued) {
                 const int slot = issued % kSlots;
                 if (!wait_bar(bar(kBarSlotEmpty + slot), ((issued / kSlots) & 1) ^ 1, abort_flag)) break;
@@ -730,7 +749,7 @@ __global__ void __launch_bounds__(kThreads, 2)
                 drain_bar(bar(kBarSlotFull + k % kSlots), (k / kSlots) & 1);
         }
         __syncwarp();
-    } else if (warp == 8) {
+    } else if (warp == w_mma_p) {
         // ---------------------------------------------------- MMA: projections and Q
         if (lane == 0) {
             const uint64_t dap = desc_plain(sbase + kOffAP, 128, 1024);
@@ -765,7 +784,7 @@ __global__ void __launch_bounds__(kThreads, 2)
             if (v > 0) drain_bar(bar(kBarPFull + ((v - 1) & 1)), ((v - 1) >> 1) & 1);
         }
         __syncwarp();
-    } else if (warp == 9) {
+    } else if (warp == w_mma_d) {
         // ---------------------------------------------------- MMA: T', U', E
         if (lane == 0) {
             const uint64_t dt = desc_plain(sbase + kOffT, 128, 1024);
@@ -815,7 +834,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     tc_fence_before();
     __syncthreads();   // every role has left its loop; rho is complete
     tc_fence_after();
-    if (warp == w_prod)
+    if (warp == w_alloc)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                      "r"(kTmemCols));
     if (kGrad && warp < 4) {
@@ -1022,6 +1041,8 @@ __global__ void __launch_bounds__(kTmThreads, 2)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    if (tid == 0) pdl_launch_dependents();
+    pdl_wait();   // the tables needed parameters only; what follows reads the main pass's results
     // The chunk holding token L - 1 when it does not end there (-1: none).
     const int64_t n_part = (L % kC) ? (L - 1) / kC : -1;
 
@@ -1324,6 +1345,7 @@ __global__ void __launch_bounds__(128) k_to_channel_major(const __nv_bfloat16 *_
                                                           __nv_bfloat16 *__restrict__ dst0,
                                                           __nv_bfloat16 *__restrict__ dst1, int64_t L, int D,
                                                           int64_t Lp, int nf, int rev) {
+    pdl_launch_dependents();
     __shared__ uint32_t tile[64][33];   // [position][channel pair]
     const int64_t t0 = (int64_t)blockIdx.x * 64;
     const int c0 = blockIdx.y * 64;
@@ -1376,6 +1398,8 @@ __global__ void __launch_bounds__(128) k_to_channel_major(const __nv_bfloat16 *_
 __global__ void __launch_bounds__(128) k_to_row_major(const __nv_bfloat16 *__restrict__ srcT,
                                                       __nv_bfloat16 *__restrict__ dst, int64_t L, int D,
                                                       int64_t Lp, int rev) {
+    pdl_launch_dependents();
+    pdl_wait();
     __shared__ uint32_t tile[64][37];   // [channel][position pair]
     const int64_t t0 = (int64_t)blockIdx.x * 64;
     const int c0 = blockIdx.y * 64;
@@ -1435,6 +1459,8 @@ constexpr int kRmTokens = 128, kRmChannels = 64;
 __global__ void __launch_bounds__(256) k_to_row_major_wide(const __nv_bfloat16 *__restrict__ srcT,
                                                            __nv_bfloat16 *__restrict__ dst, int64_t L, int D,
                                                            int64_t Lp) {
+    pdl_launch_dependents();
+    pdl_wait();
     constexpr int kStride = kRmTokens / 2 + 1, kGroups = kRmTokens / 8;
     constexpr int kLoads = kRmChannels * kGroups / 256, kStores = kRmTokens * (kRmChannels / 8) / 256;
     __shared__ uint32_t tile[kRmChannels][kStride];   // [channel][position pair]
@@ -1480,11 +1506,12 @@ __global__ void __launch_bounds__(256) k_to_row_major_wide(const __nv_bfloat16 *
     }
 }
 // Its launch (D % 8 == 0, which every tcgen05 backward shape has).
-void row_major_wide(const __nv_bfloat16 *srcT, __nv_bfloat16 *dst, int64_t B, int64_t L, int D, int64_t Lp,
-                    cudaStream_t st) {
-    k_to_row_major_wide<<<dim3((unsigned)((L + kRmTokens - 1) / kRmTokens),
-                               (unsigned)((D + kRmChannels - 1) / kRmChannels), (unsigned)B),
-                          256, 0, st>>>(srcT, dst, L, D, Lp);
+cudaError_t row_major_wide(const __nv_bfloat16 *srcT, __nv_bfloat16 *dst, int64_t B, int64_t L, int D, int64_t Lp,
+                           cudaStream_t st) {
+    return launch_dependent(k_to_row_major_wide,
+                            dim3((unsigned)((L + kRmTokens - 1) / kRmTokens),
+                                 (unsigned)((D + kRmChannels - 1) / kRmChannels), (unsigned)B),
+                            256, 0, st, srcT, dst, L, D, Lp);
 }
 
 // ------------------------------------------------------------ host side
@@ -1642,13 +1669,16 @@ cudaError_t run_layout_and_scan(const CUtensorMap &mdy, const CUtensorMap &mx, B
     k_to_channel_major<<<dim3((unsigned)(Lp / 64), cg, (unsigned)(B * nf)), 128, 0, st>>>(
         src0, src1, dst0, dst1, L, D, Lp, nf, rev);
     if (kGrad) a.plan = row_plan(B, D, a.ntiles);
-    k_backward_tc<kGrad><<<(unsigned)(kGrad ? a.plan.end[2] : B * D), kThreads, kSmemBytes, st>>>(mdy, mx, a);
+    cudaError_t e = launch_dependent(k_backward_tc<kGrad>, dim3((unsigned)(kGrad ? a.plan.end[2] : B * D)), kThreads,
+                                     kSmemBytes, st, mdy, mx, a);
+    if (e != cudaSuccess) return e;
     if (rev)
-        k_to_row_major<<<dim3((unsigned)((L + 63) / 64), cg, (unsigned)B), 128, 0, st>>>(outT, out, L, D, Lp, rev);
+        e = launch_dependent(k_to_row_major, dim3((unsigned)((L + 63) / 64), cg, (unsigned)B), 128, 0, st, outT, out, L,
+                             D, Lp, rev);
     else
-        row_major_wide(outT, out, B, L, D, Lp, st);
+        e = row_major_wide(outT, out, B, L, D, Lp, st);
     count_launches(3);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace
@@ -1693,7 +1723,9 @@ cudaError_t tc_backward(const void *dy, const void *x, void *dx, int64_t B, int6
         k_to_channel_major<<<dim3((unsigned)(Lp / 64), cg, (unsigned)(B * 2)), 128, 0, st>>>(
             static_cast<const __nv_bfloat16 *>(x), static_cast<const __nv_bfloat16 *>(dy), xT, dyT, L, D, Lp, 2, 0);
         a.plan = row_plan(B, D, a.ntiles);
-        k_backward_tc<true><<<(unsigned)a.plan.end[2], kThreads, kSmemBytes, st>>>(mdy, mx, a);
+        if ((e = launch_dependent(k_backward_tc<true>, dim3((unsigned)a.plan.end[2]), kThreads, kSmemBytes, st, mdy, mx,
+                                  a)) != cudaSuccess)
+            return e;
         TermArgs ta;
         ta.plan = a.plan;
         ta.decay = decay;
@@ -1711,8 +1743,10 @@ cudaError_t tc_backward(const void *dy, const void *x, void *dx, int64_t B, int6
         ta.ntiles = (int)(Lp / kTile);
         CUtensorMap mdx;
         if (!make_chunk_map(&mdx, dxT, rows, Lp, false)) return cudaErrorInvalidValue;
-        k_terminal_tc<<<(unsigned)ta.plan.end[2], kTmThreads, kTmSmemBytes, st>>>(mx, mdx, ta);
-        row_major_wide(dxT, static_cast<__nv_bfloat16 *>(dx), B, L, D, Lp, st);
+        if ((e = launch_dependent(k_terminal_tc, dim3((unsigned)ta.plan.end[2]), kTmThreads, kTmSmemBytes, st, mx, mdx,
+                                  ta)) != cudaSuccess ||
+            (e = row_major_wide(dxT, static_cast<__nv_bfloat16 *>(dx), B, L, D, Lp, st)) != cudaSuccess)
+            return e;
         count_launches(4);   // transpose, pass, terminal-state terms, transpose
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

@@ -103,7 +103,6 @@ __device__ __forceinline__ void mix_shift(const MixStep<T> &m, const MixPart<T> 
     if (g == 0) h[(int64_t)(m.K - 2) * D] = r.xr;
 }
 
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Moves the line holding p into L2 without reading it into the thread: safe before
 // the dependency wait even if the previous grid writes the line (L2 is where the
 // writes land), and it overlaps the token's DRAM latency with the wait.
@@ -117,9 +116,6 @@ __device__ __forceinline__ void prefetch_step(const T *x_t, const MixStep<T> &mi
     if (g != 0 || bd >= BD || (bd & 63) != 0) return;
     prefetch_l2(x_t + bd);
     if (is_mix && mix.g) prefetch_l2(mix.g + bd);
-}
-__device__ __forceinline__ void pdl_launch_dependents() {
-    asm volatile("griddepcontrol.launch_dependents;" :::);
 }
 
 // M even with one mode pair per thread: a block of R
@@ -257,18 +253,8 @@ __global__ void k_state_init(float2 *__restrict__ s, float4 *__restrict__ coef, 
 
 template <typename Kern, typename... Args>
 cudaError_t launch_pdl_block(Kern kern, dim3 grid, int block, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
     count_launches(1);
-    return cudaLaunchKernelEx(&cfg, kern, args...);
+    return launch_dependent(kern, grid, (unsigned)block, 0, st, args...);
 }
 
 template <typename Kern, typename... Args>

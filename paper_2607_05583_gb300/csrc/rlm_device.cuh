@@ -50,6 +50,15 @@ __device__ __forceinline__ float2 lambda_pow(float gamma, float omega, float n) 
     return make_float2(r * fmaf(-pe, sp, cp), r * fmaf(pe, cp, sp));
 }
 
+// Programmatic dependent launch.  A kernel launched by launch_dependent() may start while
+// the kernel before it in the stream drains; it calls pdl_wait() before it touches what
+// that kernel (or one before it in the same call) writes, in every block, so that its own
+// end implies theirs.  The first kernel of a call is launched normally, so caller inputs
+// need no wait.  pdl_launch_dependents() lets the next such kernel start once every block
+// of this one has called it or ended.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" :::); }
+
 // c = A exp(i phi).
 __device__ __forceinline__ float2 mode_coef(float amp, float phase) {
     float s, c;

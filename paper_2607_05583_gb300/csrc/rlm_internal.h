@@ -19,6 +19,24 @@ int sm_count();
 // Adds n to the process-wide count of kernels this library has launched.
 void count_launches(int n);
 
+// Launches a kernel that may start before the previous kernel of the stream has ended
+// (see pdl_wait() in rlm_device.cuh); not counted here.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st,
+                             const A &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // ---- SIMT chunked scan (rlm_simt.cu) --------------------------------------
 // The chunk length in which the SIMT path's workspace contract is stated.
 int simt_chunk_len(int64_t B, int64_t L, int D);

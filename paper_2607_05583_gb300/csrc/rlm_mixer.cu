@@ -297,6 +297,7 @@ template <typename T>
 __global__ void __launch_bounds__(kBlock) k_conv_tail(const T *__restrict__ x, const T *hist, T *out, int64_t B,
                                                       int64_t L, int D, int K) {
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();   // the pass before read hist, which out may alias
     if (gid >= B * D) return;
     const int64_t b = gid / D;
     const int d = (int)(gid % D);
@@ -348,10 +349,9 @@ template <typename T>
 cudaError_t tail_t(const void *x, const void *hist, void *out, int64_t B, int64_t L, int D, int K,
                    cudaStream_t st) {
     const int64_t n = B * D;
-    k_conv_tail<T><<<(unsigned)((n + kBlock - 1) / kBlock), kBlock, 0, st>>>(
-        static_cast<const T *>(x), static_cast<const T *>(hist), static_cast<T *>(out), B, L, D, K);
     count_launches(1);
-    return cudaGetLastError();
+    return launch_dependent(k_conv_tail<T>, dim3((unsigned)((n + kBlock - 1) / kBlock)), kBlock, 0, st,
+                            static_cast<const T *>(x), static_cast<const T *>(hist), static_cast<T *>(out), B, L, D, K);
 }
 
 }  // namespace

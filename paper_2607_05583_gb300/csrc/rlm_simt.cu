@@ -330,6 +330,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
     float *kq = smem + w * kWords + 2 * kModes * kPwStride;
     float *us = kq + kKernWords;                 // drive tile, then W, then the output tile
     float *xs = us + (kX ? kFieldWords : 0);     // x tile (backward)
+    pdl_launch_dependents();
 
     // ---- tables: lambda^n, n < 64 (an exact power every 8, products between)
     {
@@ -350,6 +351,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
             }
         }
     }
+    if (kOut) pdl_wait();   // the segments' end states (the tables needed parameters only)
     // ---- the lane's modes: lambda^64, c, and the state (pair) entering the segment
     float2 lamC[NP][J], cm[NP][J], S0[NP][J], R0[BWD ? NP : 1][J];
     float2 *cs = reinterpret_cast<float2 *>(us);   // c of every mode, until the first tile is staged
@@ -796,6 +798,7 @@ __global__ void __launch_bounds__(256) k_grad_reduce(
     const float2 *__restrict__ ws_r, const float2 *__restrict__ ws_j, float *__restrict__ g_decay,
     float *__restrict__ g_freq, float *__restrict__ g_amp, float *__restrict__ g_phase) {
     const int pm = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
     if (pm >= D * M) return;
     const float am = amp[pm], ph = phase[pm];
     KahanSum gr, gi, pr, pi, jr, ji;
@@ -878,8 +881,10 @@ cudaError_t launch_scan(const ScanArgs &a, int nseg, int zdim, cudaStream_t st) 
             done.fetch_or(bit, std::memory_order_release);
         }
     }
-    k<<<dim3((unsigned)(a.D / kCh), (unsigned)nseg, (unsigned)zdim), kThreads, bytes, st>>>(a);
+    const dim3 grid((unsigned)(a.D / kCh), (unsigned)nseg, (unsigned)zdim);
     count_launches(1);
+    if (kOut && a.nseg > 1) return launch_dependent(k, grid, kThreads, bytes, st, a);
+    k<<<grid, kThreads, bytes, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -966,10 +971,9 @@ cudaError_t simt_prefill(const void *x, void *y, rlm_dtype dt, int64_t B, int64_
 cudaError_t grad_reduce(int64_t nparts, int D, int M, const float *amp, const float *phase,
                         const float2 *G, const float2 *P, const float2 *J, float *g_decay, float *g_freq,
                         float *g_amp, float *g_phase, cudaStream_t st) {
-    k_grad_reduce<<<(unsigned)((D * M + 255) / 256), 256, 0, st>>>(
-        nparts, D, M, 1, amp, phase, G, P, J, g_decay, g_freq, g_amp, g_phase);
     count_launches(1);
-    return cudaGetLastError();
+    return launch_dependent(k_grad_reduce, dim3((unsigned)((D * M + 255) / 256)), 256, 0, st, nparts, D, M, 1, amp, phase,
+                            G, P, J, g_decay, g_freq, g_amp, g_phase);
 }
 
 cudaError_t simt_backward(const void *dy, const void *x, void *dx, rlm_dtype dt, int64_t B,
