@@ -262,37 +262,42 @@ cudaError_t launch_pdl(Kern kern, dim3 grid, cudaStream_t st, Args... args) {
     return launch_pdl_block(kern, grid, kDecodeBlock, st, args...);
 }
 
-// One decode step with head coupling (Sec. 3.4) in a single launch, one block per
-// batch row, for rows of at most 512 channels and 4096 modes.  Right after the
-// dependency wait every load of the step is issued at once: the thread of channel
-// d (threadIdx.x) takes its token, gate, drive history and conv weights, and every
-// thread takes its (at most four) float4 mode pairs of the row's state slab with
-// their coefficients -- consecutive threads on consecutive pairs, so the M / 2
-// threads of a channel form one aligned shuffle group.  Phase 1 updates the
-// states and puts each channel's readout y_t[d] in shared memory (fp32); after
-// the block barrier, phase 2 forms (C y_t)[d], applies the gate and the local
-// path, shifts the history and writes z_t[d].  C depends on the parameters only,
-// so it is built before the wait.  H = 0: no coupling (the mixer step alone).
-constexpr int kCoupledBlock = 512;
-constexpr int kCoupledIters = 4;               // mode pairs per thread
-constexpr int kCoupledMaxModesPerRow = 2 * kCoupledIters * kCoupledBlock;   // D * M <= 4096
+// One decode step with head coupling (Sec. 3.4) in a single launch, for rows of at
+// most 512 channels and 4096 modes.  Coupling mixes equal positions of different heads
+// only, so a row splits into Q blocks by in-head position: block q takes positions
+// q dh / Q .. of every head, and no block needs another's readouts.  Right after the
+// dependency wait every load of the step is issued at once: the thread of a channel
+// takes its token, gate, drive history and conv weights, and every thread takes its (at
+// most kIters) float4 mode pairs of the block's states with their coefficients --
+// consecutive threads on consecutive pairs, so the M / 2 threads of a channel form one
+// aligned shuffle group.  Phase 1 updates the states and puts each channel's readout in
+// shared memory (fp32); after the block barrier, phase 2 forms C y_t, applies the gate and
+// the local path, shifts the history and writes z_t.  C depends on the parameters
+// only, so it is built before the wait.
+constexpr int kCoupledBlock = 512;             // one block per row
+constexpr int kSplitBlock = 256;               // several blocks per row
+constexpr int kCoupledMaxModesPerRow = 8 * kCoupledBlock;   // D * M <= 4096
 constexpr int kHistMax = RLM_MAX_LOCAL_K - 1;
 
-template <typename T>
-__global__ void __launch_bounds__(kCoupledBlock, 1) k_decode_coupled(
+template <typename T, int kBlock, int kIters>
+__global__ void __launch_bounds__(kBlock) k_decode_coupled(
     const T *__restrict__ x_t, T *__restrict__ z_t, int D, int M, float4 *__restrict__ s,
-    const float4 *__restrict__ coef, MixStep<T> mix, const float *__restrict__ c_raw, float lam, int H) {
+    const float4 *__restrict__ coef, MixStep<T> mix, const float *__restrict__ c_raw, float lam, int H, int Q) {
     extern __shared__ __align__(16) float smf[];
     float *C = smf;                              // [H][H]
-    float *ys = smf + ((H * H + 3) & ~3);        // [D]
-    const int64_t b = blockIdx.x;
-    if (H > 0) build_coupling(C, c_raw, lam, H);
+    float *ys = smf + ((H * H + 3) & ~3);        // [D / Q]
+    const int64_t b = blockIdx.y;
+    // Channel c of the block (head-major over its positions) is channel at(c) of the row.
+    const int dh = D / H, dq = dh / Q, n = H * dq, p0 = blockIdx.x * dq;
+    auto at = [&](int c) { return Q == 1 ? c : c / dq * dh + p0 + c % dq; };
+    build_coupling(C, c_raw, lam, H);
     pdl_wait();
     pdl_launch_dependents();
     const T *xb = x_t + b * D;
     // ---- loads: phase 2's inputs (channel d2) ...
-    const int d2 = threadIdx.x, K = mix.K;
-    const bool ch = d2 < D;
+    const int c2 = threadIdx.x, K = mix.K;
+    const bool ch = c2 < n;
+    const int d2 = ch ? at(c2) : 0;
     T xraw = T(0.0f), hv[kHistMax];
     float gv = 0.0f, sc = 0.0f, w0 = 0.0f, wj[kHistMax];   // wj[j]: the weight of history entry j
     T *hc = K > 1 ? mix.hist + b * (K - 1) * (int64_t)D + d2 : nullptr;   // used only when K > 1
@@ -314,27 +319,29 @@ __global__ void __launch_bounds__(kCoupledBlock, 1) k_decode_coupled(
     // ... and phase 1's states, coefficients and tokens.
     const int pairs = M / 2;                     // a power of two, at most 32
     const int lp = __ffs(pairs) - 1;
-    const int n4 = D * pairs;
-    float4 *sb = s + b * n4;
-    float4 stv[kCoupledIters], c0v[kCoupledIters], c1v[kCoupledIters];
-    float xv[kCoupledIters];
+    const int n4 = n * pairs;
+    float4 *sb = s + b * ((int64_t)D * pairs);
+    float4 stv[kIters], c0v[kIters], c1v[kIters];
+    float xv[kIters];
+    int dv[kIters];
 #pragma unroll
-    for (int k = 0; k < kCoupledIters; ++k) {
-        const int i = (int)threadIdx.x + k * kCoupledBlock;
-        const int d = i >> lp, g = i & (pairs - 1);
+    for (int k = 0; k < kIters; ++k) {
+        const int i = (int)threadIdx.x + k * kBlock;
+        const int g = i & (pairs - 1);
         if (i < n4) {
+            const int d = dv[k] = at(i >> lp);
             xv[k] = ld_elem(xb + d);
-            stv[k] = sb[i];
+            stv[k] = sb[d * pairs + g];
             c0v[k] = __ldg(coef + (int64_t)d * M + 2 * g);
             c1v[k] = __ldg(coef + (int64_t)d * M + 2 * g + 1);
         }
     }
     // ---- phase 1: every thread runs every iteration, so whole warps shuffle
 #pragma unroll
-    for (int k = 0; k < kCoupledIters; ++k) {
-        const int i = (int)threadIdx.x + k * kCoupledBlock;
+    for (int k = 0; k < kIters; ++k) {
+        const int i = (int)threadIdx.x + k * kBlock;
         const bool on = i < n4;
-        const int d = i >> lp, g = i & (pairs - 1);
+        const int g = i & (pairs - 1);
         float acc = 0.0f;
         if (on) {
             const float4 st = stv[k], c0 = c0v[k], c1 = c1v[k];
@@ -342,21 +349,18 @@ __global__ void __launch_bounds__(kCoupledBlock, 1) k_decode_coupled(
             const float i0 = fmaf(c0.x, st.y, c0.y * st.x);
             const float r1 = fmaf(c1.x, st.z, fmaf(-c1.y, st.w, xv[k]));
             const float i1 = fmaf(c1.x, st.w, c1.y * st.z);
-            sb[i] = make_float4(r0, i0, r1, i1);
+            sb[dv[k] * pairs + g] = make_float4(r0, i0, r1, i1);
             acc = fmaf(c0.z, r0, fmaf(-c0.w, i0, fmaf(c1.z, r1, -c1.w * i1)));
         }
         for (int o = pairs >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (on && g == 0) ys[d] = acc;
+        if (on && g == 0) ys[i >> lp] = acc;
     }
     __syncthreads();
     // ---- phase 2
     if (!ch) return;
-    float v = ys[d2];
-    if (H > 0) {
-        const int dh = D / H, gh = d2 / dh, jh = d2 % dh;
-        v = 0.0f;
-        for (int h = 0; h < H; ++h) v = fmaf(C[gh * H + h], ys[h * dh + jh], v);
-    }
+    float v = 0.0f;
+    const int gh = c2 / dq, jh = c2 % dq;
+    for (int h = 0; h < H; ++h) v = fmaf(C[gh * H + h], ys[h * dq + jh], v);
     if (mix.g) v *= gatef(gv);
     if (K > 0) {
         float l = w0 * as_float(xraw);
@@ -435,31 +439,53 @@ bool mixer_decode_coupled_supported(int D, int M) {
            (int64_t)D * M <= kCoupledMaxModesPerRow;
 }
 
+namespace {
+
+// Blocks per row: while one block a row leaves half the SMs idle, the largest power of
+// two up to 8 that divides the head width and leaves a block its 256 mode pairs.  One
+// block pulls a row's 98 KB of states and coefficients through one SM's L2 port.  CUDA
+// graph of steps (gate, K = 4, H = 8, bf16, D = 256, M = 16), us per step with 1 / 2 / 4 / 8
+// blocks a row: B = 1 3.18 / 3.07 / 2.24 / 1.96, B = 32 3.46 / 3.43 / 2.27 / 2.13, B = 64
+// 3.41 / 3.08 / 2.99 / 2.86, B = 128 3.52 / 3.85 / 4.87 / 4.87; with 512 pairs a row (fp32,
+// D = 64, B = 64) 2.10 / 1.72 / 1.96 / 2.33.
+int coupled_split(int B, int D, int M, int H) {
+    if (2 * B > sm_count()) return 1;
+    int Q = 8;
+    while (Q > 1 && ((D / H) % Q != 0 || D * (M / 2) < Q * kSplitBlock)) Q >>= 1;
+    return Q;
+}
+
+template <typename T>
+cudaError_t coupled_t(const void *x_t, void *z_t, int B, int D, int M, float *s, const float *coef, MixStep<T> m,
+                      const float *c_raw, float lambda_c, int H, cudaStream_t st) {
+    const int Q = coupled_split(B, D, M, H);
+    const dim3 grid((unsigned)Q, (unsigned)B);
+    const size_t smem = (size_t)(((H * H + 3) & ~3) + D / Q) * sizeof(float);
+    auto go = [&](auto kern, unsigned block) {
+        return launch_dependent(kern, grid, block, smem, st, static_cast<const T *>(x_t), static_cast<T *>(z_t), D, M,
+                                reinterpret_cast<float4 *>(s), reinterpret_cast<const float4 *>(coef), m, c_raw,
+                                lambda_c, H, Q);
+    };
+    count_launches(1);
+    const int iters = (D / Q * (M / 2) + kSplitBlock - 1) / kSplitBlock;
+    if (D / Q > kSplitBlock || iters > 4) return go(k_decode_coupled<T, kCoupledBlock, 4>, kCoupledBlock);
+    if (iters <= 1) return go(k_decode_coupled<T, kSplitBlock, 1>, kSplitBlock);
+    if (iters <= 2) return go(k_decode_coupled<T, kSplitBlock, 2>, kSplitBlock);
+    return go(k_decode_coupled<T, kSplitBlock, 4>, kSplitBlock);
+}
+
+}  // namespace
+
 cudaError_t mixer_decode_coupled(const void *x_t, const void *g_t, void *z_t, rlm_dtype dt, int B, int D, int M,
                                  float *s, const float *coef, void *hist, const float *conv_w, const float *scale,
                                  int K, const float *c_raw, float lambda_c, int H, cudaStream_t st) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)B);
-    cfg.blockDim = dim3(kCoupledBlock);
-    cfg.dynamicSmemBytes = (size_t)(((H * H + 3) & ~3) + D) * sizeof(float);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    count_launches(1);
-    float4 *s4 = reinterpret_cast<float4 *>(s);
-    const float4 *cf = reinterpret_cast<const float4 *>(coef);
     if (dt == RLM_BF16) {
         using T = __nv_bfloat16;
         const MixStep<T> m{static_cast<const T *>(g_t), static_cast<T *>(hist), conv_w, scale, K};
-        return cudaLaunchKernelEx(&cfg, k_decode_coupled<T>, static_cast<const T *>(x_t), static_cast<T *>(z_t), D,
-                                  M, s4, cf, m, c_raw, lambda_c, H);
+        return coupled_t<T>(x_t, z_t, B, D, M, s, coef, m, c_raw, lambda_c, H, st);
     }
     const MixStep<float> m{static_cast<const float *>(g_t), static_cast<float *>(hist), conv_w, scale, K};
-    return cudaLaunchKernelEx(&cfg, k_decode_coupled<float>, static_cast<const float *>(x_t),
-                              static_cast<float *>(z_t), D, M, s4, cf, m, c_raw, lambda_c, H);
+    return coupled_t<float>(x_t, z_t, B, D, M, s, coef, m, c_raw, lambda_c, H, st);
 }
 
 cudaError_t state_init(float *s, float *coef, int B, int D, int M, const float *decay,

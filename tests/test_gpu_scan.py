@@ -1,11 +1,13 @@
-"""The CUDA-core scan (fp32 with M > 16, M > 32, a ragged length from a state, fp32
-backward) at the edges of its tiles: chunks of 64 tokens, tiles of 1024, mode groups of
-8, 16, 32 and 64, segments of whole tiles.  Tolerances are the operator's parity bar."""
+"""Kernels at the edges of their tiles and splits.  The CUDA-core scan (fp32 with M > 16,
+M > 32, a ragged length from a state, fp32 backward): chunks of 64 tokens, tiles of 1024,
+mode groups of 8, 16, 32 and 64, segments of whole tiles, batch rows that share a tile.
+The tcgen05 backward with several rows per block, and the coupled decode step with
+several blocks per row.  Tolerances are the operator's parity bar unless said."""
 import numpy as np
 import pytest
 
 import oracle
-from synth import make_inputs
+from synth import make_inputs, make_mixer_inputs
 from tests._util import TOL, assert_close, to_dev, to_np
 
 torch = pytest.importorskip("torch")
@@ -116,3 +118,36 @@ def test_backward_rows_sharing_a_block(B, L, D, M):
     for k in total:
         # fp32 sums of the same terms in another order.
         assert_close(getattr(gr, k).cpu().numpy(), total[k].cpu().numpy(), 2e-5, k)
+
+
+# The coupled decode step split over blocks of a row: 8, 4, 2 and 1 blocks (few or many
+# rows, narrow heads, few modes), one head, odd head widths per block, K from 0 to 8.
+@pytest.mark.parametrize("B,D,M,H,K,dtype", [
+    (1, 256, 16, 8, 4, "bf16"), (3, 512, 8, 16, 8, "f32"), (70, 256, 16, 8, 2, "bf16"), (90, 256, 16, 8, 4, "bf16"),
+    (2, 64, 64, 1, 1, "f32"), (5, 120, 32, 5, 3, "f32"), (4, 48, 32, 4, 4, "bf16"), (2, 8, 2, 8, 4, "f32"),
+])
+def test_coupled_decode_split_over_blocks(B, D, M, H, K, dtype):
+    inp = make_inputs(B, 4, D, M, dtype, seed=B + D + K)
+    mx = make_mixer_inputs(inp, K, seed=B + M)
+    c_raw = np.random.default_rng(H).standard_normal((H, H))
+    x, g = to_dev(inp.x, dtype), to_dev(mx.g, dtype)
+    p = rlm.Params.from_arrays(*inp.params())
+    local = rlm.Local.from_arrays(mx.conv_w, mx.scale) if K else None
+    st = rlm.State.empty(B, D, M)
+    rlm.rlm_state_init(st, p)
+    cs = rlm.ConvState(to_dev(mx.conv_in, dtype)) if K > 1 else None
+    zs = []
+    for t in range(4):
+        z = torch.full_like(x[:, t], float("nan"))
+        rlm.rlm_mixer_decode(x[:, t].contiguous(), g[:, t].contiguous(), st, local, cs, z,
+                             coupling=rlm.Coupling.from_arrays(c_raw, 0.5))
+        zs.append(z)
+    torch.cuda.synchronize()
+    zr, sr, tr = oracle.mixer_prefill(inp.x, mx.g, *inp.params(), mx.conv_w, mx.scale,
+                                      conv_in=mx.conv_in if K > 1 else None, coupling=(c_raw, 0.5))
+    assert_close(to_np(torch.stack(zs, 1)), zr, TOL[dtype], "z")
+    s = st.complex().cpu().numpy()
+    assert_close(s.real, sr.real, TOL["f32"], "state re")
+    assert_close(s.imag, sr.imag, TOL["f32"], "state im")
+    if K > 1:
+        np.testing.assert_array_equal(to_np(cs.u), tr)
