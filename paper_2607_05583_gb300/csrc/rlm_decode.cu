@@ -279,17 +279,21 @@ constexpr int kSplitBlock = 256;               // several blocks per row
 constexpr int kCoupledMaxModesPerRow = 8 * kCoupledBlock;   // D * M <= 4096
 constexpr int kHistMax = RLM_MAX_LOCAL_K - 1;
 
+// (The bounds matter: without the minimum of four blocks of the one-iteration instance a
+// step at B = 64 took 3.85 us against 2.61.)
 template <typename T, int kBlock, int kIters>
-__global__ void __launch_bounds__(kBlock) k_decode_coupled(
+__global__ void __launch_bounds__(kBlock, kBlock == kCoupledBlock ? 1 : kIters == 1 ? 4 : kIters == 2 ? 3 : 2)
+    k_decode_coupled(
     const T *__restrict__ x_t, T *__restrict__ z_t, int D, int M, float4 *__restrict__ s,
     const float4 *__restrict__ coef, MixStep<T> mix, const float *__restrict__ c_raw, float lam, int H, int Q) {
     extern __shared__ __align__(16) float smf[];
     float *C = smf;                              // [H][H]
     float *ys = smf + ((H * H + 3) & ~3);        // [D / Q]
     const int64_t b = blockIdx.y;
+    constexpr bool kWhole = kBlock == kCoupledBlock;   // the whole row (Q = 1)
     // Channel c of the block (head-major over its positions) is channel at(c) of the row.
-    const int dh = D / H, dq = dh / Q, n = H * dq, p0 = blockIdx.x * dq;
-    auto at = [&](int c) { return Q == 1 ? c : c / dq * dh + p0 + c % dq; };
+    const int dh = D / H, dq = kWhole ? dh : dh / Q, n = kWhole ? D : H * dq, p0 = blockIdx.x * dq;
+    auto at = [&](int c) { return kWhole ? c : c / dq * dh + p0 + c % dq; };
     build_coupling(C, c_raw, lam, H);
     pdl_wait();
     pdl_launch_dependents();
@@ -323,15 +327,16 @@ __global__ void __launch_bounds__(kBlock) k_decode_coupled(
     float4 *sb = s + b * ((int64_t)D * pairs);
     float4 stv[kIters], c0v[kIters], c1v[kIters];
     float xv[kIters];
-    int dv[kIters];
+    int dv[kIters];   // (several blocks a row)
 #pragma unroll
     for (int k = 0; k < kIters; ++k) {
         const int i = (int)threadIdx.x + k * kBlock;
         const int g = i & (pairs - 1);
         if (i < n4) {
-            const int d = dv[k] = at(i >> lp);
+            const int d = at(i >> lp);
+            if (!kWhole) dv[k] = d;
             xv[k] = ld_elem(xb + d);
-            stv[k] = sb[d * pairs + g];
+            stv[k] = sb[kWhole ? i : d * pairs + g];
             c0v[k] = __ldg(coef + (int64_t)d * M + 2 * g);
             c1v[k] = __ldg(coef + (int64_t)d * M + 2 * g + 1);
         }
@@ -349,7 +354,7 @@ __global__ void __launch_bounds__(kBlock) k_decode_coupled(
             const float i0 = fmaf(c0.x, st.y, c0.y * st.x);
             const float r1 = fmaf(c1.x, st.z, fmaf(-c1.y, st.w, xv[k]));
             const float i1 = fmaf(c1.x, st.w, c1.y * st.z);
-            sb[dv[k] * pairs + g] = make_float4(r0, i0, r1, i1);
+            sb[kWhole ? i : dv[k] * pairs + g] = make_float4(r0, i0, r1, i1);
             acc = fmaf(c0.z, r0, fmaf(-c0.w, i0, fmaf(c1.z, r1, -c1.w * i1)));
         }
         for (int o = pairs >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -443,11 +448,12 @@ namespace {
 
 // Blocks per row: while one block a row leaves half the SMs idle, the largest power of
 // two up to 8 that divides the head width and leaves a block its 256 mode pairs.  One
-// block pulls a row's 98 KB of states and coefficients through one SM's L2 port.  CUDA
-// graph of steps (gate, K = 4, H = 8, bf16, D = 256, M = 16), us per step with 1 / 2 / 4 / 8
-// blocks a row: B = 1 3.18 / 3.07 / 2.24 / 1.96, B = 32 3.46 / 3.43 / 2.27 / 2.13, B = 64
-// 3.41 / 3.08 / 2.99 / 2.86, B = 128 3.52 / 3.85 / 4.87 / 4.87; with 512 pairs a row (fp32,
-// D = 64, B = 64) 2.10 / 1.72 / 1.96 / 2.33.
+// block a row pulls 98 KB of states and coefficients through one SM's L2 port.  CUDA graph
+// of steps (gate, K = 4, H = 8, bf16, D = 256, M = 16), us per step with one block a row
+// and by this rule: B = 1 2.94 / 1.88, B = 32 2.97 / 2.04, B = 64 3.02 / 2.61, B = 128 (one
+// block either way) 3.10 / 2.90; D = 512, M = 8, B = 64 3.20 / 2.59.  More rows gain nothing
+// from it (B = 128 with 2 / 4 / 8 blocks 3.85 / 4.87 / 4.87), nor do blocks of fewer pairs (fp32,
+// D = 64, B = 64: 2.10 / 1.72 / 1.96 / 2.33 with 1 / 2 / 4 / 8).
 int coupled_split(int B, int D, int M, int H) {
     if (2 * B > sm_count()) return 1;
     int Q = 8;
