@@ -44,9 +44,10 @@
 // instruction fetch are not hidden.  GB300, us per call, against the three launches of
 // token-by-token recurrences with chunk states in memory that this replaces:
 //
-//   fp32, B = 2, L = 4096, D = 512, M = 32: forward 247 -> 62, backward 303 -> 134
-//   bf16 from a state, B = 8, L = 1000, D = 256, M = 16: 75 -> 30
-//   fp32 backward with state terms, B = 3, L = 1521, D = 536, M = 32: 347 -> 197
+//   fp32, B = 2, L = 4096, D = 512, M = 32: forward 247 -> 62, backward 303 -> 133
+//   fp32, B = 4, L = 2048, D = 256, M = 48: forward and backward 176 (with the power table of
+//     a whole chunk, one block a SM, 305)
+//   bf16 from a state, B = 8, L = 1000, D = 256, M = 16: 75 -> 29
 //
 // and the error against 64 bits is a half to a third of the recurrences' (3e-6 -> 1e-6 for
 // the gradients of the first line).
@@ -67,22 +68,27 @@ constexpr int kCols = 16;            // chunks per tile
 constexpr int kTile = kC * kCols;    // 1024 tokens
 constexpr int kCh = 4;               // channels (warps) per block
 constexpr int kThreads = 32 * kCh;
-constexpr int kPwStride = 66;        // float2 per mode row of the power table: 16-byte aligned, rows 4 banks apart
+constexpr int kHalf = kC / 2;
+// The power table holds lambda^n for n < 32 only (it is what limits the blocks a SM holds):
+// products over a chunk run as two halves, joined by lambda^32.
+constexpr int kPwStride = kHalf + 2;   // float2 per mode row: n < 32, then lambda^32 and lambda^64; rows 4 banks apart
 constexpr int kFieldWords = kC * kCols;   // one channel's tile: [p / 2][column][p % 2], see slot()
 constexpr int kKernCopy = kC + 16;        // K reversed, then zeros (negative lags)
 constexpr int kKernWords = 2 * kKernCopy; // that, and the same shifted by one
 
-// Shared memory of a block, in floats: per channel the power table
-// [modes][66] (complex), the reversed lag kernel, the drive tile and (backward) the
-// x tile.
-constexpr int chan_words(int modes, bool bwd) {
-    return 2 * modes * kPwStride + kKernWords + (bwd ? 2 : 1) * kFieldWords;
+// Shared memory of a block, in floats: per channel the power table and c of every mode
+// (complex), the reversed lag kernel, and for output passes two field tiles, the drive's
+// and x's (forward: the second half's W).
+constexpr int chan_words(int modes, bool out) {
+    return 2 * modes * (kPwStride + 1) + kKernWords + (out ? 2 : 1) * kFieldWords;
 }
-// Resident blocks a SM (registers and shared memory both allow them).
+// Resident blocks a SM, for registers and shared memory alike.  (A third block at 17 to 32
+// modes, with 168 registers a thread, made the forward of B = 2, L = 4096, D = 512, M = 32 fp32 70
+// us against 62 and its backward 159 against 133.)
 __host__ __device__ constexpr int blocks_per_sm(int modes, bool bwd) {
-    return modes > 32 ? 1 : modes > 16 ? 2 : bwd ? 3 : 4;
+    return modes > 16 ? 2 : bwd ? 3 : 4;
 }
-constexpr int smem_bytes(int modes, bool bwd) { return kCh * chan_words(modes, bwd) * 4; }
+constexpr int smem_bytes(int modes, bool out) { return kCh * chan_words(modes, out) * 4; }
 
 __device__ __forceinline__ u64 pack2(float a, float b) {
     u64 r;
@@ -155,8 +161,9 @@ __device__ __forceinline__ void store4(void *f, int bf16, int64_t e, float4 v) {
 
 // Projection of the drive tile on the power table: for the lane's modes g + 8 j and
 // columns 4 cg + c, acc = sum_p lambda^e(p) x_p and (JORDAN) accq = sum_p w(p) lambda^e(p) x_p,
-// with e = 63 - p, w = 63 - p (TO_END) or e = p, w = p + 1.  pw points at the row of
-// mode g.  Per pair of positions: J + 2 16-byte shared
+// with e = 63 - p, w = 63 - p (TO_END) or e = p, w = p + 1.  The half with the larger
+// exponents runs first, on the table of the other, and is then carried by lambda^32.  pw
+// points at the row of mode g.  Per pair of positions: J + 2 16-byte shared
 // loads, the drives duplicated into both halves, 8 J (16 J) packed FMAs on (Re, Im).
 template <int J, bool JORDAN, bool TO_END>
 __device__ __forceinline__ void project(const float2 *pw, const float *xs, int cg, u64 (&acc)[J][4],
@@ -168,28 +175,48 @@ __device__ __forceinline__ void project(const float2 *pw, const float *xs, int c
             acc[j][c] = 0ull;
             if (JORDAN) accq[j][c] = 0ull;
         }
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+        if (h) {
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+                const float2 l32 = pw[8 * j * kPwStride + kHalf];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float2 a = cmul(l32, unpack2(acc[j][c]));
+                    acc[j][c] = pack2(a.x, a.y);
+                    if (JORDAN) {
+                        const float2 q = cmul(l32, unpack2(accq[j][c]));
+                        accq[j][c] = pack2(q.x, q.y);
+                    }
+                }
+            }
+        }
+        const int p0 = TO_END == (h == 0) ? 0 : kHalf;   // the half's first position
 #pragma unroll 2
-    for (int pp = 0; pp < kC / 2; ++pp) {
-        const float4 xa = *reinterpret_cast<const float4 *>(xs + slot(pp, 2 * cg));
-        const float4 xb = *reinterpret_cast<const float4 *>(xs + slot(pp, 2 * cg + 1));
-        ulonglong2 a[J];
-        const int n = TO_END ? kC - 2 - 2 * pp : 2 * pp;
+        for (int u = 0; u < kHalf / 2; ++u) {
+            const int pp = p0 / 2 + u;
+            const float4 xa = *reinterpret_cast<const float4 *>(xs + slot(pp, 2 * cg));
+            const float4 xb = *reinterpret_cast<const float4 *>(xs + slot(pp, 2 * cg + 1));
+            ulonglong2 a[J];
+            const int n = TO_END ? kHalf - 2 - 2 * u : 2 * u;
 #pragma unroll
-        for (int j = 0; j < J; ++j) a[j] = *reinterpret_cast<const ulonglong2 *>(pw + 8 * j * kPwStride + n);
-        const float v[2][4] = {{xa.x, xa.z, xb.x, xb.z}, {xa.y, xa.w, xb.y, xb.w}};
+            for (int j = 0; j < J; ++j) a[j] = *reinterpret_cast<const ulonglong2 *>(pw + 8 * j * kPwStride + n);
+            const float v[2][4] = {{xa.x, xa.z, xb.x, xb.z}, {xa.y, xa.w, xb.y, xb.w}};
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int p = 2 * pp + e;
-            const u64 w = dup2((float)(TO_END ? kC - 1 - p : p + 1));
+            for (int e = 0; e < 2; ++e) {
+                const int p = 2 * pp + e;
+                const u64 w = dup2((float)(TO_END ? kC - 1 - p : p + 1));
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const u64 d = dup2(v[e][c]);
-                const u64 dq = JORDAN ? mul2(d, w) : 0ull;
+                for (int c = 0; c < 4; ++c) {
+                    const u64 d = dup2(v[e][c]);
+                    const u64 dq = JORDAN ? mul2(d, w) : 0ull;
 #pragma unroll
-                for (int j = 0; j < J; ++j) {
-                    const u64 aj = (e == 0) == TO_END ? a[j].y : a[j].x;
-                    fma2(acc[j][c], aj, d);
-                    if (JORDAN) fma2(accq[j][c], aj, dq);
+                    for (int j = 0; j < J; ++j) {
+                        const u64 aj = (e == 0) == TO_END ? a[j].y : a[j].x;
+                        fma2(acc[j][c], aj, d);
+                        if (JORDAN) fma2(accq[j][c], aj, dq);
+                    }
                 }
             }
         }
@@ -246,25 +273,39 @@ __device__ __forceinline__ void causal(const float *kq, const float *xs, int g, 
 }
 
 // acc += Re(sum_m lambda^p W) over `modes` modes: W is staged as (Re, -Im) per column, so
-// a packed FMA on (Re lambda^p, Im lambda^p) accumulates both halves of the real part.
-__device__ __forceinline__ void up_project(const float2 *pw, const float *ws, int modes, int g, int cg, u64 (&acc)[8][4]) {
+// a packed FMA on (Re lambda^p, Im lambda^p) accumulates both halves of the real part.  Rows
+// p >= 32 take lambda^(p-32) and lambda^32 W (w2).
+__device__ __forceinline__ void up_project(const float2 *pw, const float *w1, const float *w2, int modes, int g, int cg,
+                                           u64 (&acc)[8][4]) {
 #pragma unroll 2
     for (int m = 0; m < modes; ++m) {
-        const ulonglong2 wa = *reinterpret_cast<const ulonglong2 *>(ws + slot(m, 2 * cg));
-        const ulonglong2 wb = *reinterpret_cast<const ulonglong2 *>(ws + slot(m, 2 * cg + 1));
+        ulonglong2 a[2];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(pw + m * kPwStride + 16 * j + 2 * g);
-            fma2(acc[2 * j][0], a.x, wa.x);
-            fma2(acc[2 * j][1], a.x, wa.y);
-            fma2(acc[2 * j][2], a.x, wb.x);
-            fma2(acc[2 * j][3], a.x, wb.y);
-            fma2(acc[2 * j + 1][0], a.y, wa.x);
-            fma2(acc[2 * j + 1][1], a.y, wa.y);
-            fma2(acc[2 * j + 1][2], a.y, wb.x);
-            fma2(acc[2 * j + 1][3], a.y, wb.y);
+        for (int j = 0; j < 2; ++j) a[j] = *reinterpret_cast<const ulonglong2 *>(pw + m * kPwStride + 16 * j + 2 * g);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float *ws = h ? w2 : w1;
+            const ulonglong2 wa = *reinterpret_cast<const ulonglong2 *>(ws + slot(m, 2 * cg));
+            const ulonglong2 wb = *reinterpret_cast<const ulonglong2 *>(ws + slot(m, 2 * cg + 1));
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int r = 2 * (2 * h + j);
+                fma2(acc[r][0], a[j].x, wa.x);
+                fma2(acc[r][1], a[j].x, wa.y);
+                fma2(acc[r][2], a[j].x, wb.x);
+                fma2(acc[r][3], a[j].x, wb.y);
+                fma2(acc[r + 1][0], a[j].y, wa.x);
+                fma2(acc[r + 1][1], a[j].y, wa.y);
+                fma2(acc[r + 1][2], a[j].y, wb.x);
+                fma2(acc[r + 1][3], a[j].y, wb.y);
+            }
         }
     }
+}
+
+// lambda^n, n < 64, from a mode's table row.
+__device__ __forceinline__ float2 power(const float2 *row, int n) {
+    return n < kHalf ? row[n] : cmul(row[kHalf], row[n - kHalf]);
 }
 
 // acc[n] += sum_u dy_u x_{u + 16 l + n} over the 16 positions u of block a, one column
@@ -325,14 +366,16 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
     const bool mine = (int)blockIdx.z * rpt + cg / A.gpr < A.B;
     const int64_t b = min((int)blockIdx.z * rpt + cg / A.gpr, A.B - 1);
     const int d0 = kCh * blockIdx.x, d = d0 + w, M = A.M, D = A.D;
-    constexpr int kWords = chan_words(kModes, kX);
+    constexpr int kWords = chan_words(kModes, kOut);
+    constexpr int kTableWords = 2 * kModes * (kPwStride + 1) + kKernWords;   // before the field tiles
     float2 *pw = reinterpret_cast<float2 *>(smem + w * kWords);
-    float *kq = smem + w * kWords + 2 * kModes * kPwStride;
+    float2 *cs = pw + kModes * kPwStride;        // c of every mode
+    float *kq = smem + w * kWords + 2 * kModes * (kPwStride + 1);
     float *us = kq + kKernWords;                 // drive tile, then W, then the output tile
-    float *xs = us + (kX ? kFieldWords : 0);     // x tile (backward)
+    float *xs = us + (kOut ? kFieldWords : 0);   // x tile (backward), then lambda^32 W
     pdl_launch_dependents();
 
-    // ---- tables: lambda^n, n < 64 (an exact power every 8, products between)
+    // ---- tables: lambda^n, n < 32 (an exact power every 8, products between), 32 and 64
     {
         constexpr int kLpm = kModes >= 32 ? 1 : 32 / kModes;   // lanes per mode
 #pragma unroll 1
@@ -342,19 +385,25 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
             const float ga = on ? A.decay[d * M + m] : 0.0f, om = on ? A.freq[d * M + m] : 0.0f;
             const float2 l1 = lambda_pow(ga, om, 1.0f);
 #pragma unroll 1
-            for (int n0 = 8 * (lane % kLpm); n0 < kC; n0 += 8 * kLpm) {
+            for (int n0 = 8 * (lane % kLpm); n0 < kHalf; n0 += 8 * kLpm) {
                 float2 z = lambda_pow(ga, om, (float)n0);
                 if (!on) z = make_float2(0.0f, 0.0f);
                 row[n0] = z;
 #pragma unroll
                 for (int e = 1; e < 8; ++e) row[n0 + e] = z = cmul(z, l1);
             }
+            if (lane % kLpm == 0) {
+                const float2 z = make_float2(0.0f, 0.0f);
+                row[kHalf] = on ? lambda_pow(ga, om, (float)kHalf) : z;
+                row[kHalf + 1] = on ? lambda_pow(ga, om, (float)kC) : z;
+                if (kOut) cs[m] = on ? mode_coef(A.amp[d * M + m], A.phase[d * M + m]) : z;
+            }
         }
     }
     if (kOut) pdl_wait();   // the segments' end states (the tables needed parameters only)
-    // ---- the lane's modes: lambda^64, c, and the state (pair) entering the segment
-    float2 lamC[NP][J], cm[NP][J], S0[NP][J], R0[BWD ? NP : 1][J];
-    float2 *cs = reinterpret_cast<float2 *>(us);   // c of every mode, until the first tile is staged
+    __syncwarp();
+    // ---- the state (pair) entering the segment, of the lane's modes
+    float2 S0[NP][J], R0[BWD ? NP : 1][J];
 #pragma unroll
     for (int q = 0; q < NP; ++q)
 #pragma unroll
@@ -364,8 +413,6 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
             const float ga = on ? A.decay[d * M + m] : 0.0f, om = on ? A.freq[d * M + m] : 0.0f;
             const float2 z = make_float2(0.0f, 0.0f);
             const int64_t sm = (b * D + d) * M + m;
-            lamC[q][j] = on ? lambda_pow(ga, om, (float)kC) : z;
-            cm[q][j] = kOut && on ? mode_coef(A.amp[d * M + m], A.phase[d * M + m]) : z;
             S0[q][j] = !BWD && A.enter && on && mine && seg == 0 ? A.enter[sm] : z;
             if (BWD) R0[q][j] = z;
             if (kOut && seg > 0 && on) {
@@ -383,10 +430,9 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                 S0[q][j] = S;
                 if (BWD) R0[q][j] = R;
             }
-            if (kOut && cg == 0) cs[m] = cm[q][j];
             if (!BWD && kOut && A.coef_out && blockIdx.z == 0 && seg == A.nseg - 1 && cg == 0 && on) {
-                const float2 l1 = lambda_pow(ga, om, 1.0f);
-                A.coef_out[d * M + m] = make_float4(l1.x, l1.y, cm[q][j].x, cm[q][j].y);
+                const float2 l1 = pw[m * kPwStride + 1];   // the exact lambda times lambda^0 = 1
+                A.coef_out[d * M + m] = make_float4(l1.x, l1.y, cs[m].x, cs[m].y);
             }
             // The output launch's segment 0 starts from this copy: by then a state_out that
             // is state_in's buffer may be written by the last segment's block.
@@ -398,9 +444,9 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
         // K[n] = sum_m Re(c lambda^n), stored reversed (and once more shifted by one).
         float k0 = 0.0f, k1 = 0.0f;
         for (int m = 0; m < M; ++m) {
-            const float2 c = cs[m], p0 = pw[m * kPwStride + lane], p1 = pw[m * kPwStride + lane + 32];
-            k0 = fmaf(c.x, p0.x, fmaf(-c.y, p0.y, k0));
-            k1 = fmaf(c.x, p1.x, fmaf(-c.y, p1.y, k1));
+            const float2 c = cs[m], p = pw[m * kPwStride + lane], c2 = cmul(c, pw[m * kPwStride + kHalf]);
+            k0 = fmaf(c.x, p.x, fmaf(-c.y, p.y, k0));
+            k1 = fmaf(c2.x, p.x, fmaf(-c2.y, p.y, k1));
         }
         kq[63 - lane] = k0;
         kq[31 - lane] = k1;
@@ -409,7 +455,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
         if (lane < 16) kq[kC + lane] = kq[kKernCopy + kC + lane] = 0.0f;
         if (lane == 0) kq[kKernCopy + kC - 1] = 0.0f;
     }
-    __syncthreads();   // the first tile overwrites cs
+    __syncwarp();
 
     float2 G[kX ? NP : 1][J], P[kX ? NP : 1][J], Jg[kX ? NP : 1][J];
     float rho_a = 0.0f, rho_b = 0.0f;   // lane (h, n): lags 16 h + n and 16 (3 - h) + n
@@ -456,7 +502,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                 o[3 * kWords] = v[i].w;
             }
         };
-        float *base = smem + 2 * kModes * kPwStride + kKernWords;
+        float *base = smem + kTableWords;
         if (!kAhead) fetch(A.u, tile, nextu);
         if constexpr (kX) fetch(A.x, tile, nextx);
         stage(nextu, base);
@@ -480,8 +526,9 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
             float2 Rn[BWD ? J : 1][4];
 #pragma unroll
             for (int j = 0; j < J; ++j) {
-                const float2 a = lamC[q][j], a2 = cmul(a, a), a4 = cmul(a2, a2);
-                const float2 lam = pw[(8 * J * q + 8 * j + g) * kPwStride + 1];
+                const float2 *row = pw + (8 * J * q + 8 * j + g) * kPwStride;
+                const float2 a = row[kHalf + 1], a2 = cmul(a, a), a4 = cmul(a2, a2);
+                const float2 lam = row[1];
                 // The lane's four columns from zero ...
                 float2 es = make_float2(0.0f, 0.0f), er = es;
 #pragma unroll
@@ -536,7 +583,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                                 Jg[q][j].y = fmaf((float)A.L, ji.y, Jg[q][j].y);
                             }
                             if (A.d_state_in) {
-                                const float2 v = cmul(cm[q][j], l0);
+                                const float2 v = cmul(cs[m], l0);
                                 A.d_state_in[sm] = cfma(gg, make_float2(lL.x, -lL.y), make_float2(v.x, -v.y));
                             }
                         }
@@ -546,11 +593,10 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                             float2 f = next;
                             if (tail) {
                                 // The sequence ends inside this chunk.
-                                const float2 *row = pw + m * kPwStride;
-                                f = cmul(row[tail], S);
+                                f = cmul(power(row, tail), S);
                                 for (int p = 0; p < tail; ++p) {
                                     const float v = us[slot(p >> 1, 2 * cg + (c >> 1)) + 2 * (c & 1) + (p & 1)];
-                                    const float2 z = row[tail - 1 - p];
+                                    const float2 z = power(row, tail - 1 - p);
                                     f.x = fmaf(z.x, v, f.x);
                                     f.y = fmaf(z.y, v, f.y);
                                 }
@@ -581,7 +627,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                         for (int c = 0; c < 4; ++c) {
                             const int64_t E = A.L - (int64_t)(A.nch - chunk0 - c) * kC;
                             if (E >= 0 && chunk0 + c < A.nch) {
-                                z = c == 0 || E < kC ? lambda_pow(ga, om, (float)E) : cmul(z, lamC[q][j]);
+                                z = c == 0 || E < kC ? lambda_pow(ga, om, (float)E) : cmul(z, pw[m * kPwStride + kHalf + 1]);
                                 const float2 p = unpack2(xp[j][c]), v = unpack2(xq[j][c]);
                                 const float Ef = (float)(E - 1);
                                 Jg[q][j] = cfma(z, make_float2(fmaf(Ef, p.x, v.x), fmaf(Ef, p.y, v.y)), Jg[q][j]);
@@ -594,8 +640,9 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                             for (int n = 0; n < tail; ++n) {
                                 const int p = n + kC - tail;
                                 const float v = (float)n * xs[slot(p >> 1, 2 * cg) + (p & 1)];
-                                Jg[q][j].x = fmaf(row[n].x, v, Jg[q][j].x);
-                                Jg[q][j].y = fmaf(row[n].y, v, Jg[q][j].y);
+                                const float2 z = power(row, n);
+                                Jg[q][j].x = fmaf(z.x, v, Jg[q][j].x);
+                                Jg[q][j].y = fmaf(z.y, v, Jg[q][j].y);
                             }
                         }
                     }
@@ -641,7 +688,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                 float2 W[4];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
-                    const float2 v = cmul(cm[q][j], unpack2(ls[q][j][c]));
+                    const float2 v = cmul(cs[m], unpack2(ls[q][j][c]));
                     W[c] = m < M ? make_float2(v.x, -v.y) : make_float2(0.0f, 0.0f);
                 }
                 if (kX && A.g && m < M) {
@@ -654,7 +701,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                     for (int c = 0; c < 4; ++c) {
                         const int64_t E = A.L - (int64_t)(A.nch - chunk0 - c) * kC;
                         if (E >= 0 && chunk0 + c < A.nch) {
-                            z = c == 0 || E < kC ? lambda_pow(ga, om, (float)E) : cmul(z, lamC[q][j]);
+                            z = c == 0 || E < kC ? lambda_pow(ga, om, (float)E) : cmul(z, pw[m * kPwStride + kHalf + 1]);
                             const float2 v = cmul(make_float2(gg.x, -gg.y), z);
                             W[c].x += v.x;
                             W[c].y -= v.y;
@@ -664,10 +711,16 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                 *reinterpret_cast<float4 *>(us + slot(8 * j + g, 2 * cg)) = make_float4(W[0].x, W[0].y, W[1].x, W[1].y);
                 *reinterpret_cast<float4 *>(us + slot(8 * j + g, 2 * cg + 1)) =
                     make_float4(W[2].x, W[2].y, W[3].x, W[3].y);
+                const float2 l32 = conj2(pw[m * kPwStride + kHalf]);   // (W is kept conjugated)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) W[c] = cmul(l32, W[c]);
+                *reinterpret_cast<float4 *>(xs + slot(8 * j + g, 2 * cg)) = make_float4(W[0].x, W[0].y, W[1].x, W[1].y);
+                *reinterpret_cast<float4 *>(xs + slot(8 * j + g, 2 * cg + 1)) =
+                    make_float4(W[2].x, W[2].y, W[3].x, W[3].y);
             }
             __syncwarp();
             if (kAhead && q == NP - 1 && tile + 1 < tile_end) fetch(A.u, tile + 1, nextu);
-            up_project(pw + 8 * J * q * kPwStride, us, min(8 * J, M - 8 * J * q), g, cg, acc);
+            up_project(pw + 8 * J * q * kPwStride, us, xs, min(8 * J, M - 8 * J * q), g, cg, acc);
         }
         float y[8][4];
 #pragma unroll
@@ -685,7 +738,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                 for (int r = 0; r < 8; ++r) {
                     const int n = 16 * (r >> 1) + 2 * g + (r & 1) - (kC - tail);
                     if (n >= 0) {
-                        const float2 z = pw[m * kPwStride + n];
+                        const float2 z = power(pw + m * kPwStride, n);
                         y[r][0] = fmaf(gg.x, z.x, fmaf(gg.y, z.y, y[r][0]));
                     }
                 }
@@ -747,14 +800,18 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                     const float2 gg = A.g[(b * D + d) * M + m];
                     js = cmul(make_float2(gg.x, -gg.y), js);
                 }
+                float2 gw = make_float2(0.0f, 0.0f), pn = gw;
                 for (int n = 16 * cg; n < 16 * cg + 16; ++n) {
-                    const float2 z = pw[m * kPwStride + n];
+                    const float2 z = pw[m * kPwStride + (n & (kHalf - 1))];
                     const float r = kq[n], nr = (float)n * r;
-                    gs.x = fmaf(z.x, r, gs.x);
-                    gs.y = fmaf(z.y, r, gs.y);
-                    ps.x = fmaf(z.x, nr, ps.x);
-                    ps.y = fmaf(z.y, nr, ps.y);
+                    gw.x = fmaf(z.x, r, gw.x);
+                    gw.y = fmaf(z.y, r, gw.y);
+                    pn.x = fmaf(z.x, nr, pn.x);
+                    pn.y = fmaf(z.y, nr, pn.y);
                 }
+                const float2 up = cg < 2 ? make_float2(1.0f, 0.0f) : pw[m * kPwStride + kHalf];
+                gs = cfma(up, gw, gs);
+                ps = cfma(up, pn, ps);
 #pragma unroll
                 for (int o = 8; o <= 16; o <<= 1) {
                     gs.x += __shfl_xor_sync(0xffffffffu, gs.x, o);
@@ -866,7 +923,7 @@ Geometry geometry(int64_t B, int64_t L, int D, int M, bool bwd, int max_seg) {
 
 template <int J, int NP, bool BWD, bool kOut>
 cudaError_t launch_scan(const ScanArgs &a, int nseg, int zdim, cudaStream_t st) {
-    constexpr int bytes = smem_bytes(8 * J * NP, BWD && kOut);
+    constexpr int bytes = smem_bytes(8 * J * NP, kOut);
     auto *k = k_scan<J, NP, BWD, kOut>;
     if (bytes > 48 * 1024) {
         // Once per device (a bit each; devices past 64 set it on every call).
