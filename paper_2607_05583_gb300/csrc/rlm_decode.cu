@@ -103,12 +103,6 @@ __device__ __forceinline__ void mix_shift(const MixStep<T> &m, const MixPart<T> 
     if (g == 0) h[(int64_t)(m.K - 2) * D] = r.xr;
 }
 
-// Moves the line holding p into L2 without reading it into the thread: safe before
-// the dependency wait even if the previous grid writes the line (L2 is where the
-// writes land), and it overlaps the token's DRAM latency with the wait.
-__device__ __forceinline__ void prefetch_l2(const void *p) {
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
 // The step's fresh inputs (token and gate rows: one line per 64 (b, d) pairs).
 template <typename T>
 __device__ __forceinline__ void prefetch_step(const T *x_t, const MixStep<T> &mix, bool is_mix, int64_t bd,

@@ -59,6 +59,13 @@ __device__ __forceinline__ float2 lambda_pow(float gamma, float omega, float n) 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" :::); }
 
+// Moves the line holding p into L2 without reading it into the thread: safe before
+// the dependency wait even if the previous grid writes the line (L2 is where the
+// writes land), and it overlaps the DRAM latency with the wait.
+__device__ __forceinline__ void prefetch_l2(const void *p) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+}
+
 // c = A exp(i phi).
 __device__ __forceinline__ float2 mode_coef(float amp, float phase) {
     float s, c;

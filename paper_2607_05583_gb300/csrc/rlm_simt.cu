@@ -308,6 +308,33 @@ __device__ __forceinline__ float2 power(const float2 *row, int n) {
     return n < kHalf ? row[n] : cmul(row[kHalf], row[n - kHalf]);
 }
 
+// sum_{p < tail} lambda^(tail-1-p) x_p of one column, in every lane: the four lanes of a mode
+// take every fourth power, and lambda^(n+32) shares the table entry of lambda^n.  (A single
+// lane walking the positions took up to 10 us of a call: B = 2, L = 4095, D = 512, M = 32 fp32
+// 76.4 us against 66.2 at L = 4096.)
+__device__ __forceinline__ float2 partial_end(const float2 *row, const float *xs, int col, int tail, int cg) {
+    float2 lo = make_float2(0.0f, 0.0f), hi = lo;
+    auto x = [&](int p) {
+        return p >= 0 ? xs[slot(p >> 1, col >> 1) + 2 * (col & 1) + (p & 1)] : 0.0f;
+    };
+#pragma unroll 4
+    for (int n = cg; n < kHalf; n += 4) {
+        const float2 z = row[n];
+        const float v = x(tail - 1 - n), w = x(tail - 1 - n - kHalf);
+        lo.x = fmaf(z.x, v, lo.x);
+        lo.y = fmaf(z.y, v, lo.y);
+        hi.x = fmaf(z.x, w, hi.x);
+        hi.y = fmaf(z.y, w, hi.y);
+    }
+    lo = cfma(row[kHalf], hi, lo);
+#pragma unroll
+    for (int o = 8; o <= 16; o <<= 1) {
+        lo.x += __shfl_xor_sync(0xffffffffu, lo.x, o);
+        lo.y += __shfl_xor_sync(0xffffffffu, lo.y, o);
+    }
+    return lo;
+}
+
 // acc[n] += sum_u dy_u x_{u + 16 l + n} over the 16 positions u of block a, one column
 // (the lane's); positions past the chunk count as zero.
 __device__ __forceinline__ void correlate(const float *dys, const float *xs, int col, int a, int l, float (&acc)[16]) {
@@ -375,6 +402,41 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
     float *xs = us + (kOut ? kFieldWords : 0);   // x tile (backward), then lambda^32 W
     pdl_launch_dependents();
 
+    const int tail = (int)(A.L & (kC - 1));                 // tokens of the partial last chunk
+    const int tile_end = min(A.ntiles, (seg + 1) * A.tps);
+    // The thread's 8 tokens of a tile, 4 channels each (zeros outside the sequence).
+    const int Li = (int)A.L, t_last = A.nch * kC - 1;
+    // The thread's column: its batch row, and its first token's tau in tile 0.
+    const int fcol = tid & (kCols - 1), frow = (int)blockIdx.z * rpt + fcol / (4 * A.gpr);
+    const int ftau = (fcol & (4 * A.gpr - 1)) * kC + (tid >> 4);
+    const int64_t fbase = (int64_t)frow * A.L;
+    auto fetch = [&](const void *f, int tile, float4 (&v)[8]) {
+        const int tau = tile * kTile + ftau;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int t = A.rev ? t_last - tau - 8 * i : tau + 8 * i;
+            v[i] = t >= 0 && t < Li && frow < A.B ? load4(f, A.bf16, (fbase + t) * D + d0)
+                                                  : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+    };
+    // The 32-mode forward loads the next tile's drive ahead of this tile's outputs (67 -> 62
+    // us at B = 2, L = 4096, D = 512, M = 32 fp32).  The backward has no registers for it
+    // (132 -> 143 us), the smaller forward needs them for its fourth block a SM.  There the
+    // first tile's lines move to L2 while the tables are built (later tiles' made the M = 16 fp32
+    // backward of B = 4, L = 8000, D = 256 189 us against 183).
+    if (!kAhead && frow < A.B) {
+        const int tau = seg * A.tps * kTile + ftau, e = A.bf16 ? 2 : 4;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int t = A.rev ? t_last - tau - 8 * i : tau + 8 * i;
+            if (t < 0 || t >= Li) continue;
+            const int64_t at = ((fbase + t) * D + d0) * e;
+            prefetch_l2(static_cast<const char *>(A.u) + at);
+            if (kX) prefetch_l2(static_cast<const char *>(A.x) + at);
+        }
+    }
+    float4 nextu[8], nextx[kX ? 8 : 1];
+
     // ---- tables: lambda^n, n < 32 (an exact power every 8, products between), 32 and 64
     {
         constexpr int kLpm = kModes >= 32 ? 1 : 32 / kModes;   // lanes per mode
@@ -383,6 +445,9 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
             float2 *row = pw + m * kPwStride;
             const bool on = m < M;
             const float ga = on ? A.decay[d * M + m] : 0.0f, om = on ? A.freq[d * M + m] : 0.0f;
+            const float am = kOut && on ? A.amp[d * M + m] : 0.0f, ph = kOut && on ? A.phase[d * M + m] : 0.0f;
+            if (!BWD && A.enter && on)   // used after the tables
+                prefetch_l2(A.enter + ((int64_t)min((int)blockIdx.z * rpt, A.B - 1) * D + d) * M + m);
             const float2 l1 = lambda_pow(ga, om, 1.0f);
 #pragma unroll 1
             for (int n0 = 8 * (lane % kLpm); n0 < kHalf; n0 += 8 * kLpm) {
@@ -396,7 +461,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                 const float2 z = make_float2(0.0f, 0.0f);
                 row[kHalf] = on ? lambda_pow(ga, om, (float)kHalf) : z;
                 row[kHalf + 1] = on ? lambda_pow(ga, om, (float)kC) : z;
-                if (kOut) cs[m] = on ? mode_coef(A.amp[d * M + m], A.phase[d * M + m]) : z;
+                if (kOut) cs[m] = on ? mode_coef(am, ph) : z;
             }
         }
     }
@@ -465,27 +530,6 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
 #pragma unroll
             for (int j = 0; j < J; ++j) G[q][j] = P[q][j] = Jg[q][j] = make_float2(0.0f, 0.0f);
     }
-    const int tail = (int)(A.L & (kC - 1));                 // tokens of the partial last chunk
-    const int tile_end = min(A.ntiles, (seg + 1) * A.tps);
-    // The thread's 8 tokens of a tile, 4 channels each (zeros outside the sequence).
-    const int Li = (int)A.L, t_last = A.nch * kC - 1;
-    // The thread's column: its batch row, and its first token's tau in tile 0.
-    const int fcol = tid & (kCols - 1), frow = (int)blockIdx.z * rpt + fcol / (4 * A.gpr);
-    const int ftau = (fcol & (4 * A.gpr - 1)) * kC + (tid >> 4);
-    const int64_t fbase = (int64_t)frow * A.L;
-    auto fetch = [&](const void *f, int tile, float4 (&v)[8]) {
-        const int tau = tile * kTile + ftau;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int t = A.rev ? t_last - tau - 8 * i : tau + 8 * i;
-            v[i] = t >= 0 && t < Li && frow < A.B ? load4(f, A.bf16, (fbase + t) * D + d0)
-                                                  : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        }
-    };
-    // The 32-mode forward loads the next tile's drive ahead of this tile's outputs (67 -> 62
-    // us at B = 2, L = 4096, D = 512, M = 32 fp32).  The backward has no registers for it
-    // (132 -> 143 us), the smaller forward needs them for its fourth block a SM.
-    float4 nextu[8], nextx[kX ? 8 : 1];
     if (kAhead) fetch(A.u, seg * A.tps, nextu);
     for (int tile = seg * A.tps; tile < tile_end; ++tile) {
         // ---- stage the tile: thread (column, position), 4 channels each
@@ -539,7 +583,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                     es = cfma(a, es, unpack2(acc[j][c]));
                 }
                 // ... the state entering them (over the mode's lanes in this row) ...
-                float2 T = S0[q][j], U = BWD ? R0[q][j] : T, S = T, R = U;
+                float2 T = S0[q][j], U = BWD ? R0[q][j] : T, S = T, R = U, send = T;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     if (i >= A.gpr) break;   // the same for every lane
@@ -589,23 +633,22 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                         }
                     } else {
                         const float2 next = cfma(a, S, unpack2(acc[j][c]));
-                        if (chunk0 + c == A.nch - 1 && on && mine && A.state_out) {
-                            float2 f = next;
-                            if (tail) {
-                                // The sequence ends inside this chunk.
-                                f = cmul(power(row, tail), S);
-                                for (int p = 0; p < tail; ++p) {
-                                    const float v = us[slot(p >> 1, 2 * cg + (c >> 1)) + 2 * (c & 1) + (p & 1)];
-                                    const float2 z = power(row, tail - 1 - p);
-                                    f.x = fmaf(z.x, v, f.x);
-                                    f.y = fmaf(z.y, v, f.y);
-                                }
-                            }
-                            A.state_out[(b * D + d) * M + m] = f;
+                        if (chunk0 + c == A.nch - 1) {
+                            if (tail)
+                                send = S;
+                            else if (on && mine && A.state_out)
+                                A.state_out[(b * D + d) * M + m] = next;
                         }
                         S = next;
                     }
                 }
+                if (!BWD && kOut && tail && tile == A.ntiles - 1 && A.state_out)
+                    for (int r = 0; r < rpt; ++r) {
+                        const int col = r * 4 * A.gpr + (A.nch - 1 - tile * kCols);   // row r's last chunk
+                        const float2 f = partial_end(row, us, col, tail, cg);
+                        if (cg == col >> 2 && on && mine)
+                            A.state_out[(b * D + d) * M + m] = cfma(power(row, tail), send, f);
+                    }
             }
             if (kX) {
                 u64 xp[J][4], xq[J][4];
@@ -633,13 +676,14 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                                 Jg[q][j] = cfma(z, make_float2(fmaf(Ef, p.x, v.x), fmaf(Ef, p.y, v.y)), Jg[q][j]);
                             }
                         }
-                        if (tail && chunk0 == 0) {
+                        if (tail && tile == 0) {
                             // The partial last chunk (the row's first column): its tokens are
-                            // positions p >= 64 - tail, L - 1 - t = p - (64 - tail).
+                            // positions p >= 64 - tail, L - 1 - t = p - (64 - tail), shared out
+                            // among the row's lanes.
                             const float2 *row = pw + m * kPwStride;
-                            for (int n = 0; n < tail; ++n) {
+                            for (int n = cg - gbase; n < tail; n += A.gpr) {
                                 const int p = n + kC - tail;
-                                const float v = (float)n * xs[slot(p >> 1, 2 * cg) + (p & 1)];
+                                const float v = (float)n * xs[slot(p >> 1, 2 * gbase) + (p & 1)];
                                 const float2 z = power(row, n);
                                 Jg[q][j].x = fmaf(z.x, v, Jg[q][j].x);
                                 Jg[q][j].y = fmaf(z.y, v, Jg[q][j].y);

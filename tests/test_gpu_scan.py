@@ -55,6 +55,26 @@ def test_prefill_from_a_state_at_tile_edges(B, L, D, M, dtype):
     assert_close(s.imag, s_ref.imag, TOL["f32"], "state im")
 
 
+# The terminal state of a sequence that ends inside a chunk: its powers are shared out among
+# four lanes and two halves of the table (n < 32 and above), with one, two or four batch
+# rows in a tile and the end in a first, middle or second tile.
+@pytest.mark.parametrize("tail", [2, 31, 32, 33, 62])
+@pytest.mark.parametrize("B,chunks,M", [(5, 0, 16), (3, 6, 8), (1, 9, 32), (2, 17, 64)])
+def test_terminal_state_of_a_partial_chunk(B, chunks, M, tail):
+    L, D = 64 * chunks + tail, 8
+    inp = make_inputs(B, L, D, M, "f32", seed=L + M)
+    st, s0 = _state(B, D, M, L)
+    x = to_dev(inp.x, "f32")
+    y, so = torch.empty_like(x), rlm.State.empty(B, D, M)
+    rlm.rlm_mix_prefill_from(x, rlm.Params.from_arrays(*inp.params()), st, y, so)
+    torch.cuda.synchronize()
+    y_ref, s_ref = oracle.rec_prefill(inp.x, *inp.params(), state_in=s0)
+    assert_close(to_np(y), y_ref, TOL["f32"], "y")
+    s = so.complex().cpu().numpy()
+    assert_close(s.real, s_ref.real, TOL["f32"], "state re")
+    assert_close(s.imag, s_ref.imag, TOL["f32"], "state im")
+
+
 @pytest.mark.parametrize("bad", [float("nan"), float("inf")])
 @pytest.mark.parametrize("t", [0, 70, 1030])
 def test_a_non_finite_drive_leaves_earlier_outputs_alone(bad, t):
