@@ -39,15 +39,16 @@
 // launch forms each segment's end state from zero, and the second enters segment s
 // with the combination of the states before it.
 //
-// What bounds it: the FMA pipe's floor is a third of the time; with two warps a
-// scheduler (tables and accumulators allow no more at M = 32) shared-load latency and
-// instruction fetch are not hidden.  GB300, us per call, against the three launches of
-// token-by-token recurrences with chunk states in memory that this replaces:
+// What bounds it: shared-load wavefronts (four a 16-byte load of a warp: at M = 32 about 1900 a
+// warp and tile forward, against 1350 cycles of FMA) at 40-50 % of their rate, since two
+// warps a scheduler (tables and accumulators allow no more at M = 32) do not hide the loads'
+// latency.  GB300, us per call, against the three launches of token-by-token recurrences with
+// chunk states in memory that this replaces:
 //
-//   fp32, B = 2, L = 4096, D = 512, M = 32: forward 247 -> 62, backward 303 -> 133
-//   fp32, B = 4, L = 2048, D = 256, M = 48: forward and backward 176 (with the power table of
+//   fp32, B = 2, L = 4096, D = 512, M = 32: forward 247 -> 56, backward 303 -> 125
+//   fp32, B = 4, L = 2048, D = 256, M = 48: forward and backward 164 (with the power table of
 //     a whole chunk, one block a SM, 305)
-//   bf16 from a state, B = 8, L = 1000, D = 256, M = 16: 75 -> 29
+//   bf16 from a state, B = 8, L = 1000, D = 256, M = 16: 75 -> 27
 //
 // and the error against 64 bits is a half to a third of the recurrences' (3e-6 -> 1e-6 for
 // the gradients of the first line).
@@ -72,7 +73,8 @@ constexpr int kHalf = kC / 2;
 // The power table holds lambda^n for n < 32 only (it is what limits the blocks a SM holds):
 // products over a chunk run as two halves, joined by lambda^32.
 constexpr int kPwStride = kHalf + 2;   // float2 per mode row: n < 32, then lambda^32 and lambda^64; rows 4 banks apart
-constexpr int kFieldWords = kC * kCols;   // one channel's tile: [p / 2][column][p % 2], see slot()
+// One channel's tile: [p / 2][column][p % 2] in rows of 32 words and 4 of padding, see slot().
+constexpr int kRowWords = 2 * kCols + 4, kFieldWords = kHalf * kRowWords;
 constexpr int kKernCopy = kC + 16;        // K reversed, then zeros (negative lags)
 constexpr int kKernWords = 2 * kKernCopy; // that, and the same shifted by one
 
@@ -109,10 +111,12 @@ __device__ __forceinline__ u64 mul2(u64 a, u64 b) {
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
-// Word of columns 2 h, 2 h + 1 in row r of a field tile (rows of 32 words: position pairs,
-// or modes of W).  The 16-byte slots of a row are permuted by its number, so that the
-// column groups that eight lanes write into eight rows fall into different banks.
-__device__ __forceinline__ int slot(int r, int h) { return r * 2 * kCols + ((h ^ (r & 7)) << 2); }
+// Word of columns 2 h, 2 h + 1 in row r of a field tile (rows are position pairs, or modes
+// of W).  The padding puts the 16-byte words that eight lanes write into eight rows in
+// different banks, and leaves every address of the product loops a constant from the lane's.
+// (Permuted 16-byte words of unpadded rows cost an XOR, a shift and an add a load: forward and
+// backward of B = 2, L = 4096, D = 512, M = 32 fp32 60.1 and 135 us against 57.7 and 127.)
+__device__ __forceinline__ int slot(int r, int h) { return r * kRowWords + 4 * h; }
 __device__ __forceinline__ float2 shfl2(float2 v, int src) {
     return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
@@ -165,6 +169,7 @@ __device__ __forceinline__ void store4(void *f, int bf16, int64_t e, float4 v) {
 // exponents runs first, on the table of the other, and is then carried by lambda^32.  pw
 // points at the row of mode g.  Per pair of positions: J + 2 16-byte shared
 // loads, the drives duplicated into both halves, 8 J (16 J) packed FMAs on (Re, Im).
+// (Four pairs unrolled in the 32-mode forward: 57.7 -> 56.4 us; in its backward 127 -> 131.)
 template <int J, bool JORDAN, bool TO_END>
 __device__ __forceinline__ void project(const float2 *pw, const float *xs, int cg, u64 (&acc)[J][4],
                                         u64 (&accq)[JORDAN ? J : 1][4]) {
@@ -193,7 +198,7 @@ __device__ __forceinline__ void project(const float2 *pw, const float *xs, int c
             }
         }
         const int p0 = TO_END == (h == 0) ? 0 : kHalf;   // the half's first position
-#pragma unroll 2
+#pragma unroll (J == 4 && !JORDAN ? 4 : 2)
         for (int u = 0; u < kHalf / 2; ++u) {
             const int pp = p0 / 2 + u;
             const float4 xa = *reinterpret_cast<const float4 *>(xs + slot(pp, 2 * cg));
@@ -229,42 +234,58 @@ __device__ __forceinline__ void project(const float2 *pw, const float *xs, int c
 // after; the copy behind it, shifted by one, keeps the pairs of even rows aligned).
 // In the diagonal 16-row blocks the zeros stand for the later drives.  kGuard: a tile
 // with an infinite or NaN drive skips them instead, so that earlier outputs stay clean.
-template <bool kGuard>
+// A pair of K serves every (row block, position block) with the same distance l, so SG
+// position blocks are held at once: shared-load wavefronts bound these products, 576 with
+// one at a time, 448 with two and 384 with four.  (One against two in the forward: 57.7 ->
+// 55.6 us at B = 2, L = 4096, D = 512, M = 32 fp32; against four in its backward: 127.7 -> 125.)
+template <bool kGuard, int SG>
 __device__ __forceinline__ void causal(const float *kq, const float *xs, int g, int cg, u64 (&acc)[8][4]) {
 #pragma unroll
-    for (int s = 0; s < 4; ++s) {
-#pragma unroll 2
+    for (int s0 = 0; s0 < 4; s0 += SG) {
+#pragma unroll (SG == 4 ? 2 : 1)
         for (int u = 0; u < 8; ++u) {
-            const int pp = 8 * s + u;   // positions 2 pp, 2 pp + 1
-            const ulonglong2 xa = *reinterpret_cast<const ulonglong2 *>(xs + slot(pp, 2 * cg));
-            const ulonglong2 xb = *reinterpret_cast<const ulonglong2 *>(xs + slot(pp, 2 * cg + 1));
-            const u64 x[4] = {xa.x, xa.y, xb.x, xb.y};
+            u64 x[SG][4];   // positions 16 (s0 + i) + 2 u and the next
 #pragma unroll
-            for (int j = s; j < 4; ++j) {
-                const int q1 = kC - 1 - (16 * j + 2 * g + 1) + 2 * pp;   // row e = 1: even
+            for (int i = 0; i < SG; ++i) {
+                const float *row = xs + slot(8 * (s0 + i) + u, 2 * cg);
+                const ulonglong2 xa = *reinterpret_cast<const ulonglong2 *>(row);
+                const ulonglong2 xb = *reinterpret_cast<const ulonglong2 *>(row + 4);
+                x[i][0] = xa.x;
+                x[i][1] = xa.y;
+                x[i][2] = xb.x;
+                x[i][3] = xb.y;
+            }
+#pragma unroll
+            for (int l = 0; l < 4 - s0; ++l) {
+                const int q1 = kC - 1 - (16 * l + 2 * g + 1) + 2 * u;   // row e = 1: even
                 const u64 k1 = *reinterpret_cast<const u64 *>(kq + q1);
                 const u64 k0 = *reinterpret_cast<const u64 *>(kq + kKernCopy + q1);   // row e = 0: kq[q1 + 1], kq[q1 + 2]
-                if (kGuard && j == s) {
-                    // Rows 2 g, 2 g + 1 of the block against its positions 2 u, 2 u + 1.
-                    const float2 f0 = unpack2(k0), f1 = unpack2(k1);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const float2 v = unpack2(x[c]);
-                        float2 a0 = unpack2(acc[2 * j][c]), a1 = unpack2(acc[2 * j + 1][c]);
-                        if (u <= g) {
-                            a0.x = fmaf(f0.x, v.x, a0.x);
-                            a1.x = fmaf(f1.x, v.x, a1.x);
-                            a1.y = fmaf(f1.y, v.y, a1.y);
+                for (int i = 0; i < SG; ++i) {
+                    const int j = s0 + i + l;
+                    if (j >= 4) continue;
+                    if (kGuard && l == 0) {
+                        // Rows 2 g, 2 g + 1 of the block against its positions 2 u, 2 u + 1.
+                        const float2 f0 = unpack2(k0), f1 = unpack2(k1);
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const float2 v = unpack2(x[i][c]);
+                            float2 a0 = unpack2(acc[2 * j][c]), a1 = unpack2(acc[2 * j + 1][c]);
+                            if (u <= g) {
+                                a0.x = fmaf(f0.x, v.x, a0.x);
+                                a1.x = fmaf(f1.x, v.x, a1.x);
+                                a1.y = fmaf(f1.y, v.y, a1.y);
+                            }
+                            if (u < g) a0.y = fmaf(f0.y, v.y, a0.y);
+                            acc[2 * j][c] = pack2(a0.x, a0.y);
+                            acc[2 * j + 1][c] = pack2(a1.x, a1.y);
                         }
-                        if (u < g) a0.y = fmaf(f0.y, v.y, a0.y);
-                        acc[2 * j][c] = pack2(a0.x, a0.y);
-                        acc[2 * j + 1][c] = pack2(a1.x, a1.y);
-                    }
-                } else {
+                    } else {
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        fma2(acc[2 * j][c], k0, x[c]);
-                        fma2(acc[2 * j + 1][c], k1, x[c]);
+                        for (int c = 0; c < 4; ++c) {
+                            fma2(acc[2 * j][c], k0, x[i][c]);
+                            fma2(acc[2 * j + 1][c], k1, x[i][c]);
+                        }
                     }
                 }
             }
@@ -384,6 +405,7 @@ template <int J, int NP, bool BWD, bool kOut>
 __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_scan(const ScanArgs A) {
     constexpr int kModes = 8 * J * NP;
     constexpr bool kX = BWD && kOut;   // the x tile is needed
+    constexpr int kSG = BWD && J == 4 ? 4 : 2;   // (see causal(); the forward with four: 55.6 -> 57.7 us)
     constexpr bool kAhead = !BWD && J == 4;   // the next tile's drive is loaded a tile ahead
     extern __shared__ __align__(16) float smem[];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -720,9 +742,9 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[r][c] = 0ull;
         if (guard)
-            causal<true>(kq, us, g, cg, acc);
+            causal<true, kSG>(kq, us, g, cg, acc);
         else
-            causal<false>(kq, us, g, cg, acc);
+            causal<false, kSG>(kq, us, g, cg, acc);
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
             __syncwarp();   // the warp is done reading the tile (or the previous W)
