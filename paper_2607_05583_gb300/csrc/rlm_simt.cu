@@ -26,7 +26,7 @@
 // Every sum over positions or modes is a small matrix product, which costs 2 FMA per
 // token and mode (4 with the Jordan partner) where the token-by-token recurrence
 // costs 4 (8) plus 2 for the readout: at M = 32 about 170 FMA per token-channel
-// forward and 410 backward, against 320 and 830.  They are bound by the FMA pipe.
+// forward and 410 backward, against 320 and 830.
 //
 // One warp owns one channel and a tile of 16 chunks (1024 tokens); its products are
 // register tiles (lane = 8 row groups x 4 column groups, columns = chunks) over
@@ -45,8 +45,8 @@
 // latency.  GB300, us per call, against the three launches of token-by-token recurrences with
 // chunk states in memory that this replaces:
 //
-//   fp32, B = 2, L = 4096, D = 512, M = 32: forward 247 -> 56, backward 303 -> 125
-//   fp32, B = 4, L = 2048, D = 256, M = 48: forward and backward 164 (with the power table of
+//   fp32, B = 2, L = 4096, D = 512, M = 32: forward 247 -> 56, backward 303 -> 117
+//   fp32, B = 4, L = 2048, D = 256, M = 48: forward and backward 162 (with the power table of
 //     a whole chunk, one block a SM, 305)
 //   bf16 from a state, B = 8, L = 1000, D = 256, M = 16: 75 -> 27
 //
@@ -106,11 +106,7 @@ __device__ __forceinline__ float2 unpack2(u64 v) {
 __device__ __forceinline__ void fma2(u64 &d, u64 a, u64 b) {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
 }
-__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
-    u64 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
+__device__ __forceinline__ void add2(u64 &d, u64 a) { asm("add.rn.f32x2 %0, %0, %1;" : "+l"(d) : "l"(a)); }
 // Word of columns 2 h, 2 h + 1 in row r of a field tile (rows are position pairs, or modes
 // of W).  The padding puts the 16-byte words that eight lanes write into eight rows in
 // different banks, and leaves every address of the product loops a constant from the lane's.
@@ -166,10 +162,15 @@ __device__ __forceinline__ void store4(void *f, int bf16, int64_t e, float4 v) {
 // Projection of the drive tile on the power table: for the lane's modes g + 8 j and
 // columns 4 cg + c, acc = sum_p lambda^e(p) x_p and (JORDAN) accq = sum_p w(p) lambda^e(p) x_p,
 // with e = 63 - p, w = 63 - p (TO_END) or e = p, w = p + 1.  The half with the larger
-// exponents runs first, on the table of the other, and is then carried by lambda^32.  pw
-// points at the row of mode g.  Per pair of positions: J + 2 16-byte shared
-// loads, the drives duplicated into both halves, 8 J (16 J) packed FMAs on (Re, Im).
-// (Four pairs unrolled in the 32-mode forward: 57.7 -> 56.4 us; in its backward 127 -> 131.)
+// exponents runs first, on the table of the other, and is then carried by lambda^32.  The
+// weights are never formed: accq adds up acc before every position (TO_END; after every
+// position), which counts position p 63 - p (p + 1) times.  pw points at the row of
+// mode g.  Per pair of positions: J + 2 16-byte shared loads, the drives duplicated into both
+// halves, 8 J packed FMAs (and as many adds) on (Re, Im).
+// Weighted products instead of the sums: backward of B = 4, L = 8000, D = 256, M = 16 fp32 166 us
+// against 147, of B = 2, L = 4096, D = 512, M = 32 125 against 117.  (Four pairs unrolled against
+// two: the 32-mode forward 57.7 -> 56.4 us, the 16-mode backward 147 -> 145, but the backward of
+// M = 48 118 -> 120.)
 template <int J, bool JORDAN, bool TO_END>
 __device__ __forceinline__ void project(const float2 *pw, const float *xs, int cg, u64 (&acc)[J][4],
                                         u64 (&accq)[JORDAN ? J : 1][4]) {
@@ -198,29 +199,28 @@ __device__ __forceinline__ void project(const float2 *pw, const float *xs, int c
             }
         }
         const int p0 = TO_END == (h == 0) ? 0 : kHalf;   // the half's first position
-#pragma unroll (J == 4 && !JORDAN ? 4 : 2)
+#pragma unroll (J == 4 && JORDAN ? 2 : 4)
         for (int u = 0; u < kHalf / 2; ++u) {
-            const int pp = p0 / 2 + u;
+            const int v0 = TO_END ? u : kHalf / 2 - 1 - u, pp = p0 / 2 + v0;
             const float4 xa = *reinterpret_cast<const float4 *>(xs + slot(pp, 2 * cg));
             const float4 xb = *reinterpret_cast<const float4 *>(xs + slot(pp, 2 * cg + 1));
             ulonglong2 a[J];
-            const int n = TO_END ? kHalf - 2 - 2 * u : 2 * u;
+            const int n = TO_END ? kHalf - 2 - 2 * v0 : 2 * v0;
 #pragma unroll
             for (int j = 0; j < J; ++j) a[j] = *reinterpret_cast<const ulonglong2 *>(pw + 8 * j * kPwStride + n);
             const float v[2][4] = {{xa.x, xa.z, xb.x, xb.z}, {xa.y, xa.w, xb.y, xb.w}};
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int p = 2 * pp + e;
-                const u64 w = dup2((float)(TO_END ? kC - 1 - p : p + 1));
+            for (int i = 0; i < 2; ++i) {
+                const int e = TO_END ? i : 1 - i;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     const u64 d = dup2(v[e][c]);
-                    const u64 dq = JORDAN ? mul2(d, w) : 0ull;
 #pragma unroll
                     for (int j = 0; j < J; ++j) {
                         const u64 aj = (e == 0) == TO_END ? a[j].y : a[j].x;
+                        if (JORDAN && TO_END) add2(accq[j][c], acc[j][c]);
                         fma2(acc[j][c], aj, d);
-                        if (JORDAN) fma2(accq[j][c], aj, dq);
+                        if (JORDAN && !TO_END) add2(accq[j][c], acc[j][c]);
                     }
                 }
             }
