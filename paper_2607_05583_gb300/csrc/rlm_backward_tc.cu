@@ -314,8 +314,8 @@ __device__ __forceinline__ void store_pair_row(uint32_t buf, int r, int g, const
 // channels from 0 on, the next ones r[1] rows of channels from ch[1] on, and so on, fewer
 // rows each, so that the large units start first and small ones fill the tail.  Same box,
 // one row per block and now: B = 8, L = 4096, D = 256, M = 16 with both state terms (this
-// kernel and k_terminal_tc) 157 -> 96 us; B = 4, L = 32768, D = 512, M = 32 (16 tiles a
-// row) with the forward 445 -> 416; B = 7, L = 465, D = 160, M = 32 66 -> 49.
+// kernel and k_terminal_tc) 157 -> 96 us; B = 7, L = 465, D = 160, M = 32 66 -> 49.  kMaxWalk
+// bounds the walk: rows of more than 8 tiles stay alone.
 struct RowPlan {
     int r[3];       // rows per block of the level
     int end[3];     // one past the level's last block
@@ -1572,8 +1572,12 @@ size_t tc_backward_ws_bytes(int64_t B, int64_t L, int D, int M) {
 
 namespace {
 
-// Longest walk of a block over several rows, in tiles (Q and E accumulate over it).
-constexpr int kMaxWalk = 64;
+// Longest walk of a block over several rows, in tiles.  Q and E accumulate over it in TMEM,
+// whose additions truncate, so the error of the sums grows with their number: relative error
+// of dA against 64 bits at B = 16, L = 8192, D = 256, M = 32 (4 tiles a row) 2.6e-6 with one row a
+// block, 2.6e-6, 3.0e-6 and 4.3e-6 with walks of up to 16, 32 and 64 tiles (B = 4, L = 32768,
+// D = 512: 2.8e-6 with 16, one row, and 3.8e-6 with 64, four rows, which takes 25 us less).
+constexpr int kMaxWalk = 16;
 
 cudaError_t configure_once() {
     static std::mutex mu;
