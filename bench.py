@@ -656,8 +656,8 @@ def _bench_mixer(rlm, torch, dev, hbm_peak, flush, mix_ms, with_decode=True):
             rlm.rlm_mixer_decode(toks[t], gts[t], dst, dlocal, hist, outs[t], coupling=dcp)
     lps = (rlm.rlm_kernels_launched() - n0) / T
     uc = replay_us(graph_c)
-    decode_coupled = {"workload": f"mixer decode with head coupling H={H}, B={Bd} D={D} M={M} K={K}: one block "
-                                  f"per batch row (recurrence step, coupling, gate, local path); {T} steps, "
+    decode_coupled = {"workload": f"mixer decode with head coupling H={H}, B={Bd} D={D} M={M} K={K}: one launch "
+                                  f"(recurrence step, coupling, gate, local path); {T} steps, "
                                   f"CUDA graph",
                       "us_per_step": round(uc, 4), "tok_s": round(Bd / (uc * 1e-6), 1), "launches_per_step": lps}
     return {"prefill_gate": prefill_gate, "prefill": prefill, "prefill_coupled": prefill_coupled, "decode": decode,

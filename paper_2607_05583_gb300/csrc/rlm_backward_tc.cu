@@ -61,7 +61,7 @@
 //              sums of Q.
 //   warp 6     TMA producer, which loads while the others build the tables (with the
 //              producer in warp 7 the call at B = 4, L = 32768, D = 512 took 329 us
-//              against 319; the MMA warps in 6-7 or exchanged, 325-333).
+//              against 319, four rows a block; the MMA warps in 6-7 or exchanged, 325-333).
 //   warp 7     TMEM allocation (and the tables, with warps 0-5 and 8-9).
 //   The kernel may start while the input transposes drain (pdl_wait): only the producer
 //   waits for them, so the tables are built meanwhile.  Backward calls, launches one after
