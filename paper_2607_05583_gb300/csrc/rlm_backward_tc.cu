@@ -1395,7 +1395,7 @@ __global__ void __launch_bounds__(128) k_to_channel_major(const __nv_bfloat16 *_
 // [B*D][Lp] -> [B][L][D] for tokens t < L, token t read from position t, or from
 // L - 1 - t when rev.  A tile covers 64 tokens x 64 channels; it loads the
 // 8-aligned window of 72 positions that holds its (reversed) positions.
-__global__ void __launch_bounds__(128) k_to_row_major(const __nv_bfloat16 *__restrict__ srcT,
+__global__ void __launch_bounds__(128) k_to_row_major(const __nv_bfloat16 *srcT,
                                                       __nv_bfloat16 *__restrict__ dst, int64_t L, int D,
                                                       int64_t Lp, int rev) {
     pdl_launch_dependents();
@@ -1419,7 +1419,7 @@ __global__ void __launch_bounds__(128) k_to_row_major(const __nv_bfloat16 *__res
         const int64_t sp = s_lo + 8 * vq;
         val[k] = make_uint4(0, 0, 0, 0);
         if (it < nload && c < D && sp >= 0 && sp < Lp)
-            val[k] = __ldg(reinterpret_cast<const uint4 *>(srcT + ((int64_t)b * D + c) * Lp + sp));
+            val[k] = *reinterpret_cast<const uint4 *>(srcT + ((int64_t)b * D + c) * Lp + sp);
     }
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
@@ -1456,7 +1456,7 @@ __global__ void __launch_bounds__(128) k_to_row_major(const __nv_bfloat16 *__res
 // the dx transpose 14 us shorter (0.380 -> 0.365 ms per call).  The same widening
 // of the channel-major transpose made it slower.
 constexpr int kRmTokens = 128, kRmChannels = 64;
-__global__ void __launch_bounds__(256) k_to_row_major_wide(const __nv_bfloat16 *__restrict__ srcT,
+__global__ void __launch_bounds__(256) k_to_row_major_wide(const __nv_bfloat16 *srcT,
                                                            __nv_bfloat16 *__restrict__ dst, int64_t L, int D,
                                                            int64_t Lp) {
     pdl_launch_dependents();
@@ -1475,7 +1475,7 @@ __global__ void __launch_bounds__(256) k_to_row_major_wide(const __nv_bfloat16 *
         const int c = c0 + cr;
         const int64_t sp = t0 + 8 * vq;
         val[k] = make_uint4(0, 0, 0, 0);
-        if (c < D && sp < Lp) val[k] = __ldg(reinterpret_cast<const uint4 *>(srcT + ((int64_t)b * D + c) * Lp + sp));
+        if (c < D && sp < Lp) val[k] = *reinterpret_cast<const uint4 *>(srcT + ((int64_t)b * D + c) * Lp + sp);
     }
 #pragma unroll
     for (int k = 0; k < kLoads; ++k) {

@@ -30,6 +30,10 @@ namespace {
 
 constexpr int kDecodeBlock = 256;
 
+// A step may start while the kernel before it runs, and that kernel may write any of its
+// inputs: all are read by plain loads (see rlm_device.cuh).  The read-only pointers
+// carry no __restrict__; the written ones do, so that loads may still pass earlier stores.
+
 // The mixer's per-step inputs (null g: no gate; K = 0: no local path).
 template <typename T>
 struct MixStep {
@@ -71,8 +75,8 @@ __device__ __forceinline__ MixPart<T> mix_part(const MixStep<T> &m, int64_t b, i
         if (g == 0) {
             // Every load of the step is issued here, before the reductions.
             r.xr = x_t[bd];
-            r.sc = __ldg(m.scale + d);
-            r.l = __ldg(w) * as_float(r.xr);
+            r.sc = m.scale[d];
+            r.l = w[0] * as_float(r.xr);
         }
         const T *h = m.hist + b * (m.K - 1) * (int64_t)D + d;
 #pragma unroll
@@ -80,7 +84,7 @@ __device__ __forceinline__ MixPart<T> mix_part(const MixStep<T> &m, int64_t b, i
             const int j = g + i * tpg;              // entry j holds u_{t-(K-1-j)}
             if (j < m.K - 1) {
                 r.hv[i] = h[(int64_t)j * D];
-                r.l = fmaf(__ldg(w + (m.K - 1 - j)), as_float(r.hv[i]), r.l);
+                r.l = fmaf(w[m.K - 1 - j], as_float(r.hv[i]), r.l);
             }
         }
     }
@@ -131,8 +135,8 @@ __device__ __forceinline__ void prefetch_step(const T *x_t, const MixStep<T> &mi
 // 11.1 us a step at B = 64, D = 2048, M = 16 against 10.6.
 template <typename T, int R, bool kMix>
 __global__ void __launch_bounds__(R * 32, 2048 / (R * 32)) k_decode_tile(
-    const T *__restrict__ x_t, T *__restrict__ y_t, int B, int D, int M, int log2_tpg,
-    float4 *__restrict__ s, const float4 *__restrict__ coef, MixStep<T> mix, bool late) {
+    const T *x_t, T *__restrict__ y_t, int B, int D, int M, int log2_tpg,
+    float4 *__restrict__ s, const float4 *coef, MixStep<T> mix, bool late) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tpg = 1 << log2_tpg;
     const int g = lane & (tpg - 1);
@@ -159,8 +163,8 @@ __global__ void __launch_bounds__(R * 32, 2048 / (R * 32)) k_decode_tile(
     if (kMix && rowok) mp = mix_part(mix, (int64_t)b, d, bd, D, g, tpg, x_t);  // every rank, with or without modes
     float acc = 0.0f;
     if (on) {
-        const float4 c0 = __ldg(coef + d * M + 2 * g);
-        const float4 c1 = __ldg(coef + d * M + 2 * g + 1);
+        const float4 c0 = coef[d * M + 2 * g];
+        const float4 c1 = coef[d * M + 2 * g + 1];
         const float xv = ld_elem(x_t + bd);
         const int64_t si = (bd * M) / 2 + g;
         const float4 q = s[si];
@@ -190,8 +194,8 @@ __global__ void __launch_bounds__(R * 32, 2048 / (R * 32)) k_decode_tile(
 // Any M: each thread owns up to MPT modes, accessed as float2.
 template <typename T, bool kMix>
 __global__ void __launch_bounds__(kDecodeBlock) k_decode_any(
-    const T *__restrict__ x_t, T *__restrict__ y_t, int64_t BD, int D, int M, int log2_tpg,
-    int mpt, float2 *__restrict__ s, const float4 *__restrict__ coef, MixStep<T> mix) {
+    const T *x_t, T *__restrict__ y_t, int64_t BD, int D, int M, int log2_tpg,
+    int mpt, float2 *__restrict__ s, const float4 *coef, MixStep<T> mix) {
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t bd = gid >> log2_tpg;
     const int g = (int)(gid & ((1 << log2_tpg) - 1));
@@ -209,7 +213,7 @@ __global__ void __launch_bounds__(kDecodeBlock) k_decode_any(
         for (int j = 0; j < mpt; ++j) {
             const int m = g * mpt + j;
             if (m >= M) break;
-            const float4 cf = __ldg(coef + d * M + m);
+            const float4 cf = coef[d * M + m];
             const float2 st = s[bd * M + m];
             const float re = fmaf(cf.x, st.x, fmaf(-cf.y, st.y, xv));
             const float im = fmaf(cf.x, st.y, cf.y * st.x);
@@ -278,8 +282,8 @@ constexpr int kHistMax = RLM_MAX_LOCAL_K - 1;
 template <typename T, int kBlock, int kIters>
 __global__ void __launch_bounds__(kBlock, kBlock == kCoupledBlock ? 1 : kIters == 1 ? 4 : kIters == 2 ? 3 : 2)
     k_decode_coupled(
-    const T *__restrict__ x_t, T *__restrict__ z_t, int D, int M, float4 *__restrict__ s,
-    const float4 *__restrict__ coef, MixStep<T> mix, const float *__restrict__ c_raw, float lam, int H, int Q) {
+    const T *x_t, T *__restrict__ z_t, int D, int M, float4 *__restrict__ s,
+    const float4 *coef, MixStep<T> mix, const float *c_raw, float lam, int H, int Q) {
     extern __shared__ __align__(16) float smf[];
     float *C = smf;                              // [H][H]
     float *ys = smf + ((H * H + 3) & ~3);        // [D / Q]
@@ -303,13 +307,13 @@ __global__ void __launch_bounds__(kBlock, kBlock == kCoupledBlock ? 1 : kIters =
         xraw = xb[d2];
         if (mix.g) gv = ld_elem(mix.g + b * D + d2);
         if (K > 0) {
-            sc = __ldg(mix.scale + d2);
-            w0 = __ldg(mix.conv_w + (int64_t)d2 * K);
+            sc = mix.scale[d2];
+            w0 = mix.conv_w[(int64_t)d2 * K];
 #pragma unroll
             for (int j = 0; j < kHistMax; ++j) {
                 if (j < K - 1) {
                     hv[j] = hc[(int64_t)j * D];
-                    wj[j] = __ldg(mix.conv_w + (int64_t)d2 * K + (K - 1 - j));
+                    wj[j] = mix.conv_w[(int64_t)d2 * K + (K - 1 - j)];
                 }
             }
         }
@@ -331,8 +335,8 @@ __global__ void __launch_bounds__(kBlock, kBlock == kCoupledBlock ? 1 : kIters =
             if (!kWhole) dv[k] = d;
             xv[k] = ld_elem(xb + d);
             stv[k] = sb[kWhole ? i : d * pairs + g];
-            c0v[k] = __ldg(coef + (int64_t)d * M + 2 * g);
-            c1v[k] = __ldg(coef + (int64_t)d * M + 2 * g + 1);
+            c0v[k] = coef[(int64_t)d * M + 2 * g];
+            c1v[k] = coef[(int64_t)d * M + 2 * g + 1];
         }
     }
     // ---- phase 1: every thread runs every iteration, so whole warps shuffle

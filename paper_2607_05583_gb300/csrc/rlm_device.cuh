@@ -10,10 +10,10 @@ namespace rlm {
 template <typename T>
 __device__ __forceinline__ float ld_elem(const T *p);
 template <>
-__device__ __forceinline__ float ld_elem<float>(const float *p) { return __ldg(p); }
+__device__ __forceinline__ float ld_elem<float>(const float *p) { return *p; }
 template <>
 __device__ __forceinline__ float ld_elem<__nv_bfloat16>(const __nv_bfloat16 *p) {
-    return __bfloat162float(__ldg(p));
+    return __bfloat162float(*p);
 }
 
 template <typename T>
@@ -56,6 +56,10 @@ __device__ __forceinline__ float2 lambda_pow(float gamma, float omega, float n) 
 // end implies theirs.  The first kernel of a call is launched normally, so caller inputs
 // need no wait.  pdl_launch_dependents() lets the next such kernel start once every block
 // of this one has called it or ended.
+// Such a kernel's life overlaps the writes of the one before it, so it reads what that
+// kernel writes by plain loads through pointers that are not const __restrict__: __ldg() (which
+// the compiler also uses for const __restrict__ parameters) needs data that nobody
+// writes while the kernel lives, and a load taken for invariant may be moved above the wait.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" :::); }
 

@@ -254,11 +254,10 @@ __global__ void __launch_bounds__(kBlock) k_couple_small(T *z, const float *__re
 // step wrote y_t into z_t: coupling, gate, local path (the thread of channel d
 // owns its history column, so it reads it all before shifting it).
 template <typename T>
-__global__ void __launch_bounds__(kBlock) k_mixer_finish(const T *__restrict__ x_t, const T *__restrict__ g_t,
+__global__ void __launch_bounds__(kBlock) k_mixer_finish(const T *x_t, const T *g_t,
                                                          T *__restrict__ z_t, T *hist,
-                                                         const float *__restrict__ conv_w,
-                                                         const float *__restrict__ scale, int K,
-                                                         const float *__restrict__ c_raw, float lam, int H, int D) {
+                                                         const float *conv_w, const float *scale, int K,
+                                                         const float *c_raw, float lam, int H, int D) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" :::);
     extern __shared__ __align__(16) uint8_t sm[];
@@ -276,16 +275,16 @@ __global__ void __launch_bounds__(kBlock) k_mixer_finish(const T *__restrict__ x
         if (g_t) v *= gatef(as_f(g_t[b * D + d]));
         if (K > 0) {
             const float xv = as_f(x_t[b * D + d]);
-            float l = __ldg(conv_w + (int64_t)d * K) * xv;
+            float l = conv_w[(int64_t)d * K] * xv;
             T *hc = hist + b * (K - 1) * (int64_t)D + d;    // entry j: u_{t-(K-1-j)}
             T hv[kMaxK];
             for (int j2 = 0; j2 < K - 1; ++j2) {
                 hv[j2] = hc[(int64_t)j2 * D];
-                l = fmaf(__ldg(conv_w + (int64_t)d * K + (K - 1 - j2)), as_f(hv[j2]), l);
+                l = fmaf(conv_w[(int64_t)d * K + (K - 1 - j2)], as_f(hv[j2]), l);
             }
             for (int j2 = 1; j2 < K - 1; ++j2) hc[(int64_t)(j2 - 1) * D] = hv[j2];
             if (K > 1) hc[(int64_t)(K - 2) * D] = x_t[b * D + d];
-            v = fmaf(__ldg(scale + d), l, v);
+            v = fmaf(scale[d], l, v);
         }
         st_elem(z_t + b * D + d, v);
     }

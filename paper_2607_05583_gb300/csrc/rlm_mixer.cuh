@@ -14,7 +14,7 @@ __device__ __forceinline__ float gatef(float v) { return __fdividef(1.0f, 1.0f +
 __device__ __forceinline__ void build_coupling(float *C, const float *c_raw, float lam, int H) {
     const float k = lam * rsqrtf((float)H);
     for (int i = threadIdx.x; i < H * H; i += blockDim.x)
-        C[i] = (i / H == i % H ? 1.0f : 0.0f) + k * tanhf(__ldg(c_raw + i));
+        C[i] = (i / H == i % H ? 1.0f : 0.0f) + k * tanhf(c_raw[i]);
 }
 
 }  // namespace rlm

@@ -917,8 +917,7 @@ struct KahanSum {
 };
 __global__ void __launch_bounds__(256) k_grad_reduce(
     int64_t B, int D, int M, int nch, const float *__restrict__ amp,
-    const float *__restrict__ phase, const float2 *__restrict__ ws_s,
-    const float2 *__restrict__ ws_r, const float2 *__restrict__ ws_j, float *__restrict__ g_decay,
+    const float *__restrict__ phase, const float2 *ws_s, const float2 *ws_r, const float2 *ws_j, float *__restrict__ g_decay,
     float *__restrict__ g_freq, float *__restrict__ g_amp, float *__restrict__ g_phase) {
     const int pm = blockIdx.x * blockDim.x + threadIdx.x;
     pdl_wait();

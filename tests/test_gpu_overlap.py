@@ -1,0 +1,110 @@
+"""Calls queued back to back.  Decode steps, and every launch of a call but its first, may
+start while the kernel before them still runs, so a chain in which each call reads what the
+one before wrote (fields, states, coefficients, drive history) must give the same bits as
+the chain with a device synchronisation after every call, and as its captured graph."""
+import numpy as np
+import pytest
+
+from synth import make_inputs, make_mixer_inputs
+from tests._util import to_dev
+
+torch = pytest.importorskip("torch")
+rlm = pytest.importorskip("paper_2607_05583_gb300")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    from paper_2607_05583_gb300 import build
+    build.build()
+    return rlm.load_library()
+
+
+def _fields(L, D, M, dtype, K=4):
+    inp = make_inputs(1, L, D, M, dtype, seed=L + M, with_dy=True)
+    mx = make_mixer_inputs(inp, K, seed=M)
+    return dict(p=rlm.Params.from_arrays(*inp.params()), x=to_dev(inp.x, dtype), dy=to_dev(inp.dy, dtype),
+                g=to_dev(mx.g, dtype), local=rlm.Local.from_arrays(mx.conv_w, mx.scale),
+                c_raw=np.random.default_rng(M).standard_normal((8, 8)), L=L, D=D, M=M, K=K)
+
+
+def _buffers(f):
+    e = lambda: torch.zeros_like(f["x"])
+    t = lambda: torch.zeros_like(f["x"][0, :1])
+    return dict(y=e(), dx=e(), s=rlm.State.empty(1, f["D"], f["M"]), gr=rlm.Grads.empty(f["D"], f["M"]),
+                conv=rlm.ConvState.empty(1, f["D"], f["K"], dtype=f["x"].dtype), a=t(), b=t(),
+                ws=torch.empty(64 << 20, dtype=torch.uint8, device="cuda"))
+
+
+# Each chain yields after every call.
+def _scan_decode(f, o):
+    rlm.rlm_mix_prefill(f["x"], f["p"], o["y"], o["s"], workspace=o["ws"])
+    yield
+    rlm.rlm_mix_decode(o["y"][0, -1:], o["s"], o["a"])   # the layer above takes the last output
+    yield
+    rlm.rlm_mix_decode(o["a"], o["s"], o["b"])
+    yield
+
+
+def _mixer_decode(f, o):
+    c = rlm.Coupling(f["cr"], 0.5)
+    rlm.rlm_mixer_prefill(f["x"], f["g"], f["p"], f["local"], o["y"], state_out=o["s"], conv_out=o["conv"],
+                          workspace=o["ws"], coupling=c)
+    yield
+    rlm.rlm_mixer_decode(o["y"][0, -1:], f["g"][0, -1:], o["s"], f["local"], o["conv"], o["a"], coupling=c)
+    yield
+    rlm.rlm_mixer_decode(o["a"], f["g"][0, :1], o["s"], f["local"], o["conv"], o["b"], coupling=c)
+    yield
+
+
+def _backward_decode(f, o):
+    rlm.rlm_state_init(o["s"], f["p"])
+    yield
+    rlm.rlm_mix_decode(f["x"][0, :1], o["s"], o["a"])
+    yield
+    rlm.rlm_mix_backward(f["dy"], f["x"], f["p"], o["dx"], o["gr"], workspace=o["ws"])
+    yield
+    rlm.rlm_mix_decode(o["dx"][0, -1:], o["s"], o["b"])
+    yield
+    rlm.rlm_mix_prefill(o["dx"], f["p"], o["y"], None, workspace=o["ws"])
+    yield
+
+
+def _results(o):
+    return [t.clone() for t in (o["y"], o["dx"], o["s"].s, o["conv"].u, o["a"], o["b"], o["gr"].decay, o["gr"].freq,
+                                o["gr"].amp, o["gr"].phase)]
+
+
+@pytest.mark.parametrize("chain", [_scan_decode, _mixer_decode, _backward_decode])
+@pytest.mark.parametrize("L,D,M,dtype", [(5000, 64, 20, "f32"), (3000, 256, 16, "bf16"), (2500, 128, 32, "bf16"),
+                                         (700, 64, 33, "bf16")])
+def test_a_queued_chain_equals_the_synchronised_one(chain, L, D, M, dtype):
+    f = _fields(L, D, M, dtype)
+    f["cr"] = torch.from_numpy(f["c_raw"].astype(np.float32)).cuda()
+    zero = lambda o: [t.zero_() for t in (o["y"], o["dx"], o["s"].s, o["s"].coef, o["conv"].u, o["a"], o["b"],
+                                          o["gr"].decay, o["gr"].freq, o["gr"].amp, o["gr"].phase)]
+    o = _buffers(f)
+    zero(o)
+    for _ in chain(f, o):
+        torch.cuda.synchronize()
+    want = _results(o)
+    for _ in range(3):
+        zero(o)
+        for _ in chain(f, o):
+            pass
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(want, _results(o)))
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        graph.capture_begin()
+        for _ in chain(f, o):
+            pass
+        graph.capture_end()
+    torch.cuda.current_stream().wait_stream(side)
+    for _ in range(2):
+        zero(o)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(want, _results(o)))
