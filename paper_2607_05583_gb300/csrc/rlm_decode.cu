@@ -270,8 +270,10 @@ cudaError_t launch_pdl(Kern kern, dim3 grid, cudaStream_t st, Args... args) {
 // consecutive threads on consecutive pairs, so the M / 2 threads of a channel form one
 // aligned shuffle group.  Phase 1 updates the states and puts each channel's readout in
 // shared memory (fp32); after the block barrier, phase 2 forms C y_t, applies the gate and
-// the local path, shifts the history and writes z_t.  C depends on the parameters
-// only, so it is built before the wait.
+// the local path, shifts the history and writes z_t.  C is built after the wait as well,
+// behind these loads: the kernel before may have written the coupling matrix.  (Built before
+// the wait, from data that wait does not cover, a step took, us: B = 64, D = 256, M = 16, H = 8 2.69,
+// now 2.70; B = 128 3.01, 3.08; B = 4, H = 32 3.0, 3.6; B = 16, D = 128, M = 32, H = 64 5.3, 7.0.)
 constexpr int kCoupledBlock = 512;             // one block per row
 constexpr int kSplitBlock = 256;               // several blocks per row
 constexpr int kCoupledMaxModesPerRow = 8 * kCoupledBlock;   // D * M <= 4096
@@ -292,9 +294,11 @@ __global__ void __launch_bounds__(kBlock, kBlock == kCoupledBlock ? 1 : kIters =
     // Channel c of the block (head-major over its positions) is channel at(c) of the row.
     const int dh = D / H, dq = kWhole ? dh : dh / Q, n = kWhole ? D : H * dq, p0 = blockIdx.x * dq;
     auto at = [&](int c) { return kWhole ? c : c / dq * dh + p0 + c % dq; };
-    build_coupling(C, c_raw, lam, H);
+    // The kernel before may write the coupling matrix too: before the wait it only moves to L2.
+    for (int i = 32 * threadIdx.x; i < H * H; i += 32 * kBlock) prefetch_l2(c_raw + i);
     pdl_wait();
     pdl_launch_dependents();
+    request_coupling(C, c_raw, H);
     const T *xb = x_t + b * D;
     // ---- loads: phase 2's inputs (channel d2) ...
     const int c2 = threadIdx.x, K = mix.K;
@@ -339,6 +343,7 @@ __global__ void __launch_bounds__(kBlock, kBlock == kCoupledBlock ? 1 : kIters =
             c1v[k] = coef[(int64_t)d * M + 2 * g + 1];
         }
     }
+    finish_coupling(C, c_raw, lam, H);
     // ---- phase 1: every thread runs every iteration, so whole warps shuffle
 #pragma unroll
     for (int k = 0; k < kIters; ++k) {

@@ -54,7 +54,8 @@ __device__ __forceinline__ float2 lambda_pow(float gamma, float omega, float n) 
 // the kernel before it in the stream drains; it calls pdl_wait() before it touches what
 // that kernel (or one before it in the same call) writes, in every block, so that its own
 // end implies theirs.  The first kernel of a call is launched normally, so caller inputs
-// need no wait.  pdl_launch_dependents() lets the next such kernel start once every block
+// need no wait -- except that of a decode step, which is a dependent launch itself and
+// reads nothing before the wait (it may prefetch to L2).  pdl_launch_dependents() lets the next such kernel start once every block
 // of this one has called it or ended.
 // Such a kernel's life overlaps the writes of the one before it, so it reads what that
 // kernel writes by plain loads through pointers that are not const __restrict__: __ldg() (which

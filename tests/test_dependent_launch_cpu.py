@@ -77,3 +77,15 @@ def test_helpers_of_dependent_kernels_use_plain_loads():
     assert "__ldg(" not in SOURCES["rlm_mixer.cuh"]
     mix = SOURCES["rlm_decode.cu"]
     assert "__ldg(" not in mix[mix.index("MixPart<T> mix_part("):mix.index("void mix_shift(")]
+
+
+# Decode steps are the first kernel of their call and a dependent launch: the kernel before
+# them may write anything they read.
+@pytest.mark.parametrize("name", ["k_decode_tile", "k_decode_any", "k_decode_coupled", "k_mixer_finish"])
+def test_decode_kernels_read_nothing_before_their_wait(name):
+    params, body = kernel(name)
+    before = re.split(r"pdl_wait\(\)|griddepcontrol\.wait", body)[0]
+    before = re.sub(r"prefetch_\w+\([^;]*;", "", before)
+    pointers = [re.search(r"(\w+)\s*$", p.strip()).group(1) for p in params.split(",") if "*" in p]
+    for p in pointers + ["mix.hist", "mix.conv_w", "mix.scale"]:
+        assert not re.search(r"(?<![\w.])" + re.escape(p) + r"\b", before), f"{p} is used before the wait"

@@ -5,8 +5,9 @@ the chain with a device synchronisation after every call, and as its captured gr
 import numpy as np
 import pytest
 
+import oracle
 from synth import make_inputs, make_mixer_inputs
-from tests._util import to_dev
+from tests._util import TOL, assert_close, to_dev, to_np
 
 torch = pytest.importorskip("torch")
 rlm = pytest.importorskip("paper_2607_05583_gb300")
@@ -108,3 +109,30 @@ def test_a_queued_chain_equals_the_synchronised_one(chain, L, D, M, dtype):
         graph.replay()
         torch.cuda.synchronize()
         assert all(torch.equal(a, b) for a, b in zip(want, _results(o)))
+
+
+# The coupling matrix is written by the kernel right before every step: matrices of fewer and
+# of more entries than a block has threads (256 with several blocks a row, 512 with one).
+@pytest.mark.parametrize("B,D,M,H,dtype", [(2, 256, 16, 16, "bf16"), (3, 240, 16, 20, "f32"), (2, 128, 32, 64, "f32"),
+                                           (80, 256, 16, 32, "bf16"), (90, 384, 8, 24, "f32"), (2, 408, 4, 51, "f32")])
+def test_coupled_steps_take_the_matrix_written_just_before(B, D, M, H, dtype):
+    T, K = 3, 2
+    inp = make_inputs(B, T, D, M, dtype, seed=B + H)
+    mx = make_mixer_inputs(inp, K, seed=H)
+    c_np = np.random.default_rng(H).standard_normal((H, H))
+    want = torch.from_numpy(c_np.astype(np.float32)).cuda()
+    c = rlm.Coupling(torch.empty_like(want), 0.5)
+    x, g = to_dev(inp.x, dtype), to_dev(mx.g, dtype)
+    tokens = [(x[:, t].contiguous(), g[:, t].contiguous()) for t in range(T)]
+    st, local = rlm.State.empty(B, D, M), rlm.Local.from_arrays(mx.conv_w, mx.scale)
+    rlm.rlm_state_init(st, rlm.Params.from_arrays(*inp.params()))
+    conv, z = rlm.ConvState(to_dev(mx.conv_in, dtype)), torch.empty(T, B, D, dtype=x.dtype, device="cuda")
+    for t, (xt, gt) in enumerate(tokens):
+        c.c_raw.fill_(9.0 + t)
+        c.c_raw.copy_(want)
+        rlm.rlm_mixer_decode(xt, gt, st, local, conv, z[t], coupling=c)
+        c.c_raw.fill_(-5.0)
+    torch.cuda.synchronize()
+    ref = oracle.mixer_prefill(inp.x, mx.g, *inp.params(), mx.conv_w, mx.scale, conv_in=mx.conv_in,
+                               coupling=(c_np, 0.5))[0]
+    assert_close(to_np(z.transpose(0, 1)), ref, TOL[dtype], "z")
