@@ -323,10 +323,19 @@ def _check(status: int, where: str):
         raise RlmError(status, where, load_library().rlm_last_error().decode())
 
 
-def _workspace(nbytes: int, device) -> torch.Tensor | None:
+def _workspace(nbytes: int, device, stream=None) -> torch.Tensor | None:
+    """A fresh workspace for a call on ``stream``.  The allocator gives a freed block to
+    later work of the stream that was current when the block was allocated, so that has to
+    be the call's own stream: the caller drops the block as soon as the call is enqueued."""
     if nbytes == 0:
         return None
-    return torch.empty(nbytes, dtype=torch.uint8, device=device)
+    handle = _stream(stream)
+    if handle == torch.cuda.current_stream(device).cuda_stream:
+        return torch.empty(nbytes, dtype=torch.uint8, device=device)
+    # Handles 0 and 1 (cudaStreamLegacy) are the default stream.
+    own = torch.cuda.default_stream(device) if handle in (0, 1) else torch.cuda.ExternalStream(handle, device=device)
+    with torch.cuda.stream(own):
+        return torch.empty(nbytes, dtype=torch.uint8, device=device)
 
 
 # --------------------------------------------------------------- entry points
@@ -366,7 +375,7 @@ def rlm_mix_prefill(x: torch.Tensor, params: Params, y: torch.Tensor,
     xt, yt = _field(x), _field(y)
     if workspace is None:
         workspace = _workspace(lib.rlm_prefill_workspace_size(xt.B, xt.L, xt.D, params.M, xt.dtype),
-                               x.device)
+                               x.device, stream)
     st = state_out._c() if state_out is not None else None
     _check(lib.rlm_mix_prefill(ctypes.byref(xt), ctypes.byref(params._c()), ctypes.byref(yt),
                                ctypes.byref(st) if st is not None else None,
@@ -388,7 +397,7 @@ def rlm_mix_prefill_from(x: torch.Tensor, params: Params, state_in: State | None
     xt, yt = _field(x), _field(y)
     if workspace is None:
         workspace = _workspace(lib.rlm_prefill_workspace_size(xt.B, xt.L, xt.D, params.M, xt.dtype),
-                               x.device)
+                               x.device, stream)
     si = state_in._c() if state_in is not None else None
     so = state_out._c() if state_out is not None else None
     _check(lib.rlm_mix_prefill_from(ctypes.byref(xt), ctypes.byref(params._c()),
@@ -442,7 +451,7 @@ def rlm_mix_backward(dy: torch.Tensor, x: torch.Tensor, params: Params, dx: torc
     dyt, xt, dxt = _field(dy), _field(x), _field(dx)
     if workspace is None:
         workspace = _workspace(lib.rlm_backward_workspace_size(xt.B, xt.L, xt.D, params.M,
-                                                               xt.dtype), x.device)
+                                                               xt.dtype), x.device, stream)
     _check(lib.rlm_mix_backward(ctypes.byref(dyt), ctypes.byref(xt), ctypes.byref(params._c()),
                                 ctypes.byref(dxt), ctypes.byref(dparams._c()),
                                 ctypes.byref(_launch(stream, workspace))), "rlm_mix_backward")
@@ -465,7 +474,7 @@ def rlm_mix_backward_from(dy: torch.Tensor, x: torch.Tensor, params: Params, sta
     dyt, xt, dxt = _field(dy), _field(x), _field(dx)
     if workspace is None:
         workspace = _workspace(lib.rlm_backward_workspace_size(xt.B, xt.L, xt.D, params.M, xt.dtype),
-                               x.device)
+                               x.device, stream)
     opt = lambda st: ctypes.byref(st._c()) if st is not None else None
     _check(lib.rlm_mix_backward_from(ctypes.byref(dyt), ctypes.byref(xt), ctypes.byref(params._c()),
                                      opt(state_in), opt(d_state_out), ctypes.byref(dxt),
@@ -502,7 +511,7 @@ def rlm_mixer_prefill(x: torch.Tensor, g: torch.Tensor | None, params: Params, l
     gt = _field(g) if g is not None else None
     if workspace is None:
         workspace = _workspace(lib.rlm_prefill_workspace_size(xt.B, xt.L, xt.D, params.M, xt.dtype),
-                               x.device)
+                               x.device, stream)
     ref = lambda c: ctypes.byref(c) if c is not None else None
     opt = lambda o: ref(o._c()) if o is not None else None
     _check(lib.rlm_mixer_prefill(ctypes.byref(xt), ref(gt), ctypes.byref(params._c()), opt(local), opt(coupling),

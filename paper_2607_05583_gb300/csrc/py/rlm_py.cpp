@@ -12,7 +12,7 @@
 // checks and raises its own error.
 //
 // No object, pointer or size is kept from one call to the next: only the interned
-// attribute names, torch's dtype objects and three torch functions.
+// attribute names, torch's dtype objects and five torch functions.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -21,9 +21,9 @@
 namespace {
 
 PyObject *s_dtype, *s_is_cuda, *s_is_contiguous, *s_shape, *s_data_ptr, *s_device, *s_cuda_stream;
-PyObject *s_decay, *s_freq, *s_amp, *s_phase, *s_s, *s_coef, *s_conv_w, *s_scale, *s_c_raw, *s_lambda_c, *s_u;
+PyObject *s_decay, *s_freq, *s_amp, *s_phase, *s_s, *s_coef, *s_conv_w, *s_scale, *s_c_raw, *s_lambda_c, *s_u, *s_index;
 PyObject *g_f32, *g_bf16, *g_u8;                  // torch dtypes
-PyObject *g_get_device, *g_get_stream, *g_empty;  // torch functions
+PyObject *g_get_device, *g_get_stream, *g_empty, *g_raw_alloc, *g_raw_delete;  // torch functions
 PyObject *g_empty_kw;                             // ("dtype", "device")
 PyObject *g_numel, *g_element_size;
 
@@ -207,26 +207,81 @@ bool stream_handle(PyObject *o, void **st) {
     return ok;
 }
 
-// The launch context.  Without a workspace of the caller's, a fresh one of `need` bytes
-// from torch's allocator; *own then holds it until the call has been enqueued (the
-// allocator is stream-ordered).
-bool launch(PyObject *stream, PyObject *ws, size_t need, PyObject *like, rlm_launch *ln, PyObject **own) {
-    *own = nullptr;
+// The workspace of a call that brought none, given back once the call has been enqueued.
+// torch's allocator hands a block that was freed to later work of the stream the block was
+// allocated under, so it is allocated under the stream that the call runs on: by torch.empty
+// when that is the current one, else by the allocator's entry that takes a stream.
+struct Scratch {
+    PyObject *tensor = nullptr;   // torch.empty's, or
+    PyObject *raw = nullptr;      // the address from raw_alloc
+    void release() {
+        Py_XDECREF(tensor);
+        if (raw) {
+            PyObject *r = PyObject_CallOneArg(g_raw_delete, raw);
+            if (!r) PyErr_WriteUnraisable(g_raw_delete);
+            Py_XDECREF(r);
+            Py_DECREF(raw);
+        }
+        tensor = raw = nullptr;
+    }
+};
+
+// Whether st is the current stream of the current device, and that device's index.
+bool current(void *st, long *device, bool *is) {
+    PyObject *dev = PyObject_CallNoArgs(g_get_device);
+    if (!dev) return false;
+    *device = PyLong_AsLong(dev);
+    void *now = nullptr;
+    PyObject *v = PyObject_CallOneArg(g_get_stream, dev);
+    Py_DECREF(dev);
+    if (!v) return false;
+    now = reinterpret_cast<void *>(PyLong_AsUnsignedLongLong(v));
+    Py_DECREF(v);
+    *is = now == st;
+    return !PyErr_Occurred();
+}
+
+bool allocate(size_t need, PyObject *stream, PyObject *like, rlm_launch *ln, Scratch *own) {
+    long device = 0;
+    bool same = true;
+    if (stream != Py_None && !current(ln->stream, &device, &same)) return false;
+    PyObject *n = PyLong_FromSize_t(need), *dev = PyObject_GetAttr(like, s_device);
+    bool ok = n && dev;
+    if (ok && same) {
+        PyObject *args[3] = {n, g_u8, dev};
+        own->tensor = PyObject_Vectorcall(g_empty, args, 1, g_empty_kw);
+        PyObject *p = own->tensor ? PyObject_CallMethodNoArgs(own->tensor, s_data_ptr) : nullptr;
+        if (p) ln->workspace = reinterpret_cast<void *>(PyLong_AsUnsignedLongLong(p));
+        Py_XDECREF(p);
+        ok = p && !PyErr_Occurred();
+    } else if (ok) {
+        // raw_alloc takes the current device's memory: the fields' device, or not the plain case.
+        PyObject *idx = PyObject_GetAttr(dev, s_index);
+        ok = idx && PyLong_Check(idx) && PyLong_AsLong(idx) == device;
+        Py_XDECREF(idx);
+        PyObject *handle = ok ? PyLong_FromVoidPtr(ln->stream) : nullptr;
+        PyObject *args[2] = {n, handle};
+        own->raw = handle ? PyObject_Vectorcall(g_raw_alloc, args, 2, nullptr) : nullptr;
+        Py_XDECREF(handle);
+        if (own->raw) ln->workspace = PyLong_AsVoidPtr(own->raw);
+        ok = own->raw && !PyErr_Occurred();
+    }
+    Py_XDECREF(n);
+    Py_XDECREF(dev);
+    if (!ok) {
+        PyErr_Clear();   // the call takes the Python route, which raises its own
+        own->release();
+    }
+    ln->workspace_bytes = need;
+    return ok;
+}
+
+// The launch context: the caller's workspace, or a fresh one of `need` bytes.
+bool launch(PyObject *stream, PyObject *ws, size_t need, PyObject *like, rlm_launch *ln, Scratch *own) {
     ln->workspace = nullptr;
     ln->workspace_bytes = 0;
     if (!stream_handle(stream, &ln->stream)) return false;
-    if (ws == Py_None && need > 0) {
-        PyObject *n = PyLong_FromSize_t(need), *dev = PyObject_GetAttr(like, s_device);
-        if (n && dev) {
-            PyObject *args[3] = {n, g_u8, dev};
-            *own = PyObject_Vectorcall(g_empty, args, 1, g_empty_kw);
-        }
-        Py_XDECREF(n);
-        Py_XDECREF(dev);
-        if (!*own) return false;
-        ws = *own;
-    }
-    if (ws == Py_None) return true;
+    if (ws == Py_None) return need == 0 || allocate(need, stream, like, ln, own);
     PyObject *p = PyObject_CallMethodNoArgs(ws, s_data_ptr);
     PyObject *n = p ? PyObject_CallMethodNoArgs(ws, g_numel) : nullptr;
     PyObject *e = n ? PyObject_CallMethodNoArgs(ws, g_element_size) : nullptr;
@@ -247,12 +302,12 @@ PyObject *other() {
 }
 
 template <typename F>
-PyObject *finish(PyObject *own, F call) {
+PyObject *finish(Scratch &own, F call) {
     rlm_status s;
     Py_BEGIN_ALLOW_THREADS
     s = call();
     Py_END_ALLOW_THREADS
-    Py_XDECREF(own);
+    own.release();
     return PyLong_FromLong((long)s);
 }
 
@@ -262,7 +317,7 @@ PyObject *mix_prefill(PyObject *, PyObject *const *a, Py_ssize_t n) {
     rlm_params p;
     rlm_state si, so, *psi, *pso;
     rlm_launch ln;
-    PyObject *own;
+    Scratch own;
     if (n != 7 || !field(a[0], &x) || !params(a[1], &p) || !state(a[2], &si, &psi) || !field(a[3], &y) ||
         !state(a[4], &so, &pso) || x.D > 0x7fffffff)
         return other();
@@ -276,7 +331,7 @@ PyObject *mix_decode(PyObject *, PyObject *const *a, Py_ssize_t n) {
     rlm_tensor x, y;
     rlm_state s, *ps;
     rlm_launch ln;
-    PyObject *own;
+    Scratch own;
     if (n != 4 || !field(a[0], &x) || !state(a[1], &s, &ps) || !ps || !field(a[2], &y) ||
         !launch(a[3], Py_None, 0, a[0], &ln, &own))
         return other();
@@ -290,7 +345,7 @@ PyObject *mix_backward(PyObject *, PyObject *const *a, Py_ssize_t n) {
     rlm_state si, go, ds, *psi, *pgo, *pds;
     rlm_grads g;
     rlm_launch ln;
-    PyObject *own;
+    Scratch own;
     if (n != 10 || !field(a[0], &dy) || !field(a[1], &x) || !params(a[2], &p) || !state(a[3], &si, &psi) ||
         !state(a[4], &go, &pgo) || !field(a[5], &dx) || !grads(a[6], &g) || !state(a[7], &ds, &pds) ||
         x.D > 0x7fffffff)
@@ -309,7 +364,7 @@ PyObject *mixer_prefill(PyObject *, PyObject *const *a, Py_ssize_t n) {
     rlm_state si, so, *psi, *pso;
     rlm_conv_state ci, co, *pci, *pco;
     rlm_launch ln;
-    PyObject *own;
+    Scratch own;
     if (n != 12 || !field(a[0], &x) || !opt_field(a[1], &g, &pg) || !params(a[2], &p) ||
         !local_path(a[3], &l, &pl) || !coupling(a[4], &c, &pc) || !state(a[5], &si, &psi) ||
         !conv_state(a[6], &ci, &pci) || !field(a[7], &z) || !state(a[8], &so, &pso) ||
@@ -328,7 +383,7 @@ PyObject *mixer_decode(PyObject *, PyObject *const *a, Py_ssize_t n) {
     rlm_coupling c, *pc;
     rlm_conv_state cv, *pcv;
     rlm_launch ln;
-    PyObject *own;
+    Scratch own;
     if (n != 8 || !field(a[0], &x) || !opt_field(a[1], &g, &pg) || !state(a[2], &s, &ps) || !ps ||
         !local_path(a[3], &l, &pl) || !coupling(a[4], &c, &pc) || !conv_state(a[5], &cv, &pcv) || !field(a[6], &z) ||
         !launch(a[7], Py_None, 0, a[0], &ln, &own))
@@ -352,7 +407,7 @@ PyMODINIT_FUNC PyInit__rlm_py(void) {
                  {&s_cuda_stream, "cuda_stream"}, {&s_decay, "decay"}, {&s_freq, "freq"},
                  {&s_amp, "amp"},         {&s_phase, "phase"},       {&s_s, "s"},
                  {&s_coef, "coef"},       {&s_conv_w, "conv_w"},     {&s_scale, "scale"},
-                 {&s_c_raw, "c_raw"},     {&s_lambda_c, "lambda_c"}, {&s_u, "u"},
+                 {&s_c_raw, "c_raw"},     {&s_lambda_c, "lambda_c"}, {&s_u, "u"},               {&s_index, "index"},
                  {&g_numel, "numel"},     {&g_element_size, "element_size"}};
     for (auto &v : names)
         if (!(*v.to = PyUnicode_InternFromString(v.name))) return nullptr;
@@ -362,6 +417,8 @@ PyMODINIT_FUNC PyInit__rlm_py(void) {
         !(g_u8 = PyObject_GetAttrString(torch, "uint8")) || !(g_empty = PyObject_GetAttrString(torch, "empty")) ||
         !(g_get_device = PyObject_GetAttrString(c, "_cuda_getDevice")) ||
         !(g_get_stream = PyObject_GetAttrString(c, "_cuda_getCurrentRawStream")) ||
+        !(g_raw_alloc = PyObject_GetAttrString(c, "_cuda_cudaCachingAllocator_raw_alloc")) ||
+        !(g_raw_delete = PyObject_GetAttrString(c, "_cuda_cudaCachingAllocator_raw_delete")) ||
         !(g_empty_kw = Py_BuildValue("(ss)", "dtype", "device")))
         return nullptr;
     Py_DECREF(torch);

@@ -136,3 +136,65 @@ def test_coupled_steps_take_the_matrix_written_just_before(B, D, M, H, dtype):
     ref = oracle.mixer_prefill(inp.x, mx.g, *inp.params(), mx.conv_w, mx.scale, conv_in=mx.conv_in,
                                coupling=(c_np, 0.5))[0]
     assert_close(to_np(z.transpose(0, 1)), ref, TOL[dtype], "z")
+
+
+# A call on another stream than the current one, without a workspace: its workspace is neither
+# a block that work of the current stream still uses, nor given to that stream while the call runs.
+@pytest.mark.parametrize("native", [True, False])
+@pytest.mark.parametrize("handle", [False, True])
+@pytest.mark.parametrize("B,L,D,M,dtype", [(1, 9000, 64, 20, "f32"), (2, 2000, 128, 32, "bf16")])
+def test_workspace_of_a_call_on_a_side_stream(monkeypatch, native, handle, B, L, D, M, dtype):
+    if not native:
+        monkeypatch.setattr(rlm, "_native", _NoNative())
+    inp = make_inputs(B, L, D, M, dtype, seed=L, with_dy=True)
+    p, x, dy = rlm.Params.from_arrays(*inp.params()), to_dev(inp.x, dtype), to_dev(inp.dy, dtype)
+    need = rlm.rlm_prefill_workspace_size(B, L, D, M, x.dtype), rlm.rlm_backward_workspace_size(B, L, D, M, x.dtype)
+    assert min(need) > 0
+
+    def calls(stream, y, dx, gr):
+        rlm.rlm_mix_prefill(x, p, y, stream=stream)
+        rlm.rlm_mix_backward(dy, x, p, dx, gr, stream=stream)
+
+    outs = [(torch.zeros_like(x), torch.zeros_like(x), rlm.Grads.empty(D, M)) for _ in range(2)]
+    calls(None, *outs[0])
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    for n in need:   # blocks of these sizes are free, and the current stream still writes them
+        block = torch.empty(n, dtype=torch.uint8, device="cuda")
+        torch.cuda._sleep(2_000_000)
+        block.fill_(0x7f)
+        del block
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(1_000_000)   # the current stream's later work runs first
+    calls(side.cuda_stream if handle else side, *outs[1])
+    for n in need:
+        torch.empty(n, dtype=torch.uint8, device="cuda").fill_(0x7f)
+    torch.cuda.synchronize()
+    for a, b in zip(outs[0][:2], outs[1][:2]):
+        assert torch.equal(a, b)
+    for k in ("decay", "freq", "amp", "phase"):
+        assert torch.equal(getattr(outs[0][2], k), getattr(outs[1][2], k))
+
+
+class _NoNative:
+    """Hands every call to the ctypes route."""
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
+@pytest.mark.parametrize("native", [True, False])
+def test_default_stream_by_handle_while_another_is_current(monkeypatch, native):
+    if not native:
+        monkeypatch.setattr(rlm, "_native", _NoNative())
+    inp = make_inputs(1, 5000, 64, 20, "f32", seed=1)
+    p, x = rlm.Params.from_arrays(*inp.params()), to_dev(inp.x, "f32")
+    want, y = torch.zeros_like(x), torch.zeros_like(x)
+    rlm.rlm_mix_prefill(x, p, want)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        for h in (0, 1):
+            y.zero_()
+            torch.cuda.synchronize()
+            rlm.rlm_mix_prefill(x, p, y, stream=h)
+            torch.cuda.synchronize()
+            assert torch.equal(y, want)
