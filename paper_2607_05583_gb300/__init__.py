@@ -3,9 +3,10 @@
 Argument marshalling only: every step of the operator runs in the library's
 CUDA kernels, reached through the C ABI declared in ``include/rlm.h`` with the
 same function names.  Calls with plain arguments (contiguous CUDA tensors) are
-marshalled by ``_rlm_py`` (``csrc/py/rlm_py.cpp``); what it hands back (None) takes the
-ctypes route below, which also raises the errors.  PyTorch supplies device memory and the current stream.
-There is no fallback: if the compiled library is missing the calls raise.
+marshalled by ``_rlm_py`` (``csrc/py/rlm_py.cpp``); what it hands back (None), and everything
+where it is not built, takes the ctypes route below, which also raises the errors.  PyTorch
+supplies device memory and the current stream.  There is no fallback for the kernels: if the
+compiled library is missing the calls raise.
 
 Names follow the paper (ResonatorLM, arxiv 2607.05583): x is the drive field
 [B][L][D]; decay gamma, frequency omega, amplitude A and phase phi are the
@@ -18,6 +19,7 @@ import ctypes
 import importlib.machinery
 import importlib.util
 import os
+import warnings
 from dataclasses import dataclass
 
 import torch
@@ -92,17 +94,18 @@ def library_path() -> str:
 
 
 def load_library(build_if_missing: bool = False) -> ctypes.CDLL:
-    """Load librlm.so (raises if it has not been built)."""
+    """Load librlm.so (raises if it has not been built) and, where it was built, the native
+    call path beside it."""
     global _lib, _native
     if _lib is not None:
         return _lib
     path = _build_mod.LIB
-    if not os.path.exists(path):
-        if not build_if_missing:
-            raise RuntimeError(
-                f"the CUDA library {path} is not built; run "
-                "`python -c 'import __graft_entry__ as g; g.build()'` first")
+    if build_if_missing and not (os.path.exists(path) and os.path.exists(_build_mod.PYLIB)):
         _build_mod.build()
+    if not os.path.exists(path):
+        raise RuntimeError(
+            f"the CUDA library {path} is not built; run "
+            "`python -c 'import __graft_entry__ as g; g.build()'` first")
     lib = ctypes.CDLL(path)
     P = ctypes.POINTER
     lib.rlm_mix_prefill.argtypes = [P(_Tensor), P(_Params), P(_Tensor), P(_State), P(_Launch)]
@@ -137,12 +140,30 @@ def load_library(build_if_missing: bool = False) -> ctypes.CDLL:
     lib.rlm_mix_prefill_noalloc.argtypes = [P(_Tensor), P(_Params), P(_Tensor), P(_State),
                                             ctypes.c_void_p]
     lib.rlm_mix_prefill_noalloc.restype = ctypes.c_int
-    spec = importlib.util.spec_from_file_location(
-        "_rlm_py", _build_mod.PYLIB, loader=importlib.machinery.ExtensionFileLoader("_rlm_py", _build_mod.PYLIB))
-    native = importlib.util.module_from_spec(spec)
-    spec.loader.exec_module(native)
-    _native, _lib = native, lib
+    _native, _lib = _load_native(), lib
     return lib
+
+
+class _CtypesOnly:
+    """Stands for the _rlm_py module where it is not built: every call takes the ctypes route."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
+def _load_native():
+    path = _build_mod.PYLIB
+    if not os.path.exists(path):   # built without Python's headers
+        return _CtypesOnly()
+    spec = importlib.util.spec_from_file_location(
+        "_rlm_py", path, loader=importlib.machinery.ExtensionFileLoader("_rlm_py", path))
+    try:
+        native = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(native)
+    except ImportError as e:   # another Python's, say
+        warnings.warn(f"{path} cannot be loaded ({e}); calls take the slower ctypes route")
+        return _CtypesOnly()
+    return native
 
 
 # --------------------------------------------------------------- containers

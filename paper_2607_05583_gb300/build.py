@@ -42,10 +42,17 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def _python_include():
+    """Directory of Python's C headers, or None where they are not installed."""
+    path = sysconfig.get_paths()["include"]
+    return path if os.path.exists(os.path.join(path, "Python.h")) else None
+
+
 def _stale() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(PYLIB):
+    libs = [LIB, PYLIB] if _python_include() else [LIB]
+    if not all(os.path.exists(p) for p in libs):
         return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(PYLIB))
+    t = min(os.path.getmtime(p) for p in libs)
     deps = [PYSRC] + sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh"))
     deps += glob.glob(os.path.join(INCLUDE, "*.h"))
     return any(os.path.getmtime(p) > t for p in deps)
@@ -79,10 +86,16 @@ def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
     if res.returncode != 0:
         raise RuntimeError(f"link failed:\n{res.stdout}\n{res.stderr}")
     os.replace(tmp, LIB)
-    # The binding's call path links against librlm.so beside it.
+    # The binding's call path links against librlm.so beside it.  Without Python's headers the
+    # package makes its calls through ctypes (and not through an older build of the binding).
+    include = _python_include()
+    if include is None:
+        if os.path.exists(PYLIB):
+            os.remove(PYLIB)
+        return LIB
     tmp = PYLIB + f".{os.getpid()}.tmp"
     cmd = [nvcc, "-O2", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "-cudart", "none",
-           "-I", sysconfig.get_paths()["include"], "-shared", PYSRC, "-o", tmp, LIB,
+           "-I", include, "-shared", PYSRC, "-o", tmp, LIB,
            "-Xlinker", "-rpath", "-Xlinker", "$ORIGIN"]
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
