@@ -334,6 +334,12 @@ RLM_API const char *rlm_status_string(rlm_status status);
  * copies to device symbols on the current device); not for production use. */
 RLM_API rlm_status rlm_test_stall_segments(int on);
 
+/* Test hook: how the tcgen05 backward (bf16, M <= 32) shares B batch rows of `ntiles`
+ * 2048-token tiles among its blocks on the current device.  Returns the number of
+ * blocks; with 0 <= block < that, out receives the block's channel, first row, number
+ * of rows and level.  Host only, launches nothing. */
+RLM_API int rlm_test_backward_plan(int64_t B, int D, int ntiles, int block, int out[4]);
+
 /* Human-readable reason for the last non-OK status returned on this host
  * thread (valid until the next call on the thread). */
 RLM_API const char *rlm_last_error(void);

@@ -124,6 +124,8 @@ def load_library(build_if_missing: bool = False) -> ctypes.CDLL:
     lib.rlm_validate_params.argtypes = [P(_Params)]
     lib.rlm_get_device_status.argtypes = [P(_Launch)]
     lib.rlm_test_stall_segments.argtypes = [ctypes.c_int]
+    lib.rlm_test_backward_plan.argtypes = [ctypes.c_int64, ctypes.c_int, ctypes.c_int, ctypes.c_int, P(ctypes.c_int)]
+    lib.rlm_test_backward_plan.restype = ctypes.c_int
     for f in ("rlm_prefill_workspace_size", "rlm_backward_workspace_size"):
         getattr(lib, f).argtypes = [ctypes.c_int64, ctypes.c_int64, ctypes.c_int,
                                     ctypes.c_int, ctypes.c_int]

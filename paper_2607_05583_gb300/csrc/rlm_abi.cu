@@ -600,6 +600,11 @@ rlm_status rlm_get_device_status(const rlm_launch *ln) {
     return RLM_OK;
 }
 
+int rlm_test_backward_plan(int64_t B, int D, int ntiles, int block, int out[4]) {
+    return B < 1 || B > 65535 || D < 1 || D > (1 << 20) || ntiles < 1 || !out ? 0
+                                                                              : backward_plan_block(B, D, ntiles, block, out);
+}
+
 rlm_status rlm_test_stall_segments(int on) {
     const cudaError_t e = set_segment_stall(on ? 1 : 0);
     if (e != cudaSuccess) return cuda_fail(e, "rlm_test_stall_segments");

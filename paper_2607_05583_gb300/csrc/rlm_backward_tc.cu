@@ -53,21 +53,25 @@
 // writes the [B][L][D] field.
 //
 // One CTA = one channel of one or more batch rows (RowPlan below; the tables are the
-// channel's, Q and E accumulate over all rows, the carry restarts at each), two CTAs per
-// SM (256 TMEM columns each):
-//   warps 0-3  reverse scan; at the end they read E and form the cross-chunk
-//              (G, P).
-//   warps 4-5  dx epilogue (quarters 0, 1: positions 0-63), then the diagonal
-//              sums of Q.
-//   warp 6     TMA producer, which loads while the others build the tables (with the
-//              producer in warp 7 the call at B = 4, L = 32768, D = 512 took 329 us
-//              against 319, four rows a block; the MMA warps in 6-7 or exchanged, 325-333).
+// channel's, the carry and the sums Q and E restart at each row), two CTAs per SM (256
+// TMEM columns each):
+//   warps 0-3  reverse scan; at a row's end they read E, form the cross-chunk (G, P), add
+//              rho and write the row's partials.
+//   warps 4-5  dx epilogue (quarters 0, 1: positions 0-63); at a row's end the diagonal
+//              sums rho of Q.
+//   warp 6     TMA producer, which loads while the others build the tables.
 //   warp 7     TMEM allocation (and the tables, with warps 0-5 and 8-9).
-//   The kernel may start while the input transposes drain (pdl_wait): only the producer
-//   waits for them, so the tables are built meanwhile.  Backward calls, launches one after
-//   the other and now (us): B = 1, L = 122, D = 424, M = 8 33 -> 26; B = 8, L = 2048, D = 256,
-//   M = 16 42 -> 35; B = 8, L = 4096, D = 256, M = 16 with state terms 97 -> 88.
 //   warp 8     MMA issue: projections and Q; warp 9: T', U' and E.
+//   The kernel may start while the input transposes drain (pdl_wait): only the producer
+//   waits for them, so the tables are built meanwhile.
+// Several rows a CTA (kRows): TMEM additions truncate, so Q and E are summed over one row
+// only, as with one row a CTA, and the rows' (G, P) are added in compensated fp32 by
+// k_grad_reduce.  Both leave TMEM while the next row's first tile is projected and
+// scanned; Q moves to warp 9, whose next products overwrite them.  (Summed over up to 16
+// tiles in TMEM the error of dA against 64 bits at B = 8, L = 4096, D = 256, M = 16 was 2.68e-6
+// against 2.59e-6, mean of 8 seeds; now 2.59e-6.  That took 51 us a call where this takes 70 and one
+// row a CTA 90; 85, 104 and 145 with both state terms.  Q and E issued by warp 7 instead:
+// as fast for several rows, 20 us slower for one of 16 tiles.)
 //
 // Every wait is bounded: after kWaitLimitCycles the waiting thread sets a shared
 // abort flag and the device status word (RLM_ERR_TIMEOUT); all roles then leave
@@ -132,8 +136,11 @@ constexpr int kSlotBytes = 8192;
 // K = the 16 S^n rows, LBO 512).
 constexpr int kOffBs = kOffRing + kSlots * kSlotBytes;   // [2] x (hi 8 KB, lo 8 KB)
 constexpr int kBsBuf = 16384;
-constexpr int kOffRho = kOffBs + 2 * kBsBuf;             // [64] fp32: rho[n]
-constexpr int kOffBar = kOffRho + 64 * 4;
+// rho[n] of a row, double-buffered: the part of each epilogue warp's 32 rows of Q.
+constexpr int kOffRho = kOffBs + 2 * kBsBuf;             // [2][2][64] fp32
+constexpr int kQsStride = 17;                            // 16 columns of Q staged per warp, one word of padding
+constexpr int kOffQs = kOffRho + 2 * 2 * 64 * 4;         // [2 warps][32][17] fp32
+constexpr int kOffBar = kOffQs + 2 * 32 * kQsStride * 4;
 constexpr int kNumBars = 32;
 constexpr int kOffMisc = kOffBar + kNumBars * 8;
 constexpr int kSmemBytes = kOffMisc + 64 + 1024;         // + alignment slack
@@ -146,18 +153,21 @@ constexpr int kOffPw = kOffBs;                                  // [32][65] floa
 constexpr int kOffCf = kOffPw + kMaxModes * kPwStride * 8;      // [32] float2
 constexpr int kOffK = kOffCf + kMaxModes * 8;                   // [64] float
 static_assert(kOffK + 64 * 4 <= kOffRho, "prologue scratch does not fit");
-static_assert(kC * 65 * 4 <= kSlots * kSlotBytes, "Q staging (end of the walk) does not fit in the ring");
 
 // Barrier indices.
 constexpr int kBarSlotFull = 0;                  // [kSlots]
 constexpr int kBarSlotEmpty = kSlots;            // [kSlots]: scan warp 0 + epilogue warp 4
-constexpr int kBarPFull = 2 * kSlots;            // [2]: projections and Q committed
+constexpr int kBarPFull = 2 * kSlots;            // [2]: projections (one row a block: and Q) committed
 constexpr int kBarPEmpty = kBarPFull + 2;        // [2]: 4 scan warps read them
 constexpr int kBarSFull = kBarPEmpty + 2;        // [2]: 4 scan warps wrote [S^n ; R^n]
 constexpr int kBarBsEmpty = kBarSFull + 2;       // [2]: U' and E products done with it
 constexpr int kBarDFull = kBarBsEmpty + 2;       // [2]: dx accumulator (and E) complete
 constexpr int kBarDEmpty = kBarDFull + 2;        // [2]: 2 epilogue warps read it
-static_assert(kBarDEmpty + 2 <= kNumBars, "too many barriers");
+constexpr int kBarRowFull = kBarDEmpty + 2;      // a row's Q and E complete
+constexpr int kBarRowFree = kBarRowFull + 1;     // ... and read: 4 scan + 2 epilogue warps
+constexpr int kBarRhoFull = kBarRowFree + 1;     // [2]: 2 epilogue warps wrote rho of a row
+constexpr int kBarRhoEmpty = kBarRhoFull + 2;    // [2]: 4 scan warps read it
+static_assert(kBarRhoEmpty + 2 <= kNumBars, "too many barriers");
 
 // ------------------------------------------------------------ PTX wrappers
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -197,6 +207,10 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile
             return false;
         }
     }
+}
+// The same for a whole warp: one answer for all its lanes, which then stay together.
+__device__ __forceinline__ bool wait_bar_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag) {
+    return __all_sync(0xffffffffu, wait_bar(bar, parity, abort_flag));
 }
 // Drain wait (teardown): bounded, no abort check.
 __device__ __forceinline__ void drain_bar(uint32_t bar, uint32_t parity) {
@@ -258,6 +272,11 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
           "=r"(v[14]), "=r"(v[15])
         : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&v)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                 : "r"(taddr));
+}
 __device__ __forceinline__ void tmem_wait_ld() {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
@@ -313,21 +332,33 @@ __device__ __forceinline__ void store_pair_row(uint32_t buf, int r, int g, const
 // prologues saved.  Up to three levels: blocks below end[0] take r[0] rows each, of
 // channels from 0 on, the next ones r[1] rows of channels from ch[1] on, and so on, fewer
 // rows each, so that the large units start first and small ones fill the tail.  Same box,
-// one row per block and now: B = 8, L = 4096, D = 256, M = 16 with both state terms (this
-// kernel and k_terminal_tc) 157 -> 96 us; B = 7, L = 465, D = 160, M = 32 66 -> 49.  kMaxWalk
-// bounds the walk: rows of more than 8 tiles stay alone.
+// one row per block and now, us: B = 8, L = 4096, D = 256, M = 16 with both state terms (this
+// kernel and k_terminal_tc) 145 -> 104; B = 7, L = 465, D = 160, M = 32 45 -> 36; B = 64, L = 200,
+// D = 512, M = 16 1012 -> 481.
 struct RowPlan {
     int r[3];       // rows per block of the level
     int end[3];     // one past the level's last block
     int ch[3];      // the level's first channel
     int B, D;
 };
-__device__ __forceinline__ void rows_of(const RowPlan &p, int blk, int &d, int &b0, int &nrows) {
-    const int l = blk < p.end[0] ? 0 : blk < p.end[1] ? 1 : 2;
+__host__ __device__ __forceinline__ int level_of(const RowPlan &p, int blk) {
+    return blk < p.end[0] ? 0 : blk < p.end[1] ? 1 : 2;
+}
+__host__ __device__ __forceinline__ void rows_of(const RowPlan &p, int blk, int &d, int &b0, int &nrows) {
+    const int l = level_of(p, blk);
     const int r = p.r[l], u = (p.B + r - 1) / r, at = blk - (l ? p.end[l - 1] : 0);
     d = p.ch[l] + at / u;
     b0 = at % u * r;
-    nrows = min(r, p.B - b0);
+    nrows = r < p.B - b0 ? r : p.B - b0;
+}
+
+// Q += [DY^T ; X^T] X over a tile's 32 chunks (K = chunks): MN-major views of the swizzled
+// dy and x tiles at sdy; rows 64-127 (X^T X) are not read.
+__device__ __forceinline__ void add_q(uint32_t tmem, uint32_t sdy, bool accum) {
+    const uint64_t dqa = desc_sw128(sdy, 4096, 1024), dqb = desc_sw128(sdy + 4096, 16, 1024);
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks)
+        umma_ss(tmem + kColQ, dqa + ks * (2048 >> 4), dqb + ks * (2048 >> 4), kIdescQ, (accum || ks > 0) ? 1u : 0u);
 }
 
 struct BwdArgs {
@@ -353,7 +384,7 @@ struct BwdArgs {
 // s_in joins the pair entering the chunk that ends at L' = L rounded up to a
 // chunk (|lambda^(L-L')| <= exp(63 gamma)), which gives lambda^(t+1) s_in at
 // token t and lambda^L s_in in the end state; positions >= L are never stored.
-template <bool kGrad>
+template <bool kGrad, bool kRows>
 __global__ void __launch_bounds__(kThreads, 2)
     k_backward_tc(const __grid_constant__ CUtensorMap tmap_dy, const __grid_constant__ CUtensorMap tmap_x,
                   const BwdArgs args) {
@@ -364,10 +395,10 @@ __global__ void __launch_bounds__(kThreads, 2)
     // The time-reversed prefill keeps one row per CTA: it serves few rows, and the row
     // bookkeeping cost it 3 %.
     int d = blockIdx.x % args.D, b0 = blockIdx.x / args.D, nrows = 1;
-    if (kGrad) rows_of(args.plan, blockIdx.x, d, b0, nrows);
+    if (kRows) rows_of(args.plan, blockIdx.x, d, b0, nrows);
     const int row0 = b0 * args.D + d;           // b * D + d of the first row; the next ones D apart
     const int M = args.M, ntiles = args.ntiles;
-    const int nv = kGrad ? nrows * ntiles : ntiles;   // tiles of the walk: each row's in reverse, row after row
+    const int nv = kRows ? nrows * ntiles : ntiles;   // tiles of the walk: each row's in reverse, row after row
     constexpr int w_prod = 6, w_alloc = 7, w_mma_p = 8, w_mma_d = 9;
     // Threads that build the tables: all but the producer's.
     constexpr int kBuilders = kThreads - 32;
@@ -391,7 +422,11 @@ __global__ void __launch_bounds__(kThreads, 2)
             bar_init(bar(kBarBsEmpty + i), 1);
             bar_init(bar(kBarDFull + i), 1);
             bar_init(bar(kBarDEmpty + i), 2);
+            bar_init(bar(kBarRhoFull + i), 2);
+            bar_init(bar(kBarRhoEmpty + i), 4);
         }
+        bar_init(bar(kBarRowFull), 1);
+        bar_init(bar(kBarRowFree), 6);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == w_alloc) {
@@ -407,7 +442,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 
     // Tile v of the walk is tile ntiles - 1 - v % ntiles of row v / ntiles.
     auto load_tile = [&](int v) {
-        const int slot = v % kSlots, rr = kGrad ? v / ntiles : 0;
+        const int slot = v % kSlots, rr = kRows ? v / ntiles : 0;
         const int chunk0 = (ntiles - 1 - (v - rr * ntiles)) * kNT, row = row0 + rr * args.D;
         const uint32_t dst = sbase + kOffRing + slot * kSlotBytes;
         bar_expect_tx(bar(kBarSlotFull + slot), kGrad ? 8192u : 4096u);
@@ -449,7 +484,6 @@ __global__ void __launch_bounds__(kThreads, 2)
         cf[m] = m >= M ? make_float2(0.0f, 0.0f)
                              : mode_coef(args.amp[d * M + m], args.phase[d * M + m]);
     }
-    if (bt < 64) reinterpret_cast<float *>(smem + kOffRho)[bt] = 0.0f;
     sync_builders();
     // Stage 2: K[n] (Eq. 1 at integer lags, modes summed in a fixed order), the
     // projection table and the up-projection U', one 16-byte core-matrix row
@@ -524,16 +558,14 @@ __global__ void __launch_bounds__(kThreads, 2)
     const int last = nv - 1;
     // Scan lanes: lane l of quarter q owns row 32 q + l of the projections and of
     // [S^n ; R^n] (mode mE = 8 q + (l % 16) / 2; role s = 2 (l >= 16) + l % 2:
-    // Re / Im of Dp and S^n, of Dq and R^n); their cross-chunk (G, P) from E is
-    // kept for the final combination.
-    const int s = ((lane >> 4) << 1) | (lane & 1), mE = 8 * (warp & 3) + ((lane & 15) >> 1);
-    const bool onE = warp < 4 && mE < M;
-    const float gamE = onE ? args.decay[d * M + mE] : 0.0f, omgE = onE ? args.freq[d * M + mE] : 0.0f;
-    float gr = 0.0f, gi = 0.0f, pr = 0.0f, pi = 0.0f;
-    // The adjoint pair of the scan lanes; after a row's last tile it is (S_0, R_0).
-    float2 S = make_float2(0.0f, 0.0f), R = make_float2(0.0f, 0.0f);
+    // Re / Im of Dp and S^n, of Dq and R^n).
     if (warp < 4) {
         // ---------------------------------------------------- reverse chunk scan
+        const int s = ((lane >> 4) << 1) | (lane & 1), mE = 8 * warp + ((lane & 15) >> 1);
+        const bool onE = mE < M;
+        const float gamE = onE ? args.decay[d * M + mE] : 0.0f, omgE = onE ? args.freq[d * M + mE] : 0.0f;
+        // The adjoint pair; after a row's last tile it is (S_0, R_0).
+        float2 S = make_float2(0.0f, 0.0f), R = make_float2(0.0f, 0.0f);
         const int q = warp, base = lane & 14;   // the mode's rows: base, base + 1, base + 16, base + 17
         const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16);
         const float2 a = lambda_pow(gamE, omgE, (float)kC);
@@ -548,69 +580,181 @@ __global__ void __launch_bounds__(kThreads, 2)
                 inj = cmul(lambda_pow(gamE, omgE, (float)(args.L - Lr)), args.state_in[(int64_t)row0 * M + mE]);
         }
         bool ok = true;
-        int row = row0, tv = 0;   // the current row and its tile
-        for (int v = 0; v < nv && ok; ++v) {
-            const int bb = v & 1;
-            if (kGrad && tv == 0) S = R = make_float2(0.0f, 0.0f);
-            if (!wait_bar(bar(kBarPFull + bb), (v >> 1) & 1, abort_flag)) break;
+        // Row r of the walk: E = [S^n ; R^n] X over the row and the within-chunk rho leave TMEM
+        // for fp32 and become the row's (G, P); the next row's first products then overwrite
+        // both accumulators.
+        const float2 l1 = lambda_pow(gamE, omgE, 1.0f);
+        const float2 l4 = lambda_pow(gamE, omgE, 4.0f), l32 = lambda_pow(gamE, omgE, 32.0f),
+                     ls0 = lambda_pow(gamE, omgE, (float)s);
+        float gin = 0.0f, gii = 0.0f, pin = 0.0f, pii = 0.0f;   // the initial state's share of (G, P), role 0
+        auto finish_row = [&](int r) {
+            if (!wait_bar_warp(bar(kBarRowFull), r & 1, abort_flag)) return false;
             tc_fence_after();
-            if (warp == 0 && lane == 0) bar_arrive(bar(kBarSlotEmpty + v % kSlots));
-            const uint32_t pb = sbase + kOffBs + bb * kBsBuf;
-            const int cinj = kinj - (last - v) * kNT;   // chunk of this tile that takes s_in, if any
+            // Weights lambda^(C-i), C - i = 16 (3 - h) + k with k = 1 .. 16: the four blocks h of 16
+            // columns share the powers lambda^k, and Horner steps of lambda^16 join them.
+            float2 w = l1, z = l1;
+            float2 A[4], J[4];   // sum lambda^k x, sum k lambda^k x
 #pragma unroll
-            for (int h = 1; h >= 0; --h) {   // chunks 31 .. 0
-                uint32_t pv[16];
-                tmem_ld16(tl + kColP + 32 * bb + 16 * h, pv);
+            for (int h = 0; h < 4; ++h) A[h] = J[h] = make_float2(0.0f, 0.0f);
+#pragma unroll 1
+            for (int eg = 3; eg >= 0; --eg) {
+                uint32_t ev[4][4];
+#pragma unroll
+                for (int h = 0; h < 4; ++h) tmem_ld4(tl + kColE + 16 * h + 4 * eg, ev[h]);
                 tmem_wait_ld();
-                if (h == 1) {
-                    if (!wait_bar(bar(kBarBsEmpty + bb), ((v >> 1) & 1) ^ 1, abort_flag)) {
-                        ok = false;
-                        break;
-                    }
-                } else {
+                if (kRows && eg == 0) {
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) bar_arrive(bar(kBarPEmpty + bb));
+                    if (lane == 0) bar_arrive(bar(kBarRowFree));
                 }
 #pragma unroll
-                for (int g = 1; g >= 0; --g) {
-                    float own[8];
+                for (int e = 3; e >= 0; --e) {
+                    const float k = (float)(16 - 4 * eg - e);
+                    const float2 kw = make_float2(k * w.x, k * w.y);
 #pragma unroll
-                    for (int n = 7; n >= 0; --n) {
-                        const float p = __uint_as_float(pv[8 * g + n]);
-                        const float dpr = __shfl_sync(0xffffffffu, p, base);
-                        const float dpi = __shfl_sync(0xffffffffu, p, base + 1);
-                        const float dqr = __shfl_sync(0xffffffffu, p, base + 16);
-                        const float dqi = __shfl_sync(0xffffffffu, p, base + 17);
-                        // The pair entering chunk 16 h + 8 g + n from the right.
-                        if (!kGrad && 16 * h + 8 * g + n == cinj) S = make_float2(S.x + inj.x, S.y + inj.y);
-                        own[n] = (s & 2) ? ((s & 1) ? R.y : R.x) : ((s & 1) ? S.y : S.x);
-                        const float2 w = make_float2(fmaf((float)kC, S.x, R.x), fmaf((float)kC, S.y, R.y));
-                        R = cfma(a, w, make_float2(dqr, dqi));
-                        S = cfma(a, S, make_float2(dpr, dpi));
+                    for (int h = 0; h < 4; ++h) {
+                        const float x = __uint_as_float(ev[h][e]);
+                        A[h].x = fmaf(w.x, x, A[h].x);
+                        A[h].y = fmaf(w.y, x, A[h].y);
+                        J[h].x = fmaf(kw.x, x, J[h].x);
+                        J[h].y = fmaf(kw.y, x, J[h].y);
                     }
-                    store_pair_row(pb, prow, 2 * h + g, own);
+                    z = w;
+                    w = cmul(w, l1);
                 }
             }
-            if (!ok) break;
-            fence_async_smem();
+            float2 a = A[0], j = J[0];   // z = lambda^16
+#pragma unroll
+            for (int h = 1; h < 4; ++h) {
+                j = cfma(z, make_float2(fmaf(16.0f, a.x, j.x), fmaf(16.0f, a.y, j.y)), J[h]);
+                a = cfma(z, a, A[h]);
+            }
+            // G = sum w (E_S.re + i E_S.im), P = sum w E_R + sum (C - i) w E_S.
+            float gr = 0.0f, gi = 0.0f, pr, pi;
+            if (s == 0) { gr = a.x; gi = a.y; pr = j.x; pi = j.y; }
+            else if (s == 1) { gr = -a.y; gi = a.x; pr = -j.y; pi = j.x; }
+            else if (s == 2) { pr = a.x; pi = a.y; }
+            else { pr = -a.y; pi = a.x; }
+            // Within-chunk terms: lags n = s, s + 4, ... < 32 from rho, and n + 32, which share
+            // lambda^n (steps of lambda^4 from the exact lambda^s) and take lambda^32 at the end.
+            if (!wait_bar_warp(bar(kBarRhoFull + (r & 1)), (r >> 1) & 1, abort_flag)) return false;
+            const float *rho = reinterpret_cast<const float *>(smem + kOffRho) + (r & 1) * 128;
+            float2 ln = ls0;
+            float2 gh = make_float2(0.0f, 0.0f), ph = gh;
+#pragma unroll 4
+            for (int e = 0; e < kC / 8; ++e) {
+                const int n = 4 * e + s;
+                const float v = rho[n] + rho[64 + n], u = rho[96 + n], nv = v * (float)n, nu = u * (float)n;
+                gr = fmaf(v, ln.x, gr);
+                gi = fmaf(v, ln.y, gi);
+                pr = fmaf(nv, ln.x, pr);
+                pi = fmaf(nv, ln.y, pi);
+                gh.x = fmaf(u, ln.x, gh.x);
+                gh.y = fmaf(u, ln.y, gh.y);
+                ph.x = fmaf(nu, ln.x, ph.x);
+                ph.y = fmaf(nu, ln.y, ph.y);
+                ln = cmul(ln, l4);
+            }
+            const float2 g2 = cfma(l32, gh, make_float2(gr, gi));
+            const float2 p2 = cfma(l32, make_float2(fmaf(32.0f, gh.x, ph.x), fmaf(32.0f, gh.y, ph.y)), make_float2(pr, pi));
+            gr = g2.x;
+            gi = g2.y;
+            pr = p2.x;
+            pi = p2.y;
             __syncwarp();
-            if (lane == 0) bar_arrive(bar(kBarSFull + bb));
-            if (!kGrad || ++tv < ntiles) continue;
+            if (kRows && lane == 0) bar_arrive(bar(kBarRhoEmpty + (r & 1)));
+            gr += gin;
+            gi += gii;
+            pr += pin;
+            pi += pii;
+            // The sum over the mode's four lanes; role 0 writes the row's partials.
+#pragma unroll
+            for (int o = 1; o <= 16; o <<= 4) {
+                gr += __shfl_xor_sync(0xffffffffu, gr, o);
+                gi += __shfl_xor_sync(0xffffffffu, gi, o);
+                pr += __shfl_xor_sync(0xffffffffu, pr, o);
+                pi += __shfl_xor_sync(0xffffffffu, pi, o);
+            }
+            if (s == 0 && onE) {
+                const int64_t at = (int64_t)(row0 + r * args.D) * M + mE;
+                args.part_g[at] = make_float2(gr, gi);
+                args.part_p[at] = make_float2(pr, pi);
+            }
+            return true;
+        };
+        int row = row0, tv = 0;   // the current row and its tile
+        int ended = 0;            // rows whose last tile has been scanned
+        bool pending = false;     // the last of them waits for finish_row
+        // (Several rows: one pass more than there are tiles, so that finish_row is inlined once.)
+        for (int v = 0; v < nv + (kRows ? 1 : 0); ++v) {
+            if (!kRows || v < nv) {
+                const int bb = v & 1;
+                if (kRows && tv == 0) S = R = make_float2(0.0f, 0.0f);
+                if (!wait_bar(bar(kBarPFull + bb), (v >> 1) & 1, abort_flag)) break;
+                tc_fence_after();
+                if (warp == 0 && lane == 0) bar_arrive(bar(kBarSlotEmpty + v % kSlots));
+                const uint32_t pb = sbase + kOffBs + bb * kBsBuf;
+                const int cinj = kinj - (last - v) * kNT;   // chunk of this tile that takes s_in, if any
+#pragma unroll
+                for (int h = 1; h >= 0; --h) {   // chunks 31 .. 0
+                    uint32_t pv[16];
+                    tmem_ld16(tl + kColP + 32 * bb + 16 * h, pv);
+                    tmem_wait_ld();
+                    if (h == 1) {
+                        if (!wait_bar(bar(kBarBsEmpty + bb), ((v >> 1) & 1) ^ 1, abort_flag)) {
+                            ok = false;
+                            break;
+                        }
+                    } else {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) bar_arrive(bar(kBarPEmpty + bb));
+                    }
+#pragma unroll
+                    for (int g = 1; g >= 0; --g) {
+                        float own[8];
+#pragma unroll
+                        for (int n = 7; n >= 0; --n) {
+                            const float p = __uint_as_float(pv[8 * g + n]);
+                            const float dpr = __shfl_sync(0xffffffffu, p, base);
+                            const float dpi = __shfl_sync(0xffffffffu, p, base + 1);
+                            const float dqr = __shfl_sync(0xffffffffu, p, base + 16);
+                            const float dqi = __shfl_sync(0xffffffffu, p, base + 17);
+                            // The pair entering chunk 16 h + 8 g + n from the right.
+                            if (!kGrad && 16 * h + 8 * g + n == cinj) S = make_float2(S.x + inj.x, S.y + inj.y);
+                            own[n] = (s & 2) ? ((s & 1) ? R.y : R.x) : ((s & 1) ? S.y : S.x);
+                            const float2 w = make_float2(fmaf((float)kC, S.x, R.x), fmaf((float)kC, S.y, R.y));
+                            R = cfma(a, w, make_float2(dqr, dqi));
+                            S = cfma(a, S, make_float2(dpr, dpi));
+                        }
+                        store_pair_row(pb, prow, 2 * h + g, own);
+                    }
+                }
+                if (!ok) break;
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) bar_arrive(bar(kBarSFull + bb));
+            }
+            if (!kGrad) continue;
+            // A row is finished after the next one's first tile, whose scan hides the last products.
+            if (kRows && pending) {
+                pending = false;
+                if (!finish_row(ended - 1)) break;
+            }
+            if ((kRows && v == nv) || ++tv < ntiles) continue;
             // The row's end: (S, R) is the adjoint pair at token 0.  The forward's initial
             // state s_in (Sec. 3.2-3.3): G += s_in lambda S_0, P += s_in lambda (R_0 + S_0),
             // once per mode; the gradient of s_in is conj(c lambda S_0).
             if (s == 0 && onE && (args.state_in || args.d_state_in)) {
                 const int64_t at = (int64_t)row * M + mE;
-                const float2 l1 = lambda_pow(gamE, omgE, 1.0f);
                 const float2 ls = cmul(l1, S);
                 if (args.state_in) {
                     const float2 si = args.state_in[at];
-                    const float2 gin = cmul(si, ls), pin = cmul(si, cmul(l1, make_float2(R.x + S.x, R.y + S.y)));
-                    gr += gin.x;
-                    gi += gin.y;
-                    pr += pin.x;
-                    pi += pin.y;
+                    const float2 g0 = cmul(si, ls), p0 = cmul(si, cmul(l1, make_float2(R.x + S.x, R.y + S.y)));
+                    gin = g0.x;
+                    gii = g0.y;
+                    pin = p0.x;
+                    pii = p0.y;
                 }
                 if (args.d_state_in) {
                     const float2 c = mode_coef(args.amp[d * M + mE], args.phase[d * M + mE]);
@@ -619,61 +763,30 @@ __global__ void __launch_bounds__(kThreads, 2)
                 }
             }
             __syncwarp();   // the next tile's tensor-memory loads are warp-wide
+            ++ended;
+            pending = true;
             tv = 0;
             row += args.D;
         }
+        if (kGrad && !kRows && pending) finish_row(0);
         if (!kGrad && ok && s == 0 && onE) {
             // The adjoint state after the first chunk is the prompt's terminal state.
             if (args.state_out) args.state_out[(int64_t)row0 * M + mE] = S;
             if (args.coef_out && row0 < args.D) {
-                const float2 l1 = lambda_pow(gamE, omgE, 1.0f);
                 const float2 c = mode_coef(args.amp[d * M + mE], args.phase[d * M + mE]);
                 args.coef_out[d * M + mE] = make_float4(l1.x, l1.y, c.x, c.y);
             }
-        }
-        if (kGrad && ok && wait_bar(bar(kBarDFull + (last & 1)), (last >> 1) & 1, abort_flag)) {
-            // E = [S^n ; R^n] X over the sequence, complete with the last dx product.
-            tc_fence_after();
-            // Weights lambda^(C-i), i = 63 .. 0, by successive products.
-            const float2 l1 = lambda_pow(gamE, omgE, 1.0f);
-            float2 w = l1;
-            float a1 = 0.0f, a2 = 0.0f, a3 = 0.0f, a4 = 0.0f;
-#pragma unroll 1
-            for (int h = 3; h >= 0; --h) {
-                uint32_t ev[16];
-                tmem_ld16(tl + kColE + 16 * h, ev);
-                tmem_wait_ld();
-#pragma unroll
-                for (int e = 15; e >= 0; --e) {
-                    const float x = __uint_as_float(ev[e]);
-                    const float ci = (float)(kC - (16 * h + e));
-                    a1 = fmaf(w.x, x, a1);
-                    a2 = fmaf(w.y, x, a2);
-                    a3 = fmaf(ci * w.x, x, a3);
-                    a4 = fmaf(ci * w.y, x, a4);
-                    w = cmul(w, l1);
-                }
-            }
-            // G = sum w (E_S.re + i E_S.im), P = sum w E_R + sum (C - i) w E_S.
-            if (s == 0) { gr += a1; gi += a2; pr += a3; pi += a4; }
-            else if (s == 1) { gr = -a2; gi = a1; pr = -a4; pi = a3; }
-            else if (s == 2) { pr = a1; pi = a2; }
-            else { pr = -a2; pi = a1; }
         }
     } else if (warp < 6) {
         // ---------------------------------------------------- dx epilogue
         const int q = warp & 3;   // 0 or 1: positions 32 q + lane
         const uint32_t tl = tmem + ((uint32_t)(32 * q) << 16);
-        bool ok = true;
         // The tile's positions in dxT: rows D apart, tiles from the end of each.
         __nv_bfloat16 *rowp = args.dxT + (int64_t)row0 * args.Lp + 32 * q + lane;
-        int tile = ntiles - 1;
+        int tile = ntiles - 1, r = 0;   // r: row of the walk
         for (int v = 0; v < nv; ++v) {
             const int bb = v & 1;
-            if (!wait_bar(bar(kBarDFull + bb), (v >> 1) & 1, abort_flag)) {
-                ok = false;
-                break;
-            }
+            if (!wait_bar(bar(kBarDFull + bb), (v >> 1) & 1, abort_flag)) break;
             tc_fence_after();
             uint32_t r0[16], r1[16];
             tmem_ld16(tl + kColD + 32 * bb, r0);
@@ -695,44 +808,47 @@ __global__ void __launch_bounds__(kThreads, 2)
                 out[k * kC] = __float2bfloat16_rn(__uint_as_float(r0[k]));
                 out[(k + 16) * kC] = __float2bfloat16_rn(__uint_as_float(r1[k]));
             }
-            if (--tile < 0 && kGrad) {
-                tile = ntiles - 1;
-                rowp += (int64_t)args.D * args.Lp;
-            }
-        }
-        // Diagonal sums of Q (accumulated over the whole sequence; its last
-        // product precedes the last dx product).  Both warps stage the rows of
-        // Q's lower triangle in the ring, which no load or product touches any
-        // more (row stride 65 words: the row writes and the diagonal reads each
-        // hit 32 banks), then thread n sums diagonal n: rho[n] = sum_k Q[n+k][k].
-        // (Adding row by row into rho, one dependent shared-memory update per
-        // element, cost ~3k cycles at the end of every CTA.)
-        if (kGrad) {
-            const int i = 32 * q + lane;
-            float *qs = reinterpret_cast<float *>(smem + kOffRing);
-            if (ok) {
-                tc_fence_after();
-                for (int h = 0; h < 2 + 2 * q; ++h) {
-                    uint32_t qv[16];
-                    tmem_ld16(tl + kColQ + 16 * h, qv);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) qs[i * 65 + 16 * h + e] = __uint_as_float(qv[e]);
+            if (--tile >= 0 || !kGrad) continue;
+            // The row's end: diagonal sums of Q over the row,
+            // rho[n] = sum_k Q[n+k][k].  Each warp takes its 32 rows, 16 columns at a time
+            // through its own staging buffer (row stride 17 words: the row writes and the
+            // diagonal reads each hit 32 banks), lane l the diagonals n = l and, in the lower
+            // rows, l + 32; the readers add the two warps' parts.
+            float *qs = reinterpret_cast<float *>(smem + kOffQs) + q * 32 * kQsStride;
+            if (!wait_bar_warp(bar(kBarRowFull), r & 1, abort_flag)) break;
+            tc_fence_after();
+            float d0[4] = {0.0f, 0.0f, 0.0f, 0.0f}, d1[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 1
+            for (int h = 0; h < 2 + 2 * q; ++h) {
+                uint32_t qv[16];
+                tmem_ld16(tl + kColQ + 16 * h, qv);
+                tmem_wait_ld();
+                if (kRows && h == 1 + 2 * q) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) bar_arrive(bar(kBarRowFree));
                 }
+#pragma unroll
+                for (int e = 0; e < 16; ++e) qs[lane * kQsStride + e] = __uint_as_float(qv[e]);
+                __syncwarp();
+                // Column 16 h + e meets diagonal n in row n + 16 h + e, this warp's row w0 + e (+ 32).
+                const int w0 = lane + 16 * h - 32 * q;
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                    if ((unsigned)(w0 + e) < 32u) d0[e & 3] += qs[(w0 + e) * kQsStride + e];
+                    if ((unsigned)(w0 + 32 + e) < 32u) d1[e & 3] += qs[(w0 + 32 + e) * kQsStride + e];
+                }
+                __syncwarp();
             }
-            // Both epilogue warps arrive here whether or not their loop completed.
-            asm volatile("bar.sync 1, 64;" ::: "memory");
-            float r0 = 0.0f, r1 = 0.0f, r2 = 0.0f, r3 = 0.0f;
-            int k = 0;
-            for (; k + 4 <= kC - i; k += 4) {
-                const float *p = qs + (i + k) * 65 + k;
-                r0 += p[0];
-                r1 += p[66];
-                r2 += p[132];
-                r3 += p[198];
-            }
-            for (; k < kC - i; ++k) r0 += qs[(i + k) * 65 + k];
-            if (ok) reinterpret_cast<float *>(smem + kOffRho)[i] = (r0 + r1) + (r2 + r3);
+            if (kRows && !wait_bar_warp(bar(kBarRhoEmpty + (r & 1)), ((r >> 1) & 1) ^ 1, abort_flag)) break;
+            float *rho = reinterpret_cast<float *>(smem + kOffRho) + (r & 1) * 128 + q * 64;
+            rho[lane] = (d0[0] + d0[1]) + (d0[2] + d0[3]);
+            rho[lane + 32] = (d1[0] + d1[1]) + (d1[2] + d1[3]);
+            __syncwarp();
+            if (lane == 0) bar_arrive(bar(kBarRhoFull + (r & 1)));
+            ++r;
+            tile = ntiles - 1;
+            rowp += (int64_t)args.D * args.Lp;
         }
     } else if (warp == w_prod) {
         // ---------------------------------------------------- TMA producer
@@ -750,7 +866,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
         __syncwarp();
     } else if (warp == w_mma_p) {
-        // ---------------------------------------------------- MMA: projections and Q
+        // ---------------------------------------------------- MMA: projections (and Q)
         if (lane == 0) {
             const uint64_t dap = desc_plain(sbase + kOffAP, 128, 1024);
             const uint64_t dapl = desc_plain(sbase + kOffAPlo, 128, 1024);
@@ -768,16 +884,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 #pragma unroll
                 for (int ks = 0; ks < 4; ++ks)
                     umma_ss(tmem + kColP + 32 * bb, dapl + ks * 16, ddy + ks * 2, kIdescN32M64, 1u);
-                // Q += [DY^T ; X^T] X over this tile's 32 chunks (K = chunks):
-                // MN-major views of the same swizzled tiles; rows 64-127 (X^T X)
-                // are not read.
-                if (kGrad) {
-                    const uint64_t dqa = desc_sw128(sdy, 4096, 1024), dqb = desc_sw128(sdy + 4096, 16, 1024);
-#pragma unroll
-                    for (int ks = 0; ks < 2; ++ks)
-                        umma_ss(tmem + kColQ, dqa + ks * (2048 >> 4), dqb + ks * (2048 >> 4), kIdescQ,
-                                (v > 0 || ks > 0) ? 1u : 0u);
-                }
+                if (kGrad && !kRows) add_q(tmem, sdy, v > 0);
                 umma_commit(bar(kBarPFull + bb));
             }
             // Drain: the last group's completion implies all earlier ones.
@@ -785,7 +892,7 @@ __global__ void __launch_bounds__(kThreads, 2)
         }
         __syncwarp();
     } else if (warp == w_mma_d) {
-        // ---------------------------------------------------- MMA: T', U', E
+        // ---------------------------------------------------- MMA: T', U', E (and Q)
         if (lane == 0) {
             const uint64_t dt = desc_plain(sbase + kOffT, 128, 1024);
             const uint64_t du = desc_plain(sbase + kOffU, 128, 1024);
@@ -796,10 +903,15 @@ __global__ void __launch_bounds__(kThreads, 2)
                 if (!wait_bar(bar(kBarDEmpty + bb), ((v >> 1) & 1) ^ 1, abort_flag)) break;
                 tc_fence_after();
                 const uint32_t sdy = sbase + kOffRing + slot * kSlotBytes;
-                const uint64_t ddy = desc_sw128(sdy, 16, 1024), dxm = desc_sw128(sdy + 4096, 16, 1024);
+                const uint64_t ddy = desc_sw128(sdy, 16, 1024);
 #pragma unroll
                 for (int ks = 0; ks < 4; ++ks)
                     umma_ss(tmem + kColD + 32 * bb, dt + ks * 16, ddy + ks * 2, kIdescN32, ks > 0);
+                // Several rows a block: Q is issued here, so that a row's first products, which
+                // overwrite Q and E, hold up dx alone until the row before has left both.
+                const int tv = kRows ? v % ntiles : v;
+                const bool fresh = kRows && tv == 0 && v > 0;
+                if (kRows && !fresh) add_q(tmem, sdy, tv > 0);
                 if (!wait_bar(bar(kBarSFull + bb), (v >> 1) & 1, abort_flag)) {
                     umma_commit(bar(kBarDFull + bb));   // so that the drain below tracks T'
                     ++v;
@@ -807,23 +919,41 @@ __global__ void __launch_bounds__(kThreads, 2)
                 }
                 tc_fence_after();
                 const uint32_t pb = sbase + kOffBs + bb * kBsBuf;
-#pragma unroll
-                for (int part = 0; part < 2; ++part) {   // high parts, then low parts
-                    const uint32_t pp = pb + part * 8192;
+                auto add_u = [&](int part) {
                     // dx += U' S^n: B = the S^n rows of quarter ks (MN-major).
-                    const uint64_t dbu = desc_plain(pp, 512, 128);
+                    const uint64_t dbu = desc_plain(pb + part * 8192, 512, 128);
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks)
                         umma_ss(tmem + kColD + 32 * bb, du + ks * 16, dbu + ks * (2048 >> 4), kIdescU, 1u);
+                };
+                auto add_e = [&](int part) {
                     // E += [S^n ; R^n] X (K = chunks).
-                    if (kGrad) {
-                        const uint64_t dea = desc_plain(pp, 128, 512);
+                    const uint64_t dea = desc_plain(pb + part * 8192, 128, 512), dxm = desc_sw128(sdy + 4096, 16, 1024);
 #pragma unroll
-                        for (int ks = 0; ks < 2; ++ks)
-                            umma_ss(tmem + kColE, dea + ks * (256 >> 4), dxm + ks * (2048 >> 4), kIdescE,
-                                    (v > 0 || part > 0 || ks > 0) ? 1u : 0u);
+                    for (int ks = 0; ks < 2; ++ks)
+                        umma_ss(tmem + kColE, dea + ks * (256 >> 4), dxm + ks * (2048 >> 4), kIdescE,
+                                (tv > 0 || part > 0 || ks > 0) ? 1u : 0u);
+                };
+                if (kRows && fresh) {
+                    add_u(0);
+                    add_u(1);
+                    if (!wait_bar(bar(kBarRowFree), (v / ntiles - 1) & 1, abort_flag)) {
+                        umma_commit(bar(kBarDFull + bb));
+                        ++v;
+                        break;
+                    }
+                    tc_fence_after();
+                    add_q(tmem, sdy, false);
+                    add_e(0);
+                    add_e(1);
+                } else {
+#pragma unroll
+                    for (int part = 0; part < 2; ++part) {   // high parts, then low parts
+                        add_u(part);
+                        if (kGrad) add_e(part);
                     }
                 }
+                if (kGrad && (kRows ? tv == ntiles - 1 : v == nv - 1)) umma_commit(bar(kBarRowFull));
                 umma_commit(bar(kBarDFull + bb));
             }
             if (v > 0) drain_bar(bar(kBarDFull + ((v - 1) & 1)), ((v - 1) >> 1) & 1);
@@ -832,44 +962,11 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
 
     tc_fence_before();
-    __syncthreads();   // every role has left its loop; rho is complete
+    __syncthreads();   // every role has left its loop
     tc_fence_after();
     if (warp == w_alloc)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                      "r"(kTmemCols));
-    if (kGrad && warp < 4) {
-        // Within-chunk terms: lags n = s, s + 4, ... from rho, then the sum over
-        // the mode's four lanes; role 0 writes the partials.  lambda^n by steps of
-        // lambda^4 from the exact lambda^s (at most 15 products).
-        const float *rho = reinterpret_cast<const float *>(smem + kOffRho);
-        const float2 l4 = lambda_pow(gamE, omgE, 4.0f);
-        float2 ln = lambda_pow(gamE, omgE, (float)s);
-#pragma unroll 4
-        for (int e = 0; e < kC / 4; ++e) {
-            const int n = 4 * e + s;
-            const float r = rho[n];
-            gr = fmaf(r, ln.x, gr);
-            gi = fmaf(r, ln.y, gi);
-            pr = fmaf(r * (float)n, ln.x, pr);
-            pi = fmaf(r * (float)n, ln.y, pi);
-            ln = cmul(ln, l4);
-        }
-#pragma unroll
-        for (int o = 1; o <= 16; o <<= 4) {
-            gr += __shfl_xor_sync(0xffffffffu, gr, o);
-            gi += __shfl_xor_sync(0xffffffffu, gi, o);
-            pr += __shfl_xor_sync(0xffffffffu, pr, o);
-            pi += __shfl_xor_sync(0xffffffffu, pi, o);
-        }
-        if (s == 0 && onE) {
-            // The sums of all rows in the first one's place, zeros in the others'.
-            for (int r = 0; r < nrows; ++r) {
-                const int64_t at = (int64_t)(row0 + r * args.D) * M + mE;
-                args.part_g[at] = r ? make_float2(0.0f, 0.0f) : make_float2(gr, gi);
-                args.part_p[at] = r ? make_float2(0.0f, 0.0f) : make_float2(pr, pi);
-            }
-        }
-    }
 }
 
 // ------------------------------------------------------------ terminal-state gradient
@@ -1160,51 +1257,48 @@ __global__ void __launch_bounds__(kTmThreads, 2)
                 ji[c & 3] = fmaf(ri ? w[c].x : w[c].y, val, ji[c & 3]);
             }
             if (++tv < ntiles) continue;
-            // The row's end, one lane per mode: the part of J of the chunk that holds
-            // token L - 1 (L % 64 != 0) directly, and the state terms.
-            if (on && !jordan && ri == 0) {
-                if (n_part >= 0) {
-                    const __nv_bfloat16 *xp = args.xT + (int64_t)row * args.Lp + n_part * kC;
-                    const int cnt = (int)(L - n_part * kC);   // tokens of the chunk before L
-                    float pr = 0.0f, pi = 0.0f;
-                    for (int i = 0; i < cnt; ++i) {
-                        const int e = cnt - 1 - i;
-                        const float xv = __bfloat162float(xp[i]) * (float)e;
-                        const float2 p = pw[m * kPwStride + e];
-                        pr = fmaf(p.x, xv, pr);
-                        pi = fmaf(p.y, xv, pi);
-                    }
-                    const float2 t = cmul(gc, make_float2(pr, pi));
-                    jr[0] += t.x;
-                    ji[0] += t.y;
+            // The row's end: conj(g) J of the row, over the mode's four lanes; one of them adds the
+            // part of the chunk that holds token L - 1 (L % 64 != 0) directly, and the state terms.
+            const bool lead = on && !jordan && ri == 0;
+            if (lead && n_part >= 0) {
+                const __nv_bfloat16 *xp = args.xT + (int64_t)row * args.Lp + n_part * kC;
+                const int cnt = (int)(L - n_part * kC);   // tokens of the chunk before L
+                float pr = 0.0f, pi = 0.0f;
+                for (int i = 0; i < cnt; ++i) {
+                    const int e = cnt - 1 - i;
+                    const float xv = __bfloat162float(xp[i]) * (float)e;
+                    const float2 p = pw[m * kPwStride + e];
+                    pr = fmaf(p.x, xv, pr);
+                    pi = fmaf(p.y, xv, pi);
                 }
+                const float2 t = cmul(gc, make_float2(pr, pi));
+                jr[0] += t.x;
+                ji[0] += t.y;
+            }
+            float jsr = (jr[0] + jr[1]) + (jr[2] + jr[3]), jsi = (ji[0] + ji[1]) + (ji[2] + ji[3]);
+            jsr += __shfl_xor_sync(0xffffffffu, jsr, 1);
+            jsi += __shfl_xor_sync(0xffffffffu, jsi, 1);
+            jsr += __shfl_xor_sync(0xffffffffu, jsr, 16);
+            jsi += __shfl_xor_sync(0xffffffffu, jsi, 16);
+            if (lead) {
                 const float2 lL = lambda_pow(gam, omg, (float)L);
                 const int64_t at = (int64_t)row * M + m;
                 if (args.state_in) {
                     const float2 t = cmul(gc, cmul(args.state_in[at], lL));
-                    jr[1] = fmaf((float)L, t.x, jr[1]);
-                    ji[1] = fmaf((float)L, t.y, ji[1]);
+                    jsr = fmaf((float)L, t.x, jsr);
+                    jsi = fmaf((float)L, t.y, jsi);
                 }
+                args.part_j[at] = make_float2(jsr, jsi);
                 if (args.d_state_in) {
                     const float2 prev = args.d_state_in[at];
                     args.d_state_in[at] = cfma(conj2(gc), conj2(lL), prev);
                 }
             }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) jr[k] = ji[k] = 0.0f;
             __syncwarp();   // the next tile's tensor-memory loads are warp-wide
             tv = 0;
             row += args.D;
-        }
-        float jsr = (jr[0] + jr[1]) + (jr[2] + jr[3]), jsi = (ji[0] + ji[1]) + (ji[2] + ji[3]);
-        // The mode's four rows.
-        jsr += __shfl_xor_sync(0xffffffffu, jsr, 1);
-        jsi += __shfl_xor_sync(0xffffffffu, jsi, 1);
-        jsr += __shfl_xor_sync(0xffffffffu, jsr, 16);
-        jsi += __shfl_xor_sync(0xffffffffu, jsi, 16);
-        if (ok && on && !jordan && ri == 0) {
-            // The sum of all rows in the first one's place, zeros in the others'.
-            for (int r = 0; r < nrows; ++r)
-                args.part_j[(int64_t)(row0 + r * args.D) * M + m] =
-                    r ? make_float2(0.0f, 0.0f) : make_float2(jsr, jsi);   // conj(g) J
         }
     } else if (warp < 6) {
         // ---------------------------------------------------- dx epilogue
@@ -1572,11 +1666,9 @@ size_t tc_backward_ws_bytes(int64_t B, int64_t L, int D, int M) {
 
 namespace {
 
-// Longest walk of a block over several rows, in tiles.  Q and E accumulate over it in TMEM,
-// whose additions truncate, so the error of the sums grows with their number: relative error
-// of dA against 64 bits at B = 16, L = 8192, D = 256, M = 32 (4 tiles a row) 2.6e-6 with one row a
-// block, 2.6e-6, 3.0e-6 and 4.3e-6 with walks of up to 16, 32 and 64 tiles (B = 4, L = 32768,
-// D = 512: 2.8e-6 with 16, one row, and 3.8e-6 with 64, four rows, which takes 25 us less).
+// Longest walk of a block over several rows, in tiles; rows of more than 8 tiles stay alone.
+// At 16 the fill (6 tiles) is about a quarter of a block's time; longer walks have not been
+// measured with the rows handed over one by one.
 constexpr int kMaxWalk = 16;
 
 cudaError_t configure_once() {
@@ -1587,9 +1679,9 @@ cudaError_t configure_once() {
     std::lock_guard<std::mutex> lock(mu);
     if ((int)configured.size() <= dev) configured.resize(dev + 1, 0);
     if (!configured[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(k_backward_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_backward_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+        cudaError_t e = cudaSuccess;
+        for (auto *k : {k_backward_tc<true, true>, k_backward_tc<true, false>, k_backward_tc<false, false>})
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_terminal_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTmSmemBytes);
         if (e != cudaSuccess) return e;
@@ -1659,6 +1751,27 @@ RowPlan row_plan(int64_t B, int D, int ntiles) {
     return best;
 }
 
+}  // namespace
+
+int backward_plan_block(int64_t B, int D, int ntiles, int blk, int out[4]) {
+    const RowPlan p = row_plan(B, D, ntiles);
+    if (blk >= 0 && blk < p.end[2]) {
+        rows_of(p, blk, out[0], out[1], out[2]);
+        out[3] = level_of(p, blk);
+    }
+    return p.end[2];
+}
+
+namespace {
+
+// The backward kernel for the call's plan.  Blocks of one row each keep the instance without
+// the hand-over between rows (340 us a call at B = 4, L = 32768, D = 512, M = 32, against 365 on the other).
+cudaError_t launch_backward(const CUtensorMap &mdy, const CUtensorMap &mx, const BwdArgs &a, cudaStream_t st) {
+    const dim3 grid((unsigned)a.plan.end[2]);
+    if (a.plan.r[0] > 1) return launch_dependent(k_backward_tc<true, true>, grid, kThreads, kSmemBytes, st, mdy, mx, a);
+    return launch_dependent(k_backward_tc<true, false>, grid, kThreads, kSmemBytes, st, mdy, mx, a);
+}
+
 // One call: transpose in (nf fields: x, or x and dy), the tcgen05 kernel, transpose
 // out, in stream order.  (Running the transposes of one part of the problem beside
 // the tcgen05 kernel of another gained nothing: beside two tcgen05 CTAs an SM has
@@ -1673,8 +1786,9 @@ cudaError_t run_layout_and_scan(const CUtensorMap &mdy, const CUtensorMap &mx, B
     k_to_channel_major<<<dim3((unsigned)(Lp / 64), cg, (unsigned)(B * nf)), 128, 0, st>>>(
         src0, src1, dst0, dst1, L, D, Lp, nf, rev);
     if (kGrad) a.plan = row_plan(B, D, a.ntiles);
-    cudaError_t e = launch_dependent(k_backward_tc<kGrad>, dim3((unsigned)(kGrad ? a.plan.end[2] : B * D)), kThreads,
-                                     kSmemBytes, st, mdy, mx, a);
+    cudaError_t e = cudaSuccess;
+    if constexpr (kGrad) e = launch_backward(mdy, mx, a, st);
+    else e = launch_dependent(k_backward_tc<false, false>, dim3((unsigned)(B * D)), kThreads, kSmemBytes, st, mdy, mx, a);
     if (e != cudaSuccess) return e;
     if (rev)
         e = launch_dependent(k_to_row_major, dim3((unsigned)((L + 63) / 64), cg, (unsigned)B), 128, 0, st, outT, out, L,
@@ -1727,9 +1841,7 @@ cudaError_t tc_backward(const void *dy, const void *x, void *dx, int64_t B, int6
         k_to_channel_major<<<dim3((unsigned)(Lp / 64), cg, (unsigned)(B * 2)), 128, 0, st>>>(
             static_cast<const __nv_bfloat16 *>(x), static_cast<const __nv_bfloat16 *>(dy), xT, dyT, L, D, Lp, 2, 0);
         a.plan = row_plan(B, D, a.ntiles);
-        if ((e = launch_dependent(k_backward_tc<true>, dim3((unsigned)a.plan.end[2]), kThreads, kSmemBytes, st, mdy, mx,
-                                  a)) != cudaSuccess)
-            return e;
+        if ((e = launch_backward(mdy, mx, a, st)) != cudaSuccess) return e;
         TermArgs ta;
         ta.plan = a.plan;
         ta.decay = decay;

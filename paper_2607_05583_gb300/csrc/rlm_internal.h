@@ -81,6 +81,9 @@ cudaError_t read_and_clear_tc32_status(int *status, cudaStream_t st);
 // ---- tcgen05 backward (rlm_backward_tc.cu) -----------------------------------
 bool tc_backward_supported(int64_t B, int64_t L, int D, int M, rlm_dtype dt);
 size_t tc_backward_ws_bytes(int64_t B, int64_t L, int D, int M);
+// Its plan for rows of ntiles 2048-token tiles on the current device: the number of blocks,
+// and in out the channel, first row, rows and level of block blk (untouched past the last).
+int backward_plan_block(int64_t B, int D, int ntiles, int blk, int out[4]);
 // state_in (the forward's initial state), d_state_out (the loss gradient of the
 // terminal state) and d_state_in (output) may be null.
 cudaError_t tc_backward(const void *dy, const void *x, void *dx, int64_t B, int64_t L, int D, int M,
