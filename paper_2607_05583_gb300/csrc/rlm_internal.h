@@ -37,6 +37,17 @@ cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, unsigned block, size
     return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
+// ---- Sequences of at most 8 tokens (rlm_short.cu), for simt_prefill / simt_backward ----
+bool short_supported(int64_t L);
+cudaError_t short_prefill(const void *x, void *y, rlm_dtype dt, int64_t B, int64_t L, int D, int M, const float *decay,
+                          const float *freq, const float *amp, const float *phase, const float *state_in, float *state_out,
+                          float *coef_out, cudaStream_t st);
+// Writes the rows' partials G and P (and conj(g) J with d_state_out), [B][D][M] each.
+cudaError_t short_backward(const void *dy, const void *x, void *dx, rlm_dtype dt, int64_t B, int64_t L, int D, int M,
+                           const float *decay, const float *freq, const float *amp, const float *phase,
+                           const float *state_in, const float *d_state_out, float *d_state_in, float2 *part_g,
+                           float2 *part_p, float2 *part_j, cudaStream_t st);
+
 // ---- SIMT chunked scan (rlm_simt.cu) --------------------------------------
 // The chunk length in which the SIMT path's workspace contract is stated.
 int simt_chunk_len(int64_t B, int64_t L, int D);

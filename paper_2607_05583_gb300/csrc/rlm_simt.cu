@@ -28,6 +28,12 @@
 // costs 4 (8) plus 2 for the readout: at M = 32 about 170 FMA per token-channel
 // forward and 410 backward, against 320 and 830.
 //
+// Sequences of at most 8 tokens take rlm_short.cu.  Up to 20 chunks, a wide tile's positions and
+// columns would be mostly padding: there the narrow tile (4 chunks, one column a lane) is
+// taken where use_narrow() says so.  In it a partial chunk alone leaves out the
+// position blocks and chunk sums that it does not need, and above 32 modes two warps share
+// a channel, 32 modes each.
+//
 // One warp owns one channel and a tile of 16 chunks (1024 tokens); its products are
 // register tiles (lane = 8 row groups x 4 column groups, columns = chunks) over
 // tables and drives in shared memory, issued as packed two-lane FMAs
@@ -49,6 +55,10 @@
 //   fp32, B = 4, L = 2048, D = 256, M = 48: forward and backward 162 (with the power table of
 //     a whole chunk, one block a SM, 305)
 //   bf16 from a state, B = 8, L = 1000, D = 256, M = 16: 75 -> 27
+//   short or few: fp32 backward B = 8, L = 24, D = 768, M = 32 44 -> 13 (wide tiles 64); from a
+//     state B = 64, L = 33, D = 768, M = 16 103 -> 52 (109).  Still slower than those: M > 32 in the
+//     backward of one row of 64 channels at L = 500 to 1025 (1.2 to 1.9 x), M = 1 at B = 64, D = 2048,
+//     L = 9 to 17 (1.2 to 1.5 x).
 //
 // and the error against 64 bits is a half to a third of the recurrences' (3e-6 -> 1e-6 for
 // the gradients of the first line).
@@ -65,32 +75,44 @@ namespace {
 typedef unsigned long long u64;
 
 constexpr int kC = 64;               // chunk length
-constexpr int kCols = 16;            // chunks per tile
-constexpr int kTile = kC * kCols;    // 1024 tokens
 constexpr int kCh = 4;               // channels (warps) per block
 constexpr int kThreads = 32 * kCh;
 constexpr int kHalf = kC / 2;
 // The power table holds lambda^n for n < 32 only (it is what limits the blocks a SM holds):
 // products over a chunk run as two halves, joined by lambda^32.
 constexpr int kPwStride = kHalf + 2;   // float2 per mode row: n < 32, then lambda^32 and lambda^64; rows 4 banks apart
-// One channel's tile: [p / 2][column][p % 2] in rows of 32 words and 4 of padding, see slot().
-constexpr int kRowWords = 2 * kCols + 4, kFieldWords = kHalf * kRowWords;
+// A tile of one channel, NC columns (chunks) a lane: 16 chunks (1024 tokens), or 4 (256) where
+// the sequences are short or few, see geometry(): [p / 2][column][p % 2].  Row r holds
+// positions 2 r and 2 r + 1, or mode r of W.  The padding puts the words that eight lanes
+// write into eight rows in different banks, and leaves every address of the product loops a
+// constant from the lane's.  (Permuted 16-byte words of unpadded rows cost an XOR, a shift
+// and an add a load: forward and backward of B = 2, L = 4096, D = 512, M = 32 fp32 60.1 and 135
+// us against 57.7 and 127.)
+template <int NC>
+struct Tile {
+    static constexpr int kCols = 4 * NC, kTokens = kC * kCols;
+    static constexpr int kRowWords = 2 * kCols + 4, kFieldWords = kHalf * kRowWords;
+    static __device__ __forceinline__ constexpr int at(int r, int col) { return r * kRowWords + 2 * col; }
+};
 constexpr int kKernCopy = kC + 16;        // K reversed, then zeros (negative lags)
 constexpr int kKernWords = 2 * kKernCopy; // that, and the same shifted by one
 
 // Shared memory of a block, in floats: per channel the power table and c of every mode
 // (complex), the reversed lag kernel, and for output passes two field tiles, the drive's
 // and x's (forward: the second half's W).
-constexpr int chan_words(int modes, bool out) {
-    return 2 * modes * (kPwStride + 1) + kKernWords + (out ? 2 : 1) * kFieldWords;
+// With the modes of a channel shared between two warps (hw = 2) each warp has tiles of its own
+// for W as well.
+constexpr int chan_words(int modes, int nc, int hw, bool out) {
+    return 2 * modes * (kPwStride + 1) + kKernWords + (hw == 2 ? 6 : out ? 2 : 1) * (kHalf * (8 * nc + 4));
 }
 // Resident blocks a SM, for registers and shared memory alike.  (A third block at 17 to 32
 // modes, with 168 registers a thread, made the forward of B = 2, L = 4096, D = 512, M = 32 fp32 70
-// us against 62 and its backward 159 against 133.)
-__host__ __device__ constexpr int blocks_per_sm(int modes, bool bwd) {
-    return modes > 16 ? 2 : bwd ? 3 : 4;
+// us against 62 and its backward 159 against 133.)  Narrow tiles (nc = 1) need fewer registers; at
+// more than 32 modes their blocks have 256 threads.
+__host__ __device__ constexpr int blocks_per_sm(int modes, int nc, bool bwd) {
+    return nc == 1 ? (modes > 32 ? 2 : modes > 16 ? 4 : modes > 8 ? 5 : 6) : modes > 16 ? 2 : bwd ? 3 : 4;
 }
-constexpr int smem_bytes(int modes, bool out) { return kCh * chan_words(modes, out) * 4; }
+constexpr int smem_bytes(int modes, int nc, int hw, bool out) { return kCh * chan_words(modes, nc, hw, out) * 4; }
 
 __device__ __forceinline__ u64 pack2(float a, float b) {
     u64 r;
@@ -107,12 +129,30 @@ __device__ __forceinline__ void fma2(u64 &d, u64 a, u64 b) {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
 }
 __device__ __forceinline__ void add2(u64 &d, u64 a) { asm("add.rn.f32x2 %0, %0, %1;" : "+l"(d) : "l"(a)); }
-// Word of columns 2 h, 2 h + 1 in row r of a field tile (rows are position pairs, or modes
-// of W).  The padding puts the 16-byte words that eight lanes write into eight rows in
-// different banks, and leaves every address of the product loops a constant from the lane's.
-// (Permuted 16-byte words of unpadded rows cost an XOR, a shift and an add a load: forward and
-// backward of B = 2, L = 4096, D = 512, M = 32 fp32 60.1 and 135 us against 57.7 and 127.)
-__device__ __forceinline__ int slot(int r, int h) { return r * kRowWords + 4 * h; }
+// The (even, odd) position pairs of a lane's NC columns, cg its column group; and back.
+template <int NC>
+__device__ __forceinline__ void load_columns(const float *xs, int r, int cg, u64 (&v)[NC]) {
+    const float *row = xs + Tile<NC>::at(r, NC * cg);
+    if constexpr (NC == 4) {
+        const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(row), b = *reinterpret_cast<const ulonglong2 *>(row + 4);
+        v[0] = a.x;
+        v[1] = a.y;
+        v[2] = b.x;
+        v[3] = b.y;
+    } else {
+        v[0] = *reinterpret_cast<const u64 *>(row);
+    }
+}
+template <int NC>
+__device__ __forceinline__ void store_columns(float *xs, int r, int cg, const float2 (&v)[NC]) {
+    float *row = xs + Tile<NC>::at(r, NC * cg);
+    if constexpr (NC == 4) {
+        *reinterpret_cast<float4 *>(row) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+        *reinterpret_cast<float4 *>(row + 4) = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
+    } else {
+        *reinterpret_cast<float2 *>(row) = v[0];
+    }
+}
 __device__ __forceinline__ float2 shfl2(float2 v, int src) {
     return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
@@ -171,13 +211,13 @@ __device__ __forceinline__ void store4(void *f, int bf16, int64_t e, float4 v) {
 // against 147, of B = 2, L = 4096, D = 512, M = 32 125 against 117.  (Four pairs unrolled against
 // two: the 32-mode forward 57.7 -> 56.4 us, the 16-mode backward 147 -> 145, but the backward of
 // M = 48 118 -> 120.)
-template <int J, bool JORDAN, bool TO_END>
-__device__ __forceinline__ void project(const float2 *pw, const float *xs, int cg, u64 (&acc)[J][4],
-                                        u64 (&accq)[JORDAN ? J : 1][4]) {
+template <int NC, int J, bool JORDAN, bool TO_END>
+__device__ __forceinline__ void project(const float2 *pw, const float *xs, int cg, u64 (&acc)[J][NC],
+                                        u64 (&accq)[JORDAN ? J : 1][NC]) {
 #pragma unroll
     for (int j = 0; j < J; ++j)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 0; c < NC; ++c) {
             acc[j][c] = 0ull;
             if (JORDAN) accq[j][c] = 0ull;
         }
@@ -188,7 +228,7 @@ __device__ __forceinline__ void project(const float2 *pw, const float *xs, int c
             for (int j = 0; j < J; ++j) {
                 const float2 l32 = pw[8 * j * kPwStride + kHalf];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
+                for (int c = 0; c < NC; ++c) {
                     const float2 a = cmul(l32, unpack2(acc[j][c]));
                     acc[j][c] = pack2(a.x, a.y);
                     if (JORDAN) {
@@ -202,19 +242,19 @@ __device__ __forceinline__ void project(const float2 *pw, const float *xs, int c
 #pragma unroll (J == 4 && JORDAN ? 2 : 4)
         for (int u = 0; u < kHalf / 2; ++u) {
             const int v0 = TO_END ? u : kHalf / 2 - 1 - u, pp = p0 / 2 + v0;
-            const float4 xa = *reinterpret_cast<const float4 *>(xs + slot(pp, 2 * cg));
-            const float4 xb = *reinterpret_cast<const float4 *>(xs + slot(pp, 2 * cg + 1));
+            u64 x[NC];
+            load_columns<NC>(xs, pp, cg, x);
             ulonglong2 a[J];
             const int n = TO_END ? kHalf - 2 - 2 * v0 : 2 * v0;
 #pragma unroll
             for (int j = 0; j < J; ++j) a[j] = *reinterpret_cast<const ulonglong2 *>(pw + 8 * j * kPwStride + n);
-            const float v[2][4] = {{xa.x, xa.z, xb.x, xb.z}, {xa.y, xa.w, xb.y, xb.w}};
 #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 const int e = TO_END ? i : 1 - i;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const u64 d = dup2(v[e][c]);
+                for (int c = 0; c < NC; ++c) {
+                    const float2 v = unpack2(x[c]);
+                    const u64 d = dup2(e ? v.y : v.x);
 #pragma unroll
                     for (int j = 0; j < J; ++j) {
                         const u64 aj = (e == 0) == TO_END ? a[j].y : a[j].x;
@@ -238,25 +278,20 @@ __device__ __forceinline__ void project(const float2 *pw, const float *xs, int c
 // position blocks are held at once: shared-load wavefronts bound these products, 576 with
 // one at a time, 448 with two and 384 with four.  (One against two in the forward: 57.7 ->
 // 55.6 us at B = 2, L = 4096, D = 512, M = 32 fp32; against four in its backward: 127.7 -> 125.)
-template <bool kGuard, int SG>
-__device__ __forceinline__ void causal(const float *kq, const float *xs, int g, int cg, u64 (&acc)[8][4]) {
+// Only blocks lo .. hi - 1 of 16 positions hold drives (NC = 1; else all four).
+template <int NC, bool kGuard, int SG>
+__device__ __forceinline__ void causal(const float *kq, const float *xs, int g, int cg, int lo, int hi, u64 (&acc)[8][NC]) {
 #pragma unroll
     for (int s0 = 0; s0 < 4; s0 += SG) {
+        if (NC == 1 && (s0 + SG <= lo || s0 >= hi)) continue;
 #pragma unroll (SG == 4 ? 2 : 1)
         for (int u = 0; u < 8; ++u) {
-            u64 x[SG][4];   // positions 16 (s0 + i) + 2 u and the next
+            u64 x[SG][NC];   // positions 16 (s0 + i) + 2 u and the next
 #pragma unroll
-            for (int i = 0; i < SG; ++i) {
-                const float *row = xs + slot(8 * (s0 + i) + u, 2 * cg);
-                const ulonglong2 xa = *reinterpret_cast<const ulonglong2 *>(row);
-                const ulonglong2 xb = *reinterpret_cast<const ulonglong2 *>(row + 4);
-                x[i][0] = xa.x;
-                x[i][1] = xa.y;
-                x[i][2] = xb.x;
-                x[i][3] = xb.y;
-            }
+            for (int i = 0; i < SG; ++i) load_columns<NC>(xs, 8 * (s0 + i) + u, cg, x[i]);
 #pragma unroll
             for (int l = 0; l < 4 - s0; ++l) {
+                if (NC == 1 && s0 + l >= hi) break;
                 const int q1 = kC - 1 - (16 * l + 2 * g + 1) + 2 * u;   // row e = 1: even
                 const u64 k1 = *reinterpret_cast<const u64 *>(kq + q1);
                 const u64 k0 = *reinterpret_cast<const u64 *>(kq + kKernCopy + q1);   // row e = 0: kq[q1 + 1], kq[q1 + 2]
@@ -268,7 +303,7 @@ __device__ __forceinline__ void causal(const float *kq, const float *xs, int g, 
                         // Rows 2 g, 2 g + 1 of the block against its positions 2 u, 2 u + 1.
                         const float2 f0 = unpack2(k0), f1 = unpack2(k1);
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
+                        for (int c = 0; c < NC; ++c) {
                             const float2 v = unpack2(x[i][c]);
                             float2 a0 = unpack2(acc[2 * j][c]), a1 = unpack2(acc[2 * j + 1][c]);
                             if (u <= g) {
@@ -282,7 +317,7 @@ __device__ __forceinline__ void causal(const float *kq, const float *xs, int g, 
                         }
                     } else {
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
+                        for (int c = 0; c < NC; ++c) {
                             fma2(acc[2 * j][c], k0, x[i][c]);
                             fma2(acc[2 * j + 1][c], k1, x[i][c]);
                         }
@@ -295,9 +330,10 @@ __device__ __forceinline__ void causal(const float *kq, const float *xs, int g, 
 
 // acc += Re(sum_m lambda^p W) over `modes` modes: W is staged as (Re, -Im) per column, so
 // a packed FMA on (Re lambda^p, Im lambda^p) accumulates both halves of the real part.  Rows
-// p >= 32 take lambda^(p-32) and lambda^32 W (w2).
+// p >= 32 take lambda^(p-32) and lambda^32 W (w2).  Rows of blocks hi and up are left out (NC = 1).
+template <int NC>
 __device__ __forceinline__ void up_project(const float2 *pw, const float *w1, const float *w2, int modes, int g, int cg,
-                                           u64 (&acc)[8][4]) {
+                                           int hi, u64 (&acc)[8][NC]) {
 #pragma unroll 2
     for (int m = 0; m < modes; ++m) {
         ulonglong2 a[2];
@@ -305,20 +341,17 @@ __device__ __forceinline__ void up_project(const float2 *pw, const float *w1, co
         for (int j = 0; j < 2; ++j) a[j] = *reinterpret_cast<const ulonglong2 *>(pw + m * kPwStride + 16 * j + 2 * g);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const float *ws = h ? w2 : w1;
-            const ulonglong2 wa = *reinterpret_cast<const ulonglong2 *>(ws + slot(m, 2 * cg));
-            const ulonglong2 wb = *reinterpret_cast<const ulonglong2 *>(ws + slot(m, 2 * cg + 1));
+            if (NC == 1 && 2 * h >= hi) break;
+            u64 w[NC];
+            load_columns<NC>(h ? w2 : w1, m, cg, w);
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 const int r = 2 * (2 * h + j);
-                fma2(acc[r][0], a[j].x, wa.x);
-                fma2(acc[r][1], a[j].x, wa.y);
-                fma2(acc[r][2], a[j].x, wb.x);
-                fma2(acc[r][3], a[j].x, wb.y);
-                fma2(acc[r + 1][0], a[j].y, wa.x);
-                fma2(acc[r + 1][1], a[j].y, wa.y);
-                fma2(acc[r + 1][2], a[j].y, wb.x);
-                fma2(acc[r + 1][3], a[j].y, wb.y);
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    fma2(acc[r][c], a[j].x, w[c]);
+                    fma2(acc[r + 1][c], a[j].y, w[c]);
+                }
             }
         }
     }
@@ -329,40 +362,55 @@ __device__ __forceinline__ float2 power(const float2 *row, int n) {
     return n < kHalf ? row[n] : cmul(row[kHalf], row[n - kHalf]);
 }
 
-// sum_{p < tail} lambda^(tail-1-p) x_p of one column, in every lane: the four lanes of a mode
-// take every fourth power, and lambda^(n+32) shares the table entry of lambda^n.  (A single
-// lane walking the positions took up to 10 us of a call: B = 2, L = 4095, D = 512, M = 32 fp32
-// 76.4 us against 66.2 at L = 4096.)
-__device__ __forceinline__ float2 partial_end(const float2 *row, const float *xs, int col, int tail, int cg) {
-    float2 lo = make_float2(0.0f, 0.0f), hi = lo;
-    auto x = [&](int p) {
-        return p >= 0 ? xs[slot(p >> 1, col >> 1) + 2 * (col & 1) + (p & 1)] : 0.0f;
-    };
-#pragma unroll 4
-    for (int n = cg; n < kHalf; n += 4) {
-        const float2 z = row[n];
-        const float v = x(tail - 1 - n), w = x(tail - 1 - n - kHalf);
-        lo.x = fmaf(z.x, v, lo.x);
-        lo.y = fmaf(z.y, v, lo.y);
-        hi.x = fmaf(z.x, w, hi.x);
-        hi.y = fmaf(z.y, w, hi.y);
-    }
-    lo = cfma(row[kHalf], hi, lo);
+// Sums over the partial chunk in one column, for the lane's J modes of a group, in every
+// lane: sum_{p < tail} lambda^(tail-1-p) x_p, or (JT) sum_{n < tail} n lambda^n x_{n + 64 - tail}.
+// The four lanes of a mode take every fourth power, and lambda^(n+32) shares the table entry
+// of lambda^n.  (A single lane walking the positions took up to 10 us of a call: B = 2, L = 4095,
+// D = 512, M = 32 fp32 76.4 us against 66.2 at L = 4096.)
+template <int NC, int J, bool JT>
+__device__ __forceinline__ void partial_sums(const float2 *pw, const float *xs, int col, int tail, int cg, float2 (&f)[J]) {
+    float2 hi[J];
 #pragma unroll
-    for (int o = 8; o <= 16; o <<= 1) {
-        lo.x += __shfl_xor_sync(0xffffffffu, lo.x, o);
-        lo.y += __shfl_xor_sync(0xffffffffu, lo.y, o);
+    for (int j = 0; j < J; ++j) f[j] = hi[j] = make_float2(0.0f, 0.0f);
+    auto x = [&](int n) {
+        const int p = JT ? n + kC - tail : tail - 1 - n;
+        return (JT ? p < kC : p >= 0) ? xs[Tile<NC>::at(p >> 1, col) + (p & 1)] : 0.0f;
+    };
+#pragma unroll (J == 1 ? 4 : 2)
+    for (int n = cg; n < kHalf && n < tail; n += 4) {
+        float v = x(n), w = x(n + kHalf);
+        if (JT) {
+            v *= (float)n;
+            w *= (float)(n + kHalf);
+        }
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const float2 z = pw[8 * j * kPwStride + n];
+            f[j].x = fmaf(z.x, v, f[j].x);
+            f[j].y = fmaf(z.y, v, f[j].y);
+            hi[j].x = fmaf(z.x, w, hi[j].x);
+            hi[j].y = fmaf(z.y, w, hi[j].y);
+        }
     }
-    return lo;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+        f[j] = cfma(pw[8 * j * kPwStride + kHalf], hi[j], f[j]);
+#pragma unroll
+        for (int o = 8; o <= 16; o <<= 1) {
+            f[j].x += __shfl_xor_sync(0xffffffffu, f[j].x, o);
+            f[j].y += __shfl_xor_sync(0xffffffffu, f[j].y, o);
+        }
+    }
 }
 
 // acc[n] += sum_u dy_u x_{u + 16 l + n} over the 16 positions u of block a, one column
 // (the lane's); positions past the chunk count as zero.
+template <int NC>
 __device__ __forceinline__ void correlate(const float *dys, const float *xs, int col, int a, int l, float (&acc)[16]) {
     float dv[16], xv[32];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-        const float2 v = *reinterpret_cast<const float2 *>(dys + slot(8 * a + u, col >> 1) + 2 * (col & 1));
+        const float2 v = *reinterpret_cast<const float2 *>(dys + Tile<NC>::at(8 * a + u, col));
         dv[2 * u] = v.x;
         dv[2 * u + 1] = v.y;
     }
@@ -371,7 +419,7 @@ __device__ __forceinline__ void correlate(const float *dys, const float *xs, int
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const float2 v = a + l + h < 4
-                                 ? *reinterpret_cast<const float2 *>(xs + slot(8 * (a + l + h) + u, col >> 1) + 2 * (col & 1))
+                                 ? *reinterpret_cast<const float2 *>(xs + Tile<NC>::at(8 * (a + l + h) + u, col))
                                  : make_float2(0.0f, 0.0f);
             xv[16 * h + 2 * u] = v.x;
             xv[16 * h + 2 * u + 1] = v.y;
@@ -382,61 +430,79 @@ __device__ __forceinline__ void correlate(const float *dys, const float *xs, int
         for (int n = 0; n < 16; ++n) acc[n] = fmaf(dv[u], xv[u + n], acc[n]);
 }
 
-// v[n] summed over the 16 columns (lanes of one half); lane `col` receives lag n = col.
-__device__ __forceinline__ float sum_columns(float (&v)[16], int col) {
+// v[n] summed over the tile's columns (4 NC consecutive lanes); lane `col` of them receives the
+// lags n = 4 col / NC .. of the first 4 / NC entries.
+template <int NC>
+__device__ __forceinline__ void sum_columns(float (&v)[16], int col) {
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) {
+    for (int o = 2 * NC, k = 8; o > 0; o >>= 1, k >>= 1) {
         const bool up = col & o;
 #pragma unroll
-        for (int n = 0; n < o; ++n) {
-            const float keep = up ? v[n + o] : v[n], send = up ? v[n] : v[n + o];
+        for (int n = 0; n < k; ++n) {
+            const float keep = up ? v[n + k] : v[n], send = up ? v[n] : v[n + k];
             v[n] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
     }
-    return v[0];
 }
 
 // One block: channels 4 blockIdx.x .. + 3 of batch row blockIdx.z, segment blockIdx.y.
-// Sequences of at most 4 (8) chunks leave most of a tile's 16 columns empty, so there a
+// Sequences of at most NC (2 NC) chunks leave most of a tile's columns empty, so there a
 // tile holds 4 (2) batch rows, one (two) column groups each, and blockIdx.z counts
 // tiles: b below is then the lane's own row, clamped; `mine` says whether it exists.
-// kOut: write outputs (else only the segment's end state, from zero).
-template <int J, int NP, bool BWD, bool kOut>
-__global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_scan(const ScanArgs A) {
-    constexpr int kModes = 8 * J * NP;
+// kOut: write outputs (else only the segment's end state, from zero).  HW = 2: the warp of
+// modes 0 .. 31 forms the causal products, that of the others the lag correlation; both parts of K
+// and of the outputs are added in shared memory.
+template <int NC, int J, int NP, int HW, bool BWD, bool kOut>
+__global__ void __launch_bounds__(HW * kThreads, blocks_per_sm(8 * J * NP * HW, NC, BWD)) k_scan(const ScanArgs A) {
+    static_assert(HW == 1 || (NC == 1 && kOut), "two warps a channel: narrow tiles only");
+    constexpr int kModes = 8 * J * NP;   // of a warp
+    using T = Tile<NC>;
+    constexpr int kCols = T::kCols, kTile = T::kTokens, kFieldWords = T::kFieldWords;
+    constexpr int kPass = HW * kThreads / kCols, kPasses = kC / kPass;   // positions the threads stage at once
     constexpr bool kX = BWD && kOut;   // the x tile is needed
     constexpr int kSG = BWD && J == 4 ? 4 : 2;   // (see causal(); the forward with four: 55.6 -> 57.7 us)
-    constexpr bool kAhead = !BWD && J == 4;   // the next tile's drive is loaded a tile ahead
+    constexpr bool kAhead = NC == 4 && !BWD && J == 4;   // the next tile's drive is loaded a tile ahead
     extern __shared__ __align__(16) float smem[];
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, w = (tid >> 5) & (kCh - 1);
+    const int hm = HW == 2 ? tid >> 7 : 0;   // which of the channel's warps, modes 32 hm ..
     const int g = lane & 7, cg = lane >> 3;
     const int seg = blockIdx.y;
     const int rpt = 4 / A.gpr, gbase = cg & ~(A.gpr - 1);   // batch rows of a tile; the row's first column group
     const bool mine = (int)blockIdx.z * rpt + cg / A.gpr < A.B;
     const int64_t b = min((int)blockIdx.z * rpt + cg / A.gpr, A.B - 1);
-    const int d0 = kCh * blockIdx.x, d = d0 + w, M = A.M, D = A.D;
-    constexpr int kWords = chan_words(kModes, kOut);
-    constexpr int kTableWords = 2 * kModes * (kPwStride + 1) + kKernWords;   // before the field tiles
-    float2 *pw = reinterpret_cast<float2 *>(smem + w * kWords);
+    const int nrows = min(rpt, A.B - (int)blockIdx.z * rpt);   // rows that exist
+    const int d0 = kCh * blockIdx.x, d = d0 + w, D = A.D;
+    const int M = HW == 2 ? min(kModes, A.M - kModes * hm) : A.M;   // the warp's modes, from these on:
+    const int pm0 = d * A.M + kModes * hm;
+    const int64_t bm0 = (b * D + d) * A.M + kModes * hm;
+    constexpr int kWords = chan_words(HW * kModes, NC, HW, kOut), kTable = 2 * kModes * (kPwStride + 1);
+    constexpr int kTableWords = HW * kTable + kKernWords;   // before the field tiles
+    float2 *pw = reinterpret_cast<float2 *>(smem + w * kWords + hm * kTable);
     float2 *cs = pw + kModes * kPwStride;        // c of every mode
-    float *kq = smem + w * kWords + 2 * kModes * (kPwStride + 1);
-    float *us = kq + kKernWords;                 // drive tile, then W, then the output tile
-    float *xs = us + (kOut ? kFieldWords : 0);   // x tile (backward), then lambda^32 W
+    float *kq = smem + w * kWords + HW * kTable;
+    float *us = kq + kKernWords;                 // drive tile; HW = 1: then W, then the output tile
+    float *xs = us + (kOut ? kFieldWords : 0);   // x tile (backward); HW = 1: then lambda^32 W
+    float *w1 = HW == 2 ? xs + (1 + 2 * hm) * kFieldWords : us, *w2 = HW == 2 ? w1 + kFieldWords : xs;
     pdl_launch_dependents();
 
     const int tail = (int)(A.L & (kC - 1));                 // tokens of the partial last chunk
+    // A sequence of one partial chunk (on the narrow tile): drives in blocks lo .. hi - 1 of 16
+    // positions only, no chunk before or after, so the chunk sums serve the state terms alone.
+    const bool single = NC == 1 && A.nch == 1 && tail != 0;
+    const bool ends = !single || (BWD && (A.state_in || A.d_state_in)), enters = !single || (!BWD && A.enter);
+    const int lo = single && BWD ? (kC - tail) >> 4 : 0, hi = single && !BWD ? (tail + 15) >> 4 : 4;
     const int tile_end = min(A.ntiles, (seg + 1) * A.tps);
-    // The thread's 8 tokens of a tile, 4 channels each (zeros outside the sequence).
+    // The thread's tokens of a tile, 4 channels each (zeros outside the sequence).
     const int Li = (int)A.L, t_last = A.nch * kC - 1;
     // The thread's column: its batch row, and its first token's tau in tile 0.
-    const int fcol = tid & (kCols - 1), frow = (int)blockIdx.z * rpt + fcol / (4 * A.gpr);
-    const int ftau = (fcol & (4 * A.gpr - 1)) * kC + (tid >> 4);
+    const int fcol = tid & (kCols - 1), frow = (int)blockIdx.z * rpt + fcol / (NC * A.gpr);
+    const int ftau = (fcol & (NC * A.gpr - 1)) * kC + tid / kCols;
     const int64_t fbase = (int64_t)frow * A.L;
-    auto fetch = [&](const void *f, int tile, float4 (&v)[8]) {
+    auto fetch = [&](const void *f, int tile, float4 (&v)[kPasses]) {
         const int tau = tile * kTile + ftau;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int t = A.rev ? t_last - tau - 8 * i : tau + 8 * i;
+        for (int i = 0; i < kPasses; ++i) {
+            const int t = A.rev ? t_last - tau - kPass * i : tau + kPass * i;
             v[i] = t >= 0 && t < Li && frow < A.B ? load4(f, A.bf16, (fbase + t) * D + d0)
                                                   : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
@@ -449,15 +515,15 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
     if (!kAhead && frow < A.B) {
         const int tau = seg * A.tps * kTile + ftau, e = A.bf16 ? 2 : 4;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int t = A.rev ? t_last - tau - 8 * i : tau + 8 * i;
+        for (int i = 0; i < kPasses; ++i) {
+            const int t = A.rev ? t_last - tau - kPass * i : tau + kPass * i;
             if (t < 0 || t >= Li) continue;
             const int64_t at = ((fbase + t) * D + d0) * e;
             prefetch_l2(static_cast<const char *>(A.u) + at);
             if (kX) prefetch_l2(static_cast<const char *>(A.x) + at);
         }
     }
-    float4 nextu[8], nextx[kX ? 8 : 1];
+    float4 nextu[kPasses], nextx[kX ? kPasses : 1];
 
     // ---- tables: lambda^n, n < 32 (an exact power every 8, products between), 32 and 64
     {
@@ -466,15 +532,15 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
         for (int m = lane / kLpm; m < kModes; m += 32) {
             float2 *row = pw + m * kPwStride;
             const bool on = m < M;
-            const float ga = on ? A.decay[d * M + m] : 0.0f, om = on ? A.freq[d * M + m] : 0.0f;
-            const float am = kOut && on ? A.amp[d * M + m] : 0.0f, ph = kOut && on ? A.phase[d * M + m] : 0.0f;
+            const float ga = on ? A.decay[pm0 + m] : 0.0f, om = on ? A.freq[pm0 + m] : 0.0f;
+            const float am = kOut && on ? A.amp[pm0 + m] : 0.0f, ph = kOut && on ? A.phase[pm0 + m] : 0.0f;
             if (!BWD && A.enter && on)   // used after the tables
-                prefetch_l2(A.enter + ((int64_t)min((int)blockIdx.z * rpt, A.B - 1) * D + d) * M + m);
+                prefetch_l2(A.enter + ((int64_t)min((int)blockIdx.z * rpt, A.B - 1) * D + d) * A.M + kModes * hm + m);
             const float2 l1 = lambda_pow(ga, om, 1.0f);
 #pragma unroll 1
             for (int n0 = 8 * (lane % kLpm); n0 < kHalf; n0 += 8 * kLpm) {
-                float2 z = lambda_pow(ga, om, (float)n0);
-                if (!on) z = make_float2(0.0f, 0.0f);
+                float2 z = make_float2(0.0f, 0.0f);
+                if (on && !(single && n0 > tail)) z = lambda_pow(ga, om, (float)n0);   // (zeros past a short sequence)
                 row[n0] = z;
 #pragma unroll
                 for (int e = 1; e < 8; ++e) row[n0 + e] = z = cmul(z, l1);
@@ -497,16 +563,16 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
         for (int j = 0; j < J; ++j) {
             const int m = 8 * J * q + 8 * j + g;
             const bool on = m < M;
-            const float ga = on ? A.decay[d * M + m] : 0.0f, om = on ? A.freq[d * M + m] : 0.0f;
+            const float ga = on ? A.decay[pm0 + m] : 0.0f, om = on ? A.freq[pm0 + m] : 0.0f;
             const float2 z = make_float2(0.0f, 0.0f);
-            const int64_t sm = (b * D + d) * M + m;
+            const int64_t sm = bm0 + m;
             S0[q][j] = !BWD && A.enter && on && mine && seg == 0 ? A.enter[sm] : z;
             if (BWD) R0[q][j] = z;
             if (kOut && seg > 0 && on) {
                 // The earlier segments' end states, each carried over the segments between.
                 const float nf = (float)(A.tps * kTile);
                 const float2 lN = lambda_pow(ga, om, nf);
-                const int64_t st = (int64_t)A.B * D * M;
+                const int64_t st = (int64_t)A.B * D * A.M;
                 float2 S = z, R = z;
 #pragma unroll 4
                 for (int r = 0; r < seg; ++r) {
@@ -519,33 +585,55 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
             }
             if (!BWD && kOut && A.coef_out && blockIdx.z == 0 && seg == A.nseg - 1 && cg == 0 && on) {
                 const float2 l1 = pw[m * kPwStride + 1];   // the exact lambda times lambda^0 = 1
-                A.coef_out[d * M + m] = make_float4(l1.x, l1.y, cs[m].x, cs[m].y);
+                A.coef_out[pm0 + m] = make_float4(l1.x, l1.y, cs[m].x, cs[m].y);
             }
             // The output launch's segment 0 starts from this copy: by then a state_out that
             // is state_in's buffer may be written by the last segment's block.
             if (!kOut && !BWD && seg == 0 && A.enter && cg == 0 && on)
-                A.seg_s[sm + (int64_t)(A.nseg - 1) * A.B * D * M] = S0[q][j];
+                A.seg_s[sm + (int64_t)(A.nseg - 1) * A.B * D * A.M] = S0[q][j];
         }
     __syncwarp();
     if (kOut) {
         // K[n] = sum_m Re(c lambda^n), stored reversed (and once more shifted by one).
         float k0 = 0.0f, k1 = 0.0f;
-        for (int m = 0; m < M; ++m) {
+        auto add = [&](int m) {
             const float2 c = cs[m], p = pw[m * kPwStride + lane], c2 = cmul(c, pw[m * kPwStride + kHalf]);
             k0 = fmaf(c.x, p.x, fmaf(-c.y, p.y, k0));
             k1 = fmaf(c2.x, p.x, fmaf(-c2.y, p.y, k1));
+        };
+        if constexpr (NC == 4) {   // (unrolled, the 16-mode backward of L = 8000 took 148 us against 144)
+            for (int m = 0; m < M; ++m) add(m);
+        } else {
+#pragma unroll 4
+            for (int m = 0; m < M; ++m) add(m);
         }
-        kq[63 - lane] = k0;
-        kq[31 - lane] = k1;
-        kq[kKernCopy + 62 - lane] = k0;
-        if (lane < 31) kq[kKernCopy + 30 - lane] = k1;
-        if (lane < 16) kq[kC + lane] = kq[kKernCopy + kC + lane] = 0.0f;
-        if (lane == 0) kq[kKernCopy + kC - 1] = 0.0f;
+        if constexpr (HW == 2) {   // the first warp adds the second's part
+            if (hm) {
+                w1[lane] = k0;
+                w1[32 + lane] = k1;
+            }
+            __syncthreads();
+            if (!hm) {
+                const float *o = w1 + 2 * kFieldWords;
+                k0 += o[lane];
+                k1 += o[32 + lane];
+            }
+        }
+        if (!hm) {
+            kq[63 - lane] = k0;
+            kq[31 - lane] = k1;
+            kq[kKernCopy + 62 - lane] = k0;
+            if (lane < 31) kq[kKernCopy + 30 - lane] = k1;
+            if (lane < 16) kq[kC + lane] = kq[kKernCopy + kC + lane] = 0.0f;
+            if (lane == 0) kq[kKernCopy + kC - 1] = 0.0f;
+        }
     }
     __syncwarp();
 
     float2 G[kX ? NP : 1][J], P[kX ? NP : 1][J], Jg[kX ? NP : 1][J];
-    float rho_a = 0.0f, rho_b = 0.0f;   // lane (h, n): lags 16 h + n and 16 (3 - h) + n
+    // NC = 4: lane (h, n): lags 16 h + n and 16 (3 - h) + n.  NC = 1: lane (h, col): lags
+    // 4 col + i of the lag blocks that group h correlates.
+    float rho_a[4 / NC] = {}, rho_b[4 / NC] = {};
     if (kX) {
 #pragma unroll
         for (int q = 0; q < NP; ++q)
@@ -557,11 +645,11 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
         // ---- stage the tile: thread (column, position), 4 channels each
         const int t0 = tile * kTile + ftau;   // tau of the thread's first token
         bool odd = false;   // an infinite or NaN drive
-        auto stage = [&](const float4 (&v)[8], float *base) {
+        auto stage = [&](const float4 (&v)[kPasses], float *base) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int p = (tid >> 4) + 8 * i, col = tid & (kCols - 1);
-                float *o = base + slot(p >> 1, col >> 1) + 2 * (col & 1) + (p & 1);
+            for (int i = 0; i < kPasses; ++i) {
+                const int p = tid / kCols + kPass * i, col = tid & (kCols - 1);
+                float *o = base + T::at(p >> 1, col) + (p & 1);
                 o[0] = v[i].x;
                 o[kWords] = v[i].y;
                 o[2 * kWords] = v[i].z;
@@ -573,7 +661,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
         if constexpr (kX) fetch(A.x, tile, nextx);
         stage(nextu, base);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < kPasses; ++i) {
             // x - x is zero for a finite x.
             const float z = (nextu[i].x - nextu[i].x) + (nextu[i].y - nextu[i].y) + (nextu[i].z - nextu[i].z) +
                             (nextu[i].w - nextu[i].w);
@@ -583,49 +671,66 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
         const bool guard = __syncthreads_or(kOut && odd);
 
         // ---- chunk-local states, carry over the 16 columns (and G, P)
-        const int chunk0 = tile * kCols + 4 * (cg - gbase);   // the lane's first chunk
-        u64 ls[NP][J][4];   // lambda S of the state entering each of the lane's columns
+        const int chunk0 = tile * kCols + NC * (cg - gbase);   // the lane's first chunk
+        u64 ls[NP][J][NC];   // lambda S of the state entering each of the lane's columns
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
-            u64 acc[J][4], accq[BWD ? J : 1][4];
-            project<J, BWD, true>(pw + (8 * J * q + g) * kPwStride, us, cg, acc, accq);
-            float2 Rn[BWD ? J : 1][4];
+            u64 acc[J][NC], accq[BWD ? J : 1][NC];
+            if (ends) {
+                project<NC, J, BWD, true>(pw + (8 * J * q + g) * kPwStride, us, cg, acc, accq);
+            } else {
+#pragma unroll
+                for (int j = 0; j < J; ++j)
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        acc[j][c] = 0ull;
+                        if (BWD) accq[j][c] = 0ull;
+                    }
+            }
+            float2 Rn[BWD ? J : 1][NC], send[BWD ? 1 : J];   // send: the state entering the partial last chunk
 #pragma unroll
             for (int j = 0; j < J; ++j) {
+                if (!ends) {   // nothing but the state entering the sequence
+                    const float2 v = BWD ? make_float2(0.0f, 0.0f) : cmul(pw[(8 * J * q + 8 * j + g) * kPwStride + 1], S0[q][j]);
+                    ls[q][j][0] = pack2(v.x, v.y);
+                    if (!BWD) send[j] = S0[q][j];
+                    continue;
+                }
                 const float2 *row = pw + (8 * J * q + 8 * j + g) * kPwStride;
-                const float2 a = row[kHalf + 1], a2 = cmul(a, a), a4 = cmul(a2, a2);
+                const float2 a = row[kHalf + 1], a2 = cmul(a, a), a4 = NC == 4 ? cmul(a2, a2) : a;   // a^NC
                 const float2 lam = row[1];
-                // The lane's four columns from zero ...
+                // The lane's columns from zero ...
                 float2 es = make_float2(0.0f, 0.0f), er = es;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
+                for (int c = 0; c < NC; ++c) {
                     if (BWD)
                         er = cfma(a, make_float2(fmaf((float)kC, es.x, er.x), fmaf((float)kC, es.y, er.y)),
                                   unpack2(accq[j][c]));
                     es = cfma(a, es, unpack2(acc[j][c]));
                 }
                 // ... the state entering them (over the mode's lanes in this row) ...
-                float2 T = S0[q][j], U = BWD ? R0[q][j] : T, S = T, R = U, send = T;
+                float2 V = S0[q][j], U = BWD ? R0[q][j] : V, S = V, R = U;
+                if (!BWD) send[j] = V;
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     if (i >= A.gpr) break;   // the same for every lane
                     if (gbase + i == cg) {
-                        S = T;
+                        S = V;
                         R = U;
                     }
                     const float2 ei = shfl2(es, g + 8 * (gbase + i));
                     if (BWD)
-                        U = cfma(a4, make_float2(fmaf(4.0f * kC, T.x, U.x), fmaf(4.0f * kC, T.y, U.y)),
+                        U = cfma(a4, make_float2(fmaf((float)(NC * kC), V.x, U.x), fmaf((float)(NC * kC), V.y, U.y)),
                                  shfl2(er, g + 8 * (gbase + i)));
-                    T = cfma(a4, T, ei);
+                    V = cfma(a4, V, ei);
                 }
-                S0[q][j] = T;
+                S0[q][j] = V;
                 if (BWD) R0[q][j] = U;
                 // ... and entering each of them.
                 const int m = 8 * J * q + 8 * j + g;
                 const bool on = m < M;
 #pragma unroll
-                for (int c = 0; c < (kOut ? 4 : 0); ++c) {
+                for (int c = 0; c < (kOut ? NC : 0); ++c) {
                     const float2 lsv = cmul(lam, S);
                     ls[q][j][c] = pack2(lsv.x, lsv.y);
                     if (kX) {
@@ -635,11 +740,11 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                         S = cfma(a, S, unpack2(acc[j][c]));
                         if (chunk0 + c == A.nch - 1 && on && mine) {
                             // The chunk of token 0: (S, R) is the adjoint pair there.
-                            const int64_t sm = (b * D + d) * M + m;
+                            const int64_t sm = bm0 + m;
                             const float2 l0 = cmul(lam, S);
                             const float2 gg = A.g ? A.g[sm] : make_float2(0.0f, 0.0f);
                             const float2 lL =
-                                A.g ? lambda_pow(A.decay[d * M + m], A.freq[d * M + m], (float)A.L) : gg;
+                                A.g ? lambda_pow(A.decay[pm0 + m], A.freq[pm0 + m], (float)A.L) : gg;
                             if (A.state_in) {
                                 const float2 si = A.state_in[sm];
                                 G[q][j] = cfma(si, l0, G[q][j]);
@@ -657,39 +762,44 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                         const float2 next = cfma(a, S, unpack2(acc[j][c]));
                         if (chunk0 + c == A.nch - 1) {
                             if (tail)
-                                send = S;
+                                send[j] = S;
                             else if (on && mine && A.state_out)
-                                A.state_out[(b * D + d) * M + m] = next;
+                                A.state_out[bm0 + m] = next;
                         }
                         S = next;
                     }
                 }
-                if (!BWD && kOut && tail && tile == A.ntiles - 1 && A.state_out)
-                    for (int r = 0; r < rpt; ++r) {
-                        const int col = r * 4 * A.gpr + (A.nch - 1 - tile * kCols);   // row r's last chunk
-                        const float2 f = partial_end(row, us, col, tail, cg);
-                        if (cg == col >> 2 && on && mine)
-                            A.state_out[(b * D + d) * M + m] = cfma(power(row, tail), send, f);
-                    }
             }
-            if (kX) {
-                u64 xp[J][4], xq[J][4];
-                project<J, true, false>(pw + (8 * J * q + g) * kPwStride, xs, cg, xp, xq);
+            if (!BWD && kOut && tail && tile == A.ntiles - 1 && A.state_out)
+                for (int r = 0; r < nrows; ++r) {
+                    const int col = r * NC * A.gpr + (A.nch - 1 - tile * kCols);   // row r's last chunk
+                    float2 f[J];
+                    partial_sums<NC, J, false>(pw + (8 * J * q + g) * kPwStride, us, col, tail, cg, f);
+#pragma unroll
+                    for (int j = 0; j < J; ++j) {
+                        const int m = 8 * J * q + 8 * j + g;
+                        if (cg == col / NC && m < M)
+                            A.state_out[bm0 + m] = cfma(power(pw + m * kPwStride, tail), send[j], f[j]);
+                    }
+                }
+            if (kX && !single) {
+                u64 xp[J][NC], xq[J][NC];
+                project<NC, J, true, false>(pw + (8 * J * q + g) * kPwStride, xs, cg, xp, xq);
 #pragma unroll
                 for (int j = 0; j < J; ++j) {
                     const int m = 8 * J * q + 8 * j + g;
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
+                    for (int c = 0; c < NC; ++c) {
                         const float2 s = unpack2(ls[q][j][c]), p = unpack2(xp[j][c]), v = unpack2(xq[j][c]);
                         G[q][j] = cfma(p, s, G[q][j]);
                         P[q][j] = cfma(p, Rn[j][c], cfma(v, s, P[q][j]));
                     }
                     if (A.g && m < M) {
                         // J over the whole chunks: L - 1 - t = E + p with E = L minus the chunk's end.
-                        const float ga = A.decay[d * M + m], om = A.freq[d * M + m];
+                        const float ga = A.decay[pm0 + m], om = A.freq[pm0 + m];
                         float2 z = make_float2(0.0f, 0.0f);
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) {
+                        for (int c = 0; c < NC; ++c) {
                             const int64_t E = A.L - (int64_t)(A.nch - chunk0 - c) * kC;
                             if (E >= 0 && chunk0 + c < A.nch) {
                                 z = c == 0 || E < kC ? lambda_pow(ga, om, (float)E) : cmul(z, pw[m * kPwStride + kHalf + 1]);
@@ -698,19 +808,31 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                                 Jg[q][j] = cfma(z, make_float2(fmaf(Ef, p.x, v.x), fmaf(Ef, p.y, v.y)), Jg[q][j]);
                             }
                         }
-                        if (tail && tile == 0) {
-                            // The partial last chunk (the row's first column): its tokens are
-                            // positions p >= 64 - tail, L - 1 - t = p - (64 - tail), shared out
-                            // among the row's lanes.
-                            const float2 *row = pw + m * kPwStride;
-                            for (int n = cg - gbase; n < tail; n += A.gpr) {
-                                const int p = n + kC - tail;
-                                const float v = (float)n * xs[slot(p >> 1, 2 * gbase) + (p & 1)];
-                                const float2 z = power(row, n);
-                                Jg[q][j].x = fmaf(z.x, v, Jg[q][j].x);
-                                Jg[q][j].y = fmaf(z.y, v, Jg[q][j].y);
-                            }
+                    }
+                }
+            }
+            if (kX && A.g && tail && tile == 0) {
+                // The partial last chunk (each row's first column): its tokens are
+                // positions p >= 64 - tail, with L - 1 - t = p - (64 - tail).
+                if constexpr (NC == 4) {   // (most rows of a wide tile exist: shared out among a row's lanes)
+#pragma unroll
+                    for (int j = 0; j < J; ++j) {
+                        const float2 *row = pw + (8 * J * q + 8 * j + g) * kPwStride;
+                        for (int n = cg - gbase; n < tail; n += A.gpr) {
+                            const int p = n + kC - tail;
+                            const float v = (float)n * xs[T::at(p >> 1, NC * gbase) + (p & 1)];
+                            const float2 z = power(row, n);
+                            Jg[q][j].x = fmaf(z.x, v, Jg[q][j].x);
+                            Jg[q][j].y = fmaf(z.y, v, Jg[q][j].y);
                         }
+                    }
+                } else {
+                    for (int r = 0; r < nrows; ++r) {
+                        float2 f[J];
+                        partial_sums<NC, J, true>(pw + (8 * J * q + g) * kPwStride, xs, r * NC * A.gpr, tail, cg, f);
+#pragma unroll
+                        for (int j = 0; j < J; ++j)
+                            if (cg == r * A.gpr) Jg[q][j] = make_float2(Jg[q][j].x + f[j].x, Jg[q][j].y + f[j].y);
                     }
                 }
             }
@@ -720,51 +842,66 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
             __syncthreads();   // every warp is done with the tile
             continue;
         }
-        if (kX) {
-            // Lag correlation: lane = (column, half); the half takes lag blocks {0, 3} or
-            // {1, 2}, whose 10 non-empty (u block, lag block) pairs fall in 4 + 2 steps.
-            const int col = lane & 15, h = lane >> 4;
+        if (kX && hm == HW - 1) {
             float r0[16], r1[16];
 #pragma unroll
             for (int n = 0; n < 16; ++n) r0[n] = r1[n] = 0.0f;
+            const int col = lane & (kCols - 1), h = lane / kCols;
+            if constexpr (NC == 4) {
+                // Lag correlation: lane = (column, half); the half takes lag blocks {0, 3} or
+                // {1, 2}, whose 10 non-empty (u block, lag block) pairs fall in 4 + 2 steps.
 #pragma unroll 1
-            for (int a = 0; a < 4; ++a) correlate(us, xs, col, a, h, r0);
+                for (int a = 0; a < 4; ++a) correlate<NC>(us, xs, col, a, h, r0);
 #pragma unroll 1
-            for (int a = 0; a < 2; ++a) correlate(us, xs, col, a, 3 - h, r1);
-            rho_a += sum_columns(r0, col);
-            rho_b += sum_columns(r1, col);
+                for (int a = 0; a < 2; ++a) correlate<NC>(us, xs, col, a, 3 - h, r1);
+            } else {
+                // Eight lane groups h take one pair each, then two of them the rest (lag block 2):
+                // (h, 0), h < 4; (h - 4, 1), h < 7; (0, 3); (h, 2), h < 2.
+                correlate<NC>(us, xs, col, h == 7 ? 0 : h & 3, h < 4 ? 0 : h < 7 ? 1 : 3, r0);
+                if (hi - lo > 2 && h < 2) correlate<NC>(us, xs, col, h, 2, r1);
+            }
+            sum_columns<NC>(r0, col);
+            sum_columns<NC>(r1, col);
+#pragma unroll
+            for (int i = 0; i < 4 / NC; ++i) {
+                rho_a[i] += r0[i];
+                rho_b[i] += r1[i];
+            }
         }
 
         // ---- outputs
-        u64 acc[8][4];
+        u64 acc[8][NC];
 #pragma unroll
         for (int r = 0; r < 8; ++r)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[r][c] = 0ull;
-        if (guard)
-            causal<true, kSG>(kq, us, g, cg, acc);
-        else
-            causal<false, kSG>(kq, us, g, cg, acc);
+            for (int c = 0; c < NC; ++c) acc[r][c] = 0ull;
+        if (hm == 0) {
+            if (guard)
+                causal<NC, true, kSG>(kq, us, g, cg, lo, hi, acc);
+            else
+                causal<NC, false, kSG>(kq, us, g, cg, lo, hi, acc);
+        }
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
+            if (!enters) break;
             __syncwarp();   // the warp is done reading the tile (or the previous W)
 #pragma unroll
             for (int j = 0; j < J; ++j) {
                 const int m = 8 * J * q + 8 * j + g;
-                float2 W[4];
+                float2 W[NC];
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
+                for (int c = 0; c < NC; ++c) {
                     const float2 v = cmul(cs[m], unpack2(ls[q][j][c]));
                     W[c] = m < M ? make_float2(v.x, -v.y) : make_float2(0.0f, 0.0f);
                 }
                 if (kX && A.g && m < M) {
                     // Terminal-state gradient: its adjoint conj(g) lambda^(L-1-t) enters a
                     // whole chunk as conj(g) lambda^E with E = L minus the chunk's end.
-                    const float ga = A.decay[d * M + m], om = A.freq[d * M + m];
-                    const float2 gg = A.g[(b * D + d) * M + m];
+                    const float ga = A.decay[pm0 + m], om = A.freq[pm0 + m];
+                    const float2 gg = A.g[bm0 + m];
                     float2 z = make_float2(0.0f, 0.0f);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
+                    for (int c = 0; c < NC; ++c) {
                         const int64_t E = A.L - (int64_t)(A.nch - chunk0 - c) * kC;
                         if (E >= 0 && chunk0 + c < A.nch) {
                             z = c == 0 || E < kC ? lambda_pow(ga, om, (float)E) : cmul(z, pw[m * kPwStride + kHalf + 1]);
@@ -774,32 +911,37 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                         }
                     }
                 }
-                *reinterpret_cast<float4 *>(us + slot(8 * j + g, 2 * cg)) = make_float4(W[0].x, W[0].y, W[1].x, W[1].y);
-                *reinterpret_cast<float4 *>(us + slot(8 * j + g, 2 * cg + 1)) =
-                    make_float4(W[2].x, W[2].y, W[3].x, W[3].y);
+                store_columns<NC>(w1, 8 * j + g, cg, W);
                 const float2 l32 = conj2(pw[m * kPwStride + kHalf]);   // (W is kept conjugated)
 #pragma unroll
-                for (int c = 0; c < 4; ++c) W[c] = cmul(l32, W[c]);
-                *reinterpret_cast<float4 *>(xs + slot(8 * j + g, 2 * cg)) = make_float4(W[0].x, W[0].y, W[1].x, W[1].y);
-                *reinterpret_cast<float4 *>(xs + slot(8 * j + g, 2 * cg + 1)) =
-                    make_float4(W[2].x, W[2].y, W[3].x, W[3].y);
+                for (int c = 0; c < NC; ++c) W[c] = cmul(l32, W[c]);
+                store_columns<NC>(w2, 8 * j + g, cg, W);
             }
             __syncwarp();
             if (kAhead && q == NP - 1 && tile + 1 < tile_end) fetch(A.u, tile + 1, nextu);
-            up_project(pw + 8 * J * q * kPwStride, us, xs, min(8 * J, M - 8 * J * q), g, cg, acc);
+            up_project<NC>(pw + 8 * J * q * kPwStride, w1, w2, min(8 * J, M - 8 * J * q), g, cg, hi, acc);
         }
-        float y[8][4];
+        float y[8][NC];
 #pragma unroll
         for (int r = 0; r < 8; ++r)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
+            for (int c = 0; c < NC; ++c) {
                 const float2 v = unpack2(acc[r][c]);
                 y[r][c] = v.x + v.y;
             }
-        if (kX && A.g && tail && chunk0 == 0) {
-            // The terminal-state term of the partial last chunk.
-            for (int m = 0; m < M; ++m) {
-                const float2 gg = A.g[(b * D + d) * M + m];
+        if (kX && A.g && tail && tile == 0) {
+            // The terminal-state term of the partial last chunk.  Narrow tiles, whose blocks are few
+            // and wait for nothing else here, take g through the tiles' memory (free by now) so
+            // that its loads are in flight together: one after the other
+            // they took 50k cycles of a block at M = 64, L = 48.
+            float2 *gs = reinterpret_cast<float2 *>(w1);   // [mode][row]
+            if constexpr (NC == 1) {
+                __syncwarp();
+                for (int m = g; m < M && chunk0 == 0; m += 8) gs[m * 4 + cg] = A.g[bm0 + m];
+                __syncwarp();
+            }
+            for (int m = 0; m < M && chunk0 == 0; ++m) {
+                const float2 gg = NC == 1 ? gs[m * 4 + cg] : A.g[bm0 + m];
 #pragma unroll
                 for (int r = 0; r < 8; ++r) {
                     const int n = 16 * (r >> 1) + 2 * g + (r & 1) - (kC - tail);
@@ -811,21 +953,41 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
             }
         }
         __syncwarp();
+        auto store_y = [&] {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            *reinterpret_cast<float4 *>(us + slot(8 * j + g, 2 * cg)) =
-                make_float4(y[2 * j][0], y[2 * j + 1][0], y[2 * j][1], y[2 * j + 1][1]);
-            *reinterpret_cast<float4 *>(us + slot(8 * j + g, 2 * cg + 1)) =
-                make_float4(y[2 * j][2], y[2 * j + 1][2], y[2 * j][3], y[2 * j + 1][3]);
+            for (int j = 0; j < 4; ++j) {
+                float2 v[NC];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) v[c] = make_float2(y[2 * j][c], y[2 * j + 1][c]);
+                store_columns<NC>(w1, 8 * j + g, cg, v);
+            }
+        };
+        if constexpr (HW == 2) {   // the first warp adds the second's part
+            if (hm) store_y();
+            __syncthreads();
+            if (!hm) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    u64 o[NC];
+                    load_columns<NC>(w1 + 2 * kFieldWords, 8 * j + g, cg, o);
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        const float2 v = unpack2(o[c]);
+                        y[2 * j][c] += v.x;
+                        y[2 * j + 1][c] += v.y;
+                    }
+                }
+            }
         }
+        if (hm == 0) store_y();
         __syncthreads();
-        // A thread reads here the words it wrote when staging, and writes them again for
-        // the next tile: no barrier is needed between.
+        // HW = 1: a thread reads here the words it wrote when staging, and writes them again for
+        // the next tile: no barrier is needed between.  HW = 2: staging writes other words.
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int p = (tid >> 4) + 8 * i, col = tid & (kCols - 1);
-            const float *o = base + slot(p >> 1, col >> 1) + 2 * (col & 1) + (p & 1);
-            const int t = A.rev ? t_last - t0 - 8 * i : t0 + 8 * i;
+        for (int i = 0; i < kPasses; ++i) {
+            const int p = tid / kCols + kPass * i, col = tid & (kCols - 1);
+            const float *o = base + (HW == 2 ? 2 * kFieldWords : 0) + T::at(p >> 1, col) + (p & 1);
+            const int t = A.rev ? t_last - t0 - kPass * i : t0 + kPass * i;
             if (t >= 0 && t < Li && frow < A.B)
                 store4(A.out, A.bf16, (fbase + t) * D + d0, make_float4(o[0], o[kWords], o[2 * kWords], o[3 * kWords]));
         }
@@ -838,7 +1000,7 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
 #pragma unroll
                 for (int j = 0; j < J; ++j) {
                     const int m = 8 * J * q + 8 * j + g;
-                    const int64_t o = (((int64_t)seg * A.B + b) * D + d) * M + m;
+                    const int64_t o = (((int64_t)seg * A.B + b) * D + d) * A.M + m;
                     if (m < M) {
                         A.seg_s[o] = S0[q][j];
                         if (BWD) A.seg_r[o] = R0[q][j];
@@ -850,34 +1012,56 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
     if (kX) {
         // The within-chunk terms: lane cg takes lags 16 cg .. 16 cg + 15 of its modes; the
         // sums over cg complete G, P and J.
-        const int h = lane >> 4;
+        const int h = lane / kCols, col = lane & (kCols - 1);
         __syncwarp();
-        kq[16 * h + (lane & 15)] = rho_a;
-        kq[16 * (3 - h) + (lane & 15)] = rho_b;
+        if (hm != HW - 1) {
+        } else if constexpr (NC == 4) {
+            kq[16 * h + col] = rho_a[0];
+            kq[16 * (3 - h) + col] = rho_b[0];
+        } else {
+            kq[lane] = kq[32 + lane] = 0.0f;
+#pragma unroll 1
+            for (int k = 0; k < 8; ++k) {   // the groups of a lag block one after the other
+                __syncwarp();
+                if (k != h) continue;
+                float *o = kq + 16 * (h < 4 ? 0 : h < 7 ? 1 : 3) + 4 * col, *o2 = kq + 32 + 4 * col;
+#pragma unroll
+                for (int i = 0; i < 4 / NC; ++i) {
+                    o[i] += rho_a[i];
+                    if (h < 2) o2[i] += rho_b[i];
+                }
+            }
+        }
+        if (HW == 2) __syncthreads();
         __syncwarp();
 #pragma unroll
-        for (int q = 0; q < NP; ++q)
+        for (int q = 0; q < NP; ++q) {
+            float2 gw[J], pn[J];
+#pragma unroll
+            for (int j = 0; j < J; ++j) gw[j] = pn[j] = make_float2(0.0f, 0.0f);
+#pragma unroll 2
+            for (int n = 16 * cg; n < 16 * cg + 16; ++n) {
+                const float r = kq[n], nr = (float)n * r;
+#pragma unroll
+                for (int j = 0; j < J; ++j) {
+                    const float2 z = pw[(8 * J * q + 8 * j + g) * kPwStride + (n & (kHalf - 1))];
+                    gw[j].x = fmaf(z.x, r, gw[j].x);
+                    gw[j].y = fmaf(z.y, r, gw[j].y);
+                    pn[j].x = fmaf(z.x, nr, pn[j].x);
+                    pn[j].y = fmaf(z.y, nr, pn[j].y);
+                }
+            }
 #pragma unroll
             for (int j = 0; j < J; ++j) {
                 const int m = 8 * J * q + 8 * j + g;
-                float2 gs = G[q][j], ps = P[q][j], js = Jg[q][j];
-                if (A.g && m < M) {
-                    // conj(g) J, g the lane's row's (Jg of a row that does not exist is zero).
-                    const float2 gg = A.g[(b * D + d) * M + m];
+                float2 js = Jg[q][j];
+                if (A.g && m < M && mine) {
+                    // conj(g) J, g the lane's row's.
+                    const float2 gg = A.g[bm0 + m];
                     js = cmul(make_float2(gg.x, -gg.y), js);
                 }
-                float2 gw = make_float2(0.0f, 0.0f), pn = gw;
-                for (int n = 16 * cg; n < 16 * cg + 16; ++n) {
-                    const float2 z = pw[m * kPwStride + (n & (kHalf - 1))];
-                    const float r = kq[n], nr = (float)n * r;
-                    gw.x = fmaf(z.x, r, gw.x);
-                    gw.y = fmaf(z.y, r, gw.y);
-                    pn.x = fmaf(z.x, nr, pn.x);
-                    pn.y = fmaf(z.y, nr, pn.y);
-                }
                 const float2 up = cg < 2 ? make_float2(1.0f, 0.0f) : pw[m * kPwStride + kHalf];
-                gs = cfma(up, gw, gs);
-                ps = cfma(up, pn, ps);
+                float2 gs = cfma(up, gw[j], G[q][j]), ps = cfma(up, pn[j], P[q][j]);
 #pragma unroll
                 for (int o = 8; o <= 16; o <<= 1) {
                     gs.x += __shfl_xor_sync(0xffffffffu, gs.x, o);
@@ -888,12 +1072,13 @@ __global__ void __launch_bounds__(kThreads, blocks_per_sm(8 * J * NP, BWD)) k_sc
                     js.y += __shfl_xor_sync(0xffffffffu, js.y, o);
                 }
                 if (cg == 0 && m < M) {
-                    const int64_t o = (((int64_t)blockIdx.z * A.nseg + seg) * D + d) * M + m;
+                    const int64_t o = (((int64_t)blockIdx.z * A.nseg + seg) * D + d) * A.M + kModes * hm + m;
                     A.part_g[o] = gs;
                     A.part_p[o] = ps;
                     if (A.g) A.part_j[o] = js;
                 }
             }
+        }
     }
 }
 
@@ -966,30 +1151,55 @@ __global__ void __launch_bounds__(256) k_grad_reduce(
 // are only taken when at least two of them fit.
 struct Geometry {
     int nch, ntiles, nseg, tps, gpr;
-    int zdim;   // blocks along the batch
+    int zdim;      // blocks along the batch
+    bool narrow;   // tiles of 4 chunks
 };
+
+// Whether narrow tiles (4 chunks) are faster than wide ones (16): estimated walks, in wide
+// tiles.  A narrow tile takes `tile` of a wide one's time, and from `share` blocks a SM on
+// blocks share the SM's time; fitted to 73 to 438 shapes a line (B = 1 to 64, L = 65 to 1025,
+// D = 64 to 2048).  Beyond 20 chunks wide tiles win, by their segments too.  Us a call in fp32,
+// wide and narrow: backward B = 1, L = 65, D = 64, M = 64 55 and 19; B = 1, L = 193, D = 256, M = 17
+// 28 and 16; forward from a state B = 1, L = 65, D = 256, M = 64 20 and 12; wide is taken for the
+// backward of B = 64, L = 193, D = 64, M = 16, 26 and 42.
+bool use_narrow(int64_t B, int nch, int D, int M, bool bwd) {
+    struct Cost {
+        double tile, share1, share4;
+    };
+    static const Cost kCost[2][4] = {{{0.55, 1.5, 1.25}, {0.5, 1.0, 1.0}, {0.6, 1.5, 1.25}, {0.5, 1.0, 1.0}},
+                                     {{0.6, 1.5, 1.25}, {0.65, 1.5, 1.25}, {0.4, 2.0, 1.5}, {0.3, 1.25, 1.25}}};
+    const Cost &c = kCost[bwd][M <= 8 ? 0 : M <= 16 ? 1 : M <= 32 ? 2 : 3];
+    auto walk = [&](int nc, double share) {
+        const int gpr = nch <= nc ? 1 : nch <= 2 * nc ? 2 : 4;
+        const double blocks = (double)((B * gpr + 3) / 4 * (D / kCh));
+        return ((nch + 4 * nc - 1) / (4 * nc)) * std::max(1.0, blocks / (share * sm_count()));
+    };
+    return nch == 1 || (nch <= 20 && c.tile * walk(1, c.share1) < walk(4, c.share4));
+}
 
 Geometry geometry(int64_t B, int64_t L, int D, int M, bool bwd, int max_seg) {
     Geometry q;
     q.nch = (int)((L + kC - 1) / kC);
-    q.ntiles = (q.nch + kCols - 1) / kCols;
-    const int64_t slots = (int64_t)sm_count() * blocks_per_sm(M, bwd);
+    q.narrow = use_narrow(B, q.nch, D, M, bwd);
+    const int nc = q.narrow ? 1 : 4;
+    q.ntiles = (q.nch + 4 * nc - 1) / (4 * nc);
+    const int64_t slots = (int64_t)sm_count() * blocks_per_sm(M, nc, bwd);
     const int64_t groups = B * (D / kCh);
-    q.nseg = (int)std::max<int64_t>(1, std::min<int64_t>({slots / groups, (int64_t)q.ntiles, (int64_t)max_seg}));
+    q.nseg = q.narrow ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>({slots / groups, (int64_t)q.ntiles, (int64_t)max_seg}));
     q.tps = (q.ntiles + q.nseg - 1) / q.nseg;
     q.nseg = (q.ntiles + q.tps - 1) / q.tps;
     // Packed rows cost a block nothing and divide their number by up to four: at B = 22,
     // L = 74, D = 88, M = 16 (fp32 backward with state terms) 484 blocks, just over one
     // wave, become 132: 63.6 -> 32.8 us.
-    q.gpr = q.nch <= 4 ? 1 : q.nch <= 8 ? 2 : 4;
+    q.gpr = q.nch <= nc ? 1 : q.nch <= 2 * nc ? 2 : 4;
     q.zdim = (int)((B * q.gpr + 3) / 4);
     return q;
 }
 
-template <int J, int NP, bool BWD, bool kOut>
+template <int NC, int J, int NP, int HW, bool BWD, bool kOut>
 cudaError_t launch_scan(const ScanArgs &a, int nseg, int zdim, cudaStream_t st) {
-    constexpr int bytes = smem_bytes(8 * J * NP, kOut);
-    auto *k = k_scan<J, NP, BWD, kOut>;
+    constexpr int bytes = smem_bytes(8 * J * NP * HW, NC, HW, kOut);
+    auto *k = k_scan<NC, J, NP, HW, BWD, kOut>;
     if (bytes > 48 * 1024) {
         // Once per device (a bit each; devices past 64 set it on every call).
         static std::atomic<unsigned long long> done{0};
@@ -1005,26 +1215,29 @@ cudaError_t launch_scan(const ScanArgs &a, int nseg, int zdim, cudaStream_t st) 
     }
     const dim3 grid((unsigned)(a.D / kCh), (unsigned)nseg, (unsigned)zdim);
     count_launches(1);
-    if (kOut && a.nseg > 1) return launch_dependent(k, grid, kThreads, bytes, st, a);
-    k<<<grid, kThreads, bytes, st>>>(a);
+    if (kOut && a.nseg > 1) return launch_dependent(k, grid, HW * kThreads, bytes, st, a);
+    k<<<grid, HW * kThreads, bytes, st>>>(a);
     return cudaGetLastError();
 }
 
+template <int NC, bool BWD, bool kOut>
+cudaError_t pass_scan(const ScanArgs &a, int nseg, int zdim, cudaStream_t st) {
+    if (a.M <= 8) return launch_scan<NC, 1, 1, 1, BWD, kOut>(a, nseg, zdim, st);
+    if (a.M <= 16) return launch_scan<NC, 2, 1, 1, BWD, kOut>(a, nseg, zdim, st);
+    if (a.M <= 32) return launch_scan<NC, 4, 1, 1, BWD, kOut>(a, nseg, zdim, st);
+    if constexpr (NC == 1) return launch_scan<1, 4, 1, 2, BWD, kOut>(a, nseg, zdim, st);
+    else return launch_scan<NC, 4, 2, 1, BWD, kOut>(a, nseg, zdim, st);
+}
+
 template <bool BWD>
-cudaError_t run_scan(ScanArgs &a, int zdim, cudaStream_t st) {
-    auto pass = [&](auto out, int nseg) {
-        constexpr bool kOut = decltype(out)::value;
-        if (a.M <= 8) return launch_scan<1, 1, BWD, kOut>(a, nseg, zdim, st);
-        if (a.M <= 16) return launch_scan<2, 1, BWD, kOut>(a, nseg, zdim, st);
-        if (a.M <= 32) return launch_scan<4, 1, BWD, kOut>(a, nseg, zdim, st);
-        return launch_scan<4, 2, BWD, kOut>(a, nseg, zdim, st);
-    };
+cudaError_t run_scan(ScanArgs &a, const Geometry &q, cudaStream_t st) {
+    if (q.narrow) return pass_scan<1, BWD, true>(a, 1, q.zdim, st);
     if (a.nseg > 1) {
-        const cudaError_t e = pass(std::false_type{}, a.nseg - 1);
+        const cudaError_t e = pass_scan<4, BWD, false>(a, a.nseg - 1, q.zdim, st);
         if (e != cudaSuccess) return e;
         if (!BWD && a.enter) a.enter = a.seg_s + (int64_t)(a.nseg - 1) * a.B * a.D * a.M;
     }
-    return pass(std::true_type{}, a.nseg);
+    return pass_scan<4, BWD, true>(a, a.nseg, q.zdim, st);
 }
 
 }  // namespace
@@ -1065,6 +1278,8 @@ cudaError_t simt_prefill(const void *x, void *y, rlm_dtype dt, int64_t B, int64_
                          int M, const float *decay, const float *freq, const float *amp,
                          const float *phase, const float *state_in, float *state_out, float *coef_out,
                          void *ws, cudaStream_t st) {
+    if (short_supported(L))
+        return short_prefill(x, y, dt, B, L, D, M, decay, freq, amp, phase, state_in, state_out, coef_out, st);
     const Geometry q = geometry(B, L, D, M, false, 1 << 15);
     ScanArgs a = {};
     a.u = x;
@@ -1087,7 +1302,7 @@ cudaError_t simt_prefill(const void *x, void *y, rlm_dtype dt, int64_t B, int64_
     a.enter = reinterpret_cast<const float2 *>(state_in);
     a.state_out = reinterpret_cast<float2 *>(state_out);
     a.coef_out = reinterpret_cast<float4 *>(coef_out);
-    return run_scan<false>(a, q.zdim, st);
+    return run_scan<false>(a, q, st);
 }
 
 cudaError_t grad_reduce(int64_t nparts, int D, int M, const float *amp, const float *phase,
@@ -1103,6 +1318,14 @@ cudaError_t simt_backward(const void *dy, const void *x, void *dx, rlm_dtype dt,
                           const float *amp, const float *phase, const float *state_in,
                           const float *d_state_out, float *d_state_in, float *g_decay,
                           float *g_freq, float *g_amp, float *g_phase, void *ws, cudaStream_t st) {
+    if (short_supported(L)) {
+        const int64_t n = B * D * M;   // the contract holds three units a row
+        float2 *pg = static_cast<float2 *>(ws), *pp = pg + n, *pj = pp + n;
+        const cudaError_t e = short_backward(dy, x, dx, dt, B, L, D, M, decay, freq, amp, phase, state_in, d_state_out,
+                                             d_state_in, pg, pp, pj, st);
+        if (e != cudaSuccess) return e;
+        return grad_reduce(B, D, M, amp, phase, pg, pp, d_state_out ? pj : nullptr, g_decay, g_freq, g_amp, g_phase, st);
+    }
     // A segment needs five workspace units (its pair, and its G, P and J partials)
     // where the contract states three a chunk; one segment keeps no pair.
     const Geometry q = geometry(B, L, D, M, true, std::max(1, 3 * bwd_ws_chunks(B, L, D) / 5));
@@ -1134,7 +1357,7 @@ cudaError_t simt_backward(const void *dy, const void *x, void *dx, rlm_dtype dt,
     a.state_in = reinterpret_cast<const float2 *>(state_in);
     a.g = reinterpret_cast<const float2 *>(d_state_out);
     a.d_state_in = reinterpret_cast<float2 *>(d_state_in);
-    const cudaError_t e = run_scan<true>(a, q.zdim, st);
+    const cudaError_t e = run_scan<true>(a, q, st);
     if (e != cudaSuccess) return e;
     return grad_reduce((int64_t)q.zdim * q.nseg, D, M, amp, phase, a.part_g, a.part_p, d_state_out ? a.part_j : nullptr, g_decay,
                        g_freq, g_amp, g_phase, st);
