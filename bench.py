@@ -815,7 +815,7 @@ def run_kernels_only(args):
       fp32_prefill        B=4 L=32768 D=256 M=16 fp32: k_prefill_tc32
       fp32_prefill_state  the same with an initial state: k_prefill_tc32
       fp32_prefill_state_ragged  B=4 L=32767 with an initial state (the SIMT chunked scan):
-                          k_chunk_local, k_chunk_carry, k_chunk_output
+                          k_scan
       decode_b64 / b1     one plain decode step: k_decode_tile
       mixer_decode_plain  mixer step without coupling, B=64 D=2048 K=4 (rows past the
                           one-block step): k_decode_tile (mixer)

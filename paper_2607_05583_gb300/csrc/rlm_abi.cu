@@ -137,11 +137,6 @@ rlm_status check_workspace(const rlm_launch *ln, size_t need) {
     return RLM_OK;
 }
 
-int simt_chunks(int64_t B, int64_t L, int D) {
-    const int C = simt_chunk_len(B, L, D);
-    return (int)((L + C - 1) / C);
-}
-
 // The complex [B][D][M] buffer of an optional state argument (only ->s is used).
 rlm_status check_state_s(const rlm_state *st, int64_t B, int64_t D, int M, const char *name) {
     if (!st) return RLM_OK;
@@ -317,8 +312,6 @@ rlm_status rlm_mix_prefill_from(const rlm_tensor *x, const rlm_params *p, const 
     if ((s = check_params(p, x->D)) != RLM_OK) return s;
     if ((s = check_prefill_states(x, y, p, state_in, state_out)) != RLM_OK) return s;
     const PrefillPath path = prefill_path(x, p->M, state_in != nullptr);
-    if (path == PrefillPath::kSimt && simt_chunks(x->B, x->L, (int)x->D) > 65535)
-        return fail(RLM_ERR_UNSUPPORTED, "sequence too long for the chunk grid");
     const size_t need = rlm_prefill_workspace_size(x->B, x->L, (int)x->D, p->M, x->dtype);
     if ((s = check_workspace(ln, need)) != RLM_OK) return s;
     cudaError_t e = launch_prefill(path, x, p, state_in ? state_in->s : nullptr, y->ptr,
@@ -362,8 +355,6 @@ rlm_status rlm_mixer_prefill(const rlm_tensor *x, const rlm_tensor *g, const rlm
             return fail(RLM_ERR_INVALID_ARG, "conv_in and conv_out overlap without being the same buffer");
     }
     const PrefillPath path = prefill_path(x, p->M, state_in != nullptr);
-    if (path == PrefillPath::kSimt && simt_chunks(x->B, x->L, (int)x->D) > 65535)
-        return fail(RLM_ERR_UNSUPPORTED, "sequence too long for the chunk grid");
     const size_t need = rlm_prefill_workspace_size(x->B, x->L, (int)x->D, p->M, x->dtype);
     if ((s = check_workspace(ln, need)) != RLM_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(ln->stream);
@@ -464,8 +455,8 @@ rlm_status rlm_mixer_decode(const rlm_tensor *x_t, const rlm_tensor *g_t, rlm_st
     }
     cudaStream_t st = static_cast<cudaStream_t>(ln->stream);
     cudaError_t e;
-    // One block per batch row serves the coupled step; the uncoupled step runs on
-    // the row-tiled decode kernel.
+    // The coupled step has a kernel of its own (one to eight blocks per batch row); the
+    // uncoupled step runs on the row-tiled decode kernel.
     const bool row_block = coupling != nullptr;
     if (row_block && mixer_decode_coupled_supported((int)x_t->D, state->M)) {
         // One launch: recurrence step, coupling (if any), gate, local path.
@@ -548,8 +539,6 @@ rlm_status rlm_mix_backward_from(const rlm_tensor *dy, const rlm_tensor *x, cons
     float *dsin = d_state_in ? d_state_in->s : nullptr;
     const int D = (int)x->D, M = p->M;
     const bool tc = tc_backward_supported(x->B, x->L, D, M, x->dtype);
-    if (!tc && simt_chunks(x->B, x->L, D) > 65535)
-        return fail(RLM_ERR_UNSUPPORTED, "sequence too long for the chunk grid");
     const size_t need = rlm_backward_workspace_size(x->B, x->L, D, M, x->dtype);
     if ((s = check_workspace(ln, need)) != RLM_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(ln->stream);

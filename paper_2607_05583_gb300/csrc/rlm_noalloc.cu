@@ -119,8 +119,9 @@ extern "C" rlm_status rlm_mix_prefill_noalloc(const rlm_tensor *x, const rlm_par
                           sdev, dev);
     }
     const int D = (int)x->D, M = p->M;
+    // Sequences of more than 65535 of the chunks that the scratch is counted in are refused.
     const int C = simt_chunk_len(x->B, x->L, D);
-    if ((x->L + C - 1) / C > 65535) return reject(RLM_ERR_UNSUPPORTED, "sequence too long for the chunk grid");
+    if ((x->L + C - 1) / C > 65535) return reject(RLM_ERR_UNSUPPORTED, "sequence of more than 65535 chunks");
     const size_t need = simt_prefill_ws_bytes(x->B, x->L, D, M);
     if (need > kNoAllocScratchBytes)
         return reject(RLM_ERR_UNSUPPORTED,

@@ -48,7 +48,7 @@
 // What bounds it: shared-load wavefronts (four a 16-byte load of a warp: at M = 32 about 1900 a
 // warp and tile forward, against 1350 cycles of FMA) at 40-50 % of their rate, since two
 // warps a scheduler (tables and accumulators allow no more at M = 32) do not hide the loads'
-// latency.  GB300, us per call, against the three launches of token-by-token recurrences with
+// latency.  The wide backward above 32 modes also spills: 255 registers, 0.4 KB a thread.  GB300, us per call, against the three launches of token-by-token recurrences with
 // chunk states in memory that this replaces:
 //
 //   fp32, B = 2, L = 4096, D = 512, M = 32: forward 247 -> 56, backward 303 -> 117
@@ -1082,10 +1082,9 @@ __global__ void __launch_bounds__(HW * kThreads, blocks_per_sm(8 * J * NP * HW, 
     }
 }
 
-// One thread per (d, m): fixed-order sum of the partials
-// over (b, k), then the four gradients.  The sums are compensated (Kahan) fp32
-// sums, so the result is reproducible and its error stays near one rounding
-// however many partials are added; the combination with
+// One thread per (d, m): fixed-order sum of its n partials, then the four gradients.  The
+// sums are compensated (Kahan) fp32 sums, so the result is reproducible and its error stays
+// near one rounding however many partials are added; the combination with
 // c = A e^{i phi} (formed as the forward forms it, fp32 sincosf) uses fmaf for
 // the differences.  Double precision made this launch 3-4x slower on this part
 // (low FP64 rate): 4.8 against 1.4 us at D = 512, M = 32, four partials.
@@ -1101,7 +1100,7 @@ struct KahanSum {
     }
 };
 __global__ void __launch_bounds__(256) k_grad_reduce(
-    int64_t B, int D, int M, int nch, const float *__restrict__ amp,
+    int64_t n, int D, int M, const float *__restrict__ amp,
     const float *__restrict__ phase, const float2 *ws_s, const float2 *ws_r, const float2 *ws_j, float *__restrict__ g_decay,
     float *__restrict__ g_freq, float *__restrict__ g_amp, float *__restrict__ g_phase) {
     const int pm = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1109,7 +1108,7 @@ __global__ void __launch_bounds__(256) k_grad_reduce(
     if (pm >= D * M) return;
     const float am = amp[pm], ph = phase[pm];
     KahanSum gr, gi, pr, pi, jr, ji;
-    const int64_t n = B * nch, stride = (int64_t)D * M;
+    const int64_t stride = (int64_t)D * M;
     // Four partials' loads in flight before their adds (the sum order is fixed).
     for (int64_t bk0 = 0; bk0 < n; bk0 += 4) {
         float2 g[4], p[4], j[4];
@@ -1309,7 +1308,7 @@ cudaError_t grad_reduce(int64_t nparts, int D, int M, const float *amp, const fl
                         const float2 *G, const float2 *P, const float2 *J, float *g_decay, float *g_freq,
                         float *g_amp, float *g_phase, cudaStream_t st) {
     count_launches(1);
-    return launch_dependent(k_grad_reduce, dim3((unsigned)((D * M + 255) / 256)), 256, 0, st, nparts, D, M, 1, amp, phase,
+    return launch_dependent(k_grad_reduce, dim3((unsigned)((D * M + 255) / 256)), 256, 0, st, nparts, D, M, amp, phase,
                             G, P, J, g_decay, g_freq, g_amp, g_phase);
 }
 
