@@ -69,8 +69,8 @@
 // k_grad_reduce.  Both leave TMEM while the next row's first tile is projected and
 // scanned; Q moves to warp 9, whose next products overwrite them.  (Summed over up to 16
 // tiles in TMEM the error of dA against 64 bits at B = 8, L = 4096, D = 256, M = 16 was 2.68e-6
-// against 2.59e-6, mean of 8 seeds; now 2.59e-6.  That took 51 us a call where this takes 70 and one
-// row a CTA 90; 85, 104 and 145 with both state terms.  Q and E issued by warp 7 instead:
+// against 2.59e-6, mean of 8 seeds; now 2.59e-6.  That took 51 us a call where this takes 68 and one
+// row a CTA 90; 85, 105 and 145 with both state terms.  Q and E issued by warp 7 instead:
 // as fast for several rows, 20 us slower for one of 16 tiles.)
 //
 // Every wait is bounded: after kWaitLimitCycles the waiting thread sets a shared
@@ -138,9 +138,11 @@ constexpr int kOffBs = kOffRing + kSlots * kSlotBytes;   // [2] x (hi 8 KB, lo 8
 constexpr int kBsBuf = 16384;
 // rho[n] of a row, double-buffered: the part of each epilogue warp's 32 rows of Q.
 constexpr int kOffRho = kOffBs + 2 * kBsBuf;             // [2][2][64] fp32
-constexpr int kQsStride = 17;                            // 16 columns of Q staged per warp, one word of padding
-constexpr int kOffQs = kOffRho + 2 * 2 * 64 * 4;         // [2 warps][32][17] fp32
-constexpr int kOffBar = kOffQs + 2 * 32 * kQsStride * 4;
+// 16 columns of an epilogue warp's 32 rows of Q, row i - c of element (i, c): every row is a
+// diagonal.  Cells that no element meets stay zero.
+constexpr int kQsRows = 47, kQsStride = 18;
+constexpr int kOffQs = kOffRho + 2 * 2 * 64 * 4;         // [2 warps][47][18] fp32
+constexpr int kOffBar = kOffQs + 2 * kQsRows * kQsStride * 4;
 constexpr int kNumBars = 32;
 constexpr int kOffMisc = kOffBar + kNumBars * 8;
 constexpr int kSmemBytes = kOffMisc + 64 + 1024;         // + alignment slack
@@ -333,8 +335,8 @@ __device__ __forceinline__ void store_pair_row(uint32_t buf, int r, int g, const
 // channels from 0 on, the next ones r[1] rows of channels from ch[1] on, and so on, fewer
 // rows each, so that the large units start first and small ones fill the tail.  Same box,
 // one row per block and now, us: B = 8, L = 4096, D = 256, M = 16 with both state terms (this
-// kernel and k_terminal_tc) 145 -> 104; B = 7, L = 465, D = 160, M = 32 45 -> 36; B = 64, L = 200,
-// D = 512, M = 16 1012 -> 481.
+// kernel and k_terminal_tc) 145 -> 105; B = 7, L = 465, D = 160, M = 32 45 -> 36; B = 64, L = 200,
+// D = 512, M = 16 1012 -> 470.
 struct RowPlan {
     int r[3];       // rows per block of the level
     int end[3];     // one past the level's last block
@@ -459,6 +461,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     float2 *pw = reinterpret_cast<float2 *>(smem + kOffPw);
     float2 *cf = reinterpret_cast<float2 *>(smem + kOffCf);
     float *kt = reinterpret_cast<float *>(smem + kOffK);
+    if (kGrad)
+        for (int i = bt; i < 2 * kQsRows * kQsStride; i += kBuilders) reinterpret_cast<float *>(smem + kOffQs)[i] = 0.0f;
     static_assert(kMaxModes * 9 == kBuilders, "one builder per mode and group of powers");
     {
         const int m = bt / 9, g = bt % 9;
@@ -809,15 +813,17 @@ __global__ void __launch_bounds__(kThreads, 2)
                 out[(k + 16) * kC] = __float2bfloat16_rn(__uint_as_float(r1[k]));
             }
             if (--tile >= 0 || !kGrad) continue;
-            // The row's end: diagonal sums of Q over the row,
-            // rho[n] = sum_k Q[n+k][k].  Each warp takes its 32 rows, 16 columns at a time
-            // through its own staging buffer (row stride 17 words: the row writes and the
-            // diagonal reads each hit 32 banks), lane l the diagonals n = l and, in the lower
-            // rows, l + 32; the readers add the two warps' parts.
-            float *qs = reinterpret_cast<float *>(smem + kOffQs) + q * 32 * kQsStride;
+            // The row's end: diagonal sums of Q over the row, rho[n] = sum_k Q[n+k][k].  Each warp
+            // takes its 32 rows, 16 columns at a time, through its own staging buffer, where a row
+            // holds a diagonal's cells (row stride 18 words: the 8-byte reads hit 32 banks), and
+            // adds them into its part of rho; the readers add the two warps' parts.  (Rows kept as
+            // rows, with a range check a cell: B = 8, L = 4096, D = 256, M = 16 69.7 us against 68.1.)
+            float *qs = reinterpret_cast<float *>(smem + kOffQs) + q * kQsRows * kQsStride;
+            float *rho = reinterpret_cast<float *>(smem + kOffRho) + (r & 1) * 128 + q * 64;
             if (!wait_bar_warp(bar(kBarRowFull), r & 1, abort_flag)) break;
             tc_fence_after();
-            float d0[4] = {0.0f, 0.0f, 0.0f, 0.0f}, d1[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            if (kRows && !wait_bar_warp(bar(kBarRhoEmpty + (r & 1)), ((r >> 1) & 1) ^ 1, abort_flag)) break;
+            rho[lane] = rho[lane + 32] = 0.0f;
 #pragma unroll 1
             for (int h = 0; h < 2 + 2 * q; ++h) {
                 uint32_t qv[16];
@@ -829,21 +835,25 @@ __global__ void __launch_bounds__(kThreads, 2)
                     if (lane == 0) bar_arrive(bar(kBarRowFree));
                 }
 #pragma unroll
-                for (int e = 0; e < 16; ++e) qs[lane * kQsStride + e] = __uint_as_float(qv[e]);
+                for (int e = 0; e < 16; ++e) qs[(lane - e + 15) * kQsStride + e] = __uint_as_float(qv[e]);
                 __syncwarp();
-                // Column 16 h + e meets diagonal n in row n + 16 h + e, this warp's row w0 + e (+ 32).
-                const int w0 = lane + 16 * h - 32 * q;
+                // Element (32 q + i, 16 h + e) went to row i - e + 15: row k is diagonal k + at.
+                const int at = 32 * q - 16 * h - 15;
+                auto add = [&](int k) {
+                    if (k >= kQsRows || k + at < 0) return;
+                    float a = 0.0f, b = 0.0f;
 #pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    if ((unsigned)(w0 + e) < 32u) d0[e & 3] += qs[(w0 + e) * kQsStride + e];
-                    if ((unsigned)(w0 + 32 + e) < 32u) d1[e & 3] += qs[(w0 + 32 + e) * kQsStride + e];
-                }
+                    for (int e = 0; e < 16; e += 2) {
+                        const float2 v = *reinterpret_cast<const float2 *>(qs + k * kQsStride + e);
+                        a += v.x;
+                        b += v.y;
+                    }
+                    rho[k + at] += a + b;
+                };
+                add(lane);
+                add(lane + 32);
                 __syncwarp();
             }
-            if (kRows && !wait_bar_warp(bar(kBarRhoEmpty + (r & 1)), ((r >> 1) & 1) ^ 1, abort_flag)) break;
-            float *rho = reinterpret_cast<float *>(smem + kOffRho) + (r & 1) * 128 + q * 64;
-            rho[lane] = (d0[0] + d0[1]) + (d0[2] + d0[3]);
-            rho[lane + 32] = (d1[0] + d1[1]) + (d1[2] + d1[3]);
             __syncwarp();
             if (lane == 0) bar_arrive(bar(kBarRhoFull + (r & 1)));
             ++r;
