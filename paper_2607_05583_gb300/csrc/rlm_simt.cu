@@ -472,9 +472,11 @@ __global__ void __launch_bounds__(HW * kThreads, blocks_per_sm(8 * J * NP * HW, 
     const int64_t b = min((int)blockIdx.z * rpt + cg / A.gpr, A.B - 1);
     const int nrows = min(rpt, A.B - (int)blockIdx.z * rpt);   // rows that exist
     const int d0 = kCh * blockIdx.x, d = d0 + w, D = A.D;
-    const int M = HW == 2 ? min(kModes, A.M - kModes * hm) : A.M;   // the warp's modes, from these on:
-    const int pm0 = d * A.M + kModes * hm;
-    const int64_t bm0 = (b * D + d) * A.M + kModes * hm;
+    const int M = HW == 2 ? min(kModes, A.M - kModes * hm) : A.M;   // the warp's modes, its m-th at pm(m), bm(m)
+    // (Formed where they are used: kept in registers they cost the fp32 training step at B = 2,
+    // L = 4096, D = 512, M = 32 four of 175 us.)
+    auto pm = [&](int m) { return d * A.M + kModes * hm + m; };
+    auto bm = [&](int m) { return (b * D + d) * A.M + kModes * hm + m; };
     constexpr int kWords = chan_words(HW * kModes, NC, HW, kOut), kTable = 2 * kModes * (kPwStride + 1);
     constexpr int kTableWords = HW * kTable + kKernWords;   // before the field tiles
     float2 *pw = reinterpret_cast<float2 *>(smem + w * kWords + hm * kTable);
@@ -532,8 +534,8 @@ __global__ void __launch_bounds__(HW * kThreads, blocks_per_sm(8 * J * NP * HW, 
         for (int m = lane / kLpm; m < kModes; m += 32) {
             float2 *row = pw + m * kPwStride;
             const bool on = m < M;
-            const float ga = on ? A.decay[pm0 + m] : 0.0f, om = on ? A.freq[pm0 + m] : 0.0f;
-            const float am = kOut && on ? A.amp[pm0 + m] : 0.0f, ph = kOut && on ? A.phase[pm0 + m] : 0.0f;
+            const float ga = on ? A.decay[pm(m)] : 0.0f, om = on ? A.freq[pm(m)] : 0.0f;
+            const float am = kOut && on ? A.amp[pm(m)] : 0.0f, ph = kOut && on ? A.phase[pm(m)] : 0.0f;
             if (!BWD && A.enter && on)   // used after the tables
                 prefetch_l2(A.enter + ((int64_t)min((int)blockIdx.z * rpt, A.B - 1) * D + d) * A.M + kModes * hm + m);
             const float2 l1 = lambda_pow(ga, om, 1.0f);
@@ -563,9 +565,9 @@ __global__ void __launch_bounds__(HW * kThreads, blocks_per_sm(8 * J * NP * HW, 
         for (int j = 0; j < J; ++j) {
             const int m = 8 * J * q + 8 * j + g;
             const bool on = m < M;
-            const float ga = on ? A.decay[pm0 + m] : 0.0f, om = on ? A.freq[pm0 + m] : 0.0f;
+            const float ga = on ? A.decay[pm(m)] : 0.0f, om = on ? A.freq[pm(m)] : 0.0f;
             const float2 z = make_float2(0.0f, 0.0f);
-            const int64_t sm = bm0 + m;
+            const int64_t sm = bm(m);
             S0[q][j] = !BWD && A.enter && on && mine && seg == 0 ? A.enter[sm] : z;
             if (BWD) R0[q][j] = z;
             if (kOut && seg > 0 && on) {
@@ -585,7 +587,7 @@ __global__ void __launch_bounds__(HW * kThreads, blocks_per_sm(8 * J * NP * HW, 
             }
             if (!BWD && kOut && A.coef_out && blockIdx.z == 0 && seg == A.nseg - 1 && cg == 0 && on) {
                 const float2 l1 = pw[m * kPwStride + 1];   // the exact lambda times lambda^0 = 1
-                A.coef_out[pm0 + m] = make_float4(l1.x, l1.y, cs[m].x, cs[m].y);
+                A.coef_out[pm(m)] = make_float4(l1.x, l1.y, cs[m].x, cs[m].y);
             }
             // The output launch's segment 0 starts from this copy: by then a state_out that
             // is state_in's buffer may be written by the last segment's block.
@@ -740,11 +742,11 @@ __global__ void __launch_bounds__(HW * kThreads, blocks_per_sm(8 * J * NP * HW, 
                         S = cfma(a, S, unpack2(acc[j][c]));
                         if (chunk0 + c == A.nch - 1 && on && mine) {
                             // The chunk of token 0: (S, R) is the adjoint pair there.
-                            const int64_t sm = bm0 + m;
+                            const int64_t sm = bm(m);
                             const float2 l0 = cmul(lam, S);
                             const float2 gg = A.g ? A.g[sm] : make_float2(0.0f, 0.0f);
                             const float2 lL =
-                                A.g ? lambda_pow(A.decay[pm0 + m], A.freq[pm0 + m], (float)A.L) : gg;
+                                A.g ? lambda_pow(A.decay[pm(m)], A.freq[pm(m)], (float)A.L) : gg;
                             if (A.state_in) {
                                 const float2 si = A.state_in[sm];
                                 G[q][j] = cfma(si, l0, G[q][j]);
@@ -764,7 +766,7 @@ __global__ void __launch_bounds__(HW * kThreads, blocks_per_sm(8 * J * NP * HW, 
                             if (tail)
                                 send[j] = S;
                             else if (on && mine && A.state_out)
-                                A.state_out[bm0 + m] = next;
+                                A.state_out[bm(m)] = next;
                         }
                         S = next;
                     }
@@ -779,7 +781,7 @@ __global__ void __launch_bounds__(HW * kThreads, blocks_per_sm(8 * J * NP * HW, 
                     for (int j = 0; j < J; ++j) {
                         const int m = 8 * J * q + 8 * j + g;
                         if (cg == col / NC && m < M)
-                            A.state_out[bm0 + m] = cfma(power(pw + m * kPwStride, tail), send[j], f[j]);
+                            A.state_out[bm(m)] = cfma(power(pw + m * kPwStride, tail), send[j], f[j]);
                     }
                 }
             if (kX && !single) {
@@ -796,7 +798,7 @@ __global__ void __launch_bounds__(HW * kThreads, blocks_per_sm(8 * J * NP * HW, 
                     }
                     if (A.g && m < M) {
                         // J over the whole chunks: L - 1 - t = E + p with E = L minus the chunk's end.
-                        const float ga = A.decay[pm0 + m], om = A.freq[pm0 + m];
+                        const float ga = A.decay[pm(m)], om = A.freq[pm(m)];
                         float2 z = make_float2(0.0f, 0.0f);
 #pragma unroll
                         for (int c = 0; c < NC; ++c) {
@@ -897,8 +899,8 @@ __global__ void __launch_bounds__(HW * kThreads, blocks_per_sm(8 * J * NP * HW, 
                 if (kX && A.g && m < M) {
                     // Terminal-state gradient: its adjoint conj(g) lambda^(L-1-t) enters a
                     // whole chunk as conj(g) lambda^E with E = L minus the chunk's end.
-                    const float ga = A.decay[pm0 + m], om = A.freq[pm0 + m];
-                    const float2 gg = A.g[bm0 + m];
+                    const float ga = A.decay[pm(m)], om = A.freq[pm(m)];
+                    const float2 gg = A.g[bm(m)];
                     float2 z = make_float2(0.0f, 0.0f);
 #pragma unroll
                     for (int c = 0; c < NC; ++c) {
@@ -937,11 +939,11 @@ __global__ void __launch_bounds__(HW * kThreads, blocks_per_sm(8 * J * NP * HW, 
             float2 *gs = reinterpret_cast<float2 *>(w1);   // [mode][row]
             if constexpr (NC == 1) {
                 __syncwarp();
-                for (int m = g; m < M && chunk0 == 0; m += 8) gs[m * 4 + cg] = A.g[bm0 + m];
+                for (int m = g; m < M && chunk0 == 0; m += 8) gs[m * 4 + cg] = A.g[bm(m)];
                 __syncwarp();
             }
             for (int m = 0; m < M && chunk0 == 0; ++m) {
-                const float2 gg = NC == 1 ? gs[m * 4 + cg] : A.g[bm0 + m];
+                const float2 gg = NC == 1 ? gs[m * 4 + cg] : A.g[bm(m)];
 #pragma unroll
                 for (int r = 0; r < 8; ++r) {
                     const int n = 16 * (r >> 1) + 2 * g + (r & 1) - (kC - tail);
@@ -1057,7 +1059,7 @@ __global__ void __launch_bounds__(HW * kThreads, blocks_per_sm(8 * J * NP * HW, 
                 float2 js = Jg[q][j];
                 if (A.g && m < M && mine) {
                     // conj(g) J, g the lane's row's.
-                    const float2 gg = A.g[bm0 + m];
+                    const float2 gg = A.g[bm(m)];
                     js = cmul(make_float2(gg.x, -gg.y), js);
                 }
                 const float2 up = cg < 2 ? make_float2(1.0f, 0.0f) : pw[m * kPwStride + kHalf];
