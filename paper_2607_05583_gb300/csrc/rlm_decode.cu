@@ -273,7 +273,8 @@ cudaError_t launch_pdl(Kern kern, dim3 grid, cudaStream_t st, Args... args) {
 // the local path, shifts the history and writes z_t.  C is built after the wait as well,
 // behind these loads: the kernel before may have written the coupling matrix.  (Built before
 // the wait, from data that wait does not cover, a step took, us: B = 64, D = 256, M = 16, H = 8 2.69,
-// now 2.70; B = 128 3.01, 3.08; B = 4, H = 32 3.0, 3.6; B = 16, D = 128, M = 32, H = 64 5.3, 7.0.)
+// now 2.68; B = 1 1.99, 2.05; B = 128 3.01, 3.08; B = 4, H = 32 3.0, 3.4; B = 16, D = 128, M = 32,
+// H = 64 5.3, 6.6.)
 constexpr int kCoupledBlock = 512;             // one block per row
 constexpr int kSplitBlock = 256;               // several blocks per row
 constexpr int kCoupledMaxModesPerRow = 8 * kCoupledBlock;   // D * M <= 4096
@@ -343,7 +344,7 @@ __global__ void __launch_bounds__(kBlock, kBlock == kCoupledBlock ? 1 : kIters =
             c1v[k] = coef[(int64_t)d * M + 2 * g + 1];
         }
     }
-    finish_coupling(C, c_raw, lam, H);
+    finish_coupling<kWhole>(C, c_raw, lam, H);
     // ---- phase 1: every thread runs every iteration, so whole warps shuffle
 #pragma unroll
     for (int k = 0; k < kIters; ++k) {
